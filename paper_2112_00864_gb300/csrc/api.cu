@@ -4,10 +4,12 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <array>
 #include <chrono>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <map>
 #include <string>
 #include <vector>
 
@@ -114,11 +116,13 @@ struct bcfmm_ctx {
   double* dens[3] = {nullptr, nullptr, nullptr};
   int* err = nullptr;                  // device error word (bounded device waits)
   size_t tc_partial_per_dens = 0;      // largest tensor-core partial-sum need over the tasks (float2)
-  // Taylor-form M2L (BCFMM_FP32): offset coefficients, prescaled moments,
-  // chunk partial sums (largest need over the tasks, floats per density)
+  // Taylor-form M2L (BCFMM_FP32 and BCFMM_FP64): offset coefficients,
+  // prescaled moments, chunk partial sums (largest need over the tasks,
+  // values per density)
   TaylorTables ty{};
-  float* ty_momp = nullptr;
-  float* ty_partial = nullptr;
+  TaylorOffsets ty_offs;               // parent offsets of the tasks' schedules (build only)
+  void* ty_momp = nullptr;             // FP32, or FP64 in a plain FP64 context
+  void* ty_partial = nullptr;
   size_t ty_partial_per_dens = 0;
   float2* tc_partial = nullptr;        // unit partial sums of the tensor-core M2L
   uint8_t* tc_momb = nullptr;          // BF16 split moments of the tensor-core M2L
@@ -385,25 +389,20 @@ static int upload_task(bcfmm_ctx* C, const HostSetup& H, int t) {
     }
     C->tc_partial_per_dens = std::max(C->tc_partial_per_dens, D.tcs.partial_per_dens);
   }
-  // Taylor-form M2L: per order, the interaction lists cut into chunks and
-  // interleaved per warp; targets of orders above the kernel's range go to
-  // the generic kernel
+  // Taylor-form M2L: per order, the sibling groups' entries cut into chunks;
+  // targets of orders above the kernel's range go to the wide kernel (FP32)
+  // or the dense one (FP64)
   for (size_t k = 0; k < T.m2l_tgt.size(); ++k)
     D.m2l_pairs_q[level_order(C->prm, H.box[T.m2l_tgt[k]].level)] += T.vl_off[k + 1] - T.vl_off[k];
-  if (C->ty.g && !T.m2l_tgt.empty()) {
+  if (C->ty.q > 0 && !T.m2l_tgt.empty()) {
     int nsm = 152;
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, C->device);
     std::vector<int> tq(T.m2l_tgt.size()), sel;
     for (size_t k = 0; k < tq.size(); ++k) tq[k] = level_order(C->prm, H.box[T.m2l_tgt[k]].level);
     std::vector<TaylorOrderHost> sched;
     D.tys = TaylorTaskSched();
-    if (!m2l_taylor_schedule(T.m2l_tgt, T.vl_off, T.vl_src, T.vl_code, tq, C->nbox, C->ncode, nsm, sched, sel,
-                             &D.tys.cbits)) {
-      // indices too large for the packed lists: every target on the generic kernel
-      sched.clear();
-      sel.resize(T.m2l_tgt.size());
-      for (size_t k = 0; k < sel.size(); ++k) sel[k] = (int)k;
-    }
+    const bool f64 = C->prm.precision == BCFMM_FP64;
+    m2l_taylor_schedule(H, t, tq, nsm, C->ty_offs, sched, sel);
     for (const TaylorOrderHost& O : sched) {
       TaylorOrderSched& S = D.tys.ord[O.q];
       S.q = O.q;
@@ -412,16 +411,16 @@ static int upload_task(bcfmm_ctx* C, const HostSetup& H, int t) {
       S.ntgt = (int)O.tgt.size();
       S.chunk = O.chunk;
       S.pairs = O.pairs;
-      int2* dwb;
-      int *dlc, *dtg, *dtc;
-      uint32_t* dpk;
+      int4 *dwb, *den;
+      int *dws, *dtg, *dtc;
       CU(m.upload(&dwb, O.wb.data(), O.wb.size(), st));
-      CU(m.upload(&dlc, O.lane_chunk.data(), O.lane_chunk.size(), st));
-      CU(m.upload(&dpk, O.pk.data(), O.pk.size(), st));
+      CU(m.upload(&dws, O.wslot.data(), O.wslot.size(), st));
+      CU(m.upload(&den, O.ent.data(), O.ent.size(), st));
       CU(m.upload(&dtg, O.tgt.data(), O.tgt.size(), st));
       CU(m.upload(&dtc, O.tchunk.data(), O.tchunk.size(), st));
-      S.wb = dwb; S.lane_chunk = dlc; S.pk = dpk; S.tgt = dtg; S.tchunk = dtc;
-      D.tys.partial_per_dens = std::max(D.tys.partial_per_dens, (size_t)O.nchunk * nterms_q(O.q));
+      S.wb = dwb; S.wslot = dws; S.ent = den; S.tgt = dtg; S.tchunk = dtc;
+      const int slot = f64 ? taylor_slot<double>(O.q) : taylor_slot<float>(O.q);
+      D.tys.partial_per_dens = std::max(D.tys.partial_per_dens, (size_t)O.nchunk * slot);
     }
     if (!sel.empty()) {
       int* dsel;
@@ -587,6 +586,26 @@ static int upload_task(bcfmm_ctx* C, const HostSetup& H, int t) {
     for (int k = 0; k < 5; ++k) D.p2p_src_q[k] = srcs[at[k]];
   }
   return BCFMM_OK;
+}
+
+// The Taylor form's offset coefficients: one table per order that occurs,
+// rows for every parent offset of the three tasks' schedules.
+template <typename T>
+static int upload_taylor_rows_t(bcfmm_ctx* C) {
+  for (int q = 1; q <= kTaylorMaxQ; ++q) {
+    bool used = false;
+    for (const TaskDev& D : C->task) used = used || D.tys.ord[q].nwarp > 0;
+    if (!used) continue;
+    std::vector<T> rows;
+    m2l_taylor_rows<T>(C->ty_offs, q, rows);
+    T* d;
+    CU(C->mem.upload(&d, rows.data(), rows.size(), C->st));
+    for (TaskDev& D : C->task) D.tys.ord[q].g = d;
+  }
+  return BCFMM_OK;
+}
+static int upload_taylor_rows(bcfmm_ctx* C) {
+  return C->prm.precision == BCFMM_FP64 ? upload_taylor_rows_t<double>(C) : upload_taylor_rows_t<float>(C);
 }
 
 // Blob of the learned correction: 8 uint32 (magic "BCML" little-endian,
@@ -846,20 +865,35 @@ static int build_impl(const double* verts, const int64_t* vert_off, const int32_
       return cleanup(fail(BCFMM_ERR_OOM, "build: device allocation failed (normals)"));
     G.tri_nrm = dn;
   }
-  // translation tables: M2L transposed per offset code
+  // translation tables
   {
     const int np = C->np;
     const int ncode = (int)(H.offsets.size() / 3);
     C->ncode = ncode;
-    std::vector<double> T((size_t)std::max(ncode, 1) * np * np, 0.0), Tt(T.size(), 0.0), tmp(np * np);
-    for (int code = 0; code < ncode; ++code) {
-      double od[3] = {(double)H.offsets[3 * code], (double)H.offsets[3 * code + 1], (double)H.offsets[3 * code + 2]};
-      m2l_matrix_scaled(prm.p, od, tmp.data());
-      for (int a = 0; a < np; ++a)
-        for (int b = 0; b < np; ++b) {
-          T[((size_t)code * np + a) * np + b] = tmp[a * np + b];
-          Tt[((size_t)code * np + b) * np + a] = tmp[a * np + b];
+    // the largest order of any level, and the dense M2L tables (transposed,
+    // per offset code) where a kernel reads them: the tensor-core form, the
+    // FP64 orders above the Taylor form's, and p = 0
+    int qt = 0;
+    for (int l = 0; l < C->nlevels; ++l) qt = std::max(qt, level_order(prm, l));
+    const bool dense = tc_mode || qt == 0 || (prm.precision == BCFMM_FP64 && qt > kTaylorMaxQ);
+    std::vector<double> T, Tt;
+    if (dense) {
+      T.assign((size_t)std::max(ncode, 1) * np * np, 0.0);
+      Tt.assign(T.size(), 0.0);
+#pragma omp parallel
+      {
+        std::vector<double> tmp(np * np);
+#pragma omp for schedule(static)
+        for (int code = 0; code < ncode; ++code) {
+          double od[3] = {(double)H.offsets[3 * code], (double)H.offsets[3 * code + 1], (double)H.offsets[3 * code + 2]};
+          m2l_matrix_scaled(prm.p, od, tmp.data());
+          for (int a = 0; a < np; ++a)
+            for (int b = 0; b < np; ++b) {
+              T[((size_t)code * np + a) * np + b] = tmp[a * np + b];
+              Tt[((size_t)code * np + b) * np + a] = tmp[a * np + b];
+            }
         }
+      }
     }
     // M2M and L2L run as three 1-D binomial shifts: their coefficients
     // C(n, k) (+-1/4)^(n-k), s = 0 for -1/4, s = 1 for +1/4
@@ -894,45 +928,59 @@ static int build_impl(const double* verts, const int64_t* vert_off, const int32_
         return cleanup(fail(BCFMM_ERR_CUDA, std::string("build: tensor tables: ") + cudaGetErrorString(ce)));
       }
     }
-    if (prm.precision == BCFMM_FP32) {
-      // Taylor-form M2L: D^gamma G(o), |gamma| <= the largest order of any level
-      int qt = 0;
-      for (int l = 0; l < C->nlevels; ++l) qt = std::max(qt, level_order(prm, l));
-      if (qt > 0) {
-        const int pitch = m2l_taylor_pitch(qt);
+    if (!tc_mode && qt > 0) {
+      const int pitch = m2l_taylor_pitch(qt);
+      // the one-CTA-per-target FP32 kernel's D^gamma G(o) per offset code
+      if (prm.precision == BCFMM_FP32 && qt > kTaylorMaxQ) {
         std::vector<float> g((size_t)std::max(ncode, 1) * pitch, 0.f);
-        std::vector<double> gd(nterms_q(qt));
+#pragma omp parallel for schedule(static)
         for (int code = 0; code < ncode; ++code) {
+          std::vector<double> gd(nterms_q(qt));
           const double od[3] = {(double)H.offsets[3 * code], (double)H.offsets[3 * code + 1],
                                 (double)H.offsets[3 * code + 2]};
           m2l_taylor_coeffs(qt, od, gd.data());
           for (int k = 0; k < nterms_q(qt); ++k) g[(size_t)code * pitch + k] = (float)gd[k];
         }
-        // (-1)^{|b|} / b! for the moments, 1 / a! for the locals
-        std::vector<float> fac(2 * (size_t)pitch, 0.f);
-        MultiIndex M;
-        M.init(qt);
-        for (int k = 0; k < M.n; ++k) {
-          double f = 1.0;
-          for (int n = 2; n <= M.a[k]; ++n) f *= n;
-          for (int n = 2; n <= M.b[k]; ++n) f *= n;
-          for (int n = 2; n <= M.c[k]; ++n) f *= n;
-          fac[k] = (float)(((M.a[k] + M.b[k] + M.c[k]) & 1 ? -1.0 : 1.0) / f);
-          fac[pitch + k] = (float)(1.0 / f);
-        }
-        float *dg, *df;
-        if (m.upload(&dg, g.data(), g.size(), st) != cudaSuccess || m.upload(&df, fac.data(), fac.size(), st) != cudaSuccess)
+        float* dg;
+        if (m.upload(&dg, g.data(), g.size(), st) != cudaSuccess)
           return cleanup(fail(BCFMM_ERR_OOM, "build: device allocation failed (Taylor tables)"));
         C->ty.g = dg;
-        C->ty.fac = df;
-        C->ty.gpitch = pitch;
-        C->ty.q = qt;
       }
+      // (-1)^{|b|} / b! for the moments, 1 / a! for the locals
+      std::vector<double> fac(2 * (size_t)pitch, 0.0);
+      MultiIndex M;
+      M.init(qt);
+      for (int k = 0; k < M.n; ++k) {
+        double f = 1.0;
+        for (int n = 2; n <= M.a[k]; ++n) f *= n;
+        for (int n = 2; n <= M.b[k]; ++n) f *= n;
+        for (int n = 2; n <= M.c[k]; ++n) f *= n;
+        fac[k] = ((M.a[k] + M.b[k] + M.c[k]) & 1 ? -1.0 : 1.0) / f;
+        fac[pitch + k] = 1.0 / f;
+      }
+      cudaError_t fe;
+      if (prm.precision == BCFMM_FP64) {
+        double* df;
+        fe = m.upload(&df, fac.data(), fac.size(), st);
+        C->ty.fac = df;
+      } else {
+        const std::vector<float> f32(fac.begin(), fac.end());
+        float* df;
+        fe = m.upload(&df, f32.data(), f32.size(), st);
+        C->ty.fac = df;
+      }
+      if (fe != cudaSuccess) return cleanup(fail(BCFMM_ERR_OOM, "build: device allocation failed (Taylor tables)"));
+      C->ty.gpitch = pitch;
+      C->ty.q = qt;
     }
   }
   double tn = wall();
   for (int t = 0; t < 3; ++t) {
     int rc = upload_task(C, H, t);
+    if (rc != BCFMM_OK) return cleanup(rc);
+  }
+  {
+    const int rc = upload_taylor_rows(C);
     if (rc != BCFMM_OK) return cleanup(rc);
   }
   C->sec_near_dev = wall() - tn;
@@ -1180,21 +1228,20 @@ extern "C" int bcfmm_debug_list_coverage(const double* verts, const int64_t* ver
       }
       out[6 + t] = sbad;
       // the Taylor-form schedule: every list entry of a target of orders
-      // 1..kTaylorMaxQ exactly once, in a lane whose chunk is the target's,
-      // decoding to the entry's (offset code, source box); every chunk in
-      // exactly one lane; every other target in the generic kernel's list
+      // 1..kTaylorMaxQ exactly once, in a warp whose slot is the target's, with
+      // the g row of its offset; every slot in exactly one warp; every other
+      // target in the generic kernels' list
       int64_t ybad = 0;
+      std::map<std::array<int, 3>, int> code_of;
+      for (size_t x = 0; x < H.offsets.size() / 3; ++x)
+        code_of[{H.offsets[3 * x], H.offsets[3 * x + 1], H.offsets[3 * x + 2]}] = (int)x;
       std::vector<int> tq(T.m2l_tgt.size());
       for (size_t k = 0; k < tq.size(); ++k) tq[k] = box_q[T.m2l_tgt[k]];
       for (int nsm : {1, 7, 152}) {
         std::vector<TaylorOrderHost> ys;
         std::vector<int> sel;
-        int cbits = 0;
-        if (!m2l_taylor_schedule(T.m2l_tgt, T.vl_off, T.vl_src, T.vl_code, tq, (int)H.box.size(),
-                                 (int)(H.offsets.size() / 3), nsm, ys, sel, &cbits)) {
-          ++ybad;
-          continue;
-        }
+        TaylorOffsets offs;
+        m2l_taylor_schedule(H, t, tq, nsm, offs, ys, sel);
         std::vector<std::vector<std::pair<int, int>>> got(T.m2l_tgt.size());
         std::vector<int> in_sel(T.m2l_tgt.size(), 0);
         for (int k : sel) {
@@ -1203,21 +1250,36 @@ extern "C" int bcfmm_debug_list_coverage(const double* verts, const int64_t* ver
         }
         for (const TaylorOrderHost& O : ys) {
           std::vector<int> ctgt(O.nchunk, -1), cseen(O.nchunk, 0);
-          if ((int)O.tchunk.size() != (int)O.tgt.size() + 1 || O.tchunk.back() != O.nchunk) { ++ybad; continue; }
+          if ((int)O.tchunk.size() != (int)O.tgt.size() + 1 || O.tchunk.back() != O.nchunk ||
+              O.wslot.size() != 8 * O.wb.size()) { ++ybad; continue; }
           for (size_t i = 0; i < O.tgt.size(); ++i)
             for (int c = O.tchunk[i]; c < O.tchunk[i + 1]; ++c) ctgt[c] = k_of[O.tgt[i]];
-          for (size_t w = 0; w < O.wb.size(); ++w)
-            for (int l = 0; l < 32; ++l) {
-              const int c = O.lane_chunk[w * 32 + l];
-              if (c >= O.nchunk) { ++ybad; continue; }
-              if (c >= 0) cseen[c]++;
-              for (int j = 0; j < O.wb[w].y; ++j) {
-                const uint32_t v = O.pk[(size_t)O.wb[w].x + (size_t)j * 32 + l];
-                if (v == ~0u) continue;
-                if (c < 0 || ctgt[c] < 0) { ++ybad; continue; }
-                got[ctgt[c]].push_back({(int)(v & ((1u << cbits) - 1u)), (int)(v >> cbits)});
-              }
+          for (size_t w = 0; w < O.wb.size(); ++w) {
+            const int4 B = O.wb[w];
+            if (B.x < 0 || B.y < 1 || B.y > 32 || (size_t)B.x + B.y > O.ent.size() || B.w < 1 || B.w > 8) { ++ybad; continue; }
+            for (int l = 0; l < 8; ++l) {
+              const int c = O.wslot[w * 8 + l];
+              if ((c < 0) != (l >= B.w) || c >= O.nchunk) { ++ybad; continue; }
+              if (c < 0) continue;
+              cseen[c]++;
+              const int k = ctgt[c], to = B.z >> (3 * l) & 7;
+              if (k < 0 || H.box[T.m2l_tgt[k]].octant != to) { ++ybad; continue; }
+              for (int j = B.x; j < B.x + B.y; ++j)
+                for (int i = 0; i < 4; ++i) {
+                  const unsigned sb = (unsigned)O.ent[j].z >> (8 * i) & 255u;
+                  if (!sb) continue;
+                  const int so = sb >> 3 & 7, box = O.ent[j].x + (int)(sb & 7);
+                  const int row = (to >> 2) * 9 + ((to >> 1 & 1) - (so >> 1 & 1) + 1) * 3 + (to & 1) - (so & 1) + 1;
+                  if (!(O.ent[j].w >> row & 1)) continue;
+                  if (box < 0 || box >= (int)H.box.size() || O.ent[j].y < 0 || O.ent[j].y + 18 > 27 * (int)(offs.d.size() / 3)) { ++ybad; continue; }
+                  const int gr = O.ent[j].y + row;
+                  const int* Dd = &offs.d[3 * (gr / 27)];
+                  const int o[3] = {2 * Dd[0] + gr % 3 - 1, 2 * Dd[1] + gr / 3 % 3 - 1, 2 * Dd[2] + gr / 9 % 3 - 1};
+                  const auto it = code_of.find({o[0], o[1], o[2]});
+                  got[k].push_back({it == code_of.end() ? -1 : it->second, box});
+                }
             }
+          }
           for (int v : cseen) ybad += (v != 1);
         }
         for (size_t k = 0; k < T.m2l_tgt.size(); ++k) {
@@ -1367,10 +1429,14 @@ static int ensure_work(bcfmm_ctx* C, int ndp) {
       const int kpitch = m2l_tc_kpitch(C->prm.p);
       CU(m.alloc(&C->tc_momb, (size_t)C->nbox * ndp * C->tc.nsplit * kpitch * 2));
     }
-    if (C->ty.g) {
-      CU(m.alloc(&C->ty_momp, (size_t)C->nbox * ndp * C->ty.gpitch));
-      CU(m.alloc(&C->ty_partial, std::max<size_t>((size_t)ndp * C->ty_partial_per_dens, 1)));
-    }
+  }
+  if (C->ty.q > 0) {
+    const size_t es = f64 ? sizeof(double) : sizeof(float);
+    char *mp, *pp;
+    CU(m.alloc(&mp, (size_t)C->nbox * ndp * C->ty.gpitch * es));
+    C->ty_momp = mp;
+    CU(m.alloc(&pp, std::max<size_t>((size_t)ndp * C->ty_partial_per_dens, 1) * es));
+    C->ty_partial = pp;
   }
   C->work_ndp = ndp;
   C->work_gen++;
@@ -1456,7 +1522,14 @@ static int eval_impl(bcfmm_ctx* C, int t, double* out, int out_is_device, bool s
       }
     }
     if (tm) CU(cudaEventRecord(ev[2], st));
-    if (!skip_far) CU(launch_m2l_simt<double>(G, L, C->T64, ndp, C->mom64, C->loc64, st));
+    if (!skip_far) {
+      if (C->ty.q > 0)
+        CU(launch_m2l_taylor<double>(G, L, D.tys, C->ty, ndp, C->mom64, C->loc64, (double*)C->ty_momp,
+                                     (double*)C->ty_partial, st));
+      if (C->ty.q == 0) CU(launch_m2l_simt<double>(G, L, C->T64, ndp, C->mom64, C->loc64, st));
+      else if (D.tys.nsimt > 0)
+        CU(launch_m2l_simt<double>(G, L, C->T64, ndp, C->mom64, C->loc64, st, D.tys.simt_sel, D.tys.nsimt));
+    }
     if (tm) CU(cudaEventRecord(ev[3], st));
     for (int l = 3; l < C->nlevels && !skip_far; ++l) {
       const int n = D.l2l_off[l + 1] - D.l2l_off[l];
@@ -1486,8 +1559,9 @@ static int eval_impl(bcfmm_ctx* C, int t, double* out, int out_is_device, bool s
     } else if (tc) {
       CU(launch_m2l_tc(G, L, D.tcs, C->tc, ndp, C->mom32, C->loc32, C->tc_partial, C->tc_momb, st));
       if (D.tcs.nsimt > 0) CU(launch_m2l_simt<float>(G, L, C->T32, ndp, C->mom32, C->loc32, st, D.tcs.simt_sel, D.tcs.nsimt));
-    } else if (C->ty.g) {
-      CU(launch_m2l_taylor(G, L, D.tys, C->ty, ndp, C->mom32, C->loc32, C->ty_momp, C->ty_partial, st));
+    } else if (C->ty.q > 0) {
+      CU(launch_m2l_taylor<float>(G, L, D.tys, C->ty, ndp, C->mom32, C->loc32, (float*)C->ty_momp,
+                                  (float*)C->ty_partial, st));
     } else {
       CU(launch_m2l_simt<float>(G, L, C->T32, ndp, C->mom32, C->loc32, st));
     }
@@ -1604,7 +1678,7 @@ extern "C" int bcfmm_eval_noalloc(bcfmm_ctx* C, int32_t task, const double* dens
   TaskDev& D = C->task[task];
   const DevTaskLists& L = D.L;
   const int kind = L.src_cls;
-  if (C->work_ndp < 1 || (tcp && C->tc_momb == nullptr) || (typ && C->ty.g && C->ty_momp == nullptr))
+  if (C->work_ndp < 1 || (tcp && C->tc_momb == nullptr) || (typ && C->ty.q > 0 && C->ty_momp == nullptr))
     return fail(BCFMM_ERR_STATE, "eval_noalloc: call bcfmm_set_density once first (it sizes the work buffers)");
   int dev = -1;
   CU(cudaGetDevice(&dev));
@@ -1635,8 +1709,9 @@ extern "C" int bcfmm_eval_noalloc(bcfmm_ctx* C, int32_t task, const double* dens
   if (tcp) {
     CU(launch_m2l_tc(G, L, D.tcs, C->tc, ndp, C->mom32, C->loc32, partial, C->tc_momb, st));
     if (D.tcs.nsimt > 0) CU(launch_m2l_simt<float>(G, L, C->T32, ndp, C->mom32, C->loc32, st, D.tcs.simt_sel, D.tcs.nsimt));
-  } else if (C->ty.g) {
-    CU(launch_m2l_taylor(G, L, D.tys, C->ty, ndp, C->mom32, C->loc32, C->ty_momp, reinterpret_cast<float*>(partial), st));
+  } else if (C->ty.q > 0) {
+    CU(launch_m2l_taylor<float>(G, L, D.tys, C->ty, ndp, C->mom32, C->loc32, (float*)C->ty_momp,
+                                reinterpret_cast<float*>(partial), st));
   } else {
     CU(launch_m2l_simt<float>(G, L, C->T32, ndp, C->mom32, C->loc32, st));
   }
@@ -1802,7 +1877,7 @@ extern "C" int bcfmm_stats(const bcfmm_ctx* C, char* json, size_t cap) {
     }
     per_q += "], \"taylor_orders\": [";
     bool first_ty = true;
-    for (int q = 1; q <= kTaylorMaxQ; ++q) {
+    for (int q = 1; q <= kTaylorRegQ; ++q) {
       const TaylorOrderSched& O = D.tys.ord[q];
       if (O.nwarp == 0) continue;
       if (!first_ty) per_q += ", ";
@@ -1813,7 +1888,7 @@ extern "C" int bcfmm_stats(const bcfmm_ctx* C, char* json, size_t cap) {
     }
     per_q += "], \"m2l_pairs_by_order\": [";
     for (int q = 0; q <= C->prm.p; ++q) per_q += std::to_string(D.m2l_pairs_q[q]) + (q < C->prm.p ? ", " : "");
-    per_q += "], \"generic_m2l_targets\": " + std::to_string(C->ty.g ? D.tys.nsimt : (D.tcs.nsimt > 0 ? D.tcs.nsimt : 0));
+    per_q += "], \"generic_m2l_targets\": " + std::to_string(C->ty.q > 0 ? D.tys.nsimt + D.tys.ord[kTaylorMaxQ].ntgt : (D.tcs.nsimt > 0 ? D.tcs.nsimt : 0));
     per_q += ", \"p2p_sources_per_leaf\": [";
     for (int k = 0; k < 5; ++k) per_q += std::to_string(D.p2p_src_q[k]) + (k < 4 ? ", " : "]");
     snprintf(b, sizeof b,

@@ -64,6 +64,7 @@ struct HostSetup {
   std::vector<double> qp[2], qw[2];
   // tree
   double lo[3], R0;
+  double eta0 = 0.5;                               // box-neighbour parameter of the lists
   std::vector<HostBox> box;
   std::vector<int> lvl_off;                        // box index range per level
   int nlevels = 0;

@@ -200,6 +200,7 @@ static std::vector<std::array<int, 3>> neighbour_offsets(double eta0) {
 
 void build_lists(HostSetup& H, double eta0) {
   double t0 = now_s();
+  H.eta0 = eta0;
   const auto NB = neighbour_offsets(eta0);
   auto is_nb = [&](int64_t dx, int64_t dy, int64_t dz) { return (double)(dx * dx + dy * dy + dz * dz) * eta0 * eta0 < 3.0; };
   std::unordered_map<uint64_t, int> idx;
@@ -592,7 +593,7 @@ void merge_setups(std::vector<HostSetup>& P, HostSetup& H) {
       H.qw[c].insert(H.qw[c].end(), S.qw[c].begin(), S.qw[c].end());
     }
   }
-  if (nm > 0) { std::memcpy(H.lo, P[0].lo, sizeof H.lo); H.R0 = P[0].R0; }
+  if (nm > 0) { std::memcpy(H.lo, P[0].lo, sizeof H.lo); H.R0 = P[0].R0; H.eta0 = P[0].eta0; }
   // point offsets per class: points are element-major (4 per tet, 3 per triangle)
   auto pto = [&](int m, int c) -> int { return c == 0 ? (int)(4 * H.mesh_tet_off[m]) : (int)(3 * H.mesh_tri_off[m]); };
   // boxes, level-major
