@@ -19,6 +19,7 @@
 #include "m2l_taylor.cuh"
 #include "m2l_tc.cuh"
 #include "mlp.cuh"
+#include "p2p_sym.cuh"
 
 using namespace bcfmm;
 
@@ -81,6 +82,7 @@ struct TaskDev {
   DevTaskLists L{};
   TcTaskSched tcs{};                   // tensor-core M2L launches, one per expansion order
   TaylorTaskSched tys{};               // CUDA-core Taylor-form M2L launches, one per expansion order
+  DevSym sym{};                        // symmetric near field (VtV, FP32 points; nblk 0: none)
   std::vector<int> m2m_off, l2l_off;   // host offsets into the per-level arrays
   int* m2m_parent = nullptr;
   int* l2l_child = nullptr;
@@ -290,6 +292,34 @@ static int upload_task(bcfmm_ctx* C, const HostSetup& H, int t) {
     CU(m.alloc(&scr, (size_t)K.rows * 2 * 128));     // up to two densities
     L.sp_leaf = sl; L.sp_run_off = sro; L.sp_runs = srn; L.sp_self = ss;
     L.sp_grp = sg; L.grp_info = gi; L.grp_cnt = gc; L.sp_scratch = scr;
+  }
+  if (t == 0 && C->prm.precision != BCFMM_FP64 && p2p_sym_pays(H)) {
+    // symmetric near field (one density)
+    int nsm = 152;
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, C->device);
+    HostSym Y;
+    if (build_p2p_sym(H, p2p_sym_chunk(H, nsm), Y)) {
+      DevSym& S = D.sym;
+      int *lf, *ro, *sf, *fl, *fto, *ft, *fso, *fs;
+      int2 *rn, *bs;
+      CU(m.upload(&lf, Y.leaf.data(), Y.leaf.size(), st));
+      CU(m.upload(&ro, Y.run_off.data(), Y.run_off.size(), st));
+      CU(m.upload(&rn, reinterpret_cast<const int2*>(Y.runs.data()), Y.runs.size() / 2, st));
+      CU(m.upload(&bs, reinterpret_cast<const int2*>(Y.base.data()), Y.base.size() / 2, st));
+      CU(m.upload(&sf, Y.self.data(), Y.self.size(), st));
+      CU(m.upload(&fl, Y.fin_leaf.data(), Y.fin_leaf.size(), st));
+      CU(m.upload(&fto, Y.fin_tgt_off.data(), Y.fin_tgt_off.size(), st));
+      CU(m.upload(&ft, Y.fin_tgt.data(), Y.fin_tgt.size(), st));
+      CU(m.upload(&fso, Y.fin_src_off.data(), Y.fin_src_off.size(), st));
+      CU(m.upload(&fs, Y.fin_src.data(), Y.fin_src.size(), st));
+      CU(m.alloc(&S.src, (size_t)Y.nsrc));
+      CU(m.alloc(&S.tgt, (size_t)Y.ntgt));
+      S.nblk = (int)Y.leaf.size();
+      S.nlarge = Y.nlarge;
+      S.leaf = lf; S.run_off = ro; S.runs = rn; S.base = bs; S.self = sf;
+      S.nfin = (int)Y.fin_leaf.size();
+      S.fin_leaf = fl; S.fin_tgt_off = fto; S.fin_tgt = ft; S.fin_src_off = fso; S.fin_src = fs;
+    }
   }
   L.n_m2l = (int)T.m2l_tgt.size();
   CU(m.upload(&m2l_tgt, T.m2l_tgt.data(), T.m2l_tgt.size(), st));
@@ -807,21 +837,30 @@ static int build_impl(const double* verts, const int64_t* vert_off, const int32_
   {
     const int nb = C->nbox;
     std::vector<double4_32a> cs(nb);
+    std::vector<float4> bhi(nb), blo(nb);
     std::vector<int> c0(nb), nc(nb), oc(nb), par(nb);
     std::vector<int2> rg[2] = {std::vector<int2>(nb), std::vector<int2>(nb)};
     for (int i = 0; i < nb; ++i) {
       const HostBox& B = H.box[i];
       cs[i] = make_double4_32a(B.c[0], B.c[1], B.c[2], B.s);
+      const double v[4] = {B.c[0], B.c[1], B.c[2], 1.0 / B.s};
+      float h[4], l[4];
+      for (int a = 0; a < 4; ++a) { h[a] = (float)v[a]; l[a] = (float)(v[a] - (double)h[a]); }
+      bhi[i] = make_float4(h[0], h[1], h[2], h[3]);
+      blo[i] = make_float4(l[0], l[1], l[2], l[3]);
       c0[i] = B.child0; nc[i] = B.nchild; oc[i] = B.octant; par[i] = B.parent;
       for (int c = 0; c < 2; ++c) rg[c][i] = make_int2(B.pt0[c], B.pt1[c]);
     }
     const std::vector<int>& bq = box_q;
+    float4 *dbh, *dbl;
     double4_32a* dcs; int *dc0, *dnc, *doc, *dpar, *dbq; int2 *drg0, *drg1;
     bool ok = m.upload(&dcs, cs.data(), nb, st) == cudaSuccess && m.upload(&dc0, c0.data(), nb, st) == cudaSuccess &&
               m.upload(&dnc, nc.data(), nb, st) == cudaSuccess && m.upload(&doc, oc.data(), nb, st) == cudaSuccess &&
               m.upload(&dpar, par.data(), nb, st) == cudaSuccess && m.upload(&drg0, rg[0].data(), nb, st) == cudaSuccess &&
-              m.upload(&drg1, rg[1].data(), nb, st) == cudaSuccess && m.upload(&dbq, bq.data(), nb, st) == cudaSuccess;
+              m.upload(&drg1, rg[1].data(), nb, st) == cudaSuccess && m.upload(&dbq, bq.data(), nb, st) == cudaSuccess &&
+              m.upload(&dbh, bhi.data(), nb, st) == cudaSuccess && m.upload(&dbl, blo.data(), nb, st) == cudaSuccess;
     if (!ok) return cleanup(fail(BCFMM_ERR_OOM, "build: device allocation failed (boxes)"));
+    G.box_hi = dbh; G.box_lo = dbl;
     G.box_cs = dcs; G.box_child0 = dc0; G.box_nchild = dnc; G.box_octant = doc; G.box_parent = dpar;
     G.box_rng[0] = drg0; G.box_rng[1] = drg1; G.box_q = dbq;
   }
@@ -1571,7 +1610,9 @@ static int eval_impl(bcfmm_ctx* C, int t, double* out, int out_is_device, bool s
       CU(launch_l2l<float>(G, D.l2l_child + D.l2l_off[l], n, ndp, C->loc32, st));
     }
     if (tm) CU(cudaEventRecord(ev[4], st));
-    CU(launch_p2p_l2p_f32(G, L, C->W32, nsp, ntp, ndp, C->loc32, C->phi, st));
+    if (ndp == 1 && D.sym.nblk > 0) CU(launch_p2p_sym(G, D.sym, C->W32, C->phi, st));
+    else CU(launch_p2p_f32(G, L, C->W32, nsp, ntp, ndp, C->phi, st));
+    CU(launch_l2p_f32(G, L, ntp, ndp, C->loc32, C->phi, st));
     if (dl) CU(launch_p2p_dl<float>(G, L, C->W32dl, nsp, ntp, ndp, C->phi, st));
   }
   if (tm) CU(cudaEventRecord(ev[5], st));
@@ -1719,7 +1760,9 @@ extern "C" int bcfmm_eval_noalloc(bcfmm_ctx* C, int32_t task, const double* dens
     const int n = D.l2l_off[l + 1] - D.l2l_off[l];
     CU(launch_l2l<float>(G, D.l2l_child + D.l2l_off[l], n, ndp, C->loc32, st));
   }
-  CU(launch_p2p_l2p_f32(G, L, C->W32, nsp, ntp, ndp, C->loc32, C->phi, st));
+  if (D.sym.nblk > 0) CU(launch_p2p_sym(G, D.sym, C->W32, C->phi, st));
+  else CU(launch_p2p_f32(G, L, C->W32, nsp, ntp, ndp, C->phi, st));
+  CU(launch_l2p_f32(G, L, ntp, ndp, C->loc32, C->phi, st));
   CU(launch_elem_sum(G, L, C->phi, ntp, dens_dev, 1, out_dev, st));
   C->ev_rec[task] = false;             // no stage timings recorded by this call
   return BCFMM_OK;

@@ -16,6 +16,7 @@ struct DevGeom {
   const int* mi;                 // packed multi-indices a | b << 8 | c << 16, degree-major
   const int* box_q;              // expansion order of each box's level (<= p; Sec. 4.3)
   const double4_32a* box_cs;         // centre xyz, side s
+  const float4 *box_hi, *box_lo;     // (centre xyz, 1 / s) as float hi and lo parts (FP64 arithmetic is scarce)
   const int* box_child0;
   const int* box_nchild;
   const int* box_octant;
@@ -51,7 +52,7 @@ struct DevTaskLists {
   // exceed one chunk are cut into chunks (runs split at chunk boundaries);
   // a chunk block writes its per-target sums to its scratch row and the
   // last chunk of a leaf to finish (ticket counter) adds the rows in chunk
-  // order and evaluates L2P
+  // order
   int sp_n;                      // blocks
   const int* sp_leaf;            // [sp_n] target leaf box
   const int* sp_run_off;         // [sp_n + 1] into sp_runs
@@ -78,8 +79,12 @@ cudaError_t launch_m2l_simt(const DevGeom& G, const DevTaskLists& L, const T* Tt
                             cudaStream_t st, const int* sel = nullptr, int nsel = 0);
 template <typename T>
 cudaError_t launch_l2l(const DevGeom& G, const int* children, int n, int ndp, T* loc, cudaStream_t st);
-cudaError_t launch_p2p_l2p_f32(const DevGeom& G, const DevTaskLists& L, const float* W, int64_t nsrc_pts,
-                               int64_t ntgt_pts, int ndp, const float* loc, double* phi, cudaStream_t st);
+// phi = near field / 4 pi
+cudaError_t launch_p2p_f32(const DevGeom& G, const DevTaskLists& L, const float* W, int64_t nsrc_pts, int64_t ntgt_pts,
+                           int ndp, double* phi, cudaStream_t st);
+// phi += far field (L2P of the target leaves' local expansions)
+cudaError_t launch_l2p_f32(const DevGeom& G, const DevTaskLists& L, int64_t ntgt_pts, int ndp, const float* loc,
+                           double* phi, cudaStream_t st);
 cudaError_t launch_p2p_l2p_f64(const DevGeom& G, const DevTaskLists& L, const double* W, int64_t nsrc_pts,
                                int64_t ntgt_pts, int ndp, const double* loc, double* phi, cudaStream_t st);
 // dens_dl: BtV double-layer density (subtracts its corrections L.cor_val_dl), or null

@@ -1,7 +1,7 @@
 // Evaluation kernels of the boundary-concentrated FMM (Sec. 3.3, Algorithms
 // 1-3): source weights, moments (P2M), upward pass (M2M), interaction phase
-// on CUDA cores (M2L), downward pass (L2L), evaluation fused with the near
-// field (L2P + P2P over the extended neighbour list N*), and the Galerkin
+// on CUDA cores (M2L), downward pass (L2L), evaluation (L2P) and near field
+// (P2P over the extended neighbour list N*), fused in FP64, and the Galerkin
 // element sums plus near-rule corrections.
 //
 // Expansions are box-scaled: moments m^b = sum_j W_j ((y_j - c)/s)^b, locals
@@ -391,6 +391,87 @@ __device__ __forceinline__ void l2p_and_store(const DevGeom& G, int leaf, int nd
   for (int d = 0; d < ND; ++d) phi[(int64_t)d * ntp + pos] = near[d] * kInv4Pi + (double)far[d];
 }
 
+// ------------------------------------------------ L2P (FP32 tasks)
+// sum_{|a| <= Q} l^a x^a: Horner in x for every (j, k), then the products
+// y^j z^k (about 1.5 FMA a term and no table of multi-indices)
+template <int Q>
+__device__ __forceinline__ float l2p_eval(const float* __restrict__ sl, float x, float y, float z) {
+  float far = 0.f, yp = 1.f;
+#pragma unroll
+  for (int j = 0; j <= Q; ++j) {
+    float yz = yp;
+    asm volatile("" ::: "memory");       // this j's coefficients only (registers)
+#pragma unroll
+    for (int k = 0; k <= Q - j; ++k) {
+      float h = sl[midx3(Q - j - k, j, k)];
+#pragma unroll
+      for (int i = Q - j - k - 1; i >= 0; --i) h = fmaf(h, x, sl[midx3(i, j, k)]);
+      far = fmaf(h, yz, far);
+      yz *= z;
+    }
+    yp *= y;
+  }
+  return far;
+}
+__device__ float l2p_loop(const float* sl, int q, float x, float y, float z) {
+  float far = 0.f, yp = 1.f;
+  for (int j = 0; j <= q; ++j) {
+    float yz = yp;
+    for (int k = 0; k <= q - j; ++k) {
+      float h = sl[midx3(q - j - k, j, k)];
+      for (int i = q - j - k - 1; i >= 0; --i) h = fmaf(h, x, sl[midx3(i, j, k)]);
+      far = fmaf(h, yz, far);
+      yz *= z;
+    }
+    yp *= y;
+  }
+  return far;
+}
+
+// phi += far field of the leaf's local expansion, one CTA per target leaf, one
+// target point per thread and round; the coefficients are staged in shared
+// memory (locals of boxes without an interaction list are zero).  Latency: two
+// dependent loads and some 400 instructions a CTA, so small CTAs, twelve on an
+// SM; 767,360 points at orders 6 and 7 take 35 us (as the tail of the near-
+// field CTAs, with FP64 scaling and indexed powers, it cost them about 0.1 ms).
+constexpr int kL2pThreads = 64;
+__global__ void __launch_bounds__(kL2pThreads, 12) k_l2p(DevGeom G, const int* __restrict__ leaves, int tc, int64_t ntp,
+                                                         int ndp, const float* __restrict__ loc,
+                                                         double* __restrict__ phi) {
+  __shared__ float sl[456];
+  const int leaf = leaves[blockIdx.x];
+  const float4 ch = G.box_hi[leaf], cl = G.box_lo[leaf];
+  const int2 tr = G.box_rng[tc][leaf];
+  const int q = G.box_q[leaf], nq = nterms_q(q);
+  for (int d = 0; d < ndp; ++d) {
+    if (d > 0) __syncthreads();
+    for (int a = threadIdx.x; a < nq; a += kL2pThreads) sl[a] = loc[((int64_t)leaf * ndp + d) * G.ms + a];
+    __syncthreads();
+    for (int j = tr.x + threadIdx.x; j < tr.y; j += kL2pThreads) {
+      const float4 h = G.pthi[tc][j], l = G.ptlo[tc][j];
+      float x = (h.x - ch.x) + (l.x - cl.x), y = (h.y - ch.y) + (l.y - cl.y), z = (h.z - ch.z) + (l.z - cl.z);
+      x = fmaf(x, ch.w, x * cl.w);
+      y = fmaf(y, ch.w, y * cl.w);
+      z = fmaf(z, ch.w, z * cl.w);
+      float far;
+      switch (q) {
+        case 5: far = l2p_eval<5>(sl, x, y, z); break;
+        case 6: far = l2p_eval<6>(sl, x, y, z); break;
+        case 7: far = l2p_eval<7>(sl, x, y, z); break;
+        default: far = l2p_loop(sl, q, x, y, z); break;
+      }
+      phi[(int64_t)d * ntp + j] += (double)far;
+    }
+  }
+}
+
+cudaError_t launch_l2p_f32(const DevGeom& G, const DevTaskLists& L, int64_t ntgt_pts, int ndp, const float* loc,
+                           double* phi, cudaStream_t st) {
+  if (L.n_p2p == 0) return cudaSuccess;
+  k_l2p<<<L.n_p2p, kL2pThreads, 0, st>>>(G, L.p2p_leaf, L.tgt_cls, ntgt_pts, ndp, loc, phi);
+  return cudaGetLastError();
+}
+
 // The hardware reciprocal square root (PTX rsqrt.approx.ftz.f32: maximum
 // relative error about 2^-22.9, subnormal inputs and results flushed to
 // zero).  Squared distances of distinct quadrature points lie far above the
@@ -415,9 +496,8 @@ __device__ __forceinline__ void two_sum_f(float& hi, float& lo, float x) {
 // source tile; source tiles are double-buffered (one barrier per tile); the
 // per-tile FP32 sums are folded with a compensated (hi + lo) FP32 sum.
 template <int ND>
-__global__ void __launch_bounds__(128) k_p2p_l2p_f32(DevGeom G, DevTaskLists L, const float* __restrict__ W,
-                                                     int64_t nsp, int64_t ntp, int ndp,
-                                                     const float* __restrict__ loc, double* __restrict__ phi) {
+__global__ void __launch_bounds__(128) k_p2p_f32(DevGeom G, DevTaskLists L, const float* __restrict__ W, int64_t nsp,
+                                                 int64_t ntp, double* __restrict__ phi) {
   constexpr int TPT = ND <= 2 ? 2 : 1;
   constexpr int PPT = kTile / 128;                 // source points loaded per thread per tile
   __shared__ float4 tile[2][kTile];
@@ -427,9 +507,8 @@ __global__ void __launch_bounds__(128) k_p2p_l2p_f32(DevGeom G, DevTaskLists L, 
   const int b = blockIdx.x;
   const int leaf = L.p2p_leaf[b];
   const int sc = L.src_cls, tc = L.tgt_cls;
-  const double4_32a cs = G.box_cs[leaf];
-  float chx, clx, chy, cly, chz, clz;
-  split_df(cs.x, chx, clx); split_df(cs.y, chy, cly); split_df(cs.z, chz, clz);
+  const float4 ch = G.box_hi[leaf], cl = G.box_lo[leaf];
+  const float chx = ch.x, chy = ch.y, chz = ch.z, clx = cl.x, cly = cl.y, clz = cl.z;
   const int2 tr = G.box_rng[tc][leaf];
   const int nt = tr.y - tr.x;
   // TS target slots (TPT targets each) per source group, NG = 128 / TS
@@ -562,9 +641,8 @@ __global__ void __launch_bounds__(128) k_p2p_l2p_f32(DevGeom G, DevTaskLists L, 
         }
         near[d] = (double)hi + (double)lo;
       }
-      const double inv_s = 1.0 / cs.w;
-      l2p_and_store<float, ND>(G, leaf, ndp, loc, xt[u] * inv_s, yt[u] * inv_s, zt[u] * inv_s, near, tr.x + ts + u * TS,
-                               ntp, phi);
+#pragma unroll
+      for (int d = 0; d < ND; ++d) phi[(int64_t)d * ntp + tr.x + ts + u * TS] = near[d] * kInv4Pi;
     }
   }
 }
@@ -617,9 +695,8 @@ __device__ __forceinline__ void p2p_pairs_x2(const float4* __restrict__ xy, cons
 constexpr int kTileX2 = 512;     // source points per tile of the packed kernel
 
 template <int ND, int TPT>
-__global__ void __launch_bounds__(128) k_p2p_l2p_f32x2(DevGeom G, DevTaskLists L, const float* __restrict__ W,
-                                                       int64_t nsp, int64_t ntp, int ndp,
-                                                       const float* __restrict__ loc, double* __restrict__ phi) {
+__global__ void __launch_bounds__(128) k_p2p_f32x2(DevGeom G, DevTaskLists L, const float* __restrict__ W, int64_t nsp,
+                                                   int64_t ntp, double* __restrict__ phi) {
   static_assert(ND >= 1 && ND <= 2, "packed P2P serves one or two densities");
   constexpr int kTile = kTileX2;
   constexpr int kPairs = kTile / 2;
@@ -632,9 +709,8 @@ __global__ void __launch_bounds__(128) k_p2p_l2p_f32x2(DevGeom G, DevTaskLists L
   const int b = blockIdx.x;
   const int leaf = L.sp_leaf[b];
   const int sc = L.src_cls, tc = L.tgt_cls;
-  const double4_32a cs = G.box_cs[leaf];
-  float chx, clx, chy, cly, chz, clz;
-  split_df(cs.x, chx, clx); split_df(cs.y, chy, cly); split_df(cs.z, chz, clz);
+  const float4 ch = G.box_hi[leaf], cl = G.box_lo[leaf];
+  const float chx = ch.x, chy = ch.y, chz = ch.z, clx = cl.x, cly = cl.y, clz = cl.z;
   const int2 tr = G.box_rng[tc][leaf];
   const int nt = tr.y - tr.x;
   const int TS = (nt + TPT - 1) / TPT;
@@ -752,7 +828,7 @@ __global__ void __launch_bounds__(128) k_p2p_l2p_f32x2(DevGeom G, DevTaskLists L
   __syncthreads();
   // every thread: one target, the group sums in group order; a chunk of a
   // split leaf stores them in its scratch row, and the leaf's last chunk
-  // to finish adds the rows in chunk order; then L2P
+  // to finish adds the rows in chunk order
   const int2 grp = L.sp_grp[b];
   __shared__ int last_chunk;
   if (grp.x >= 0) {
@@ -782,10 +858,8 @@ __global__ void __launch_bounds__(128) k_p2p_l2p_f32x2(DevGeom G, DevTaskLists L
     if (!last_chunk) return;
     __threadfence();
   }
-  const double inv_s = 1.0 / cs.w;
   for (int tt = threadIdx.x; tt < nt; tt += 128) {
     const int u = tt / TS, tsl = tt - u * TS;
-    double near[ND];
 #pragma unroll
     for (int d = 0; d < ND; ++d) {
       float hi = 0.f, lo = 0.f;
@@ -803,11 +877,8 @@ __global__ void __launch_bounds__(128) k_p2p_l2p_f32x2(DevGeom G, DevTaskLists L
           lo += v.y;
         }
       }
-      near[d] = (double)hi + (double)lo;
+      phi[(int64_t)d * ntp + tr.x + tt] = ((double)hi + (double)lo) * kInv4Pi;
     }
-    const float4 h = G.pthi[tc][tr.x + tt], l = G.ptlo[tc][tr.x + tt];
-    const float xt = (h.x - chx) + (l.x - clx), yt = (h.y - chy) + (l.y - cly), zt = (h.z - chz) + (l.z - clz);
-    l2p_and_store<float, ND>(G, leaf, ndp, loc, xt * inv_s, yt * inv_s, zt * inv_s, near, tr.x + tt, ntp, phi);
   }
 }
 
@@ -898,15 +969,15 @@ __global__ void __launch_bounds__(128) k_p2p_l2p_f64(DevGeom G, DevTaskLists L, 
     default: return cudaErrorInvalidValue;                                   \
   }
 
-cudaError_t launch_p2p_l2p_f32(const DevGeom& G, const DevTaskLists& L, const float* W, int64_t nsrc_pts,
-                               int64_t ntgt_pts, int ndp, const float* loc, double* phi, cudaStream_t st) {
+cudaError_t launch_p2p_f32(const DevGeom& G, const DevTaskLists& L, const float* W, int64_t nsrc_pts, int64_t ntgt_pts,
+                           int ndp, double* phi, cudaStream_t st) {
   if (L.n_p2p == 0) return cudaSuccess;
   switch (ndp) {
-    case 1: k_p2p_l2p_f32x2<1, 4><<<L.sp_n, 128, 0, st>>>(G, L, W, nsrc_pts, ntgt_pts, ndp, loc, phi); break;
-    case 2: k_p2p_l2p_f32x2<2, 2><<<L.sp_n, 128, 0, st>>>(G, L, W, nsrc_pts, ntgt_pts, ndp, loc, phi); break;
-    case 4: k_p2p_l2p_f32<4><<<L.n_p2p, 128, 0, st>>>(G, L, W, nsrc_pts, ntgt_pts, ndp, loc, phi); break;
-    case 8: k_p2p_l2p_f32<8><<<L.n_p2p, 128, 0, st>>>(G, L, W, nsrc_pts, ntgt_pts, ndp, loc, phi); break;
-    case 16: k_p2p_l2p_f32<16><<<L.n_p2p, 128, 0, st>>>(G, L, W, nsrc_pts, ntgt_pts, ndp, loc, phi); break;
+    case 1: k_p2p_f32x2<1, 4><<<L.sp_n, 128, 0, st>>>(G, L, W, nsrc_pts, ntgt_pts, phi); break;
+    case 2: k_p2p_f32x2<2, 2><<<L.sp_n, 128, 0, st>>>(G, L, W, nsrc_pts, ntgt_pts, phi); break;
+    case 4: k_p2p_f32<4><<<L.n_p2p, 128, 0, st>>>(G, L, W, nsrc_pts, ntgt_pts, phi); break;
+    case 8: k_p2p_f32<8><<<L.n_p2p, 128, 0, st>>>(G, L, W, nsrc_pts, ntgt_pts, phi); break;
+    case 16: k_p2p_f32<16><<<L.n_p2p, 128, 0, st>>>(G, L, W, nsrc_pts, ntgt_pts, phi); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
