@@ -85,7 +85,7 @@ struct TaskDev {
   DevSym sym{};                        // symmetric near field (VtV, FP32 points; nblk 0: none)
   std::vector<int> m2m_off, l2l_off;   // host offsets into the per-level arrays
   int* m2m_parent = nullptr;
-  int* l2l_child = nullptr;
+  int2* l2l_parent = nullptr;          // (parent, mask of the child slots with targets), by child level
   int64_t p2p_pairs = 0, near_boxes = 0, m2l_pairs = 0, nnz = 0, tc_entries = 0, tc_rows = 0;
   int64_t m2l_pairs_q[kMaxP + 1] = {};     // box pairs of the interaction phase per expansion order
   double tc_mma_flop = 0;              // executed MMA flops of the tensor-core M2L per density
@@ -338,10 +338,17 @@ static int upload_task(bcfmm_ctx* C, const HostSetup& H, int t) {
   D.m2m_off.assign(1, 0);
   for (auto& v : T.m2m_parent) { flat.insert(flat.end(), v.begin(), v.end()); D.m2m_off.push_back((int)flat.size()); }
   CU(m.upload(&D.m2m_parent, flat.data(), flat.size(), st));
-  flat.clear();
+  std::vector<int2> l2l;
   D.l2l_off.assign(1, 0);
-  for (auto& v : T.l2l_child) { flat.insert(flat.end(), v.begin(), v.end()); D.l2l_off.push_back((int)flat.size()); }
-  CU(m.upload(&D.l2l_child, flat.data(), flat.size(), st));
+  for (auto& v : T.l2l_child) {
+    for (int c : v) {                    // (children of one parent in a row)
+      const int par = H.box[c].parent;
+      if ((int)l2l.size() == D.l2l_off.back() || l2l.back().x != par) l2l.push_back(make_int2(par, 0));
+      l2l.back().y |= 1 << (c - H.box[par].child0);
+    }
+    D.l2l_off.push_back((int)l2l.size());
+  }
+  CU(m.upload(&D.l2l_parent, l2l.data(), l2l.size(), st));
   // target elements: sorted positions of their points
   const int tc = T.tgt_cls, sc = T.src_cls;
   const int nqt = tc == 0 ? 4 : 3;
@@ -843,11 +850,10 @@ static int build_impl(const double* verts, const int64_t* vert_off, const int32_
     for (int i = 0; i < nb; ++i) {
       const HostBox& B = H.box[i];
       cs[i] = make_double4_32a(B.c[0], B.c[1], B.c[2], B.s);
-      const double v[4] = {B.c[0], B.c[1], B.c[2], 1.0 / B.s};
-      float h[4], l[4];
-      for (int a = 0; a < 4; ++a) { h[a] = (float)v[a]; l[a] = (float)(v[a] - (double)h[a]); }
-      bhi[i] = make_float4(h[0], h[1], h[2], h[3]);
-      blo[i] = make_float4(l[0], l[1], l[2], l[3]);
+      float h[3], l[3];
+      for (int a = 0; a < 3; ++a) { h[a] = (float)B.c[a]; l[a] = (float)(B.c[a] - (double)h[a]); }
+      bhi[i] = make_float4(h[0], h[1], h[2], 0.f);
+      blo[i] = make_float4(l[0], l[1], l[2], 0.f);
       c0[i] = B.child0; nc[i] = B.nchild; oc[i] = B.octant; par[i] = B.parent;
       for (int c = 0; c < 2; ++c) rg[c][i] = make_int2(B.pt0[c], B.pt1[c]);
     }
@@ -870,7 +876,7 @@ static int build_impl(const double* verts, const int64_t* vert_off, const int32_
     const int64_t n = (int64_t)H.perm[c].size();
     C->npts[c] = n;
     std::vector<double4_32a> p64(n);
-    std::vector<float4> hi(n), lo(n);
+    std::vector<float4> hi(n), lo(n), xh(prm.precision == BCFMM_FP64 ? 0 : n);
     std::vector<int> el(n);
     for (int64_t j = 0; j < n; ++j) {
       const int o = H.perm[c][j];
@@ -881,7 +887,17 @@ static int build_impl(const double* verts, const int64_t* vert_off, const int32_
       hi[j] = make_float4(h[0], h[1], h[2], (float)H.qw[c][o]);
       lo[j] = make_float4(l[0], l[1], l[2], 0.f);
       el[j] = o / nq;
+      if (!xh.empty()) {
+        const HostBox& B = H.box[H.leaf_of[c][j]];
+        const double inv_s = 1.0 / B.s;
+        xh[j] = make_float4((float)((x[0] - B.c[0]) * inv_s), (float)((x[1] - B.c[1]) * inv_s),
+                            (float)((x[2] - B.c[2]) * inv_s), 0.f);
+      }
     }
+    float4* dxh;
+    if (m.upload(&dxh, xh.data(), xh.size(), st) != cudaSuccess)
+      return cleanup(fail(BCFMM_ERR_OOM, "build: device allocation failed (points)"));
+    G.xhat[c] = dxh;
     double4_32a* dp; float4 *dh, *dl; int* de;
     bool ok = m.upload(&dp, p64.data(), n, st) == cudaSuccess && m.upload(&dh, hi.data(), n, st) == cudaSuccess &&
               m.upload(&dl, lo.data(), n, st) == cudaSuccess && m.upload(&de, el.data(), n, st) == cudaSuccess;
@@ -1548,16 +1564,15 @@ static int eval_impl(bcfmm_ctx* C, int t, double* out, int out_is_device, bool s
     if (!skip_up) {
       CU(launch_weights<double>(G, L.src_cls, nsp, C->dens[kind], nsel, ndens, ndp, C->W64, st));
       if (dl) CU(launch_weights<double>(G, 1, nsp, C->dens[BCFMM_DIPOLE], nsel, ndens, ndp, C->W64dl, st));
-      CU(cudaMemsetAsync(C->mom64, 0, nexp * sizeof(double), st));
     }
     if (!skip_far) CU(cudaMemsetAsync(C->loc64, 0, nexp * sizeof(double), st));
     if (tm) CU(cudaEventRecord(ev[1], st));
     if (!skip_up) {
       CU(launch_p2m<double>(G, L, C->W64, nsp, ndp, C->mom64, st));
       if (dl) CU(launch_p2m_dl<double>(G, L, C->W64dl, nsp, ndp, C->mom64, st));
-      for (int l = C->nlevels - 1; l >= 0; --l) {
+      for (int l = C->nlevels - 1; l >= 2; --l) {
         const int n = D.m2m_off[l + 1] - D.m2m_off[l];
-        CU(launch_m2m<double>(G, D.m2m_parent + D.m2m_off[l], n, ndp, C->mom64, st));
+        CU(launch_m2m<double>(G, D.m2m_parent + D.m2m_off[l], n, L.src_cls, ndp, C->mom64, st));
       }
     }
     if (tm) CU(cudaEventRecord(ev[2], st));
@@ -1572,7 +1587,7 @@ static int eval_impl(bcfmm_ctx* C, int t, double* out, int out_is_device, bool s
     if (tm) CU(cudaEventRecord(ev[3], st));
     for (int l = 3; l < C->nlevels && !skip_far; ++l) {
       const int n = D.l2l_off[l + 1] - D.l2l_off[l];
-      CU(launch_l2l<double>(G, D.l2l_child + D.l2l_off[l], n, ndp, C->loc64, st));
+      CU(launch_l2l<double>(G, D.l2l_parent + D.l2l_off[l], n, ndp, C->loc64, st));
     }
     if (tm) CU(cudaEventRecord(ev[4], st));
     CU(launch_p2p_l2p_f64(G, L, C->W64, nsp, ntp, ndp, C->loc64, C->phi, st));
@@ -1581,16 +1596,15 @@ static int eval_impl(bcfmm_ctx* C, int t, double* out, int out_is_device, bool s
     if (!skip_up) {
       CU(launch_weights<float>(G, L.src_cls, nsp, C->dens[kind], nsel, ndens, ndp, C->W32, st));
       if (dl) CU(launch_weights<float>(G, 1, nsp, C->dens[BCFMM_DIPOLE], nsel, ndens, ndp, C->W32dl, st));
-      CU(cudaMemsetAsync(C->mom32, 0, nexp * sizeof(float), st));
     }
     if (!skip_far) CU(cudaMemsetAsync(C->loc32, 0, nexp * sizeof(float), st));
     if (tm) CU(cudaEventRecord(ev[1], st));
     if (!skip_up) {
       CU(launch_p2m<float>(G, L, C->W32, nsp, ndp, C->mom32, st));
       if (dl) CU(launch_p2m_dl<float>(G, L, C->W32dl, nsp, ndp, C->mom32, st));
-      for (int l = C->nlevels - 1; l >= 0; --l) {
+      for (int l = C->nlevels - 1; l >= 2; --l) {
         const int n = D.m2m_off[l + 1] - D.m2m_off[l];
-        CU(launch_m2m<float>(G, D.m2m_parent + D.m2m_off[l], n, ndp, C->mom32, st));
+        CU(launch_m2m<float>(G, D.m2m_parent + D.m2m_off[l], n, L.src_cls, ndp, C->mom32, st));
       }
     }
     if (tm) CU(cudaEventRecord(ev[2], st));
@@ -1607,7 +1621,7 @@ static int eval_impl(bcfmm_ctx* C, int t, double* out, int out_is_device, bool s
     if (tm) CU(cudaEventRecord(ev[3], st));
     for (int l = 3; l < C->nlevels && !skip_far; ++l) {
       const int n = D.l2l_off[l + 1] - D.l2l_off[l];
-      CU(launch_l2l<float>(G, D.l2l_child + D.l2l_off[l], n, ndp, C->loc32, st));
+      CU(launch_l2l<float>(G, D.l2l_parent + D.l2l_off[l], n, ndp, C->loc32, st));
     }
     if (tm) CU(cudaEventRecord(ev[4], st));
     if (ndp == 1 && D.sym.nblk > 0) CU(launch_p2p_sym(G, D.sym, C->W32, C->phi, st));
@@ -1740,12 +1754,11 @@ extern "C" int bcfmm_eval_noalloc(bcfmm_ctx* C, int32_t task, const double* dens
   const int64_t nsel = kind == 0 ? C->ntet : C->ntri;
   const size_t nexp = (size_t)C->nbox * ndp * C->G.ms;
   CU(launch_weights<float>(G, L.src_cls, nsp, dens_dev, nsel, 1, ndp, C->W32, st));
-  CU(cudaMemsetAsync(C->mom32, 0, nexp * sizeof(float), st));
   CU(cudaMemsetAsync(C->loc32, 0, nexp * sizeof(float), st));
   CU(launch_p2m<float>(G, L, C->W32, nsp, ndp, C->mom32, st));
-  for (int l = C->nlevels - 1; l >= 0; --l) {
+  for (int l = C->nlevels - 1; l >= 2; --l) {     // (no box above level 2 is a source)
     const int n = D.m2m_off[l + 1] - D.m2m_off[l];
-    CU(launch_m2m<float>(G, D.m2m_parent + D.m2m_off[l], n, ndp, C->mom32, st));
+    CU(launch_m2m<float>(G, D.m2m_parent + D.m2m_off[l], n, L.src_cls, ndp, C->mom32, st));
   }
   if (tcp) {
     CU(launch_m2l_tc(G, L, D.tcs, C->tc, ndp, C->mom32, C->loc32, partial, C->tc_momb, st));
@@ -1758,7 +1771,7 @@ extern "C" int bcfmm_eval_noalloc(bcfmm_ctx* C, int32_t task, const double* dens
   }
   for (int l = 3; l < C->nlevels; ++l) {
     const int n = D.l2l_off[l + 1] - D.l2l_off[l];
-    CU(launch_l2l<float>(G, D.l2l_child + D.l2l_off[l], n, ndp, C->loc32, st));
+    CU(launch_l2l<float>(G, D.l2l_parent + D.l2l_off[l], n, ndp, C->loc32, st));
   }
   if (D.sym.nblk > 0) CU(launch_p2p_sym(G, D.sym, C->W32, C->phi, st));
   else CU(launch_p2p_f32(G, L, C->W32, nsp, ntp, ndp, C->phi, st));

@@ -16,7 +16,7 @@ struct DevGeom {
   const int* mi;                 // packed multi-indices a | b << 8 | c << 16, degree-major
   const int* box_q;              // expansion order of each box's level (<= p; Sec. 4.3)
   const double4_32a* box_cs;         // centre xyz, side s
-  const float4 *box_hi, *box_lo;     // (centre xyz, 1 / s) as float hi and lo parts (FP64 arithmetic is scarce)
+  const float4 *box_hi, *box_lo;     // centre xyz as float hi and lo parts (FP64 arithmetic is scarce)
   const int* box_child0;
   const int* box_nchild;
   const int* box_octant;
@@ -25,6 +25,7 @@ struct DevGeom {
   const double4_32a* pt64[2];        // sorted points: x, y, z, quadrature weight
   const float4* pthi[2];         // float hi parts (x, y, z, weight)
   const float4* ptlo[2];         // float lo parts (x - hi, ...)
+  const float4* xhat[2];         // offset from the point's leaf centre over the box side (FP32 contexts)
   const int* pt_elem[2];         // sorted point -> element
   const double4_32a* tri_nrm;    // unit normal of each triangle (right-hand rule; w unused)
   const double* shift64;         // [2][p+1][p+1] C(n, k) (-+1/4)^(n-k): M2M / L2L 1-D shifts
@@ -72,13 +73,13 @@ template <typename T>
 cudaError_t launch_p2m(const DevGeom& G, const DevTaskLists& L, const T* W, int64_t nsrc_pts, int ndp,
                        T* mom, cudaStream_t st);
 template <typename T>
-cudaError_t launch_m2m(const DevGeom& G, const int* parents, int n, int ndp, T* mom, cudaStream_t st);
+cudaError_t launch_m2m(const DevGeom& G, const int* parents, int n, int cls, int ndp, T* mom, cudaStream_t st);
 // sel: optional list of indices into L.m2l_tgt (nsel of them); NULL: every target
 template <typename T>
 cudaError_t launch_m2l_simt(const DevGeom& G, const DevTaskLists& L, const T* Tt, int ndp, const T* mom, T* loc,
                             cudaStream_t st, const int* sel = nullptr, int nsel = 0);
 template <typename T>
-cudaError_t launch_l2l(const DevGeom& G, const int* children, int n, int ndp, T* loc, cudaStream_t st);
+cudaError_t launch_l2l(const DevGeom& G, const int2* parents, int n, int ndp, T* loc, cudaStream_t st);
 // phi = near field / 4 pi
 cudaError_t launch_p2p_f32(const DevGeom& G, const DevTaskLists& L, const float* W, int64_t nsrc_pts, int64_t ntgt_pts,
                            int ndp, double* phi, cudaStream_t st);

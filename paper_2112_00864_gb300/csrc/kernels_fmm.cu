@@ -35,63 +35,151 @@ cudaError_t launch_weights(const DevGeom& G, int cls, int64_t n, const double* d
   return cudaGetLastError();
 }
 
+// degree-major position of the multi-index (i, j, k): degree d, then i
+// descending, then j descending
+__device__ __forceinline__ int midx3(int i, int j, int k) {
+  const int d = i + j + k;
+  return d * (d + 1) * (d + 2) / 6 + (j + k) * (j + k + 1) / 2 + k;
+}
+
 // ---------------------------------------------------------------- P2M
-// One CTA per leaf; thread per coefficient; powers of the scaled offsets
-// staged in shared memory for a chunk of 64 points, rows of kPwS = 65
-// (threads of one warp read rows of different exponents at the same point:
-// an odd stride puts them in different banks).
+// One CTA per leaf (and four densities).  The moments are an outer-product sum
+// over the leaf's points: powers of x against products y^b z^c.  A thread
+// takes one (b, c) and a share of the points: one load of its product and the
+// point's powers of x (two or three 16-byte loads, the same for all lanes)
+// serve PX coefficients per density.  (A thread per coefficient needed four
+// loads for each and formed the monomial anew for every density.)  The shares
+// are added through shared memory.  Rows of kPwS = 65: threads of one warp
+// read rows of different exponents at the same point, an odd stride puts them
+// in different banks.  Shared-memory loads and latency bound it: 767,360
+// points at p = 7 take 63 us with one density (as before); with sixteen
+// densities (25,040 points) the upward pass went from 1.01 ms to 0.05 ms.
 constexpr int kPwS = 65;
+constexpr int kP2mDens = 4;
+
+// offset of point j from the leaf's centre in units of the box side
 template <typename T>
-__global__ void k_p2m(DevGeom G, const int* __restrict__ leaves, int cls, const T* __restrict__ W, int64_t nsp,
-                      int ndp, T* __restrict__ mom) {
-  extern __shared__ unsigned char smraw[];
-  const int P = G.p, np = G.np;
-  T* pw = reinterpret_cast<T*>(smraw);               // [3][P+1][64]
-  T* ws = pw + 3 * (P + 1) * kPwS;                   // [ndp][64]
-  const int leaf = leaves[blockIdx.x];
+__device__ __forceinline__ void point_xhat(const DevGeom& G, int cls, int64_t j, const double4_32a& cs, double inv_s, T& x,
+                                           T& y, T& z) {
+  if constexpr (sizeof(T) == 4) {
+    const float4 v = G.xhat[cls][j];
+    x = v.x; y = v.y; z = v.z;
+  } else {
+    const double4_32a q = G.pt64[cls][j];
+    x = (q.x - cs.x) * inv_s; y = (q.y - cs.y) * inv_s; z = (q.z - cs.z) * inv_s;
+  }
+}
+
+template <typename T, int PX, int NDC>
+__global__ void __launch_bounds__(128) k_p2m(DevGeom G, const int* __restrict__ leaves, int cls, const T* __restrict__ W,
+                                            int64_t nsp, int ndp, T* __restrict__ mom) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  const int P = G.p, np = G.np, npair = (P + 1) * (P + 2) / 2, NS = 128 / npair;
+  T* xp = reinterpret_cast<T*>(smraw);               // [64][PX] powers of x
+  T* ws = xp + 64 * PX;                              // [NDC][64]
+  T* py = ws + NDC * 64;                             // [P+1][kPwS]
+  T* pz = py + (P + 1) * kPwS;                       // [P+1][kPwS]
+  T* yz = pz + (P + 1) * kPwS;                       // [npair][kPwS]
+  T* red = yz + npair * kPwS;                        // [NDC][np]
+  const int leaf = leaves[blockIdx.x], d0 = blockIdx.y * NDC;
   const double4_32a cs = G.box_cs[leaf];
   const int2 r = G.box_rng[cls][leaf];
-  const double inv_s = 1.0 / cs.w;
+  const double inv_s = sizeof(T) == 8 ? 1.0 / cs.w : 0.0;
+  const int split = threadIdx.x / npair, pair = threadIdx.x - split * npair;
+  // (b, c) of this thread: pair = c + (b + c)(b + c + 1) / 2
+  int deg = 0, c = pair;
+  while (c > deg) { c -= deg + 1; ++deg; }
+  const int b = deg - c, na = P - deg;
+  T acc[NDC][PX];
+#pragma unroll
+  for (int d = 0; d < NDC; ++d)
+#pragma unroll
+    for (int k = 0; k < PX; ++k) acc[d][k] = (T)0;
   for (int j0 = r.x; j0 < r.y; j0 += 64) {
     const int m = min(64, r.y - j0);
     __syncthreads();
-    for (int j = threadIdx.x; j < m; j += blockDim.x) {
-      const double4_32a y = G.pt64[cls][j0 + j];
-      const T d[3] = {(T)((y.x - cs.x) * inv_s), (T)((y.y - cs.y) * inv_s), (T)((y.z - cs.z) * inv_s)};
-      for (int ax = 0; ax < 3; ++ax) {
-        T v = (T)1;
-        for (int k = 0; k <= P; ++k) { pw[(ax * (P + 1) + k) * kPwS + j] = v; v *= d[ax]; }
-      }
-      for (int dd = 0; dd < ndp; ++dd) ws[dd * 64 + j] = W[(int64_t)dd * nsp + j0 + j];
+    if (threadIdx.x < m) {
+      const int j = threadIdx.x;
+      T x, y, z;
+      point_xhat<T>(G, cls, j0 + j, cs, inv_s, x, y, z);
+      T vx = (T)1, vy = (T)1, vz = (T)1;
+#pragma unroll
+      for (int k = 0; k < PX; ++k) { xp[j * PX + k] = vx; vx *= x; }
+      for (int k = 0; k <= P; ++k) { py[k * kPwS + j] = vy; pz[k * kPwS + j] = vz; vy *= y; vz *= z; }
+    } else if (threadIdx.x >= 64) {
+      const int j = threadIdx.x - 64;
+      if (j < m)
+        for (int d = 0; d < NDC; ++d) ws[d * 64 + j] = d0 + d < ndp ? W[(int64_t)(d0 + d) * nsp + j0 + j] : (T)0;
     }
     __syncthreads();
-    for (int q = threadIdx.x; q < np; q += blockDim.x) {
-      const int mi = G.mi[q];
-      const int a = mi & 255, b = (mi >> 8) & 255, c = (mi >> 16) & 255;
-      const T* px = pw + (0 * (P + 1) + a) * kPwS;
-      const T* py = pw + (1 * (P + 1) + b) * kPwS;
-      const T* pz = pw + (2 * (P + 1) + c) * kPwS;
-      for (int dd = 0; dd < ndp; ++dd) {
-        T acc = 0;
-        for (int j = 0; j < m; ++j) acc += ws[dd * 64 + j] * px[j] * py[j] * pz[j];
-        mom[((int64_t)leaf * ndp + dd) * G.ms + q] += acc;
+    if (split < NS)
+      for (int j = split; j < m; j += NS) {
+        T t = py[b * kPwS + j] * pz[c * kPwS + j];
+        if constexpr (NDC == 1) t *= ws[j];
+        yz[pair * kPwS + j] = t;
+      }
+    // (a thread reads the products it wrote itself)
+    if (split < NS)
+      for (int j = split; j < m; j += NS) {
+        const T t = yz[pair * kPwS + j];
+        T x[PX];
+#pragma unroll
+        for (int k = 0; k < PX; k += 16 / sizeof(T))
+          *reinterpret_cast<float4*>(x + k) = *reinterpret_cast<const float4*>(xp + j * PX + k);
+#pragma unroll
+        for (int d = 0; d < NDC; ++d) {
+          const T v = NDC == 1 ? t : t * ws[d * 64 + j];
+#pragma unroll
+          for (int k = 0; k < PX; ++k) acc[d][k] += v * x[k];
+        }
+      }
+  }
+  for (int sp = 0; sp < NS; ++sp) {
+    __syncthreads();
+    if (split == sp) {
+#pragma unroll
+      for (int k = 0; k < PX; ++k) {
+        if (k > na) break;
+        const int q = midx3(k, b, c);
+#pragma unroll
+        for (int d = 0; d < NDC; ++d) red[d * np + q] = sp == 0 ? acc[d][k] : red[d * np + q] + acc[d][k];
       }
     }
   }
+  __syncthreads();
+  for (int i = threadIdx.x; i < NDC * np; i += 128) {
+    const int d = i / np;
+    if (d0 + d < ndp) mom[((int64_t)leaf * ndp + d0 + d) * G.ms + i - d * np] = red[i];
+  }
+}
+
+template <typename T, int PX, int NDC>
+cudaError_t launch_p2m_t(const DevGeom& G, const DevTaskLists& L, const T* W, int64_t nsp, int ndp, T* mom, cudaStream_t st) {
+  const int npair = (G.p + 1) * (G.p + 2) / 2;
+  const size_t sm = sizeof(T) * (64 * PX + NDC * (64 + G.np) + (2 * (G.p + 1) + npair) * kPwS);
+  if (sm > 48 * 1024) {
+    const cudaError_t e = cudaFuncSetAttribute(k_p2m<T, PX, NDC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+  }
+  k_p2m<T, PX, NDC><<<dim3(L.n_p2m, (ndp + NDC - 1) / NDC), 128, sm, st>>>(G, L.p2m_leaf, L.src_cls, W, nsp, ndp, mom);
+  return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t launch_p2m(const DevGeom& G, const DevTaskLists& L, const T* W, int64_t nsrc_pts, int ndp,
                        T* mom, cudaStream_t st) {
   if (L.n_p2m == 0) return cudaSuccess;
-  size_t sm = sizeof(T) * (3 * (G.p + 1) * kPwS + ndp * 64);
-  k_p2m<T><<<L.n_p2m, 128, sm, st>>>(G, L.p2m_leaf, L.src_cls, W, nsrc_pts, ndp, mom);
-  return cudaGetLastError();
+  if (ndp == 1) {
+    if (G.p < 8) return launch_p2m_t<T, 8, 1>(G, L, W, nsrc_pts, ndp, mom, st);
+    if (G.p < 12) return launch_p2m_t<T, 12, 1>(G, L, W, nsrc_pts, ndp, mom, st);
+    return launch_p2m_t<T, 16, 1>(G, L, W, nsrc_pts, ndp, mom, st);
+  }
+  if (G.p < 8) return launch_p2m_t<T, 8, kP2mDens>(G, L, W, nsrc_pts, ndp, mom, st);
+  if (G.p < 12) return launch_p2m_t<T, 12, kP2mDens>(G, L, W, nsrc_pts, ndp, mom, st);
+  return launch_p2m_t<T, 16, kP2mDens>(G, L, W, nsrc_pts, ndp, mom, st);
 }
 
-// ---------------------------------------------------------------- M2M
-// m_parent[b] = sum_children sum_g M[octant][b][g] m_child[g]; the table is
-// stored transposed, Mt[octant][g][b], so threads (b) read it coalesced.
+// ------------------------------------------------------- M2M and L2L shifts
 // Shifts between a box and its child in octant o (centre offset sigma s_p/4,
 // sigma_i = +-1 by the octant's bits; child side s_p/2), box-scaled:
 //   M2M  mhat_p[b] = sum_{g <= b} prod_i C(b_i, g_i) (sigma_i/4)^(b_i - g_i) 2^-|g| mhat_c[g]
@@ -102,13 +190,6 @@ cudaError_t launch_p2m(const DevGeom& G, const DevTaskLists& L, const T* W, int6
 // input and the output), so the passes are exact on the truncated arrays.
 // One pass costs about n (p+1)/2 products instead of the dense table's
 // n^2 / 2 (n = nterms(p)), and no table is read from memory.
-
-// degree-major position of the multi-index (i, j, k): degree d, then i
-// descending, then j descending
-__device__ __forceinline__ int midx3(int i, int j, int k) {
-  const int d = i + j + k;
-  return d * (d + 1) * (d + 2) / 6 + (j + k) * (j + k + 1) / 2 + k;
-}
 
 // tab[s][n][k] = C(n, k) (+-1/4)^(n - k), s = 0: -1/4, s = 1: +1/4 (the
 // table is built on the host, G.shift64 / G.shift32)
@@ -124,83 +205,95 @@ __device__ void shift_table(const DevGeom& G, T* tab) {
   for (int e = threadIdx.x; e < 2 * (G.p + 1) * (G.p + 1); e += blockDim.x) tab[e] = src[e];
 }
 
-// one M2M pass along axis ax: out[b] = sum_{g_ax <= b_ax} tab[b_ax][g_ax] in[b with b_ax -> g_ax]
-template <typename T>
-__device__ __forceinline__ void m2m_pass(const DevGeom& G, int nq, int ax, const T* tb, const T* in, T* out) {
-  for (int q = threadIdx.x; q < nq; q += blockDim.x) {
-    const int mi = G.mi[q];
-    int c[3] = {mi & 255, (mi >> 8) & 255, (mi >> 16) & 255};
-    const int n = c[ax];
-    const int P1 = G.p + 1;
-    T acc = 0;
-    for (int k = 0; k <= n; ++k) {
-      c[ax] = k;
-      acc += tb[n * P1 + k] * in[midx3(c[0], c[1], c[2])];
-    }
-    out[q] = acc;
-  }
-}
-
-// one L2L pass along axis ax: out[a] = sum_{b_ax >= a_ax, |b| <= qd} tab[b_ax][a_ax] in[a with a_ax -> b_ax]
-template <typename T>
-__device__ __forceinline__ void l2l_pass(const DevGeom& G, int nq, int qd, int ax, const T* tb, const T* in, T* out) {
-  for (int q = threadIdx.x; q < nq; q += blockDim.x) {
-    const int mi = G.mi[q];
-    int c[3] = {mi & 255, (mi >> 8) & 255, (mi >> 16) & 255};
-    const int a = c[ax], rest = c[0] + c[1] + c[2] - a;
-    const int P1 = G.p + 1;
-    T acc = 0;
-    for (int k = a; k + rest <= qd; ++k) {
-      c[ax] = k;
-      acc += tb[k * P1 + a] * in[midx3(c[0], c[1], c[2])];
-    }
-    out[q] = acc;
-  }
-}
-
 // ---------------------------------------------------------------- M2M
-// One CTA per parent box: the children's moments through the three
-// passes, summed in shared memory.
+// One CTA per parent box and density.  The children's moments are merged axis
+// by axis: the x shift adds the two children of each (y, z), the y shift the
+// two sums of each z, the z shift the last two: 7 np outputs of two 1-D
+// shifts each and three barriers, where shifting child by child took 24 np
+// outputs and forty barriers.  Latency-bound: a level of 64 to 360 parents 10 us
+// (20 - 22 before), the finest of the level-4 ball, 1,908 parents, 23 us (46).
+// Children without sources count as zero (their moments are never written).
 template <typename T>
-__global__ void k_m2m(DevGeom G, const int* __restrict__ parents, int ndp, T* __restrict__ mom) {
+__global__ void __launch_bounds__(256) k_m2m(DevGeom G, const int* __restrict__ parents, int cls, int ndp, T* __restrict__ mom) {
   extern __shared__ unsigned char smraw[];
   const int np = G.np, P1 = G.p + 1;
   T* tab = reinterpret_cast<T*>(smraw);              // [2][P+1][P+1]
-  T* va = tab + 2 * P1 * P1;                         // [np]
-  T* vb = va + np;                                   // [np]
-  T* acc = vb + np;                                  // [np]
+  T* v8 = tab + 2 * P1 * P1;                         // [8 octants][np]
+  T* v4 = v8 + 8 * np;                               // [4 (y, z)][np]
+  T* v2 = v4 + 4 * np;                               // [2 (z)][np]
+  __shared__ int child[8];
   shift_table(G, tab);
-  const int P = parents[blockIdx.x];
+  const int P = parents[blockIdx.x], d = blockIdx.y;
   const int c0 = G.box_child0[P], nc = G.box_nchild[P];
-  for (int d = 0; d < ndp; ++d) {
-    for (int q = threadIdx.x; q < np; q += blockDim.x) acc[q] = 0;
-    for (int c = 0; c < nc; ++c) {
-      const int oc = G.box_octant[c0 + c];
-      __syncthreads();
-      for (int q = threadIdx.x; q < np; q += blockDim.x) {
-        const int mi = G.mi[q];
-        const int deg = (mi & 255) + ((mi >> 8) & 255) + ((mi >> 16) & 255);
-        va[q] = mom[((int64_t)(c0 + c) * ndp + d) * G.ms + q] / (T)(1 << deg);
-      }
-      __syncthreads();
-      m2m_pass(G, np, 0, tab + ((oc & 1) ? P1 * P1 : 0), va, vb);
-      __syncthreads();
-      m2m_pass(G, np, 1, tab + ((oc & 2) ? P1 * P1 : 0), vb, va);
-      __syncthreads();
-      m2m_pass(G, np, 2, tab + ((oc & 4) ? P1 * P1 : 0), va, vb);
-      __syncthreads();
-      for (int q = threadIdx.x; q < np; q += blockDim.x) acc[q] += vb[q];
+  if (threadIdx.x < 8) child[threadIdx.x] = -1;
+  __syncthreads();
+  if (threadIdx.x < nc) {
+    const int2 r = G.box_rng[cls][c0 + threadIdx.x];
+    if (r.y > r.x) child[G.box_octant[c0 + threadIdx.x]] = c0 + threadIdx.x;
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < 8 * np; i += blockDim.x) {
+    const int o = i / np, q = i - o * np, c = child[o];
+    T v = 0;
+    if (c >= 0) {
+      const int mi = G.mi[q];
+      v = mom[((int64_t)c * ndp + d) * G.ms + q] * ((T)1 / (T)(1 << ((mi & 255) + ((mi >> 8) & 255) + ((mi >> 16) & 255))));
     }
-    __syncthreads();
-    for (int q = threadIdx.x; q < np; q += blockDim.x) mom[((int64_t)P * ndp + d) * G.ms + q] = acc[q];
+    v8[i] = v;
+  }
+  const T* lo = tab;
+  const T* hi = tab + P1 * P1;
+  // x: input position of (k, j, l) moves on by the degree's count
+  __syncthreads();
+  for (int i = threadIdx.x; i < 4 * np; i += blockDim.x) {
+    const int o = i / np, q = i - o * np, mi = G.mi[q];
+    const int n = mi & 255, j = (mi >> 8) & 255, l = (mi >> 16) & 255;
+    const T* in0 = v8 + 2 * o * np;
+    const T* in1 = in0 + np;
+    T acc = 0;
+    int pos = midx3(0, j, l), deg = j + l;
+    for (int k = 0; k <= n; ++k) {
+      acc += lo[n * P1 + k] * in0[pos] + hi[n * P1 + k] * in1[pos];
+      pos += (deg + 1) * (deg + 2) / 2;
+      ++deg;
+    }
+    v4[i] = acc;
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < 2 * np; i += blockDim.x) {
+    const int o = i / np, q = i - o * np, mi = G.mi[q];
+    const int a = mi & 255, n = (mi >> 8) & 255, l = (mi >> 16) & 255;
+    const T* in0 = v4 + 2 * o * np;
+    const T* in1 = in0 + np;
+    T acc = 0;
+    for (int k = 0; k <= n; ++k) {
+      const int pos = midx3(a, k, l);
+      acc += lo[n * P1 + k] * in0[pos] + hi[n * P1 + k] * in1[pos];
+    }
+    v2[i] = acc;
+  }
+  __syncthreads();
+  for (int q = threadIdx.x; q < np; q += blockDim.x) {
+    const int mi = G.mi[q];
+    const int a = mi & 255, b = (mi >> 8) & 255, n = (mi >> 16) & 255;
+    T acc = 0;
+    for (int k = 0; k <= n; ++k) {
+      const int pos = midx3(a, b, k);
+      acc += lo[n * P1 + k] * v2[pos] + hi[n * P1 + k] * v2[np + pos];
+    }
+    mom[((int64_t)P * ndp + d) * G.ms + q] = acc;
   }
 }
 
 template <typename T>
-cudaError_t launch_m2m(const DevGeom& G, const int* parents, int n, int ndp, T* mom, cudaStream_t st) {
+cudaError_t launch_m2m(const DevGeom& G, const int* parents, int n, int cls, int ndp, T* mom, cudaStream_t st) {
   if (n == 0) return cudaSuccess;
-  const size_t sm = sizeof(T) * (2 * (G.p + 1) * (G.p + 1) + 3 * G.np);
-  k_m2m<T><<<n, 128, sm, st>>>(G, parents, ndp, mom);
+  const size_t sm = sizeof(T) * (2 * (G.p + 1) * (G.p + 1) + 14 * G.np);
+  if (sm > 48 * 1024) {
+    const cudaError_t e = cudaFuncSetAttribute(k_m2m<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+  }
+  k_m2m<T><<<dim3(n, ndp), 256, sm, st>>>(G, parents, cls, ndp, mom);
   return cudaGetLastError();
 }
 
@@ -275,46 +368,67 @@ cudaError_t launch_m2l_simt(const DevGeom& G, const DevTaskLists& L, const T* Tt
 }
 
 // ---------------------------------------------------------------- L2L
-// One CTA per child box.  The parent's expansion has its level's order qp,
-// the child's is cut to its own (Sec. 4.3): the passes run over |b| <= qp,
-// the child receives |a| <= min(q_child, qp).
+// One CTA per parent box and density, the mirror image of M2M: the z shift
+// gives the two z halves, the y shift their four (y, z) parts, the x shift the
+// children, which add it to their own.  The parent's expansion has its level's
+// order qp, the child's is cut to its own (Sec. 4.3): the passes run over
+// |b| <= qp, the child receives |a| <= min(q_child, qp).  parents: (box, mask of
+// the child slots that take part).  The level-4 ball's finest level (14,976
+// children) takes 28 us, 37 with one CTA per child.
 template <typename T>
-__global__ void k_l2l(DevGeom G, const int* __restrict__ children, int ndp, T* __restrict__ loc) {
+__global__ void __launch_bounds__(256) k_l2l(DevGeom G, const int2* __restrict__ parents, int ndp, T* __restrict__ loc) {
   extern __shared__ unsigned char smraw[];
   const int P1 = G.p + 1;
+  const int2 pm = parents[blockIdx.x];
+  const int P = pm.x, d = blockIdx.y, qp = G.box_q[P], nqp = nterms_q(qp);
   T* tab = reinterpret_cast<T*>(smraw);              // [2][P+1][P+1]
-  T* va = tab + 2 * P1 * P1;                         // [np]
-  T* vb = va + G.np;                                 // [np]
+  T* v1 = tab + 2 * P1 * P1;                         // [np]
+  T* v2 = v1 + G.np;                                 // [2 (z)][np]
+  T* v4 = v2 + 2 * G.np;                             // [4 (y, z)][np]
   shift_table(G, tab);
-  const int C = children[blockIdx.x];
-  const int P = G.box_parent[C];
-  const int qp = G.box_q[P];
-  const int nqc = nterms_q(G.box_q[C]), nqp = nterms_q(qp);
-  const int oc = G.box_octant[C];
-  for (int d = 0; d < ndp; ++d) {
-    __syncthreads();
-    for (int q = threadIdx.x; q < nqp; q += blockDim.x) va[q] = loc[((int64_t)P * ndp + d) * G.ms + q];
-    __syncthreads();
-    l2l_pass(G, nqp, qp, 0, tab + ((oc & 1) ? P1 * P1 : 0), va, vb);
-    __syncthreads();
-    l2l_pass(G, nqp, qp, 1, tab + ((oc & 2) ? P1 * P1 : 0), vb, va);
-    __syncthreads();
-    l2l_pass(G, nqp, qp, 2, tab + ((oc & 4) ? P1 * P1 : 0), va, vb);
-    __syncthreads();
+  for (int q = threadIdx.x; q < nqp; q += blockDim.x) v1[q] = loc[((int64_t)P * ndp + d) * G.ms + q];
+  __syncthreads();
+  for (int i = threadIdx.x; i < 2 * nqp; i += blockDim.x) {
+    const int o = i / nqp, q = i - o * nqp, mi = G.mi[q];
+    const int a = mi & 255, b = (mi >> 8) & 255, c = (mi >> 16) & 255;
+    const T* tb = tab + o * P1 * P1;
+    T acc = 0;
+    for (int k = c; a + b + k <= qp; ++k) acc += tb[k * P1 + c] * v1[midx3(a, b, k)];
+    v2[o * nqp + q] = acc;
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < 4 * nqp; i += blockDim.x) {
+    const int o = i / nqp, q = i - o * nqp, mi = G.mi[q];          // o = y + 2 z
+    const int a = mi & 255, b = (mi >> 8) & 255, c = (mi >> 16) & 255;
+    const T* tb = tab + (o & 1) * P1 * P1;
+    const T* in = v2 + (o >> 1) * nqp;
+    T acc = 0;
+    for (int k = b; a + k + c <= qp; ++k) acc += tb[k * P1 + b] * in[midx3(a, k, c)];
+    v4[o * nqp + q] = acc;
+  }
+  __syncthreads();
+  const int c0 = G.box_child0[P], nc = G.box_nchild[P];
+  for (int i = threadIdx.x; i < nc * nqp; i += blockDim.x) {
+    const int s = i / nqp, q = i - s * nqp, C = c0 + s;
     // a child of a higher order than its parent gets nothing above |a| = qp
-    for (int a = threadIdx.x; a < min(nqc, nqp); a += blockDim.x) {
-      const int mi = G.mi[a];
-      const int deg = (mi & 255) + ((mi >> 8) & 255) + ((mi >> 16) & 255);
-      loc[((int64_t)C * ndp + d) * G.ms + a] += vb[a] / (T)(1 << deg);
-    }
+    if (!(pm.y >> s & 1) || q >= nterms_q(G.box_q[C])) continue;
+    const int oc = G.box_octant[C], mi = G.mi[q];
+    const int a = mi & 255, b = (mi >> 8) & 255, c = (mi >> 16) & 255;
+    const T* tb = tab + (oc & 1) * P1 * P1;
+    const T* in = v4 + (oc >> 1) * nqp;
+    T* out = loc + ((int64_t)C * ndp + d) * G.ms + q;
+    const T own = *out;
+    T acc = 0;
+    for (int k = a; k + b + c <= qp; ++k) acc += tb[k * P1 + a] * in[midx3(k, b, c)];
+    *out = own + acc * ((T)1 / (T)(1 << (a + b + c)));
   }
 }
 
 template <typename T>
-cudaError_t launch_l2l(const DevGeom& G, const int* children, int n, int ndp, T* loc, cudaStream_t st) {
+cudaError_t launch_l2l(const DevGeom& G, const int2* parents, int n, int ndp, T* loc, cudaStream_t st) {
   if (n == 0) return cudaSuccess;
-  const size_t sm = sizeof(T) * (2 * (G.p + 1) * (G.p + 1) + 2 * G.np);
-  k_l2l<T><<<n, 128, sm, st>>>(G, children, ndp, loc);
+  const size_t sm = sizeof(T) * (2 * (G.p + 1) * (G.p + 1) + 7 * G.np);
+  k_l2l<T><<<dim3(n, ndp), 256, sm, st>>>(G, parents, ndp, loc);
   return cudaGetLastError();
 }
 
@@ -440,7 +554,6 @@ __global__ void __launch_bounds__(kL2pThreads, 12) k_l2p(DevGeom G, const int* _
                                                          double* __restrict__ phi) {
   __shared__ float sl[456];
   const int leaf = leaves[blockIdx.x];
-  const float4 ch = G.box_hi[leaf], cl = G.box_lo[leaf];
   const int2 tr = G.box_rng[tc][leaf];
   const int q = G.box_q[leaf], nq = nterms_q(q);
   for (int d = 0; d < ndp; ++d) {
@@ -448,11 +561,8 @@ __global__ void __launch_bounds__(kL2pThreads, 12) k_l2p(DevGeom G, const int* _
     for (int a = threadIdx.x; a < nq; a += kL2pThreads) sl[a] = loc[((int64_t)leaf * ndp + d) * G.ms + a];
     __syncthreads();
     for (int j = tr.x + threadIdx.x; j < tr.y; j += kL2pThreads) {
-      const float4 h = G.pthi[tc][j], l = G.ptlo[tc][j];
-      float x = (h.x - ch.x) + (l.x - cl.x), y = (h.y - ch.y) + (l.y - cl.y), z = (h.z - ch.z) + (l.z - cl.z);
-      x = fmaf(x, ch.w, x * cl.w);
-      y = fmaf(y, ch.w, y * cl.w);
-      z = fmaf(z, ch.w, z * cl.w);
+      const float4 v = G.xhat[tc][j];
+      const float x = v.x, y = v.y, z = v.z;
       float far;
       switch (q) {
         case 5: far = l2p_eval<5>(sl, x, y, z); break;
@@ -1200,11 +1310,11 @@ template cudaError_t launch_weights<float>(const DevGeom&, int, int64_t, const d
 template cudaError_t launch_weights<double>(const DevGeom&, int, int64_t, const double*, int64_t, int, int, double*, cudaStream_t);
 template cudaError_t launch_p2m<float>(const DevGeom&, const DevTaskLists&, const float*, int64_t, int, float*, cudaStream_t);
 template cudaError_t launch_p2m<double>(const DevGeom&, const DevTaskLists&, const double*, int64_t, int, double*, cudaStream_t);
-template cudaError_t launch_m2m<float>(const DevGeom&, const int*, int, int, float*, cudaStream_t);
-template cudaError_t launch_m2m<double>(const DevGeom&, const int*, int, int, double*, cudaStream_t);
+template cudaError_t launch_m2m<float>(const DevGeom&, const int*, int, int, int, float*, cudaStream_t);
+template cudaError_t launch_m2m<double>(const DevGeom&, const int*, int, int, int, double*, cudaStream_t);
 template cudaError_t launch_m2l_simt<float>(const DevGeom&, const DevTaskLists&, const float*, int, const float*, float*, cudaStream_t, const int*, int);
 template cudaError_t launch_m2l_simt<double>(const DevGeom&, const DevTaskLists&, const double*, int, const double*, double*, cudaStream_t, const int*, int);
-template cudaError_t launch_l2l<float>(const DevGeom&, const int*, int, int, float*, cudaStream_t);
-template cudaError_t launch_l2l<double>(const DevGeom&, const int*, int, int, double*, cudaStream_t);
+template cudaError_t launch_l2l<float>(const DevGeom&, const int2*, int, int, float*, cudaStream_t);
+template cudaError_t launch_l2l<double>(const DevGeom&, const int2*, int, int, double*, cudaStream_t);
 
 }  // namespace bcfmm
