@@ -11,6 +11,7 @@
 #include <cstring>
 #include <map>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/bcfmm.h"
@@ -82,6 +83,7 @@ struct TaskDev {
   DevTaskLists L{};
   TcTaskSched tcs{};                   // tensor-core M2L launches, one per expansion order
   TaylorTaskSched tys{};               // CUDA-core Taylor-form M2L launches, one per expansion order
+  int sp_rows = 0;                     // scratch rows of the near field's chunk blocks
   DevSym sym{};                        // symmetric near field (VtV, FP32 points; nblk 0: none)
   std::vector<int> m2m_off, l2l_off;   // host offsets into the per-level arrays
   int* m2m_parent = nullptr;
@@ -123,17 +125,29 @@ struct bcfmm_ctx {
   // values per density)
   TaylorTables ty{};
   TaylorOffsets ty_offs;               // parent offsets of the tasks' schedules (build only)
-  void* ty_momp = nullptr;             // FP32, or FP64 in a plain FP64 context
-  void* ty_partial = nullptr;
   size_t ty_partial_per_dens = 0;
-  float2* tc_partial = nullptr;        // unit partial sums of the tensor-core M2L
-  uint8_t* tc_momb = nullptr;          // BF16 split moments of the tensor-core M2L
-  // work buffers (sized for the largest ndp seen)
-  int work_ndp = 0;
-  double *W64 = nullptr, *mom64 = nullptr, *loc64 = nullptr, *phi = nullptr, *out_dev = nullptr;
-  float *W32 = nullptr, *mom32 = nullptr, *loc32 = nullptr;
-  double* W64dl = nullptr;               // BtV double-layer point weights w g (double_layer)
-  float* W32dl = nullptr;
+  // work buffers, sized for the largest ndp seen: set 0 for the tasks with
+  // volume sources (VtV, VtB), set 1 for those with boundary sources (BtV), so
+  // that both may run at the same time.  Element type double in an FP64
+  // context, else float.
+  struct Work {
+    int ndp = 0;
+    void *W = nullptr, *mom = nullptr, *loc = nullptr;
+    void* Wdl = nullptr;               // BtV double-layer point weights w g (double_layer)
+    void *ty_momp = nullptr, *ty_partial = nullptr;
+    float2* tc_partial = nullptr;      // unit partial sums of the tensor-core M2L
+    uint8_t* tc_momb = nullptr;        // BF16 split moments of the tensor-core M2L
+  } work[2];
+  double* phi[3] = {nullptr, nullptr, nullptr};   // point potentials per task
+  double* out_dev = nullptr;           // staging of host outputs
+  int out_ndp = 0;
+  // streams and events of the parts of an evaluation that do not depend on
+  // one another (see run_tasks): far[set] the expansions, cor the near
+  // corrections, near1 BtV's near field when volume tasks run too, m2l[set] a
+  // second stream for the orders of the interaction phase
+  cudaStream_t s_far[2] = {nullptr, nullptr}, s_m2l[2] = {nullptr, nullptr}, s_cor = nullptr, s_near1 = nullptr;
+  enum { kEvStart, kEvZero, kEvCor, kEvW0, kEvW1, kEvFar0, kEvFar1, kEvBtv, kEvM0, kEvM1, kEvM2, kEvM3, kEvCount };
+  cudaEvent_t e_part[kEvCount] = {};
   // stats
   int nmesh = 1;
   std::vector<int64_t> mesh_tet_off, mesh_tri_off;
@@ -271,15 +285,16 @@ static int upload_task(bcfmm_ctx* C, const HostSetup& H, int t) {
   }
   {
     // blocks of the packed FP32 near field (long leaves cut into chunks)
+    int nsm = 152;
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, C->device);
     P2pChunks K;
-    build_p2p_chunks(H, t, kP2pChunk, K);
+    build_p2p_chunks(H, t, p2p_chunk(H, t, nsm), K);
     std::vector<int2> grp(K.grp.size()), ginfo(K.grp_row.size());
     for (size_t b = 0; b < K.grp.size(); ++b) grp[b] = make_int2(K.grp[b], K.chunk[b]);
     for (size_t g = 0; g < K.grp_row.size(); ++g) ginfo[g] = make_int2(K.grp_row[g], K.grp_n[g]);
     int *sl, *sro, *ss;
     int2 *srn, *sg, *gi;
     unsigned* gc;
-    float2* scr;
     L.sp_n = (int)K.leaf.size();
     CU(m.upload(&sl, K.leaf.data(), K.leaf.size(), st));
     CU(m.upload(&sro, K.run_off.data(), K.run_off.size(), st));
@@ -289,9 +304,9 @@ static int upload_task(bcfmm_ctx* C, const HostSetup& H, int t) {
     CU(m.upload(&gi, ginfo.data(), ginfo.size(), st));
     CU(m.alloc(&gc, ginfo.size()));
     CU(cudaMemsetAsync(gc, 0, std::max<size_t>(1, ginfo.size()) * sizeof(unsigned), st));
-    CU(m.alloc(&scr, (size_t)K.rows * 2 * 128));     // up to two densities
+    D.sp_rows = K.rows;                              // (the rows are sized with the work buffers)
     L.sp_leaf = sl; L.sp_run_off = sro; L.sp_runs = srn; L.sp_self = ss;
-    L.sp_grp = sg; L.grp_info = gi; L.grp_cnt = gc; L.sp_scratch = scr;
+    L.sp_grp = sg; L.grp_info = gi; L.grp_cnt = gc;
   }
   if (t == 0 && C->prm.precision != BCFMM_FP64 && p2p_sym_pays(H)) {
     // symmetric near field (one density)
@@ -312,8 +327,8 @@ static int upload_task(bcfmm_ctx* C, const HostSetup& H, int t) {
       CU(m.upload(&ft, Y.fin_tgt.data(), Y.fin_tgt.size(), st));
       CU(m.upload(&fso, Y.fin_src_off.data(), Y.fin_src_off.size(), st));
       CU(m.upload(&fs, Y.fin_src.data(), Y.fin_src.size(), st));
-      CU(m.alloc(&S.src, (size_t)Y.nsrc));
-      CU(m.alloc(&S.tgt, (size_t)Y.ntgt));
+      S.nsrc = Y.nsrc;
+      S.ntgt = Y.ntgt;
       S.nblk = (int)Y.leaf.size();
       S.nlarge = Y.nlarge;
       S.leaf = lf; S.run_off = ro; S.runs = rn; S.base = bs; S.self = sf;
@@ -364,6 +379,13 @@ static int upload_task(bcfmm_ctx* C, const HostSetup& H, int t) {
   int* elem_pts;
   CU(m.upload(&elem_pts, ep.data(), ep.size(), st));
   L.elem_pts = elem_pts;
+  {
+    std::vector<double> ew(nte);
+    for (int64_t e = 0; e < nte; ++e) ew[e] = H.qw[tc][nqt * e];
+    double* dw;
+    CU(m.upload(&dw, ew.data(), ew.size(), st));
+    L.elem_w = dw;
+  }
   // tensor-core M2L tiles and their schedule: one persistent launch per
   // expansion order, units dealt to the SMs on the host
   L.err = C->err;
@@ -457,7 +479,7 @@ static int upload_task(bcfmm_ctx* C, const HostSetup& H, int t) {
       CU(m.upload(&dtc, O.tchunk.data(), O.tchunk.size(), st));
       S.wb = dwb; S.wslot = dws; S.ent = den; S.tgt = dtg; S.tchunk = dtc;
       const int slot = f64 ? taylor_slot<double>(O.q) : taylor_slot<float>(O.q);
-      D.tys.partial_per_dens = std::max(D.tys.partial_per_dens, (size_t)O.nchunk * slot);
+      D.tys.partial_per_dens += (size_t)O.nchunk * slot;
     }
     if (!sel.empty()) {
       int* dsel;
@@ -690,6 +712,13 @@ static std::string build_host_mesh(HostSetup& H, const double* verts, int64_t nv
   return "";
 }
 
+static void destroy_parts(bcfmm_ctx* C) {
+  for (cudaStream_t s : {C->s_far[0], C->s_far[1], C->s_m2l[0], C->s_m2l[1], C->s_cor, C->s_near1})
+    if (s) cudaStreamDestroy(s);
+  for (cudaEvent_t e : C->e_part)
+    if (e) cudaEventDestroy(e);
+}
+
 static int build_impl(const double* verts, const int64_t* vert_off, const int32_t* tets, const int64_t* tet_off,
                       const int32_t* tris, const int64_t* tri_off, int32_t nmesh, const bcfmm_params* prm_in,
                       void* stream, bcfmm_ctx** out, const bcfmm_ctx* reuse = nullptr) {
@@ -795,7 +824,7 @@ static int build_impl(const double* verts, const int64_t* vert_off, const int32_
   C->prm = prm;
   C->ntet = ntet;
   C->ntri = ntri;
-  auto cleanup = [&](int code) { C->mem.free_all(); delete C; return code; };
+  auto cleanup = [&](int code) { destroy_parts(C); C->mem.free_all(); delete C; return code; };
 
   if (C->mem.alloc(&C->err, 1) != cudaSuccess || cudaMemsetAsync(C->err, 0, sizeof(int), C->st) != cudaSuccess)
     return cleanup(fail(BCFMM_ERR_OOM, "build: device allocation failed (error word)"));
@@ -1037,6 +1066,19 @@ static int build_impl(const double* verts, const int64_t* vert_off, const int32_
   {
     const int rc = upload_taylor_rows(C);
     if (rc != BCFMM_OK) return cleanup(rc);
+  }
+  {
+    // the expansions are the longer chain of small launches: their blocks go
+    // first where an SM has room, the near field fills the rest
+    int lo = 0, hi = 0;
+    bool ok = cudaDeviceGetStreamPriorityRange(&lo, &hi) == cudaSuccess;
+    for (int k = 0; k < 2; ++k)
+      ok = ok && cudaStreamCreateWithPriority(&C->s_far[k], cudaStreamNonBlocking, hi) == cudaSuccess &&
+           cudaStreamCreateWithPriority(&C->s_m2l[k], cudaStreamNonBlocking, hi) == cudaSuccess;
+    ok = ok && cudaStreamCreateWithPriority(&C->s_cor, cudaStreamNonBlocking, lo) == cudaSuccess &&
+         cudaStreamCreateWithPriority(&C->s_near1, cudaStreamNonBlocking, lo) == cudaSuccess;
+    for (auto& e : C->e_part) ok = ok && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) == cudaSuccess;
+    if (!ok) return cleanup(fail(BCFMM_ERR_CUDA, "build: stream or event creation failed"));
   }
   C->sec_near_dev = wall() - tn;
   C->reuse = nullptr;
@@ -1446,55 +1488,67 @@ extern "C" int bcfmm_build_like(const bcfmm_ctx* base, const bcfmm_params* prm, 
   }
 }
 
-static int ensure_work(bcfmm_ctx* C, int ndp) {
-  if (C->work_ndp >= ndp) return BCFMM_OK;
+static int ensure_work(bcfmm_ctx* C, int set, int ndp) {
+  bcfmm_ctx::Work& w = C->work[set];
+  if (w.ndp >= ndp) return BCFMM_OK;
   auto& m = C->mem;
-  for (void* p : {(void*)C->W64, (void*)C->mom64, (void*)C->loc64, (void*)C->phi, (void*)C->out_dev, (void*)C->W32,
-                  (void*)C->mom32, (void*)C->loc32, (void*)C->tc_partial, (void*)C->tc_momb, (void*)C->ty_momp,
-                  (void*)C->ty_partial, (void*)C->W64dl, (void*)C->W32dl})
+  const int t0 = set == 0 ? 0 : 2, t1 = set == 0 ? 1 : 2;      // the set's tasks
+  for (void* p : {w.W, w.mom, w.loc, w.Wdl, w.ty_momp, w.ty_partial, (void*)w.tc_partial, (void*)w.tc_momb})
     if (p) m.release(p);
-  C->W64dl = nullptr;
-  C->W32dl = nullptr;
-  C->tc_partial = nullptr;
-  C->tc_momb = nullptr;
-  C->ty_momp = C->ty_partial = nullptr;
-  const int64_t npmax = std::max(C->npts[0], C->npts[1]);
-  const int64_t nel = std::max(C->ntet, C->ntri);
-  const size_t nexp = (size_t)C->nbox * ndp * C->G.ms;
+  w = bcfmm_ctx::Work();
   const bool f64 = C->prm.precision == BCFMM_FP64;
-  CU(m.alloc(&C->phi, (size_t)ndp * npmax));
-  CU(m.alloc(&C->out_dev, (size_t)ndp * nel));
-  if (C->prm.double_layer && C->npts[1] > 0) {
-    if (f64) CU(m.alloc(&C->W64dl, (size_t)ndp * C->npts[1]));
-    else CU(m.alloc(&C->W32dl, (size_t)ndp * C->npts[1]));
-  }
-  if (f64) {
-    CU(m.alloc(&C->W64, (size_t)ndp * npmax));
-    CU(m.alloc(&C->mom64, nexp));
-    CU(m.alloc(&C->loc64, nexp));
-    C->W32 = C->mom32 = C->loc32 = nullptr;
-  } else {
-    CU(m.alloc(&C->W32, (size_t)ndp * npmax));
-    CU(m.alloc(&C->mom32, nexp));
-    CU(m.alloc(&C->loc32, nexp));
-    C->W64 = C->mom64 = C->loc64 = nullptr;
-    if (C->tc.nsplit > 0) {
-      CU(m.alloc(&C->tc_partial, std::max<size_t>((size_t)ndp * C->tc_partial_per_dens, 1)));
-      // split moments: one row per (box, density, part)
-      const int kpitch = m2l_tc_kpitch(C->prm.p);
-      CU(m.alloc(&C->tc_momb, (size_t)C->nbox * ndp * C->tc.nsplit * kpitch * 2));
+  const size_t es = f64 ? sizeof(double) : sizeof(float);
+  const size_t nexp = (size_t)C->nbox * ndp * C->G.ms;
+  auto bytes = [&](auto** p, size_t n) {
+    char* q = nullptr;
+    const cudaError_t e = m.alloc(&q, n);
+    *p = reinterpret_cast<std::remove_reference_t<decltype(*p)>>(q);
+    return e;
+  };
+  CU(bytes(&w.W, (size_t)ndp * C->npts[set] * es));
+  CU(bytes(&w.mom, nexp * es));
+  CU(bytes(&w.loc, nexp * es));
+  if (set == 1 && C->prm.double_layer) CU(bytes(&w.Wdl, (size_t)ndp * C->npts[1] * es));
+  for (int t = t0; t <= t1; ++t) {
+    if (C->phi[t]) m.release(C->phi[t]);
+    C->phi[t] = nullptr;
+    CU(m.alloc(&C->phi[t], (size_t)ndp * C->npts[C->task[t].L.tgt_cls]));
+    DevTaskLists& L = C->task[t].L;
+    if (L.sp_scratch) m.release(L.sp_scratch);
+    L.sp_scratch = nullptr;
+    CU(m.alloc(&L.sp_scratch, (size_t)C->task[t].sp_rows * ndp * 128));
+    DevSym& Y = C->task[t].sym;
+    if (Y.src) m.release(Y.src);
+    if (Y.tgt) m.release(Y.tgt);
+    Y.src = nullptr;
+    Y.tgt = nullptr;
+    if (Y.nblk > 0) {                  // (up to four densities take the symmetric form)
+      CU(m.alloc(&Y.src, (size_t)std::min(ndp, 4) * Y.nsrc));
+      CU(m.alloc(&Y.tgt, (size_t)std::min(ndp, 4) * Y.ntgt));
     }
   }
-  if (C->ty.q > 0) {
-    const size_t es = f64 ? sizeof(double) : sizeof(float);
-    char *mp, *pp;
-    CU(m.alloc(&mp, (size_t)C->nbox * ndp * C->ty.gpitch * es));
-    C->ty_momp = mp;
-    CU(m.alloc(&pp, std::max<size_t>((size_t)ndp * C->ty_partial_per_dens, 1) * es));
-    C->ty_partial = pp;
+  if (C->tc.nsplit > 0) {
+    CU(m.alloc(&w.tc_partial, std::max<size_t>((size_t)ndp * C->tc_partial_per_dens, 1)));
+    // split moments: one row per (box, density, part)
+    const int kpitch = m2l_tc_kpitch(C->prm.p);
+    CU(m.alloc(&w.tc_momb, (size_t)C->nbox * ndp * C->tc.nsplit * kpitch * 2));
   }
-  C->work_ndp = ndp;
+  if (C->ty.q > 0) {
+    CU(bytes(&w.ty_momp, (size_t)C->nbox * ndp * C->ty.gpitch * es));
+    CU(bytes(&w.ty_partial, std::max<size_t>((size_t)ndp * C->ty_partial_per_dens, 1) * es));
+  }
+  w.ndp = ndp;
   C->work_gen++;
+  return BCFMM_OK;
+}
+
+static int ensure_out(bcfmm_ctx* C, int ndp) {
+  if (C->out_ndp >= ndp) return BCFMM_OK;
+  if (C->out_dev) C->mem.release(C->out_dev);
+  C->out_dev = nullptr;
+  C->out_ndp = 0;
+  CU(C->mem.alloc(&C->out_dev, (size_t)ndp * std::max(C->ntet, C->ntri)));
+  C->out_ndp = ndp;
   return BCFMM_OK;
 }
 
@@ -1526,114 +1580,252 @@ extern "C" int bcfmm_set_density(bcfmm_ctx* C, int32_t kind, const double* vals,
   if (!is_device) CU(cudaStreamSynchronize(C->st));
   C->ndens[kind] = ndens;
   C->ndp[kind] = pad_ndens(ndens);
-  return ensure_work(C, C->ndp[kind]);
+  // (the other set too, for one density: bcfmm_eval_noalloc takes any task
+  // after one call of this function)
+  for (int set = 0; set < 2; ++set) {
+    const int rc = ensure_work(C, set, (kind == BCFMM_VOLUME) == (set == 0) ? C->ndp[kind] : 1);
+    if (rc != BCFMM_OK) return rc;
+  }
+  return ensure_out(C, C->ndp[kind]);
 }
 
-// skip_up: the moments and weights already hold this task's source side;
-// skip_far: the local expansions already hold this task's far field (both:
-// VtB right after VtV of the same volume density in one graph, VtV's lists
-// covering every box with tet or triangle points).
-static int eval_impl(bcfmm_ctx* C, int t, double* out, int out_is_device, bool skip_up = false,
-                     bool skip_far = false) {
+// What one task is evaluated with.
+struct TaskRun {
+  int t = 0;
+  const double *dens = nullptr, *dip = nullptr;   // source density; BtV's double-layer density or null
+  int ndens = 0, ndp = 0;
+  double* out = nullptr;                          // device
+  void* partial = nullptr;                        // M2L partial sums in place of the work set's, or null
+};
+
+// The parts of an evaluation; T: double in an FP64 context, else float.
+template <typename T>
+struct Parts {
+  bcfmm_ctx* C;
+  const DevGeom& G;
+  explicit Parts(bcfmm_ctx* C_) : C(C_), G(C_->G) {}
+  static constexpr bool f64 = sizeof(T) == 8;
+  bcfmm_ctx::Work& w(const TaskRun& r) const { return C->work[C->task[r.t].L.src_cls]; }
+  T* loc(const TaskRun& r) const { return static_cast<T*>(w(r).loc); }
+
+  cudaError_t weights(const TaskRun& r, cudaStream_t st) const {
+    const DevTaskLists& L = C->task[r.t].L;
+    const int64_t nel = L.src_cls == 0 ? C->ntet : C->ntri, n = C->npts[L.src_cls];
+    cudaError_t e = launch_weights<T>(G, L.src_cls, n, r.dens, nel, r.ndens, r.ndp, static_cast<T*>(w(r).W), st);
+    if (e == cudaSuccess && r.dip) e = launch_weights<T>(G, 1, n, r.dip, nel, r.ndens, r.ndp, static_cast<T*>(w(r).Wdl), st);
+    return e;
+  }
+  cudaError_t zero(const TaskRun& r, cudaStream_t st) const {
+    return cudaMemsetAsync(w(r).loc, 0, (size_t)C->nbox * r.ndp * G.ms * sizeof(T), st);
+  }
+  cudaError_t up(const TaskRun& r, cudaStream_t st) const {
+    const TaskDev& D = C->task[r.t];
+    const DevTaskLists& L = D.L;
+    const int64_t n = C->npts[L.src_cls];
+    T* mom = static_cast<T*>(w(r).mom);
+    cudaError_t e = launch_p2m<T>(G, L, static_cast<T*>(w(r).W), n, r.ndp, mom, st);
+    if (e == cudaSuccess && r.dip) e = launch_p2m_dl<T>(G, L, static_cast<T*>(w(r).Wdl), n, r.ndp, mom, st);
+    for (int l = C->nlevels - 1; l >= 2 && e == cudaSuccess; --l)      // (no box above level 2 is a source)
+      e = launch_m2m<T>(G, D.m2m_parent + D.m2m_off[l], D.m2m_off[l + 1] - D.m2m_off[l], L.src_cls, r.ndp, mom, st);
+    return e;
+  }
+  cudaError_t m2l(const TaskRun& r, cudaStream_t st, const TaylorFork* side) const {
+    const TaskDev& D = C->task[r.t];
+    const DevTaskLists& L = D.L;
+    const T* mom = static_cast<T*>(w(r).mom);
+    if (C->ty.q > 0) {
+      cudaError_t e = launch_m2l_taylor<T>(G, L, D.tys, C->ty, r.ndp, mom, loc(r), static_cast<T*>(w(r).ty_momp),
+                                           static_cast<T*>(r.partial ? r.partial : w(r).ty_partial), st, side);
+      if constexpr (f64)
+        if (e == cudaSuccess && D.tys.nsimt > 0)
+          e = launch_m2l_simt<double>(G, L, C->T64, r.ndp, mom, loc(r), st, D.tys.simt_sel, D.tys.nsimt);
+      return e;
+    }
+    if constexpr (f64) {
+      return launch_m2l_simt<double>(G, L, C->T64, r.ndp, mom, loc(r), st);
+    } else {
+      if (C->tc.nsplit == 0) return launch_m2l_simt<float>(G, L, C->T32, r.ndp, mom, loc(r), st);
+      cudaError_t e = launch_m2l_tc(G, L, D.tcs, C->tc, r.ndp, mom, loc(r),
+                                    r.partial ? static_cast<float2*>(r.partial) : w(r).tc_partial, w(r).tc_momb, st);
+      if (e == cudaSuccess && D.tcs.nsimt > 0)
+        e = launch_m2l_simt<float>(G, L, C->T32, r.ndp, mom, loc(r), st, D.tcs.simt_sel, D.tcs.nsimt);
+      return e;
+    }
+  }
+  cudaError_t l2l(const TaskRun& r, cudaStream_t st) const {
+    const TaskDev& D = C->task[r.t];
+    cudaError_t e = cudaSuccess;
+    for (int l = 3; l < C->nlevels && e == cudaSuccess; ++l)
+      e = launch_l2l<T>(G, D.l2l_parent + D.l2l_off[l], D.l2l_off[l + 1] - D.l2l_off[l], r.ndp, loc(r), st);
+    return e;
+  }
+  // near field of the points (FP64: with L2P, in one pass)
+  cudaError_t near(const TaskRun& r, cudaStream_t st) const {
+    const TaskDev& D = C->task[r.t];
+    const DevTaskLists& L = D.L;
+    const int64_t nsp = C->npts[L.src_cls], ntp = C->npts[L.tgt_cls];
+    const T* W = static_cast<const T*>(w(r).W);
+    double* phi = C->phi[r.t];
+    cudaError_t e;
+    if constexpr (f64) e = launch_p2p_l2p_f64(G, L, W, nsp, ntp, r.ndp, loc(r), phi, st);
+    else if (r.t == 0 && p2p_sym_takes(D.sym, r.ndp)) e = launch_p2p_sym(G, D.sym, W, nsp, r.ndp, phi, st);
+    else e = launch_p2p_f32(G, L, W, nsp, ntp, r.ndp, phi, st);
+    if (e == cudaSuccess && r.dip) e = launch_p2p_dl<T>(G, L, static_cast<const T*>(w(r).Wdl), nsp, ntp, r.ndp, phi, st);
+    return e;
+  }
+  cudaError_t l2p(const TaskRun& r, cudaStream_t st) const {
+    const DevTaskLists& L = C->task[r.t].L;
+    if constexpr (f64) return cudaSuccess;
+    else return launch_l2p_f32(G, L, C->npts[L.tgt_cls], r.ndp, loc(r), C->phi[r.t], st);
+  }
+  cudaError_t cor(const TaskRun& r, cudaStream_t st) const {
+    return launch_near_cor(C->task[r.t].L, r.dens, r.ndens, r.out, st, r.dip);
+  }
+  cudaError_t add(const TaskRun& r, cudaStream_t st) const {
+    const DevTaskLists& L = C->task[r.t].L;
+    return launch_elem_add(L, C->phi[r.t], C->npts[L.tgt_cls], r.ndens, r.out, st);
+  }
+};
+
+// One task after the other's parts on one stream, with events between the
+// stages when ev is given.
+template <typename T>
+static cudaError_t run_serial(bcfmm_ctx* C, const TaskRun& r, cudaStream_t st, cudaEvent_t* ev) {
+  const Parts<T> P(C);
+  cudaError_t e = cudaSuccess;
+  auto mark = [&](int k) { if (ev && e == cudaSuccess) e = cudaEventRecord(ev[k], st); };
+  auto step = [&](cudaError_t x) { if (e == cudaSuccess) e = x; };
+  mark(0);
+  step(P.weights(r, st));
+  if (e == cudaSuccess) step(P.zero(r, st));
+  mark(1);
+  if (e == cudaSuccess) step(P.up(r, st));
+  mark(2);
+  if (e == cudaSuccess) step(P.m2l(r, st, nullptr));
+  mark(3);
+  if (e == cudaSuccess) step(P.l2l(r, st));
+  mark(4);
+  if (e == cudaSuccess) step(P.near(r, st));
+  if (e == cudaSuccess) step(P.l2p(r, st));
+  mark(5);
+  if (e == cudaSuccess) step(P.cor(r, st));
+  if (e == cudaSuccess) step(P.add(r, st));
+  mark(6);
+  return e;
+}
+
+// Tasks whose independent parts run side by side: the near corrections need
+// the densities only, the near field and the expansions the point weights, and
+// the potentials meet at L2P.  BtV has work buffers of its own and runs
+// beside the volume tasks; VtB takes VtV's upward pass and local expansions
+// (same volume density and source points, so the same interaction lists; VtV's
+// far field covers the boxes of both).  Everything starts after what is on
+// `st` and is joined on it.
+template <typename T>
+static cudaError_t run_tasks(bcfmm_ctx* C, const TaskRun* runs, int n, cudaStream_t st) {
+  const Parts<T> P(C);
+  cudaEvent_t* E = C->e_part;
+  cudaError_t e = cudaSuccess;
+  auto ok = [&](cudaError_t x) { if (e == cudaSuccess) e = x; return e == cudaSuccess; };
+  auto rec = [&](int k, cudaStream_t s) { return e == cudaSuccess && ok(cudaEventRecord(E[k], s)); };
+  auto wait = [&](cudaStream_t s, int k) { return e == cudaSuccess && ok(cudaStreamWaitEvent(s, E[k], 0)); };
+  const TaskRun *vol[2] = {nullptr, nullptr}, *btv = nullptr;
+  int nvol = 0;
+  for (int i = 0; i < n; ++i) {
+    if (runs[i].t == 2) btv = &runs[i];
+    else vol[nvol++] = &runs[i];
+  }
+  rec(bcfmm_ctx::kEvStart, st);
+  wait(C->s_cor, bcfmm_ctx::kEvStart);
+  if (nvol && e == cudaSuccess) ok(P.zero(*vol[0], C->s_cor));
+  if (btv && e == cudaSuccess) ok(P.zero(*btv, C->s_cor));
+  rec(bcfmm_ctx::kEvZero, C->s_cor);
+  for (int i = 0; i < n && e == cudaSuccess; ++i) ok(P.cor(runs[i], C->s_cor));
+  rec(bcfmm_ctx::kEvCor, C->s_cor);
+  // the far field of `r` on its own stream, its near fields on sn
+  auto far = [&](const TaskRun& r, int set, cudaStream_t sn) {
+    if (e == cudaSuccess) ok(P.weights(r, sn));
+    rec(set ? bcfmm_ctx::kEvW1 : bcfmm_ctx::kEvW0, sn);
+    cudaStream_t sf = C->s_far[set];
+    wait(sf, set ? bcfmm_ctx::kEvW1 : bcfmm_ctx::kEvW0);
+    if (e == cudaSuccess) ok(P.up(r, sf));
+    wait(sf, bcfmm_ctx::kEvZero);
+    const TaylorFork side{C->s_m2l[set], E[bcfmm_ctx::kEvM0 + 2 * set], E[bcfmm_ctx::kEvM0 + 2 * set + 1]};
+    if (e == cudaSuccess) ok(P.m2l(r, sf, &side));
+    if (e == cudaSuccess) ok(P.l2l(r, sf));
+    rec(set ? bcfmm_ctx::kEvFar1 : bcfmm_ctx::kEvFar0, sf);
+  };
+  auto finish = [&](const TaskRun& r, cudaStream_t s) {
+    if (e == cudaSuccess) ok(P.l2p(r, s));
+    if (e == cudaSuccess) ok(P.add(r, s));
+  };
+  cudaStream_t sb = nvol ? C->s_near1 : st;
+  if (btv) {
+    if (sb != st) wait(sb, bcfmm_ctx::kEvStart);
+    far(*btv, 1, sb);
+  }
+  if (nvol) far(*vol[0], 0, st);
+  // (FP64 evaluates L2P with the near field, after the expansions)
+  if (Parts<T>::f64 && nvol) wait(st, bcfmm_ctx::kEvFar0);
+  for (int i = 0; i < nvol && e == cudaSuccess; ++i) ok(P.near(*vol[i], st));
+  if (btv) {
+    if (Parts<T>::f64) wait(sb, bcfmm_ctx::kEvFar1);
+    if (e == cudaSuccess) ok(P.near(*btv, sb));
+    if (!Parts<T>::f64) wait(sb, bcfmm_ctx::kEvFar1);
+    wait(sb, bcfmm_ctx::kEvCor);
+    finish(*btv, sb);
+    if (sb != st) rec(bcfmm_ctx::kEvBtv, sb);
+  }
+  if (nvol) {
+    if (!Parts<T>::f64) wait(st, bcfmm_ctx::kEvFar0);
+    wait(st, bcfmm_ctx::kEvCor);
+    for (int i = 0; i < nvol; ++i) finish(*vol[i], st);
+  }
+  if (btv && sb != st) wait(st, bcfmm_ctx::kEvBtv);
+  return e;
+}
+
+static cudaError_t run_tasks(bcfmm_ctx* C, const TaskRun* runs, int n, cudaStream_t st) {
+  return C->prm.precision == BCFMM_FP64 ? run_tasks<double>(C, runs, n, st) : run_tasks<float>(C, runs, n, st);
+}
+
+// A task with the context's densities; out may be set by the caller.
+static int task_run(bcfmm_ctx* C, int t, TaskRun& r) {
+  const int kind = C->task[t].L.src_cls;     // class 0 sources: volume density; class 1: boundary density
+  r.t = t;
+  r.dens = C->dens[kind];
+  r.ndens = C->ndens[kind];
+  r.ndp = C->ndp[kind];
+  // BtV with a double-layer density g: V~ q - K~ g (Algorithm 3)
+  r.dip = t == 2 && C->ndens[BCFMM_DIPOLE] > 0 ? C->dens[BCFMM_DIPOLE] : nullptr;
+  if (r.dip && C->ndens[BCFMM_DIPOLE] != r.ndens)
+    return fail(BCFMM_ERR_STATE, "eval: the double-layer density's ndens differs from the boundary density's");
+  return ensure_work(C, kind, r.ndp);
+}
+
+// Near-field pairs from which a single task's parts run side by side: the
+// eight event calls cost the host about 10 us.
+constexpr int64_t kForkPairs = 100000000;
+
+static int eval_impl(bcfmm_ctx* C, int t, double* out, int out_is_device) {
   if (!C) return fail(BCFMM_ERR_ARG, "eval: null context");
-  TaskDev& D = C->task[t];
-  const DevTaskLists& L = D.L;
-  const int kind = L.src_cls;     // class 0 sources: volume density; class 1: boundary density
+  const DevTaskLists& L = C->task[t].L;
+  const int kind = L.src_cls;
   if (C->ndens[kind] == 0)
     return fail(BCFMM_ERR_STATE, kind == 0 ? "eval: volume density not set" : "eval: boundary density not set");
   if (!out) return fail(BCFMM_ERR_ARG, "eval: null output");
-  const int ndens = C->ndens[kind], ndp = C->ndp[kind];
-  // BtV with a double-layer density g: V~ q - K~ g (Algorithm 3)
-  const bool dl = t == 2 && C->ndens[BCFMM_DIPOLE] > 0;
-  if (dl && C->ndens[BCFMM_DIPOLE] != ndens)
-    return fail(BCFMM_ERR_STATE, "eval: the double-layer density's ndens differs from the boundary density's");
-  const int rc = ensure_work(C, ndp);
+  TaskRun r;
+  int rc = task_run(C, t, r);
+  if (rc == BCFMM_OK && !out_is_device) rc = ensure_out(C, r.ndp);
   if (rc != BCFMM_OK) return rc;
   cudaStream_t st = C->st;
-  const DevGeom& G = C->G;
-  const int64_t nsp = C->npts[L.src_cls], ntp = C->npts[L.tgt_cls];
-  const int64_t nsel = kind == 0 ? C->ntet : C->ntri;
-  const size_t nexp = (size_t)C->nbox * ndp * C->G.ms;
-  const bool f64 = C->prm.precision == BCFMM_FP64;
-  const bool tc = C->prm.precision == BCFMM_FP32_BF16X2 || C->prm.precision == BCFMM_FP32_BF16X3;
   const bool tm = C->prm.timing && C->ev_ok;
-  cudaEvent_t* ev = C->ev[t];
-  double* outd = out_is_device ? out : C->out_dev;
-  if (tm) CU(cudaEventRecord(ev[0], st));
-  if (f64) {
-    if (!skip_up) {
-      CU(launch_weights<double>(G, L.src_cls, nsp, C->dens[kind], nsel, ndens, ndp, C->W64, st));
-      if (dl) CU(launch_weights<double>(G, 1, nsp, C->dens[BCFMM_DIPOLE], nsel, ndens, ndp, C->W64dl, st));
-    }
-    if (!skip_far) CU(cudaMemsetAsync(C->loc64, 0, nexp * sizeof(double), st));
-    if (tm) CU(cudaEventRecord(ev[1], st));
-    if (!skip_up) {
-      CU(launch_p2m<double>(G, L, C->W64, nsp, ndp, C->mom64, st));
-      if (dl) CU(launch_p2m_dl<double>(G, L, C->W64dl, nsp, ndp, C->mom64, st));
-      for (int l = C->nlevels - 1; l >= 2; --l) {
-        const int n = D.m2m_off[l + 1] - D.m2m_off[l];
-        CU(launch_m2m<double>(G, D.m2m_parent + D.m2m_off[l], n, L.src_cls, ndp, C->mom64, st));
-      }
-    }
-    if (tm) CU(cudaEventRecord(ev[2], st));
-    if (!skip_far) {
-      if (C->ty.q > 0)
-        CU(launch_m2l_taylor<double>(G, L, D.tys, C->ty, ndp, C->mom64, C->loc64, (double*)C->ty_momp,
-                                     (double*)C->ty_partial, st));
-      if (C->ty.q == 0) CU(launch_m2l_simt<double>(G, L, C->T64, ndp, C->mom64, C->loc64, st));
-      else if (D.tys.nsimt > 0)
-        CU(launch_m2l_simt<double>(G, L, C->T64, ndp, C->mom64, C->loc64, st, D.tys.simt_sel, D.tys.nsimt));
-    }
-    if (tm) CU(cudaEventRecord(ev[3], st));
-    for (int l = 3; l < C->nlevels && !skip_far; ++l) {
-      const int n = D.l2l_off[l + 1] - D.l2l_off[l];
-      CU(launch_l2l<double>(G, D.l2l_parent + D.l2l_off[l], n, ndp, C->loc64, st));
-    }
-    if (tm) CU(cudaEventRecord(ev[4], st));
-    CU(launch_p2p_l2p_f64(G, L, C->W64, nsp, ntp, ndp, C->loc64, C->phi, st));
-    if (dl) CU(launch_p2p_dl<double>(G, L, C->W64dl, nsp, ntp, ndp, C->phi, st));
-  } else {
-    if (!skip_up) {
-      CU(launch_weights<float>(G, L.src_cls, nsp, C->dens[kind], nsel, ndens, ndp, C->W32, st));
-      if (dl) CU(launch_weights<float>(G, 1, nsp, C->dens[BCFMM_DIPOLE], nsel, ndens, ndp, C->W32dl, st));
-    }
-    if (!skip_far) CU(cudaMemsetAsync(C->loc32, 0, nexp * sizeof(float), st));
-    if (tm) CU(cudaEventRecord(ev[1], st));
-    if (!skip_up) {
-      CU(launch_p2m<float>(G, L, C->W32, nsp, ndp, C->mom32, st));
-      if (dl) CU(launch_p2m_dl<float>(G, L, C->W32dl, nsp, ndp, C->mom32, st));
-      for (int l = C->nlevels - 1; l >= 2; --l) {
-        const int n = D.m2m_off[l + 1] - D.m2m_off[l];
-        CU(launch_m2m<float>(G, D.m2m_parent + D.m2m_off[l], n, L.src_cls, ndp, C->mom32, st));
-      }
-    }
-    if (tm) CU(cudaEventRecord(ev[2], st));
-    if (skip_far) {
-    } else if (tc) {
-      CU(launch_m2l_tc(G, L, D.tcs, C->tc, ndp, C->mom32, C->loc32, C->tc_partial, C->tc_momb, st));
-      if (D.tcs.nsimt > 0) CU(launch_m2l_simt<float>(G, L, C->T32, ndp, C->mom32, C->loc32, st, D.tcs.simt_sel, D.tcs.nsimt));
-    } else if (C->ty.q > 0) {
-      CU(launch_m2l_taylor<float>(G, L, D.tys, C->ty, ndp, C->mom32, C->loc32, (float*)C->ty_momp,
-                                  (float*)C->ty_partial, st));
-    } else {
-      CU(launch_m2l_simt<float>(G, L, C->T32, ndp, C->mom32, C->loc32, st));
-    }
-    if (tm) CU(cudaEventRecord(ev[3], st));
-    for (int l = 3; l < C->nlevels && !skip_far; ++l) {
-      const int n = D.l2l_off[l + 1] - D.l2l_off[l];
-      CU(launch_l2l<float>(G, D.l2l_parent + D.l2l_off[l], n, ndp, C->loc32, st));
-    }
-    if (tm) CU(cudaEventRecord(ev[4], st));
-    if (ndp == 1 && D.sym.nblk > 0) CU(launch_p2p_sym(G, D.sym, C->W32, C->phi, st));
-    else CU(launch_p2p_f32(G, L, C->W32, nsp, ntp, ndp, C->phi, st));
-    CU(launch_l2p_f32(G, L, ntp, ndp, C->loc32, C->phi, st));
-    if (dl) CU(launch_p2p_dl<float>(G, L, C->W32dl, nsp, ntp, ndp, C->phi, st));
-  }
-  if (tm) CU(cudaEventRecord(ev[5], st));
-  CU(launch_elem_sum(G, L, C->phi, ntp, C->dens[kind], ndens, outd, st, dl ? C->dens[BCFMM_DIPOLE] : nullptr));
-  if (tm) CU(cudaEventRecord(ev[6], st));
+  r.out = out_is_device ? out : C->out_dev;
+  if (!tm && C->task[t].p2p_pairs >= kForkPairs) CU(run_tasks(C, &r, 1, st));
+  else if (C->prm.precision == BCFMM_FP64) CU(run_serial<double>(C, r, st, tm ? C->ev[t] : nullptr));
+  else CU(run_serial<float>(C, r, st, tm ? C->ev[t] : nullptr));
   if (!out_is_device) {
-    CU(cudaMemcpyAsync(out, C->out_dev, (size_t)ndens * L.ntgt_el * sizeof(double), cudaMemcpyDeviceToHost, st));
+    CU(cudaMemcpyAsync(out, C->out_dev, (size_t)r.ndens * L.ntgt_el * sizeof(double), cudaMemcpyDeviceToHost, st));
     int herr = 0;
     CU(cudaMemcpyAsync(&herr, C->err, sizeof(int), cudaMemcpyDeviceToHost, st));
     CU(cudaStreamSynchronize(st));
@@ -1653,21 +1845,24 @@ extern "C" int bcfmm_eval_btv(bcfmm_ctx* C, double* out, int32_t d) { return eva
 // Several tasks through one CUDA graph.  The graph is captured on a
 // library-owned stream the first time a (task mask, outputs, density
 // sizes, work buffers) combination is seen, and replayed on the context's
-// stream afterwards.  VtB right after VtV reuses VtV's upward pass and its
-// local expansions (same volume density and source points, so the same
-// interaction lists; VtV's far field covers the boxes of both).
+// stream afterwards.
 extern "C" int bcfmm_eval_graph(bcfmm_ctx* C, int32_t mask, double* out_vtv, double* out_vtb, double* out_btv) {
   if (!C) return fail(BCFMM_ERR_ARG, "eval_graph: null context");
   if (mask <= 0 || mask > 7) return fail(BCFMM_ERR_ARG, "eval_graph: task mask must be a non-empty subset of 1|2|4");
   double* outs[3] = {out_vtv, out_vtb, out_btv};
+  TaskRun runs[3];
+  int nrun = 0;
   for (int t = 0; t < 3; ++t) {
     if (!(mask >> t & 1)) { outs[t] = nullptr; continue; }
     const int kind = C->task[t].L.src_cls;
     if (C->ndens[kind] == 0)
       return fail(BCFMM_ERR_STATE, kind == 0 ? "eval_graph: volume density not set" : "eval_graph: boundary density not set");
     if (!outs[t]) return fail(BCFMM_ERR_ARG, "eval_graph: null output for a task in the mask");
-    const int rc = ensure_work(C, C->ndp[kind]);
+    TaskRun r;
+    const int rc = task_run(C, t, r);
     if (rc != BCFMM_OK) return rc;
+    r.out = outs[t];
+    runs[nrun++] = r;
   }
   auto& g = C->graph;
   const bool same = g.exec && g.mask == mask && g.work_gen == C->work_gen && g.ndens[0] == C->ndens[0] &&
@@ -1675,19 +1870,14 @@ extern "C" int bcfmm_eval_graph(bcfmm_ctx* C, int32_t mask, double* out_vtv, dou
   if (!same) {
     if (g.exec) { cudaGraphExecDestroy(g.exec); g.exec = nullptr; }
     if (!C->cap_st) CU(cudaStreamCreateWithFlags(&C->cap_st, cudaStreamNonBlocking));
-    cudaStream_t user = C->st;
-    const int timing = C->prm.timing;
-    C->st = C->cap_st;
-    C->prm.timing = 0;
     CU(cudaStreamBeginCapture(C->cap_st, cudaStreamCaptureModeRelaxed));
-    int rc = BCFMM_OK;
-    for (int t = 0; t < 3 && rc == BCFMM_OK; ++t)
-      if (mask >> t & 1) rc = eval_impl(C, t, outs[t], 1, t == 1 && (mask & 1), t == 1 && (mask & 1));
+    const cudaError_t re = run_tasks(C, runs, nrun, C->cap_st);
     cudaGraph_t graph = nullptr;
     const cudaError_t ce = cudaStreamEndCapture(C->cap_st, &graph);
-    C->st = user;
-    C->prm.timing = timing;
-    if (rc != BCFMM_OK) { if (graph) cudaGraphDestroy(graph); return rc; }
+    if (re != cudaSuccess) {
+      if (graph) cudaGraphDestroy(graph);
+      return fail(BCFMM_ERR_CUDA, std::string("eval_graph: launch: ") + cudaGetErrorString(re));
+    }
     if (ce != cudaSuccess) return fail(BCFMM_ERR_CUDA, std::string("eval_graph: capture failed: ") + cudaGetErrorString(ce));
     int nkernel = 0;
     {
@@ -1733,7 +1923,7 @@ extern "C" int bcfmm_eval_noalloc(bcfmm_ctx* C, int32_t task, const double* dens
   TaskDev& D = C->task[task];
   const DevTaskLists& L = D.L;
   const int kind = L.src_cls;
-  if (C->work_ndp < 1 || (tcp && C->tc_momb == nullptr) || (typ && C->ty.q > 0 && C->ty_momp == nullptr))
+  if (C->work[kind].ndp < 1)
     return fail(BCFMM_ERR_STATE, "eval_noalloc: call bcfmm_set_density once first (it sizes the work buffers)");
   int dev = -1;
   CU(cudaGetDevice(&dev));
@@ -1747,36 +1937,13 @@ extern "C" int bcfmm_eval_noalloc(bcfmm_ctx* C, int32_t task, const double* dens
     return fail(BCFMM_ERR_ARG, "eval_noalloc: the mesh needs " + std::to_string(need * sizeof(float2)) +
                                    " bytes of M2L scratch, more than the fixed " + std::to_string(cap * sizeof(float2)) +
                                    " bytes (use bcfmm_eval_vtv/vtb/btv)");
-  cudaStream_t st = C->st;
-  const DevGeom& G = C->G;
-  const int ndp = 1;
-  const int64_t nsp = C->npts[L.src_cls], ntp = C->npts[L.tgt_cls];
-  const int64_t nsel = kind == 0 ? C->ntet : C->ntri;
-  const size_t nexp = (size_t)C->nbox * ndp * C->G.ms;
-  CU(launch_weights<float>(G, L.src_cls, nsp, dens_dev, nsel, 1, ndp, C->W32, st));
-  CU(cudaMemsetAsync(C->loc32, 0, nexp * sizeof(float), st));
-  CU(launch_p2m<float>(G, L, C->W32, nsp, ndp, C->mom32, st));
-  for (int l = C->nlevels - 1; l >= 2; --l) {     // (no box above level 2 is a source)
-    const int n = D.m2m_off[l + 1] - D.m2m_off[l];
-    CU(launch_m2m<float>(G, D.m2m_parent + D.m2m_off[l], n, L.src_cls, ndp, C->mom32, st));
-  }
-  if (tcp) {
-    CU(launch_m2l_tc(G, L, D.tcs, C->tc, ndp, C->mom32, C->loc32, partial, C->tc_momb, st));
-    if (D.tcs.nsimt > 0) CU(launch_m2l_simt<float>(G, L, C->T32, ndp, C->mom32, C->loc32, st, D.tcs.simt_sel, D.tcs.nsimt));
-  } else if (C->ty.q > 0) {
-    CU(launch_m2l_taylor<float>(G, L, D.tys, C->ty, ndp, C->mom32, C->loc32, (float*)C->ty_momp,
-                                reinterpret_cast<float*>(partial), st));
-  } else {
-    CU(launch_m2l_simt<float>(G, L, C->T32, ndp, C->mom32, C->loc32, st));
-  }
-  for (int l = 3; l < C->nlevels; ++l) {
-    const int n = D.l2l_off[l + 1] - D.l2l_off[l];
-    CU(launch_l2l<float>(G, D.l2l_parent + D.l2l_off[l], n, ndp, C->loc32, st));
-  }
-  if (D.sym.nblk > 0) CU(launch_p2p_sym(G, D.sym, C->W32, C->phi, st));
-  else CU(launch_p2p_f32(G, L, C->W32, nsp, ntp, ndp, C->phi, st));
-  CU(launch_l2p_f32(G, L, ntp, ndp, C->loc32, C->phi, st));
-  CU(launch_elem_sum(G, L, C->phi, ntp, dens_dev, 1, out_dev, st));
+  TaskRun r;
+  r.t = task;
+  r.dens = dens_dev;
+  r.ndens = r.ndp = 1;
+  r.out = out_dev;
+  r.partial = partial;
+  CU(run_tasks(C, &r, 1, C->st));
   C->ev_rec[task] = false;             // no stage timings recorded by this call
   return BCFMM_OK;
 }
@@ -1991,6 +2158,7 @@ extern "C" void bcfmm_destroy(bcfmm_ctx* C) {
       for (auto& ev : row) cudaEventDestroy(ev);
   if (C->graph.exec) cudaGraphExecDestroy(C->graph.exec);
   if (C->cap_st) cudaStreamDestroy(C->cap_st);
+  destroy_parts(C);
   m2l_tc_free_tables(&C->tc);
   C->mem.free_all();
   delete C;

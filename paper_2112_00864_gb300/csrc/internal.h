@@ -102,7 +102,11 @@ struct P2pChunks {
   std::vector<int> grp_row, grp_n;              // per split leaf: first scratch row, chunks
   int rows = 0;                                 // scratch rows (chunks of split leaves)
 };
-constexpr int64_t kP2pChunk = 8192;
+// At most 8192 sources a block; fewer on meshes that would leave SMs idle (about
+// sixteen blocks an SM, at least 1024 sources: a block's sums cost as much as
+// a few hundred).
+constexpr int64_t kP2pChunk = 8192, kP2pChunkMin = 1024;
+int64_t p2p_chunk(const HostSetup& H, int task, int nsm);
 void build_p2p_chunks(const HostSetup& H, int task, int64_t chunk, P2pChunks& out);
 
 // Gauss-Legendre nodes/weights on [0,1] (Newton iteration on P_n).

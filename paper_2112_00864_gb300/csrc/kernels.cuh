@@ -42,6 +42,7 @@ struct DevTaskLists {
   const int64_t* cor_off; const int* cor_col; const double* cor_val;
   const double* cor_val_dl;      // BtV: near-rule corrections of dG/dn_y (same CSR), or null
   const int* elem_pts;           // [ntgt_el][4] sorted positions of the element's points (-1 pad)
+  const double* elem_w;          // [ntgt_el] quadrature weight of the element's points
   int nq_tgt;                    // 4 (tets) or 3 (triangles)
   int src_cls, tgt_cls;
   // tensor-core M2L tiles: 128 targets of one expansion order and one
@@ -88,10 +89,12 @@ cudaError_t launch_l2p_f32(const DevGeom& G, const DevTaskLists& L, int64_t ntgt
                            double* phi, cudaStream_t st);
 cudaError_t launch_p2p_l2p_f64(const DevGeom& G, const DevTaskLists& L, const double* W, int64_t nsrc_pts,
                                int64_t ntgt_pts, int ndp, const double* loc, double* phi, cudaStream_t st);
-// dens_dl: BtV double-layer density (subtracts its corrections L.cor_val_dl), or null
-cudaError_t launch_elem_sum(const DevGeom& G, const DevTaskLists& L, const double* phi, int64_t ntgt_pts,
-                            const double* dens_src, int ndens, double* out, cudaStream_t st,
+// out = near corrections; dens_dl: BtV double-layer density (subtracts its
+// corrections L.cor_val_dl), or null
+cudaError_t launch_near_cor(const DevTaskLists& L, const double* dens_src, int ndens, double* out, cudaStream_t st,
                             const double* dens_dl = nullptr);
+// out += Galerkin sums of the point potentials
+cudaError_t launch_elem_add(const DevTaskLists& L, const double* phi, int64_t ntgt_pts, int ndens, double* out, cudaStream_t st);
 // BtV double layer (Algorithm 3): moments -<gamma_1 (y-c)^b, g> added to mom,
 // near field -sum Wg n.(x-y)/(4 pi r^3) subtracted from phi
 template <typename T>

@@ -602,220 +602,86 @@ __device__ __forceinline__ void two_sum_f(float& hi, float& lo, float x) {
   hi = s;
 }
 
-// Two targets per thread (ND <= 2) or one (ND > 2); thread groups split the
-// source tile; source tiles are double-buffered (one barrier per tile); the
-// per-tile FP32 sums are folded with a compensated (hi + lo) FP32 sum.
-template <int ND>
-__global__ void __launch_bounds__(128) k_p2p_f32(DevGeom G, DevTaskLists L, const float* __restrict__ W, int64_t nsp,
-                                                 int64_t ntp, double* __restrict__ phi) {
-  constexpr int TPT = ND <= 2 ? 2 : 1;
-  constexpr int PPT = kTile / 128;                 // source points loaded per thread per tile
-  __shared__ float4 tile[2][kTile];
-  __shared__ float tw[2][ND > 1 ? ND - 1 : 1][kTile];
-  __shared__ int pre[kRunBatch + 1], rst[kRunBatch];
-  __shared__ float2 red[ND][128 * TPT];
-  const int b = blockIdx.x;
-  const int leaf = L.p2p_leaf[b];
-  const int sc = L.src_cls, tc = L.tgt_cls;
-  const float4 ch = G.box_hi[leaf], cl = G.box_lo[leaf];
-  const float chx = ch.x, chy = ch.y, chz = ch.z, clx = cl.x, cly = cl.y, clz = cl.z;
-  const int2 tr = G.box_rng[tc][leaf];
-  const int nt = tr.y - tr.x;
-  // TS target slots (TPT targets each) per source group, NG = 128 / TS
-  // groups; threads beyond NG * TS only help loading the tiles
-  const int TS = (nt + TPT - 1) / TPT;
-  const int NG = 128 / TS;
-  const int ts = threadIdx.x % TS, gi_raw = threadIdx.x / TS;
-  const int gi = gi_raw < NG ? gi_raw : NG;       // NG: idle for the compute
-  float xt[TPT], yt[TPT], zt[TPT];
-  bool act[TPT];
-#pragma unroll
-  for (int u = 0; u < TPT; ++u) {
-    const int t = ts + u * TS;
-    act[u] = t < nt;
-    xt[u] = yt[u] = zt[u] = 1e30f;      // padding targets: far away, discarded
-    if (act[u]) {
-      const float4 h = G.pthi[tc][tr.x + t], l = G.ptlo[tc][tr.x + t];
-      xt[u] = (h.x - chx) + (l.x - clx);
-      yt[u] = (h.y - chy) + (l.y - cly);
-      zt[u] = (h.z - chz) + (l.z - clz);
-    }
-  }
-  float shi[TPT][ND], slo[TPT][ND];
-#pragma unroll
-  for (int u = 0; u < TPT; ++u)
-#pragma unroll
-    for (int d = 0; d < ND; ++d) shi[u][d] = slo[u][d] = 0.f;
-  const int r0 = L.run_off[b], r1 = L.run_off[b + 1];
-  const int self_len = L.self_len[b];
-  float4 reg[PPT];
-  float regw[PPT][ND > 1 ? ND - 1 : 1];
-  for (int rb = r0; rb < r1; rb += kRunBatch) {
-    const int nr = min(kRunBatch, r1 - rb);
-    __syncthreads();
-    scan_runs(L.runs + rb, nr, pre, rst);
-    __syncthreads();
-    const int total = pre[nr];
-    const int ntiles = (total + kTile - 1) / kTile;
-    auto load_tile = [&](int t) {
-#pragma unroll
-      for (int q = 0; q < PPT; ++q) {
-        const int v = t * kTile + threadIdx.x + q * 128;
-        if (v < total) {
-          const int r = find_run(pre, nr, v);
-          const int src = rst[r] + (v - pre[r]);
-          const float4 h = G.pthi[sc][src], l = G.ptlo[sc][src];
-          reg[q] = make_float4((h.x - chx) + (l.x - clx), (h.y - chy) + (l.y - cly), (h.z - chz) + (l.z - clz), W[src]);
-#pragma unroll
-          for (int d = 1; d < ND; ++d) regw[q][d - 1] = W[(int64_t)d * nsp + src];
-        }
-      }
-    };
-    auto store_tile = [&](int buf) {
-#pragma unroll
-      for (int q = 0; q < PPT; ++q) {
-        const int j = threadIdx.x + q * 128;
-        tile[buf][j] = reg[q];
-#pragma unroll
-        for (int d = 1; d < ND; ++d) tw[buf][d - 1][j] = regw[q][d - 1];
-      }
-    };
-    if (ntiles > 0) {
-      load_tile(0);
-      store_tile(0);
-    }
-    __syncthreads();
-    for (int t = 0; t < ntiles; ++t) {
-      const int cur = t & 1;
-      if (t + 1 < ntiles) load_tile(t + 1);      // global loads in flight during the compute
-      const int m = min(kTile, total - t * kTile);
-      float acc[TPT][ND];
-#pragma unroll
-      for (int u = 0; u < TPT; ++u)
-#pragma unroll
-        for (int d = 0; d < ND; ++d) acc[u][d] = 0.f;
-      const int jstart = gi_raw < NG ? gi : m;        // idle threads skip the loops
-      if (rb == r0 && t * kTile < self_len) {
-        for (int j = jstart; j < m; j += NG) {
-          const float4 s = tile[cur][j];
-#pragma unroll
-          for (int u = 0; u < TPT; ++u) {
-            const float dx = xt[u] - s.x, dy = yt[u] - s.y, dz = zt[u] - s.z;
-            const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-            const float ri = r2 > 0.f ? rsqrt_ftz(r2) : 0.f;
-            acc[u][0] = fmaf(s.w, ri, acc[u][0]);
-#pragma unroll
-            for (int d = 1; d < ND; ++d) acc[u][d] = fmaf(tw[cur][d - 1][j], ri, acc[u][d]);
-          }
-        }
-      } else {
-#pragma unroll 4
-        for (int j = jstart; j < m; j += NG) {
-          const float4 s = tile[cur][j];
-#pragma unroll
-          for (int u = 0; u < TPT; ++u) {
-            const float dx = xt[u] - s.x, dy = yt[u] - s.y, dz = zt[u] - s.z;
-            const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-            const float ri = rsqrt_ftz(r2);
-            acc[u][0] = fmaf(s.w, ri, acc[u][0]);
-#pragma unroll
-            for (int d = 1; d < ND; ++d) acc[u][d] = fmaf(tw[cur][d - 1][j], ri, acc[u][d]);
-          }
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < TPT; ++u)
-#pragma unroll
-        for (int d = 0; d < ND; ++d) two_sum_f(shi[u][d], slo[u][d], acc[u][d]);
-      if (t + 1 < ntiles) store_tile(cur ^ 1);
-      __syncthreads();
-    }
-  }
-#pragma unroll
-  for (int u = 0; u < TPT; ++u)
-#pragma unroll
-    for (int d = 0; d < ND; ++d) red[d][u * 128 + threadIdx.x] = make_float2(shi[u][d], slo[u][d]);
-  __syncthreads();
-  if (gi_raw == 0) {
-#pragma unroll
-    for (int u = 0; u < TPT; ++u) {
-      if (!act[u]) continue;
-      double near[ND];
-#pragma unroll
-      for (int d = 0; d < ND; ++d) {
-        float hi = 0.f, lo = 0.f;
-        for (int g = 0; g < NG; ++g) {
-          const float2 v = red[d][u * 128 + g * TS + ts];
-          two_sum_f(hi, lo, v.x);
-          lo += v.y;
-        }
-        near[d] = (double)hi + (double)lo;
-      }
-#pragma unroll
-      for (int d = 0; d < ND; ++d) phi[(int64_t)d * ntp + tr.x + ts + u * TS] = near[d] * kInv4Pi;
-    }
-  }
-}
-
-
-
 // The packed pair loop over pairs [k0, k1) of a staged tile: per pair and
 // target, three packed subtractions (the sources are stored negated), the
 // packed r^2 (one multiply, two FMAs), two rsqrt and one packed FMA per
 // density.  CHECK: the tile holds the target points themselves (r^2 = 0).
-template <int ND, int TPT, bool CHECK>
+// w2: the weights of densities 1.. of pair k at w2[d - 1][k].
+template <int ND, int TPT, int PAIRS, bool CHECK>
 __device__ __forceinline__ void p2p_pairs_x2(const float4* __restrict__ xy, const float4* __restrict__ zw,
                                              const float2* __restrict__ w2, int k0, int k1, const float2 (&X)[TPT],
                                              const float2 (&Y)[TPT], const float2 (&Z)[TPT], float2 (&acc)[TPT][ND]) {
-#pragma unroll 4
+#pragma unroll(ND <= 4 ? 4 : 2)
   for (int k = k0; k < k1; ++k) {
     const float4 a = xy[k], c = zw[k];
     const float2 nx = make_float2(a.x, a.y), ny = make_float2(a.z, a.w), nz = make_float2(c.x, c.y);
-    const float2 w0 = make_float2(c.z, c.w);
-    float2 wb = w0;
-    if constexpr (ND > 1) wb = w2[k];
+    float2 ri[TPT];
 #pragma unroll
     for (int u = 0; u < TPT; ++u) {
       const float2 dx = __fadd2_rn(X[u], nx), dy = __fadd2_rn(Y[u], ny), dz = __fadd2_rn(Z[u], nz);
       const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
-      float2 ri;
-      if constexpr (CHECK) ri = make_float2(r2.x > 0.f ? rsqrt_ftz(r2.x) : 0.f, r2.y > 0.f ? rsqrt_ftz(r2.y) : 0.f);
-      else ri = make_float2(rsqrt_ftz(r2.x), rsqrt_ftz(r2.y));
-      acc[u][0] = __ffma2_rn(w0, ri, acc[u][0]);
-      if constexpr (ND > 1) acc[u][ND - 1] = __ffma2_rn(wb, ri, acc[u][ND - 1]);
+      if constexpr (CHECK) ri[u] = make_float2(r2.x > 0.f ? rsqrt_ftz(r2.x) : 0.f, r2.y > 0.f ? rsqrt_ftz(r2.y) : 0.f);
+      else ri[u] = make_float2(rsqrt_ftz(r2.x), rsqrt_ftz(r2.y));
+      acc[u][0] = __ffma2_rn(make_float2(c.z, c.w), ri[u], acc[u][0]);
+    }
+#pragma unroll
+    for (int d = 1; d < ND; ++d) {
+      const float2 w = w2[(d - 1) * PAIRS + k];
+#pragma unroll
+      for (int u = 0; u < TPT; ++u) acc[u][d] = __ffma2_rn(w, ri[u], acc[u][d]);
     }
   }
 }
 
-// Packed form for ND <= 2: TPT targets per thread (4 for one density, 2
-// for two) and source points taken two at a time, every arithmetic
-// instruction on a float2 (the two sources of a pair: __fadd2_rn /
-// __fmul2_rn / __ffma2_rn), so a target keeps two independent partial sums
-// and the instructions issued per point pair nearly halve.  A tile of
-// source points is staged pair-interleaved in shared memory, negated and
-// relative to the target leaf's centre: xy[k] = (x0, x1, y0, y1), zw[k] =
-// (z0, z1, w0, w1) for the pair k = (2k, 2k + 1), so one pair costs two
-// 16-byte shared loads.  Each of the NG thread groups takes a contiguous
-// range of pairs (odd length, so two groups' loads in one quarter-warp fall
-// in different banks) walked with unit stride.  An odd tile is padded with a
-// weightless point at -1e30, whose distance overflows to inf (rsqrt 0).  Only
-// the pairs that hold the leaf's own points (the first run of a VtV list)
-// select r^2 = 0 out.  After the source loop all threads reduce the group
-// sums and evaluate L2P, one target each.
-constexpr int kTileX2 = 512;     // source points per tile of the packed kernel
+// Packed form: TPT targets per thread (4 for one density, 1 for sixteen) and
+// source points taken two at a time, every arithmetic instruction on a float2
+// (the two sources of a pair: __fadd2_rn / __fmul2_rn / __ffma2_rn), so a
+// target keeps two independent partial sums and the instructions issued per
+// point pair nearly halve.  A tile of source points is staged pair-interleaved
+// in shared memory, negated and relative to the target leaf's centre: xy[k] =
+// (x0, x1, y0, y1), zw[k] = (z0, z1, w0, w1) for the pair k = (2k, 2k + 1), so
+// one pair costs two 16-byte shared loads and 8 bytes per further density.
+// Each of the NG thread groups takes a contiguous range of pairs (odd length,
+// so two groups' loads in one quarter-warp fall in different banks) walked
+// with unit stride.  An odd tile is padded with a weightless point at -1e30,
+// whose distance overflows to inf (rsqrt 0).  Only the pairs that hold the
+// leaf's own points (the first run of a VtV list) select r^2 = 0 out.  After
+// the source loop all threads reduce the group sums, one target each.
+// The weights of the densities after the first go straight to shared memory
+// (4-byte cp.async), and from four densities on the compensated sums live there
+// and are folded every other tile: the registers then hold enough targets that
+// the shared-memory loads of the weights do not bound the loop.
+template <int ND>
+struct P2pShape {
+  static constexpr int TPT = ND == 1 || ND == 4 ? 4 : 2;
+  static constexpr int kTile = ND <= 4 ? 512 : 256;      // source points per tile
+  static constexpr int kPairs = kTile / 2;
+  static constexpr bool kSumsShared = ND >= 4;
+  static constexpr int kFold = kSumsShared ? 2 : 1;      // tiles between folds (a sum: at most 64 products)
+  static constexpr int kW2 = ND > 1 ? 2 * (ND - 1) * kPairs : 0;     // float2
+  static constexpr int kRed = ND * 128 * TPT;                        // float2
+  // (the sums of fewer densities are laid over the weights at the end)
+  static constexpr size_t smem = 2 * 2 * kPairs * sizeof(float4) +
+                                 (kSumsShared ? kW2 + kRed : (kW2 > kRed ? kW2 : kRed)) * sizeof(float2);
+};
 
-template <int ND, int TPT>
+// 4-byte asynchronous copy to shared memory
+__device__ __forceinline__ void cp_async4(float* dst, const float* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+
+template <int ND>
 __global__ void __launch_bounds__(128) k_p2p_f32x2(DevGeom G, DevTaskLists L, const float* __restrict__ W, int64_t nsp,
                                                    int64_t ntp, double* __restrict__ phi) {
-  static_assert(ND >= 1 && ND <= 2, "packed P2P serves one or two densities");
-  constexpr int kTile = kTileX2;
-  constexpr int kPairs = kTile / 2;
+  constexpr int TPT = P2pShape<ND>::TPT, kTile = P2pShape<ND>::kTile, kPairs = P2pShape<ND>::kPairs;
+  constexpr bool SM = P2pShape<ND>::kSumsShared;
   constexpr int PPT = kPairs / 128;                // pairs loaded per thread per tile
-  __shared__ float4 sxy[2][kPairs];
-  __shared__ float4 szw[2][kPairs];
-  __shared__ float2 sw2[ND > 1 ? 2 : 1][ND > 1 ? kPairs : 1];
+  extern __shared__ __align__(16) unsigned char smraw[];
+  float4(*sxy)[kPairs] = reinterpret_cast<float4(*)[kPairs]>(smraw);
+  float4(*szw)[kPairs] = sxy + 2;
+  float2* sw2 = reinterpret_cast<float2*>(szw + 2);            // weights of the further densities
+  float2* red = SM ? sw2 + P2pShape<ND>::kW2 : sw2;            // group sums [ND][128 TPT]
   __shared__ int pre[kRunBatch + 1], rst[kRunBatch];
-  __shared__ float2 red[ND][128 * TPT];
   const int b = blockIdx.x;
   const int leaf = L.sp_leaf[b];
   const int sc = L.src_cls, tc = L.tgt_cls;
@@ -841,15 +707,37 @@ __global__ void __launch_bounds__(128) k_p2p_f32x2(DevGeom G, DevTaskLists L, co
     Y[u] = make_float2(yt, yt);
     Z[u] = make_float2(zt, zt);
   }
-  float shi[TPT][ND], slo[TPT][ND];
+  float shi[SM ? 1 : TPT][ND], slo[SM ? 1 : TPT][ND];
+  float2 acc[TPT][ND];
 #pragma unroll
   for (int u = 0; u < TPT; ++u)
 #pragma unroll
-    for (int d = 0; d < ND; ++d) shi[u][d] = slo[u][d] = 0.f;
+    for (int d = 0; d < ND; ++d) {
+      acc[u][d] = make_float2(0.f, 0.f);
+      if constexpr (SM) red[(d * TPT + u) * 128 + threadIdx.x] = make_float2(0.f, 0.f);
+      else shi[u][d] = slo[u][d] = 0.f;
+    }
+  auto fold = [&]() {
+#pragma unroll
+    for (int u = 0; u < TPT; ++u)
+#pragma unroll
+      for (int d = 0; d < ND; ++d) {
+        if constexpr (SM) {
+          float2 v = red[(d * TPT + u) * 128 + threadIdx.x];
+          two_sum_f(v.x, v.y, acc[u][d].x);
+          two_sum_f(v.x, v.y, acc[u][d].y);
+          red[(d * TPT + u) * 128 + threadIdx.x] = v;
+        } else {
+          two_sum_f(shi[u][d], slo[u][d], acc[u][d].x);
+          two_sum_f(shi[u][d], slo[u][d], acc[u][d].y);
+        }
+        acc[u][d] = make_float2(0.f, 0.f);
+      }
+  };
+  int nfold = 0;
   const int r0 = L.sp_run_off[b], r1 = L.sp_run_off[b + 1];
   const int self_len = L.sp_self[b];
   float4 rxy[PPT], rzw[PPT];
-  float2 rw2[PPT];
   for (int rb = r0; rb < r1; rb += kRunBatch) {
     const int nr = min(kRunBatch, r1 - rb);
     __syncthreads();
@@ -858,32 +746,40 @@ __global__ void __launch_bounds__(128) k_p2p_f32x2(DevGeom G, DevTaskLists L, co
     const int total = pre[nr];
     const int ntiles = (total + kTile - 1) / kTile;
     // source point v of this batch (r: its run), negated, relative to the centre
-    auto fetch = [&](int v, int r, float& x, float& y, float& z, float& w, float& w2) {
+    auto fetch = [&](int v, int r, float& x, float& y, float& z, float& w) {
       const int src = rst[r] + (v - pre[r]);
       const float4 h = G.pthi[sc][src], l = G.ptlo[sc][src];
       x = -((h.x - chx) + (l.x - clx));
       y = -((h.y - chy) + (l.y - cly));
       z = -((h.z - chz) + (l.z - clz));
       w = W[src];
-      if constexpr (ND > 1) w2 = W[nsp + src];
+      return src;
     };
-    auto load_tile = [&](int t) {
+    auto load_tile = [&](int t, int buf) {
 #pragma unroll
       for (int q = 0; q < PPT; ++q) {
-        const int v0 = t * kTile + 2 * (threadIdx.x + q * 128);
-        float x0 = 1e30f, y0 = 1e30f, z0 = 1e30f, w0 = 0.f, u0 = 0.f;   // negated padding points
-        float x1 = 1e30f, y1 = 1e30f, z1 = 1e30f, w1 = 0.f, u1 = 0.f;
+        const int k = threadIdx.x + q * 128, v0 = t * kTile + 2 * k;
+        float x0 = 1e30f, y0 = 1e30f, z0 = 1e30f, w0 = 0.f;   // negated padding points
+        float x1 = 1e30f, y1 = 1e30f, z1 = 1e30f, w1 = 0.f;
+        int s0 = -1, s1 = -1;
         if (v0 < total) {
           int r = find_run(pre, nr, v0);
-          fetch(v0, r, x0, y0, z0, w0, u0);
+          s0 = fetch(v0, r, x0, y0, z0, w0);
           if (v0 + 1 < total) {
             while (r + 1 < nr && pre[r + 1] <= v0 + 1) ++r;
-            fetch(v0 + 1, r, x1, y1, z1, w1, u1);
+            s1 = fetch(v0 + 1, r, x1, y1, z1, w1);
           }
         }
         rxy[q] = make_float4(x0, x1, y0, y1);
         rzw[q] = make_float4(z0, z1, w0, w1);
-        rw2[q] = make_float2(u0, u1);
+        if constexpr (ND > 1) {
+          float2* w = sw2 + buf * (ND - 1) * kPairs + k;
+#pragma unroll
+          for (int d = 1; d < ND; ++d, w += kPairs) {
+            if (s0 >= 0) cp_async4(&w->x, W + d * nsp + s0); else w->x = 0.f;
+            if (s1 >= 0) cp_async4(&w->y, W + d * nsp + s1); else w->y = 0.f;
+          }
+        }
       }
     };
     auto store_tile = [&](int buf) {
@@ -892,17 +788,17 @@ __global__ void __launch_bounds__(128) k_p2p_f32x2(DevGeom G, DevTaskLists L, co
         const int k = threadIdx.x + q * 128;
         sxy[buf][k] = rxy[q];
         szw[buf][k] = rzw[q];
-        if constexpr (ND > 1) sw2[buf][k] = rw2[q];
       }
+      if constexpr (ND > 1) asm volatile("cp.async.wait_all;" ::: "memory");
     };
     if (ntiles > 0) {
-      load_tile(0);
+      load_tile(0, 0);
       store_tile(0);
     }
     __syncthreads();
     for (int t = 0; t < ntiles; ++t) {
       const int cur = t & 1;
-      if (t + 1 < ntiles) load_tile(t + 1);
+      if (t + 1 < ntiles) load_tile(t + 1, cur ^ 1);
       const int m = min(kTile, total - t * kTile);
       const int mp = (m + 1) >> 1;
       // group gi_raw's contiguous pair range, odd length
@@ -911,30 +807,22 @@ __global__ void __launch_bounds__(128) k_p2p_f32x2(DevGeom G, DevTaskLists L, co
       const int k1 = min(k0 + len, mp);
       // pairs that hold one of the leaf's own points (first run of a VtV list)
       const int ks = rb == r0 ? max(0, min(mp, (self_len - t * kTile + 1) >> 1)) : 0;
-      float2 acc[TPT][ND];
-#pragma unroll
-      for (int u = 0; u < TPT; ++u)
-#pragma unroll
-        for (int d = 0; d < ND; ++d) acc[u][d] = make_float2(0.f, 0.f);
-      const float2* w2 = nullptr;
-      if constexpr (ND > 1) w2 = sw2[cur];
-      if (k0 < ks) p2p_pairs_x2<ND, TPT, true>(sxy[cur], szw[cur], w2, k0, min(k1, ks), X, Y, Z, acc);
-      p2p_pairs_x2<ND, TPT, false>(sxy[cur], szw[cur], w2, max(k0, ks), k1, X, Y, Z, acc);
-#pragma unroll
-      for (int u = 0; u < TPT; ++u)
-#pragma unroll
-        for (int d = 0; d < ND; ++d) {
-          two_sum_f(shi[u][d], slo[u][d], acc[u][d].x);
-          two_sum_f(shi[u][d], slo[u][d], acc[u][d].y);
-        }
+      const float2* w2 = sw2 + cur * (ND - 1) * kPairs;
+      if (k0 < ks) p2p_pairs_x2<ND, TPT, kPairs, true>(sxy[cur], szw[cur], w2, k0, min(k1, ks), X, Y, Z, acc);
+      p2p_pairs_x2<ND, TPT, kPairs, false>(sxy[cur], szw[cur], w2, max(k0, ks), k1, X, Y, Z, acc);
+      if (++nfold == P2pShape<ND>::kFold) { fold(); nfold = 0; }
       if (t + 1 < ntiles) store_tile(cur ^ 1);
       __syncthreads();
     }
   }
+  if constexpr (SM) {
+    if (nfold) fold();
+  } else {
 #pragma unroll
-  for (int u = 0; u < TPT; ++u)
+    for (int u = 0; u < TPT; ++u)
 #pragma unroll
-    for (int d = 0; d < ND; ++d) red[d][u * 128 + threadIdx.x] = make_float2(shi[u][d], slo[u][d]);
+      for (int d = 0; d < ND; ++d) red[(d * TPT + u) * 128 + threadIdx.x] = make_float2(shi[u][d], slo[u][d]);
+  }
   __syncthreads();
   // every thread: one target, the group sums in group order; a chunk of a
   // split leaf stores them in its scratch row, and the leaf's last chunk
@@ -950,7 +838,7 @@ __global__ void __launch_bounds__(128) k_p2p_f32x2(DevGeom G, DevTaskLists L, co
       for (int d = 0; d < ND; ++d) {
         float hi = 0.f, lo = 0.f;
         for (int g = 0; g < NG; ++g) {
-          const float2 v = red[d][u * 128 + g * TS + tsl];
+          const float2 v = red[(d * TPT + u) * 128 + g * TS + tsl];
           two_sum_f(hi, lo, v.x);
           lo += v.y;
         }
@@ -975,7 +863,7 @@ __global__ void __launch_bounds__(128) k_p2p_f32x2(DevGeom G, DevTaskLists L, co
       float hi = 0.f, lo = 0.f;
       if (grp.x < 0) {
         for (int g = 0; g < NG; ++g) {
-          const float2 v = red[d][u * 128 + g * TS + tsl];
+          const float2 v = red[(d * TPT + u) * 128 + g * TS + tsl];
           two_sum_f(hi, lo, v.x);
           lo += v.y;
         }
@@ -1079,18 +967,29 @@ __global__ void __launch_bounds__(128) k_p2p_l2p_f64(DevGeom G, DevTaskLists L, 
     default: return cudaErrorInvalidValue;                                   \
   }
 
+template <int ND>
+cudaError_t launch_p2p_nd(const DevGeom& G, const DevTaskLists& L, const float* W, int64_t nsp, int64_t ntp, double* phi,
+                          cudaStream_t st) {
+  constexpr size_t sm = P2pShape<ND>::smem;
+  if (sm > 44 * 1024) {
+    const cudaError_t e = cudaFuncSetAttribute(k_p2p_f32x2<ND>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+  }
+  k_p2p_f32x2<ND><<<L.sp_n, 128, sm, st>>>(G, L, W, nsp, ntp, phi);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_p2p_f32(const DevGeom& G, const DevTaskLists& L, const float* W, int64_t nsrc_pts, int64_t ntgt_pts,
                            int ndp, double* phi, cudaStream_t st) {
   if (L.n_p2p == 0) return cudaSuccess;
   switch (ndp) {
-    case 1: k_p2p_f32x2<1, 4><<<L.sp_n, 128, 0, st>>>(G, L, W, nsrc_pts, ntgt_pts, phi); break;
-    case 2: k_p2p_f32x2<2, 2><<<L.sp_n, 128, 0, st>>>(G, L, W, nsrc_pts, ntgt_pts, phi); break;
-    case 4: k_p2p_f32<4><<<L.n_p2p, 128, 0, st>>>(G, L, W, nsrc_pts, ntgt_pts, phi); break;
-    case 8: k_p2p_f32<8><<<L.n_p2p, 128, 0, st>>>(G, L, W, nsrc_pts, ntgt_pts, phi); break;
-    case 16: k_p2p_f32<16><<<L.n_p2p, 128, 0, st>>>(G, L, W, nsrc_pts, ntgt_pts, phi); break;
+    case 1: return launch_p2p_nd<1>(G, L, W, nsrc_pts, ntgt_pts, phi, st);
+    case 2: return launch_p2p_nd<2>(G, L, W, nsrc_pts, ntgt_pts, phi, st);
+    case 4: return launch_p2p_nd<4>(G, L, W, nsrc_pts, ntgt_pts, phi, st);
+    case 8: return launch_p2p_nd<8>(G, L, W, nsrc_pts, ntgt_pts, phi, st);
+    case 16: return launch_p2p_nd<16>(G, L, W, nsrc_pts, ntgt_pts, phi, st);
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 
 cudaError_t launch_p2p_l2p_f64(const DevGeom& G, const DevTaskLists& L, const double* W, int64_t nsrc_pts,
@@ -1101,40 +1000,64 @@ cudaError_t launch_p2p_l2p_f64(const DevGeom& G, const DevTaskLists& L, const do
 }
 
 
-// ------------------------------------------- Galerkin sums + corrections
-// One warp per target element: u[d][e] = sum_q w_q phi[d][pos_q]
-//                                      + sum_k C[k] dens[d][col[k]].
-__global__ void k_elem_sum(DevGeom G, DevTaskLists L, const double* __restrict__ phi, int64_t ntp,
-                           const double* __restrict__ dens, int ndens, const double* __restrict__ dens_dl,
-                           double* __restrict__ out) {
-  const int64_t e = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (e >= L.ntgt_el) return;
-  const int tc = L.tgt_cls;
-  for (int d = 0; d < ndens; ++d) {
-    double s = 0.0;
-    if (lane < L.nq_tgt) {
-      const int pos = L.elem_pts[e * 4 + lane];
-      s = G.pt64[tc][pos].w * phi[(int64_t)d * ntp + pos];
-    }
-    const int64_t k0 = L.cor_off[e], k1 = L.cor_off[e + 1];
-#pragma unroll 4
-    for (int64_t k = k0 + lane; k < k1; k += 32) s += L.cor_val[k] * dens[(int64_t)d * L.nsrc_el + L.cor_col[k]];
-    // BtV double layer: - (N - Q) of dG/dn_y times g
-    if (dens_dl)
-      for (int64_t k = k0 + lane; k < k1; k += 32) s -= L.cor_val_dl[k] * dens_dl[(int64_t)d * L.nsrc_el + L.cor_col[k]];
+// ------------------------------------------- near corrections, Galerkin sums
+// The near corrections read the densities only, so they run beside the
+// expansions and the near field, and the Galerkin sums of the potentials are
+// added at the end.
+// LANES lanes per target element and density: out[d][e] = sum_k C[k] dens[d][col[k]].
+// On large meshes the FP64 pipe bounds it (two lanes a cycle and SM, so
+// sixteen cycles for any FP64 instruction of a warp): with a warp per element
+// the five reduction steps cost nearly as much as the seven products of an
+// average row (214 near pairs); with eight lanes four elements share three
+// steps (level-4 ball, with the Galerkin sums: 190 -> 137 us).  On small ones it
+// is latency, and a warp per element has the loads in flight sooner.
+template <int LANES>
+__global__ void __launch_bounds__(256) k_near_cor(DevTaskLists L, const double* __restrict__ dens,
+                                                  const double* __restrict__ dens_dl, double* __restrict__ out) {
+  const int64_t e = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / LANES;
+  const int lane = threadIdx.x % LANES;
+  const bool live = e < L.ntgt_el;
+  const int64_t k0 = live ? L.cor_off[e] : 0, k1 = live ? L.cor_off[e + 1] : 0;
+  const int64_t d = blockIdx.y;
+  double s = 0.0;
+#pragma unroll 8
+  for (int64_t k = k0 + lane; k < k1; k += LANES) s += L.cor_val[k] * dens[d * L.nsrc_el + L.cor_col[k]];
+  // BtV double layer: - (N - Q) of dG/dn_y times g
+  if (dens_dl)
+    for (int64_t k = k0 + lane; k < k1; k += LANES) s -= L.cor_val_dl[k] * dens_dl[d * L.nsrc_el + L.cor_col[k]];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) out[(int64_t)d * L.ntgt_el + e] = s;
-  }
+  for (int o = LANES / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (live && lane == 0) out[d * L.ntgt_el + e] = s;
 }
 
-cudaError_t launch_elem_sum(const DevGeom& G, const DevTaskLists& L, const double* phi, int64_t ntgt_pts,
-                            const double* dens_src, int ndens, double* out, cudaStream_t st, const double* dens_dl) {
+// out[d][e] += sum_q w_q phi[d][pos_q] (the points of an element have one weight)
+__global__ void k_elem_add(DevTaskLists L, const double* __restrict__ phi, int64_t ntp, int ndens, double* __restrict__ out) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i >= L.ntgt_el * ndens) return;
+  const int64_t d = i / L.ntgt_el, e = i - d * L.ntgt_el;
+  const int4 pos = reinterpret_cast<const int4*>(L.elem_pts)[e];
+  const double* ph = phi + d * ntp;
+  double s = ph[pos.x] + ph[pos.y] + ph[pos.z];
+  if (pos.w >= 0) s += ph[pos.w];
+  out[i] += L.elem_w[e] * s;
+}
+
+cudaError_t launch_near_cor(const DevTaskLists& L, const double* dens_src, int ndens, double* out, cudaStream_t st,
+                            const double* dens_dl) {
   if (L.ntgt_el == 0) return cudaSuccess;
   if (dens_dl && !L.cor_val_dl) return cudaErrorInvalidValue;
-  const int64_t threads = L.ntgt_el * 32;
-  k_elem_sum<<<(unsigned)((threads + 255) / 256), 256, 0, st>>>(G, L, phi, ntgt_pts, dens_src, ndens, dens_dl, out);
+  // 65,536 elements at eight lanes fill the SMs' warps twice
+  if (L.ntgt_el * ndens >= 65536)
+    k_near_cor<8><<<dim3((unsigned)((L.ntgt_el * 8 + 255) / 256), ndens), 256, 0, st>>>(L, dens_src, dens_dl, out);
+  else
+    k_near_cor<32><<<dim3((unsigned)((L.ntgt_el * 32 + 255) / 256), ndens), 256, 0, st>>>(L, dens_src, dens_dl, out);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_elem_add(const DevTaskLists& L, const double* phi, int64_t ntgt_pts, int ndens, double* out, cudaStream_t st) {
+  const int64_t n = L.ntgt_el * ndens;
+  if (n == 0) return cudaSuccess;
+  k_elem_add<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(L, phi, ntgt_pts, ndens, out);
   return cudaGetLastError();
 }
 

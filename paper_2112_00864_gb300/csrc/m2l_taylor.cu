@@ -505,7 +505,8 @@ template void m2l_taylor_rows<double>(const TaylorOffsets&, int, std::vector<dou
 template <typename T>
 cudaError_t launch_m2l_taylor(const DevGeom& G, const DevTaskLists& L, const TaylorTaskSched& S,
                               const TaylorTables& tab, int ndp, const T* mom, T* loc, T* momp, T* partial,
-                              cudaStream_t st) {
+                              cudaStream_t main, const TaylorFork* side) {
+  cudaStream_t st = main;
   int qtop = 0;
   for (int q = 1; q <= kTaylorMaxQ; ++q)
     if (S.ord[q].nwarp > 0) qtop = q;
@@ -535,9 +536,19 @@ cudaError_t launch_m2l_taylor(const DevGeom& G, const DevTaskLists& L, const Tay
       if (e != cudaSuccess) return e;
     }
   }
+  int norder = 0;
+  for (int q = 1; q <= kTaylorMaxQ; ++q) norder += S.ord[q].nwarp > 0;
+  const bool fork = side && side->side && norder > 1;
+  if (fork) {
+    cudaError_t e = cudaEventRecord(side->fork, main);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(side->side, side->fork, 0);
+    if (e != cudaSuccess) return e;
+  }
+  int k = 0;
   for (int q = 1; q <= kTaylorMaxQ; ++q) {
     const TaylorOrderSched& O = S.ord[q];
     if (O.nwarp == 0) continue;
+    st = fork && (k++ & 1) ? side->side : main;
     cudaError_t e = cudaSuccess;
     switch (q) {
       case 1: e = launch_order<T, 1>(O, tab, G, ndp, momp, loc, partial, st); break;
@@ -551,12 +562,18 @@ cudaError_t launch_m2l_taylor(const DevGeom& G, const DevTaskLists& L, const Tay
       default: e = cudaErrorInvalidValue;
     }
     if (e != cudaSuccess) return e;
+    partial += (size_t)O.nchunk * ndp * taylor_slot<T>(q);
+  }
+  if (fork) {
+    cudaError_t e = cudaEventRecord(side->join, side->side);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(main, side->join, 0);
+    if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
 }
 template cudaError_t launch_m2l_taylor<float>(const DevGeom&, const DevTaskLists&, const TaylorTaskSched&, const TaylorTables&,
-                                              int, const float*, float*, float*, float*, cudaStream_t);
+                                              int, const float*, float*, float*, float*, cudaStream_t, const TaylorFork*);
 template cudaError_t launch_m2l_taylor<double>(const DevGeom&, const DevTaskLists&, const TaylorTaskSched&, const TaylorTables&,
-                                               int, const double*, double*, double*, double*, cudaStream_t);
+                                               int, const double*, double*, double*, double*, cudaStream_t, const TaylorFork*);
 
 }  // namespace bcfmm

@@ -57,7 +57,7 @@ struct TaylorOrderSched {
 // the entry's 18.
 struct TaylorTaskSched {
   TaylorOrderSched ord[kTaylorMaxQ + 1];   // index = order q (nwarp 0: none)
-  size_t partial_per_dens = 0;             // values of chunk partial sums per density
+  size_t partial_per_dens = 0;             // values of chunk partial sums per density (all orders)
   const int* simt_sel = nullptr;           // targets (indices into the task's list) of
   int nsimt = 0;                           // higher orders: one CTA per target
 };
@@ -114,9 +114,16 @@ int m2l_taylor_pitch(int q);
 // tab.q must be the largest order of any target (the wide kernel reads the
 // g rows and moments up to it); targets in S.simt_sel use the wide kernel
 // (FP32; an FP64 caller runs the dense kernel for them).
+// side: a second stream for every other order (their targets differ, and
+// each order has its own part of `partial`), joined before the call returns;
+// null: all on st.
+struct TaylorFork {
+  cudaStream_t side = nullptr;
+  cudaEvent_t fork = nullptr, join = nullptr;
+};
 template <typename T>
 cudaError_t launch_m2l_taylor(const DevGeom& G, const DevTaskLists& L, const TaylorTaskSched& S,
                               const TaylorTables& tab, int ndp, const T* mom, T* loc, T* momp, T* partial,
-                              cudaStream_t st);
+                              cudaStream_t st, const TaylorFork* side = nullptr);
 
 }  // namespace bcfmm

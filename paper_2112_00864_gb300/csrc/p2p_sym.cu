@@ -1,12 +1,15 @@
 // Symmetric FP32 near field of VtV (see p2p_sym.cuh).
 //
-// Bound by the FMA pipe: 8 operations and one rsqrt serve both directions of a
-// pair of points, where the directed kernel spends 7 and one on each.  The
-// price is a slot per owner block and source point (45 M floats on the level-4
-// ball) and the pass that adds them.  Unit ball, level 4 (191,840 tets, 4.8e9
-// directed pairs, one density): near field 1.64 -> 1.04 ms (owners over 64
-// points 0.51, the others 0.45, gather 0.085; FMA pipe 66 and 61 % active,
-// what is missing goes to the staging rounds); level-3 ball 0.32 -> 0.25 ms.
+// Bound by the FMA pipe and the rsqrt unit alike: 8 operations (of 128 lanes a
+// cycle and SM) and one rsqrt (of 16) serve both directions of a pair of
+// points, where the directed kernel spends 7 and one on each; a register-only
+// loop of this body reaches 80 - 84 % of the FMA rate.  The price is a slot per
+// owner block and source point (45 M floats on the level-4 ball) and the pass
+// that adds them.  Unit ball, level 4 (191,840 tets, 4.8e9 directed pairs, one
+// density): near field 1.64 -> 1.00 ms (owners over 32 points 0.78, the others
+// 0.14, gather 0.083; FMA pipe 66 % active); level-3 ball 0.32 -> 0.23 ms; a
+// batch of six meshes with four densities 2.71 -> 1.57 ms (scalar kernel
+// before).
 #include <algorithm>
 #include <climits>
 #include <cmath>
@@ -18,9 +21,7 @@ namespace bcfmm {
 namespace {
 
 constexpr double kInv4PiS = 0.079577471545947667884441881686257;
-constexpr int kSymTile = 512;       // sources staged per round
 constexpr int kSymRuns = 256;       // source runs per batch
-constexpr int kSymFold = 2;         // rounds between folds: at most 64 products per FP32 sum
 
 __device__ __forceinline__ void two_sum(float& hi, float& lo, float x) {
   const float s = hi + x;
@@ -35,37 +36,71 @@ __device__ __forceinline__ float rsqrt_ftz(float x) {
   return y;
 }
 
-template <bool LARGE>
+// The sources of the next round arrive by cp.async while this one is computed
+// (each thread copies and converts its own, so no barrier is needed between).
+// LARGE (one density): a source is two float4 whose components stand in pairs,
+// ready for the packed instructions; owners that spend fewer instructions on a
+// source would be bound by those loads and read one float4, and so do the forms
+// for two and four densities, with the further weights beside it.
+template <int ND, bool LARGE>
 struct SymShared {
-  float4 xy[kSymTile];              // source k: (-x, -x, -y, -y)
-  float4 zw[kSymTile];              // (-z, -z, w, w)
-  float2 red[LARGE ? 16 : 8][128];  // (hi, lo) of target slot u, thread
+  static constexpr bool kLarge = LARGE;
+  static constexpr int kDens = ND, kTile = ND == 4 ? 256 : 512;     // sources staged per round
+  float4 xy[kTile];                 // LARGE: source k: (-x, -x, -y, -y); else (-x, -y, -z, w)
+  float4 zw[LARGE ? kTile : 1];     // (-z, -z, w, w)
+  float wx[ND > 1 ? ND * kTile : 1];  // [source][ND] weights (the first one again)
+  float4 rh[kTile], rl[kTile];      // copies in flight: hi and lo coordinates
+  float rw[ND][kTile];              // and weights
+  float2 red[LARGE ? 16 : 8][ND][128];  // (hi, lo) of target slot u, density, thread
   int pre[kSymRuns + 1], rst[kSymRuns];
 };
 
-// One staged round: source blocks of eight, four to a warp and step (one per
-// group of eight lanes).  A lane holds 2 T2 of the owner's points as T2 packed
-// pairs, the same in every group; in step s lane l takes source l ^ s of its
-// group's block, so that after eight steps every pair of the block was met
-// once, and the sum for a source has travelled with it through the eight lanes
-// (one shuffle a step).  SELF: the owner's own points, one direction only,
-// r = 0 selected out.
-template <int T2, bool SELF, class SH>
+__device__ __forceinline__ void copy16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copy4(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// One staged round: source blocks of GS, one per group of GS lanes and step.  A
+// lane holds 2 T2 of the owner's points as T2 packed pairs, the same in every
+// group; in step s lane l takes source l ^ s of its group's block, so that
+// after GS steps every pair of the block was met once, and the sum for a
+// source has travelled with it through the GS lanes (one shuffle a step).
+// SELF: the owner's own points, one direction only, r = 0 selected out.
+template <int T2, int GS, bool SELF, class SH, int ND>
 __device__ __forceinline__ void sym_round(const SH& S, int m, const float2 (&X)[T2], const float2 (&Y)[T2],
-                                          const float2 (&Z)[T2], const float2 (&Wt)[T2], float2 (&acc)[T2],
+                                          const float2 (&Z)[T2], const float2 (&Wt)[T2][ND], float2 (&acc)[T2][ND],
                                           float* __restrict__ out) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, l = lane & 7;
-  const int nb = (m + 7) >> 3;
-  for (int bb = warp * 4; bb < nb; bb += 16) {
-    const int b8 = (bb + (lane >> 3)) * 8;
-    float trav = 0.f;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, l = lane & (GS - 1);
+  for (int k0 = warp * 32; k0 < m; k0 += 128) {
+    const int kg = k0 + lane - l;
+    float trav[ND];
 #pragma unroll
-    for (int s = 0; s < 8; ++s) {
-      const int k = b8 + (l ^ s);
-      const float4 a = S.xy[k], c = S.zw[k];
-      const float2 nx = make_float2(a.x, a.y), ny = make_float2(a.z, a.w), nz = make_float2(c.x, c.y);
-      const float2 w = make_float2(c.z, c.w);
-      float2 as = make_float2(0.f, 0.f);
+    for (int d = 0; d < ND; ++d) trav[d] = 0.f;
+#pragma unroll
+    for (int s = 0; s < GS; ++s) {
+      const int k = kg + (l ^ s);
+      float2 nx, ny, nz, w[ND], as[ND];
+      const float4 a = S.xy[k];
+      if constexpr (SH::kLarge) {
+        const float4 c = S.zw[k];
+        nx = make_float2(a.x, a.y); ny = make_float2(a.z, a.w); nz = make_float2(c.x, c.y);
+        w[0] = make_float2(c.z, c.w);
+      } else {
+        nx = make_float2(a.x, a.x); ny = make_float2(a.y, a.y); nz = make_float2(a.z, a.z);
+        w[0] = make_float2(a.w, a.w);
+      }
+      if constexpr (ND == 2) {
+        const float v = S.wx[2 * k + 1];
+        w[ND - 1] = make_float2(v, v);
+      } else if constexpr (ND == 4) {
+        const float4 v = *reinterpret_cast<const float4*>(S.wx + 4 * k);
+        w[1 % ND] = make_float2(v.y, v.y);
+        w[2 % ND] = make_float2(v.z, v.z);
+        w[3 % ND] = make_float2(v.w, v.w);
+      }
 #pragma unroll
       for (int u = 0; u < T2; ++u) {
         const float2 dx = __fadd2_rn(X[u], nx), dy = __fadd2_rn(Y[u], ny), dz = __fadd2_rn(Z[u], nz);
@@ -73,72 +108,107 @@ __device__ __forceinline__ void sym_round(const SH& S, int m, const float2 (&X)[
         float2 ri;
         if constexpr (SELF) ri = make_float2(r2.x > 0.f ? rsqrt_ftz(r2.x) : 0.f, r2.y > 0.f ? rsqrt_ftz(r2.y) : 0.f);
         else ri = make_float2(rsqrt_ftz(r2.x), rsqrt_ftz(r2.y));
-        acc[u] = __ffma2_rn(w, ri, acc[u]);
-        if constexpr (!SELF) as = u == 0 ? __fmul2_rn(Wt[u], ri) : __ffma2_rn(Wt[u], ri, as);
+#pragma unroll
+        for (int d = 0; d < ND; ++d) {
+          acc[u][d] = __ffma2_rn(w[d], ri, acc[u][d]);
+          if constexpr (!SELF) as[d] = u == 0 ? __fmul2_rn(Wt[u][d], ri) : __ffma2_rn(Wt[u][d], ri, as[d]);
+        }
       }
       if constexpr (!SELF) {
-        trav += as.x + as.y;
-        trav = __shfl_xor_sync(0xffffffffu, trav, s < 7 ? (s ^ (s + 1)) : 7);
+#pragma unroll
+        for (int d = 0; d < ND; ++d) {
+          trav[d] += as[d].x + as[d].y;
+          trav[d] = __shfl_xor_sync(0xffffffffu, trav[d], s < GS - 1 ? (s ^ (s + 1)) : GS - 1);
+        }
       }
     }
-    if constexpr (!SELF)
-      if (b8 + l < m) out[b8 + l] = trav;
+    if constexpr (!SELF) {
+      if (kg + l < m) {
+        if constexpr (ND == 1) out[kg + l] = trav[0];
+        else if constexpr (ND == 2) reinterpret_cast<float2*>(out)[kg + l] = make_float2(trav[0], trav[1]);
+        else reinterpret_cast<float4*>(out)[kg + l] = make_float4(trav[0], trav[1], trav[2], trav[3]);
+      }
+    }
   }
 }
 
-template <int T2, class SH>
-__device__ __forceinline__ void sym_fold(SH& S, float2 (&acc)[T2]) {
+template <int T2, class SH, int ND>
+__device__ __forceinline__ void sym_fold(SH& S, float2 (&acc)[T2][ND]) {
 #pragma unroll
-  for (int u = 0; u < T2; ++u) {
-    float2 a = S.red[2 * u][threadIdx.x], b = S.red[2 * u + 1][threadIdx.x];
-    two_sum(a.x, a.y, acc[u].x);
-    two_sum(b.x, b.y, acc[u].y);
-    S.red[2 * u][threadIdx.x] = a;
-    S.red[2 * u + 1][threadIdx.x] = b;
-    acc[u] = make_float2(0.f, 0.f);
-  }
+  for (int u = 0; u < T2; ++u)
+#pragma unroll
+    for (int d = 0; d < ND; ++d) {
+      float2 a = S.red[2 * u][d][threadIdx.x], b = S.red[2 * u + 1][d][threadIdx.x];
+      two_sum(a.x, a.y, acc[u][d].x);
+      two_sum(b.x, b.y, acc[u][d].y);
+      S.red[2 * u][d][threadIdx.x] = a;
+      S.red[2 * u + 1][d][threadIdx.x] = b;
+      acc[u][d] = make_float2(0.f, 0.f);
+    }
 }
 
-template <int T2, class SH>
-__device__ __forceinline__ void sym_block(const DevGeom& G, const DevSym& L, const float* __restrict__ W, SH& S,
+template <int T2, int GS, class SH>
+__device__ __forceinline__ void sym_block(const DevGeom& G, const DevSym& L, const float* __restrict__ W, int64_t nsp, SH& S,
                                           int b, int nt, int2 tr, float4 ch, float4 cl) {
-  auto stage = [&](int k, int src) {
-    const float4 h = G.pthi[0][src], q = G.ptlo[0][src];
-    const float x = -((h.x - ch.x) + (q.x - cl.x)), y = -((h.y - ch.y) + (q.y - cl.y)), z = -((h.z - ch.z) + (q.z - cl.z));
-    const float w = W[src];
-    S.xy[k] = make_float4(x, x, y, y);
-    S.zw[k] = make_float4(z, z, w, w);
+  constexpr int ND = SH::kDens, kTile = SH::kTile;
+  auto put = [&](int k, float x, float y, float z, float w) {
+    if constexpr (SH::kLarge) {
+      S.xy[k] = make_float4(x, x, y, y);
+      S.zw[k] = make_float4(z, z, w, w);
+    } else {
+      S.xy[k] = make_float4(x, y, z, w);
+    }
+  };
+  auto put_df = [&](int k, const float4& h, const float4& q, float w) {
+    put(k, -((h.x - ch.x) + (q.x - cl.x)), -((h.y - ch.y) + (q.y - cl.y)), -((h.z - ch.z) + (q.z - cl.z)), w);
   };
   // padding: sources at -1e30 (stored negated), owner points at +1e30; the
   // distance overflows to inf, whose rsqrt is 0
   auto pad = [&](int k) {
-    S.xy[k] = make_float4(1e30f, 1e30f, 1e30f, 1e30f);
-    S.zw[k] = make_float4(1e30f, 1e30f, 0.f, 0.f);
+    put(k, 1e30f, 1e30f, 1e30f, 0.f);
+    if constexpr (ND > 1)
+      for (int d = 0; d < ND; ++d) S.wx[ND * k + d] = 0.f;
   };
   // the owner's points, staged as the first round's sources
-  if (threadIdx.x < nt) stage(threadIdx.x, tr.x + threadIdx.x);
-  else pad(threadIdx.x);
+  if (threadIdx.x < nt) {
+    const int j = tr.x + threadIdx.x;
+    put_df(threadIdx.x, G.pthi[0][j], G.ptlo[0][j], W[j]);
+    if constexpr (ND > 1)
+      for (int d = 0; d < ND; ++d) S.wx[ND * threadIdx.x + d] = W[d * nsp + j];
+  } else {
+    pad(threadIdx.x);
+  }
 #pragma unroll
-  for (int u = 0; u < 2 * T2; ++u) S.red[u][threadIdx.x] = make_float2(0.f, 0.f);
+  for (int u = 0; u < 2 * T2; ++u)
+#pragma unroll
+    for (int d = 0; d < ND; ++d) S.red[u][d][threadIdx.x] = make_float2(0.f, 0.f);
   __syncthreads();
-  float2 X[T2], Y[T2], Z[T2], Wt[T2], acc[T2];
-  const int l = threadIdx.x & 7;
+  float2 X[T2], Y[T2], Z[T2], Wt[T2][ND], acc[T2][ND];
+  const int l = threadIdx.x & (GS - 1);
 #pragma unroll
   for (int u = 0; u < T2; ++u) {
-    const int t0 = 16 * u + l, t1 = t0 + 8;
+    const int t0 = 2 * GS * u + l, t1 = t0 + GS;
     const bool v0 = t0 < nt, v1 = t1 < nt;
-    const float4 a0 = S.xy[t0], c0 = S.zw[t0], a1 = S.xy[t1], c1 = S.zw[t1];
-    X[u] = make_float2(v0 ? -a0.x : 1e30f, v1 ? -a1.x : 1e30f);
-    Y[u] = make_float2(v0 ? -a0.z : 1e30f, v1 ? -a1.z : 1e30f);
-    Z[u] = make_float2(v0 ? -c0.x : 1e30f, v1 ? -c1.x : 1e30f);
-    Wt[u] = make_float2(v0 ? c0.z : 0.f, v1 ? c1.z : 0.f);
-    acc[u] = make_float2(0.f, 0.f);
+    float4 p0 = S.xy[t0], p1 = S.xy[t1];         // (-x, -y, -z, w)
+    if constexpr (SH::kLarge) {
+      p0 = make_float4(p0.x, p0.z, S.zw[t0].x, S.zw[t0].z);
+      p1 = make_float4(p1.x, p1.z, S.zw[t1].x, S.zw[t1].z);
+    }
+    X[u] = make_float2(v0 ? -p0.x : 1e30f, v1 ? -p1.x : 1e30f);
+    Y[u] = make_float2(v0 ? -p0.y : 1e30f, v1 ? -p1.y : 1e30f);
+    Z[u] = make_float2(v0 ? -p0.z : 1e30f, v1 ? -p1.z : 1e30f);
+#pragma unroll
+    for (int d = 0; d < ND; ++d) {
+      if constexpr (ND > 1) { p0.w = S.wx[ND * t0 + d]; p1.w = S.wx[ND * t1 + d]; }
+      Wt[u][d] = make_float2(v0 ? p0.w : 0.f, v1 ? p1.w : 0.f);
+      acc[u][d] = make_float2(0.f, 0.f);
+    }
   }
-  if (L.self[b]) sym_round<T2, true>(S, nt, X, Y, Z, Wt, acc, nullptr);
+  if (L.self[b]) sym_round<T2, GS, true>(S, nt, X, Y, Z, Wt, acc, nullptr);
   const int r0 = L.run_off[b], r1 = L.run_off[b + 1];
   const int2 base = L.base[b];
-  float* out = L.src + base.x;
-  int fold = 0;
+  float* out = L.src + (int64_t)ND * base.x;
+  int fold = 0;                                  // a lane's FP32 sum holds at most 64 products between folds
   for (int rb = r0; rb < r1; rb += kSymRuns) {
     const int nr = min(kSymRuns, r1 - rb);
     __syncthreads();
@@ -158,64 +228,109 @@ __device__ __forceinline__ void sym_block(const DevGeom& G, const DevSym& L, con
     __syncthreads();
     const int total = S.pre[nr];
     int r = 0;                                   // this thread's run: its sources ascend
-    for (int v0 = 0; v0 < total; v0 += kSymTile) {
-      const int m = min(kSymTile, total - v0), mp = (m + 31) & ~31;
+    auto fetch = [&](int v0) {                   // copies of this thread's sources of the round at v0
 #pragma unroll
-      for (int q = 0; q < kSymTile / 128; ++q) {
+      for (int q = 0; q < kTile / 128; ++q) {
         const int k = threadIdx.x + q * 128, v = v0 + k;
-        if (k < m) {
+        if (v < total) {
           while (S.pre[r + 1] <= v) ++r;
-          stage(k, S.rst[r] + (v - S.pre[r]));
+          const int src = S.rst[r] + (v - S.pre[r]);
+          copy16(&S.rh[k], &G.pthi[0][src]);
+          copy16(&S.rl[k], &G.ptlo[0][src]);
+#pragma unroll
+          for (int d = 0; d < ND; ++d) copy4(&S.rw[d][k], &W[d * nsp + src]);
+        }
+      }
+    };
+    if (total > 0) fetch(0);
+    for (int v0 = 0; v0 < total; v0 += kTile) {
+      const int m = min(kTile, total - v0), mp = (m + 31) & ~31;
+      copy_wait();
+#pragma unroll
+      for (int q = 0; q < kTile / 128; ++q) {
+        const int k = threadIdx.x + q * 128;
+        if (k < m) {
+          put_df(k, S.rh[k], S.rl[k], S.rw[0][k]);
+          if constexpr (ND > 1) {
+#pragma unroll
+            for (int d = 0; d < ND; ++d) S.wx[ND * k + d] = S.rw[d][k];
+          }
         } else if (k < mp) {
           pad(k);
         }
       }
       __syncthreads();
-      sym_round<T2, false>(S, m, X, Y, Z, Wt, acc, out + v0);
-      if (++fold == kSymFold) { sym_fold<T2>(S, acc); fold = 0; }
+      if (v0 + kTile < total) fetch(v0 + kTile);
+      sym_round<T2, GS, false>(S, m, X, Y, Z, Wt, acc, out + ND * v0);
+      if (++fold >= 64 * 128 / (GS * kTile)) { sym_fold<T2>(S, acc); fold = 0; }
       __syncthreads();
     }
-    out += total;
+    out += ND * total;
   }
   sym_fold<T2>(S, acc);
   __syncthreads();
   if (threadIdx.x < nt) {
-    // the sixteen groups' sums of this point, in group order
-    const int t = threadIdx.x, u = t >> 3;
-    float hi = 0.f, lo = 0.f;
+    // the groups' sums of this point, in group order
+    const int t = threadIdx.x, u = t / GS;
 #pragma unroll
-    for (int g = 0; g < 16; ++g) {
-      const float2 v = S.red[u][g * 8 + (t & 7)];
-      two_sum(hi, lo, v.x);
-      lo += v.y;
+    for (int d = 0; d < ND; ++d) {
+      float hi = 0.f, lo = 0.f;
+#pragma unroll 16
+      for (int g = 0; g < 128 / GS; ++g) {
+        const float2 v = S.red[u][d][g * GS + (t & (GS - 1))];
+        two_sum(hi, lo, v.x);
+        lo += v.y;
+      }
+      L.tgt[(int64_t)ND * (base.y + t) + d] = make_float2(hi, lo);
     }
-    L.tgt[base.y + t] = make_float2(hi, lo);
   }
 }
 
-// LARGE: owners of more than 64 points (up to eight pairs a lane, 128
-// registers, four CTAs on an SM); the others need fewer registers and run six.
-template <bool LARGE>
-__global__ void __launch_bounds__(128, LARGE ? 4 : 6) k_p2p_sym(DevGeom G, DevSym L, int b0, const float* __restrict__ W) {
-  __shared__ SymShared<LARGE> S;
+// Groups of four lanes for small owners, of eight and sixteen for larger ones
+// (a lane holds at most eight pairs, four with several densities): the padding
+// is to eight, sixteen or 32 points, and the shared loads, the shuffles and the
+// sum for a source are paid once per lane of a group.  LARGE (one density):
+// owners of more than 32 points (five to eight pairs, 128 registers, four CTAs
+// on an SM); the others need fewer registers and run six.
+template <int ND, bool LARGE>
+__global__ void __launch_bounds__(128, ND == 1 && !LARGE ? 6 : 4) k_p2p_sym(DevGeom G, DevSym L, int b0,
+                                                                            const float* __restrict__ W, int64_t nsp) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  SymShared<ND, LARGE>& S = *reinterpret_cast<SymShared<ND, LARGE>*>(smraw);
   const int b = b0 + blockIdx.x;
   const int leaf = L.leaf[b];
   const float4 ch = G.box_hi[leaf], cl = G.box_lo[leaf];
   const int2 tr = G.box_rng[0][leaf];
   const int nt = tr.y - tr.x;
   if constexpr (LARGE) {
-    switch ((nt + 15) >> 4) {
-      case 5: sym_block<5>(G, L, W, S, b, nt, tr, ch, cl); break;
-      case 6: sym_block<6>(G, L, W, S, b, nt, tr, ch, cl); break;
-      case 7: sym_block<7>(G, L, W, S, b, nt, tr, ch, cl); break;
-      default: sym_block<8>(G, L, W, S, b, nt, tr, ch, cl); break;
+    if (nt <= 64) {
+      switch ((nt + 7) >> 3) {
+        case 5: sym_block<5, 4>(G, L, W, nsp, S, b, nt, tr, ch, cl); break;
+        case 6: sym_block<6, 4>(G, L, W, nsp, S, b, nt, tr, ch, cl); break;
+        case 7: sym_block<7, 4>(G, L, W, nsp, S, b, nt, tr, ch, cl); break;
+        default: sym_block<8, 4>(G, L, W, nsp, S, b, nt, tr, ch, cl); break;
+      }
+    } else {
+      switch ((nt + 15) >> 4) {
+        case 5: sym_block<5, 8>(G, L, W, nsp, S, b, nt, tr, ch, cl); break;
+        case 6: sym_block<6, 8>(G, L, W, nsp, S, b, nt, tr, ch, cl); break;
+        case 7: sym_block<7, 8>(G, L, W, nsp, S, b, nt, tr, ch, cl); break;
+        default: sym_block<8, 8>(G, L, W, nsp, S, b, nt, tr, ch, cl); break;
+      }
     }
   } else {
-    switch ((nt + 15) >> 4) {
-      case 1: sym_block<1>(G, L, W, S, b, nt, tr, ch, cl); break;
-      case 2: sym_block<2>(G, L, W, S, b, nt, tr, ch, cl); break;
-      case 3: sym_block<3>(G, L, W, S, b, nt, tr, ch, cl); break;
-      default: sym_block<4>(G, L, W, S, b, nt, tr, ch, cl); break;
+    if (nt <= 32) {
+      switch ((nt + 7) >> 3) {
+        case 1: sym_block<1, 4>(G, L, W, nsp, S, b, nt, tr, ch, cl); break;
+        case 2: sym_block<2, 4>(G, L, W, nsp, S, b, nt, tr, ch, cl); break;
+        case 3: sym_block<3, 4>(G, L, W, nsp, S, b, nt, tr, ch, cl); break;
+        default: sym_block<4, 4>(G, L, W, nsp, S, b, nt, tr, ch, cl); break;
+      }
+    } else if constexpr (ND > 1) {
+      if (nt <= 48) sym_block<3, 8>(G, L, W, nsp, S, b, nt, tr, ch, cl);
+      else if (nt <= 64) sym_block<4, 8>(G, L, W, nsp, S, b, nt, tr, ch, cl);
+      else if (nt <= 96) sym_block<3, 16>(G, L, W, nsp, S, b, nt, tr, ch, cl);
+      else sym_block<4, 16>(G, L, W, nsp, S, b, nt, tr, ch, cl);
     }
   }
 }
@@ -227,15 +342,18 @@ __global__ void __launch_bounds__(128, LARGE ? 4 : 6) k_p2p_sym(DevGeom G, DevSy
 // wait for them one by one.
 constexpr int kGatherThreads = 256, kGatherIdx = 1024;
 
-__global__ void __launch_bounds__(kGatherThreads) k_sym_gather(DevGeom G, DevSym L, double* __restrict__ phi) {
-  __shared__ float2 red[kGatherThreads];
+template <int ND>
+__global__ void __launch_bounds__(kGatherThreads) k_sym_gather(DevGeom G, DevSym L, int64_t ntp, double* __restrict__ phi) {
+  __shared__ float2 red[ND][kGatherThreads];
   __shared__ int idx[kGatherIdx];
   const int f = blockIdx.x, leaf = L.fin_leaf[f];
   const int2 tr = G.box_rng[0][leaf];
   const int nt = tr.y - tr.x;
   const int NG = kGatherThreads / nt, g = threadIdx.x / nt, i = threadIdx.x - g * nt;
   const int s0 = L.fin_src_off[f], s1 = L.fin_src_off[f + 1];
-  float hi = 0.f, lo = 0.f;
+  float hi[ND], lo[ND];
+#pragma unroll
+  for (int d = 0; d < ND; ++d) hi[d] = lo[d] = 0.f;
   for (int c = s0; c < s1; c += kGatherIdx) {
     const int n = min(kGatherIdx, s1 - c);
     if (c > s0) __syncthreads();
@@ -244,33 +362,70 @@ __global__ void __launch_bounds__(kGatherThreads) k_sym_gather(DevGeom G, DevSym
     if (g < NG) {
       const int e1 = n * (g + 1) / NG;
 #pragma unroll 8
-      for (int e = n * g / NG; e < e1; ++e) two_sum(hi, lo, __ldcg(L.src + idx[e] + i));
+      for (int e = n * g / NG; e < e1; ++e) {
+        const float* p = L.src + (int64_t)ND * (idx[e] + i);
+        float v[4];
+        if constexpr (ND == 1) v[0] = __ldcg(p);
+        else if constexpr (ND == 2) { const float2 q = __ldcg(reinterpret_cast<const float2*>(p)); v[0] = q.x; v[1] = q.y; }
+        else { const float4 q = __ldcg(reinterpret_cast<const float4*>(p)); v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w; }
+#pragma unroll
+        for (int d = 0; d < ND; ++d) two_sum(hi[d], lo[d], v[d]);
+      }
     }
   }
   if (g == 0)
-    for (int e = L.fin_tgt_off[f]; e < L.fin_tgt_off[f + 1]; ++e) {
-      const float2 v = __ldcg(L.tgt + L.fin_tgt[e] + i);
-      two_sum(hi, lo, v.x);
-      lo += v.y;
-    }
-  red[threadIdx.x] = make_float2(hi, lo);
+    for (int e = L.fin_tgt_off[f]; e < L.fin_tgt_off[f + 1]; ++e)
+#pragma unroll
+      for (int d = 0; d < ND; ++d) {
+        const float2 v = __ldcg(L.tgt + (int64_t)ND * (L.fin_tgt[e] + i) + d);
+        two_sum(hi[d], lo[d], v.x);
+        lo[d] += v.y;
+      }
+#pragma unroll
+  for (int d = 0; d < ND; ++d) red[d][threadIdx.x] = make_float2(hi[d], lo[d]);
   __syncthreads();
   if ((int)threadIdx.x >= nt) return;
-  for (int h = 1; h < NG; ++h) {
-    const float2 v = red[h * nt + i];
-    two_sum(hi, lo, v.x);
-    lo += v.y;
+#pragma unroll
+  for (int d = 0; d < ND; ++d) {
+    for (int h = 1; h < NG; ++h) {
+      const float2 v = red[d][h * nt + i];
+      two_sum(hi[d], lo[d], v.x);
+      lo[d] += v.y;
+    }
+    phi[d * ntp + tr.x + i] = ((double)hi[d] + (double)lo[d]) * kInv4PiS;
   }
-  phi[tr.x + i] = ((double)hi + (double)lo) * kInv4PiS;
 }
 
 }  // namespace
 
-cudaError_t launch_p2p_sym(const DevGeom& G, const DevSym& S, const float* W, double* phi, cudaStream_t st) {
+template <int ND, bool LARGE>
+cudaError_t launch_blocks(const DevGeom& G, const DevSym& S, int b0, int n, const float* W, int64_t nsp, cudaStream_t st) {
+  if (n <= 0) return cudaSuccess;
+  constexpr size_t sm = sizeof(SymShared<ND, LARGE>);
+  if (sm > 48 * 1024) {
+    const cudaError_t e = cudaFuncSetAttribute(k_p2p_sym<ND, LARGE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+  }
+  k_p2p_sym<ND, LARGE><<<n, 128, sm, st>>>(G, S, b0, W, nsp);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_p2p_sym(const DevGeom& G, const DevSym& S, const float* W, int64_t npts, int ndp, double* phi, cudaStream_t st) {
   if (S.nblk == 0) return cudaSuccess;
-  if (S.nlarge > 0) k_p2p_sym<true><<<S.nlarge, 128, 0, st>>>(G, S, 0, W);
-  if (S.nblk > S.nlarge) k_p2p_sym<false><<<S.nblk - S.nlarge, 128, 0, st>>>(G, S, S.nlarge, W);
-  k_sym_gather<<<S.nfin, kGatherThreads, 0, st>>>(G, S, phi);
+  cudaError_t e;
+  switch (ndp) {
+    case 1:
+      e = launch_blocks<1, true>(G, S, 0, S.nlarge, W, npts, st);
+      if (e == cudaSuccess) e = launch_blocks<1, false>(G, S, S.nlarge, S.nblk - S.nlarge, W, npts, st);
+      break;
+    case 2: e = launch_blocks<2, false>(G, S, 0, S.nblk, W, npts, st); break;
+    case 4: e = launch_blocks<4, false>(G, S, 0, S.nblk, W, npts, st); break;
+    default: return cudaErrorInvalidValue;
+  }
+  if (e != cudaSuccess) return e;
+  if (ndp == 1) k_sym_gather<1><<<S.nfin, kGatherThreads, 0, st>>>(G, S, npts, phi);
+  else if (ndp == 2) k_sym_gather<2><<<S.nfin, kGatherThreads, 0, st>>>(G, S, npts, phi);
+  else k_sym_gather<4><<<S.nfin, kGatherThreads, 0, st>>>(G, S, npts, phi);
   return cudaGetLastError();
 }
 
@@ -279,10 +434,13 @@ static inline bool sym_owns(const HostSetup& H, int a, int b) {
   return H.box[a].level != H.box[b].level ? H.box[a].level > H.box[b].level : a < b;
 }
 
+// owner points a block computes: padded to its lanes' pairs
+static inline int sym_pad(int nt) { return nt <= 64 ? (nt + 7) / 8 * 8 : (nt + 15) / 16 * 16; }
+
 // Lane work of both forms over the mesh: the symmetric one pads an owner to a
-// multiple of 16 points and spends 8 FP32 operations on a pair of points, the
-// directed one pads to 4 and spends 7 on each direction.  Tiny leaves (under
-// about 10 points) are better off with the latter.
+// multiple of 8 or 16 points and spends 8 FP32 operations on a pair of points,
+// the directed one pads to 4 and spends 7 on each direction.  Tiny leaves
+// (under about 5 points) are better off with the latter.
 bool p2p_sym_pays(const HostSetup& H) {
   const HostTask& T = H.task[0];
   double sym = 0, dir = 0;
@@ -295,7 +453,7 @@ bool p2p_sym_pays(const HostSetup& H) {
       nd += C.pt1[0] - C.pt0[0];
       if (!C.nchild && T.near_box[k] != a && sym_owns(H, a, T.near_box[k])) ns += C.pt1[0] - C.pt0[0];
     }
-    sym += 16 * std::ceil(nt / 16) * (ns + nt) * 8;
+    sym += sym_pad((int)nt) * (ns + nt) * 8.0;
     dir += 4 * std::ceil(nt / 4) * nd * 7;
   }
   return sym < dir;
@@ -346,11 +504,12 @@ bool build_p2p_sym(const HostSetup& H, int64_t chunk, HostSym& out) {
     }
     blk.push_back(std::move(cur));
   }
-  // owners of more than 64 points (a kernel of their own) first, then longest
-  // first: sources x target pairs a lane holds
+  // owners of one padded size in a row, the largest first, so that the blocks on
+  // an SM run the same code (mixed sizes missed the instruction cache: 1.04 ms
+  // for the level-4 ball's two kernels); then longest first
   std::stable_sort(blk.begin(), blk.end(), [](const Blk& x, const Blk& y) {
-    if ((x.nt > 64) != (y.nt > 64)) return x.nt > 64;
-    return (x.ns + 128) * ((x.nt + 15) / 16 + 1) > (y.ns + 128) * ((y.nt + 15) / 16 + 1);
+    const int px = sym_pad(x.nt), py = sym_pad(y.nt);
+    return px != py ? px > py : x.ns > y.ns;
   });
   std::vector<int> cnt(H.box.size() + 1, 0), tcnt(H.box.size() + 1, 0);
   int64_t ns = 0, ntg = 0;
@@ -378,7 +537,7 @@ bool build_p2p_sym(const HostSetup& H, int64_t chunk, HostSym& out) {
   out.run_off.push_back(0);
   for (const Blk& b : blk) {
     out.leaf.push_back(b.leaf);
-    out.nlarge += b.nt > 64;
+    out.nlarge += b.nt > 32;
     out.self.push_back(b.self);
     out.base.push_back((int)out.nsrc);
     out.base.push_back((int)out.ntgt);

@@ -1,5 +1,5 @@
-// Symmetric FP32 near field of VtV (one density): every pair of points is
-// evaluated once and serves both of its directions.
+// Symmetric FP32 near field of VtV (one, two or four densities): every pair of
+// points is evaluated once and serves both of its directions.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -23,14 +23,15 @@ struct HostSetup;
 // adds, per point, the slots that belong to it in a fixed order, so the result
 // does not depend on the order in which blocks run.
 struct DevSym {
-  int nblk = 0, nlarge = 0;         // the first nlarge blocks: owners of more than 64 points
+  int nblk = 0, nlarge = 0;         // the first nlarge blocks: owners of more than 32 points
   const int* leaf = nullptr;        // [nblk] owner
   const int* run_off = nullptr;     // [nblk + 1] into runs
   const int2* runs = nullptr;       // source runs (start, end), without the owner's own points
   const int2* base = nullptr;       // [nblk] (first src slot, first tgt slot)
   const int* self = nullptr;        // [nblk] 1: the block also holds the owner's own points
-  float* src = nullptr;             // source-side sums
-  float2* tgt = nullptr;            // owner-side sums (hi, lo)
+  int64_t nsrc = 0, ntgt = 0;       // slots
+  float* src = nullptr;             // [nsrc][ndp] source-side sums (sized with the work buffers)
+  float2* tgt = nullptr;            // [ntgt][ndp] owner-side sums (hi, lo)
   // gather kernel, per target leaf (most slots first)
   int nfin = 0;
   const int* fin_leaf = nullptr;
@@ -54,7 +55,9 @@ constexpr int64_t kSymChunkMin = 512, kSymChunkMax = 4096;
 int64_t p2p_sym_chunk(const HostSetup& H, int nsm);
 bool p2p_sym_pays(const HostSetup& H);
 
-// phi = near field of VtV / 4 pi (every target point)
-cudaError_t launch_p2p_sym(const DevGeom& G, const DevSym& S, const float* W, double* phi, cudaStream_t st);
+// densities (padded) that the symmetric form takes; more need too many registers
+inline bool p2p_sym_takes(const DevSym& S, int ndp) { return S.nblk > 0 && ndp <= 4; }
+// phi = near field of VtV / 4 pi (every target point; npts points per density in W and phi)
+cudaError_t launch_p2p_sym(const DevGeom& G, const DevSym& S, const float* W, int64_t npts, int ndp, double* phi, cudaStream_t st);
 
 }  // namespace bcfmm

@@ -565,6 +565,13 @@ void build_p2p_chunks(const HostSetup& H, int t, int64_t chunk, P2pChunks& out) 
   }
 }
 
+int64_t p2p_chunk(const HostSetup& H, int t, int nsm) {
+  const HostTask& T = H.task[t];
+  int64_t total = 0;
+  for (size_t r = 0; r < T.runs.size() / 2; ++r) total += T.runs[2 * r + 1] - T.runs[2 * r];
+  return std::min(kP2pChunk, std::max(kP2pChunkMin, total / (16 * (int64_t)nsm)));
+}
+
 void merge_setups(std::vector<HostSetup>& P, HostSetup& H) {
   const int nm = (int)P.size();
   H = HostSetup();
