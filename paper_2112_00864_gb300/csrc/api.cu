@@ -119,6 +119,7 @@ struct bcfmm_ctx {
   int ndens[3] = {0, 0, 0}, ndp[3] = {0, 0, 0};
   double* dens[3] = {nullptr, nullptr, nullptr};
   int* err = nullptr;                  // device error word (bounded device waits)
+  char* near_tabs = nullptr;           // function tables of the near rule
   size_t tc_partial_per_dens = 0;      // largest tensor-core partial-sum need over the tasks (float2)
   // Taylor-form M2L (BCFMM_FP32 and BCFMM_FP64): offset coefficients,
   // prescaled moments, chunk partial sums (largest need over the tasks,
@@ -530,7 +531,7 @@ static int upload_task(bcfmm_ctx* C, const HostSetup& H, int t) {
     CU(m.upload(&glx, gx.data(), gx.size(), st));
     CU(m.upload(&glw, gw.data(), gw.size(), st));
     CU(launch_near_rule(t, D.nnz, nullptr, cor_row, cor_col, tv, sv, tqp, tqw, sqp, sqw, glx, glw, C->prm.near_n,
-                        C->prm.near_k, 0, cor_val, st));
+                        C->prm.near_k, 0, C->near_tabs, cor_val, st));
     CU(cudaStreamSynchronize(st));
     for (void* p : {(void*)tv, (void*)sv, (void*)tqp, (void*)tqw, (void*)sqp, (void*)sqw, (void*)glx, (void*)glw,
                     (void*)cor_row})
@@ -575,7 +576,7 @@ static int upload_task(bcfmm_ctx* C, const HostSetup& H, int t) {
     D.n_learned = (int64_t)hc[1];
     D.n_singular = (int64_t)hc[3];
     CU(launch_near_rule(t, D.n_fp64, lists, cor_row, cor_col, g.tv, g.sv, g.tqp, g.tqw, g.sqp, g.sqw, g.glx, g.glw,
-                        C->prm.near_n, C->prm.near_k, 0, cor_val, st));
+                        C->prm.near_n, C->prm.near_k, 0, C->near_tabs, cor_val, st));
     if (learned) CU(launch_near_mlp(t, lists + cap, D.n_learned, cor_row, cor_col, g.tv, g.sv, par, cor_val, st));
     CU(m.alloc(&g.ns_list, std::max<int64_t>(D.n_singular, 1)));
     CU(cudaMemcpyAsync(g.ns_list, lists + 3 * cap, D.n_singular * sizeof(int64_t), cudaMemcpyDeviceToDevice, st));
@@ -615,7 +616,7 @@ static int upload_task(bcfmm_ctx* C, const HostSetup& H, int t) {
       CU(m.upload(&glx, gx.data(), gx.size(), st));
       CU(m.upload(&glw, gw.data(), gw.size(), st));
       CU(launch_near_rule(3, D.nnz, nullptr, drow, L.cor_col, tv, sv, tqp, tqw, sqp, sqw, glx, glw, C->prm.near_n,
-                          C->prm.near_k, 0, cdl, st));
+                          C->prm.near_k, 0, C->near_tabs, cdl, st));
       CU(cudaStreamSynchronize(st));
       for (void* p : {(void*)tv, (void*)sv, (void*)tqp, (void*)tqw, (void*)sqp, (void*)sqw, (void*)glx, (void*)glw,
                       (void*)drow})
@@ -828,6 +829,12 @@ static int build_impl(const double* verts, const int64_t* vert_off, const int32_
 
   if (C->mem.alloc(&C->err, 1) != cudaSuccess || cudaMemsetAsync(C->err, 0, sizeof(int), C->st) != cudaSuccess)
     return cleanup(fail(BCFMM_ERR_OOM, "build: device allocation failed (error word)"));
+  {
+    std::vector<char> tabs(near_rule_tabs_bytes());
+    near_rule_tabs_fill(tabs.data());
+    if (C->mem.upload(&C->near_tabs, tabs.data(), tabs.size(), C->st) != cudaSuccess)
+      return cleanup(fail(BCFMM_ERR_OOM, "build: device allocation failed (near-rule tables)"));
+  }
   C->nmesh = nmesh;
   C->reuse = reuse;
   for (int t = 0; t < 3; ++t) {
@@ -2007,7 +2014,7 @@ extern "C" int bcfmm_mlp_dataset(bcfmm_ctx* C, int32_t task, int64_t max_pairs, 
     e = launch_pair_data(task, sel, mcount, g.row, D.L.cor_col, g.tv, g.sv, feat, qhat, Q, bin, pairs, st);
   if (e == cudaSuccess)
     e = launch_near_rule(task, mcount, sel, g.row, D.L.cor_col, g.tv, g.sv, g.tqp, g.tqw, g.sqp, g.sqw, g.glx, g.glw,
-                         C->prm.near_n, C->prm.near_k, 1, Cv, st);
+                         C->prm.near_n, C->prm.near_k, 1, C->near_tabs, Cv, st);
   if (e == cudaSuccess) e = launch_label_ratio(Cv, Q, mcount, chat, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   cudaFree(sel);

@@ -119,7 +119,10 @@ cudaError_t launch_near_rule(int task, int64_t nnz, const int64_t* sel, const in
                              const double* tgt_v, const double* src_v,
                              const double* tgt_qp, const double* tgt_qw,
                              const double* src_qp, const double* src_qw,
-                             const double* glx, const double* glw, int n, int k, int compact,
+                             const double* glx, const double* glw, int n, int k, int compact, const void* tabs,
                              double* cor_val, cudaStream_t st);
+// tabs: device copy of the function tables (near_rule_tabs_bytes() bytes, filled on the host)
+size_t near_rule_tabs_bytes();
+void near_rule_tabs_fill(void* host);
 
 }  // namespace bcfmm
