@@ -36,7 +36,7 @@ __global__ void __launch_bounds__(kDirectThreads) k_direct_sample(DevGeom G, Dev
     for (int q = 0; q < nq; ++q) {
       const double dx = tp[q].x - y.x, dy = tp[q].y - y.y, dz = tp[q].z - y.z;
       const double r2 = dx * dx + dy * dy + dz * dz;
-      if (r2 > 0.0) g += tp[q].w / sqrt(r2);
+      if (r2 > 0.0) g += tp[q].w * rsqrt(r2);
     }
     g *= y.w;
     const int se = G.pt_elem[sc][j];
