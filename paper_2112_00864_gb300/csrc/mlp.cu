@@ -16,6 +16,8 @@
 // forward and backward passes on their BF16 roundings.
 #include <cuda_bf16.h>
 
+#include <algorithm>
+
 #include "kernels.cuh"
 #include "mlp.cuh"
 
@@ -228,93 +230,191 @@ __device__ __forceinline__ float warp_sum(float v) {
   return v;
 }
 
-// Mean loss and its gradient over n pairs (grad and loss accumulated with
-// atomics; the caller zeroes them).  One pair per thread.  Weight
-// gradients are outer-product sums over the pairs of a warp: the warp
-// stages its 32 rows of the two factors in shared memory and every lane
-// forms whole dot products over the 32 pairs (no per-parameter shuffles).
-constexpr int kStage = 65;                              // padded row of a staged factor
-constexpr int kGradSmem = (2 * kMlpParams + (kMlpThreads / 32) * 2 * 32 * kStage) * 4;
+// Mean loss and its gradient over n pairs (added with atomics to grad and
+// loss, which k_mlp_zero cleared).  A minibatch is small (about a thousand
+// pairs), so latency is the bound: a CTA of 256 threads takes P pairs (8, 16 or
+// 32, by the number of CTAs that n gives) and shares every layer among its
+// threads, activations and weights in shared memory.  With v = W3^T qhat the
+// output layer is two dot products (pred = v.h2 + b3.qhat) and its backward
+// pass is v itself: dz2 = dpred v gelu'(z2).
+// 1,024 pairs, gradient and Adam step with the copies of a caller that keeps its
+// state: 131 us with one pair per thread (eight CTAs, activations in local
+// memory), 51 us now, most of it the host's calls.
+constexpr int kGradThreads = 256;
+constexpr int kLdW2 = kMlpH + 1;                       // padded rows: W2 is read along both indexes
 
-__device__ __forceinline__ void warp_outer(const float* A, int na, const float* B, int nb, float* G, int lane) {
-  for (int idx = lane; idx < na * nb; idx += 32) {
-    const int a = idx / nb, b = idx - a * nb;
-    float s = 0.f;
-#pragma unroll 8
-    for (int p = 0; p < 32; ++p) s = fmaf(A[p * kStage + a], B[p * kStage + b], s);
-    atomicAdd(&G[idx], s);
-  }
-}
+template <int P>
+struct GradShared {
+  float W1[kMlpIn][kMlpH];                             // transposed: [k][j]
+  float W2[kMlpH][kLdW2];                              // [j][k]
+  float W3[kMlpOut][kMlpH];
+  float b1[kMlpH], b2[kMlpH], b3[kMlpOut];
+  float x[P][kMlpIn], qh[P][kMlpOut];
+  float h1[P][kMlpH], d1[P][kMlpH];                    // gelu, gelu' of layer 1 (d1: then dz1)
+  float h2[P][kMlpH], d2[P][kMlpH];                    // of layer 2 (d2: then dz2)
+  float v[P][kMlpH];
+  float part[2][P], dpred[P];
+};
 
-__device__ __forceinline__ void warp_colsum(const float* A, int na, float* G, int lane) {
-  for (int a = lane; a < na; a += 32) {
-    float s = 0.f;
-    for (int p = 0; p < 32; ++p) s += A[p * kStage + a];
-    atomicAdd(&G[a], s);
-  }
-}
-
-__global__ void __launch_bounds__(kMlpThreads) k_mlp_grad(const float* __restrict__ params,
-                                                          const float* __restrict__ feat,
-                                                          const float* __restrict__ qhat,
-                                                          const float* __restrict__ chat, int64_t n, float inv_n,
-                                                          float* __restrict__ grad, float* __restrict__ loss) {
-  extern __shared__ float sm[];
-  float* P = sm;
-  float* Gs = sm + kMlpParams;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  float* A = sm + 2 * kMlpParams + warp * 2 * 32 * kStage;
-  float* B = A + 32 * kStage;
-  load_params_bf16(params, P);
-  for (int i = threadIdx.x; i < kMlpParams; i += blockDim.x) Gs[i] = 0.f;
+template <int P>
+__global__ void __launch_bounds__(kGradThreads) k_mlp_grad(const float* __restrict__ params, const float* __restrict__ feat,
+                                                           const float* __restrict__ qhat, const float* __restrict__ chat,
+                                                           int64_t n, float inv_n, float* __restrict__ grad,
+                                                           float* __restrict__ loss) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  GradShared<P>& S = *reinterpret_cast<GradShared<P>*>(smraw);
+  const int tid = threadIdx.x, j = tid & 63, g = tid >> 6;      // unit, quarter of the pairs
+  const int64_t i0 = (int64_t)blockIdx.x * P;
+  constexpr int PQ = P / 4;
+  for (int i = tid; i < kMlpH * kMlpIn; i += kGradThreads) S.W1[i % kMlpIn][i / kMlpIn] = bf16r(params[kOffW1 + i]);
+  for (int i = tid; i < kMlpH * kMlpH; i += kGradThreads) S.W2[i / kMlpH][i % kMlpH] = bf16r(params[kOffW2 + i]);
+  for (int i = tid; i < kMlpOut * kMlpH; i += kGradThreads) S.W3[i / kMlpH][i % kMlpH] = bf16r(params[kOffW3 + i]);
+  if (tid < kMlpH) { S.b1[tid] = bf16r(params[kOffB1 + tid]); S.b2[tid] = bf16r(params[kOffB2 + tid]); }
+  if (tid < kMlpOut) S.b3[tid] = bf16r(params[kOffB3 + tid]);
+  for (int i = tid; i < P * kMlpIn; i += kGradThreads) S.x[i / kMlpIn][i % kMlpIn] = i0 + i / kMlpIn < n ? feat[i0 * kMlpIn + i] : 0.f;
+  for (int i = tid; i < P * kMlpOut; i += kGradThreads) S.qh[i / kMlpOut][i % kMlpOut] = i0 + i / kMlpOut < n ? qhat[i0 * kMlpOut + i] : 0.f;
   __syncthreads();
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  const bool live = i < n;
-  float x[kMlpIn], qh[kMlpOut], z1[kMlpH], z2[kMlpH];
-  for (int k = 0; k < kMlpIn; ++k) x[k] = live ? feat[i * kMlpIn + k] : 0.f;
-  for (int k = 0; k < kMlpOut; ++k) qh[k] = live ? qhat[i * kMlpOut + k] : 0.f;
-  const float pred = mlp_forward(P, x, qh, z1, z2);
-  const float e = live ? pred - chat[i] : 0.f;
-  const float dpred = 2.f * e * inv_n;
+  // layer 1 and v
+#pragma unroll 2
+  for (int q = 0; q < PQ; ++q) {
+    const int p = g * PQ + q;
+    float z = S.b1[j], v = 0.f;
+#pragma unroll
+    for (int k = 0; k < kMlpIn; ++k) z = fmaf(S.W1[k][j], S.x[p][k], z);
+#pragma unroll
+    for (int o = 0; o < kMlpOut; ++o) v = fmaf(S.W3[o][j], S.qh[p][o], v);
+    S.h1[p][j] = gelu(z);
+    S.d1[p][j] = gelu_d(z);
+    S.v[p][j] = v;
+  }
+  __syncthreads();
+  // layer 2 and pred
   {
-    const float l = warp_sum(e * e * inv_n);
-    if (lane == 0) atomicAdd(loss, l);
+    float z[PQ];
+#pragma unroll
+    for (int q = 0; q < PQ; ++q) z[q] = S.b2[j];
+    for (int k = 0; k < kMlpH; k += 4) {
+      float w[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) w[i] = S.W2[j][k + i];
+#pragma unroll
+      for (int q = 0; q < PQ; ++q) {
+        const float4 h = *reinterpret_cast<const float4*>(&S.h1[g * PQ + q][k]);
+        z[q] = fmaf(w[0], h.x, z[q]);
+        z[q] = fmaf(w[1], h.y, z[q]);
+        z[q] = fmaf(w[2], h.z, z[q]);
+        z[q] = fmaf(w[3], h.w, z[q]);
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < PQ; ++q) {
+      const int p = g * PQ + q;
+      const float h = gelu(z[q]);
+      S.h2[p][j] = h;
+      S.d2[p][j] = gelu_d(z[q]);
+      const float t = warp_sum(h * S.v[p][j]);
+      if ((tid & 31) == 0) S.part[(tid >> 5) & 1][p] = t;
+    }
   }
-  float* ra = A + lane * kStage;
-  float* rb = B + lane * kStage;
-  // layer 3: dy_o = dpred qhat_o;  dW3 = dy h2^T, db3 = dy
-  for (int o = 0; o < kMlpOut; ++o) ra[o] = dpred * qh[o];
-  for (int k = 0; k < kMlpH; ++k) rb[k] = gelu(z2[k]);
-  __syncwarp();
-  warp_outer(A, kMlpOut, B, kMlpH, Gs + kOffW3, lane);
-  warp_colsum(A, kMlpOut, Gs + kOffB3, lane);
-  float dz2[kMlpH];
-  for (int k = 0; k < kMlpH; ++k) {
-    float s = 0.f;
-    for (int o = 0; o < kMlpOut; ++o) s = fmaf(P[kOffW3 + o * kMlpH + k], ra[o], s);
-    dz2[k] = s * gelu_d(z2[k]);
-  }
-  __syncwarp();
-  // layer 2: dW2 = dz2 h1^T, db2 = dz2
-  for (int k = 0; k < kMlpH; ++k) { ra[k] = dz2[k]; rb[k] = gelu(z1[k]); }
-  __syncwarp();
-  warp_outer(A, kMlpH, B, kMlpH, Gs + kOffW2, lane);
-  warp_colsum(A, kMlpH, Gs + kOffB2, lane);
-  float dz1[kMlpH];
-  for (int m = 0; m < kMlpH; ++m) {
-    float s = 0.f;
-    for (int k = 0; k < kMlpH; ++k) s = fmaf(P[kOffW2 + k * kMlpH + m], ra[k], s);
-    dz1[m] = s * gelu_d(z1[m]);
-  }
-  __syncwarp();
-  // layer 1: dW1 = dz1 x^T, db1 = dz1
-  for (int m = 0; m < kMlpH; ++m) ra[m] = dz1[m];
-  for (int k = 0; k < kMlpIn; ++k) rb[k] = x[k];
-  __syncwarp();
-  warp_outer(A, kMlpH, B, kMlpIn, Gs + kOffW1, lane);
-  warp_colsum(A, kMlpH, Gs + kOffB1, lane);
   __syncthreads();
-  for (int p = threadIdx.x; p < kMlpParams; p += blockDim.x) atomicAdd(&grad[p], Gs[p]);
+  if (tid < 32) {
+    float l = 0.f;
+    for (int p = tid; p < P; p += 32) {
+      float pred = S.part[0][p] + S.part[1][p];
+#pragma unroll
+      for (int o = 0; o < kMlpOut; ++o) pred = fmaf(S.b3[o], S.qh[p][o], pred);
+      const float e = i0 + p < n ? pred - chat[i0 + p] : 0.f;
+      S.dpred[p] = 2.f * e * inv_n;
+      l = fmaf(e * e, inv_n, l);
+    }
+    l = warp_sum(l);
+    if (tid == 0) atomicAdd(loss, l);
+  }
+  __syncthreads();
+  // dz2 = dpred v gelu'(z2)
+#pragma unroll
+  for (int q = 0; q < PQ; ++q) {
+    const int p = g * PQ + q;
+    S.d2[p][j] *= S.dpred[p] * S.v[p][j];
+  }
+  __syncthreads();
+  // dz1 = (W2^T dz2) gelu'(z1); dW3, db3, dW2, db2
+  {
+    float t[PQ];
+#pragma unroll
+    for (int q = 0; q < PQ; ++q) t[q] = 0.f;
+    for (int k = 0; k < kMlpH; k += 4) {
+      float w[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) w[i] = S.W2[k + i][j];
+#pragma unroll
+      for (int q = 0; q < PQ; ++q) {
+        const float4 d = *reinterpret_cast<const float4*>(&S.d2[g * PQ + q][k]);
+        t[q] = fmaf(w[0], d.x, t[q]);
+        t[q] = fmaf(w[1], d.y, t[q]);
+        t[q] = fmaf(w[2], d.z, t[q]);
+        t[q] = fmaf(w[3], d.w, t[q]);
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < PQ; ++q) S.d1[g * PQ + q][j] *= t[q];
+  }
+  {
+    float a[16], c[4];                          // dW2[16 g + i][j], dW3[4 g + i][j]
+#pragma unroll
+    for (int i = 0; i < 16; ++i) a[i] = 0.f;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) c[i] = 0.f;
+    for (int p = 0; p < P; ++p) {
+      const float h = S.h1[p][j], u = S.h2[p][j] * S.dpred[p];
+#pragma unroll
+      for (int i = 0; i < 16; i += 4) {
+        const float4 d = *reinterpret_cast<const float4*>(&S.d2[p][16 * g + i]);
+        a[i] = fmaf(d.x, h, a[i]);
+        a[i + 1] = fmaf(d.y, h, a[i + 1]);
+        a[i + 2] = fmaf(d.z, h, a[i + 2]);
+        a[i + 3] = fmaf(d.w, h, a[i + 3]);
+      }
+      const float4 q = *reinterpret_cast<const float4*>(&S.qh[p][4 * g]);
+      c[0] = fmaf(q.x, u, c[0]);
+      c[1] = fmaf(q.y, u, c[1]);
+      c[2] = fmaf(q.z, u, c[2]);
+      c[3] = fmaf(q.w, u, c[3]);
+    }
+#pragma unroll
+    for (int i = 0; i < 16; ++i) atomicAdd(&grad[kOffW2 + (16 * g + i) * kMlpH + j], a[i]);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) atomicAdd(&grad[kOffW3 + (4 * g + i) * kMlpH + j], c[i]);
+    if (g == 0) {
+      float t = 0.f;
+      for (int p = 0; p < P; ++p) t += S.d2[p][j];
+      atomicAdd(&grad[kOffB2 + j], t);
+    } else if (g == 1 && j < kMlpOut) {
+      float t = 0.f;
+      for (int p = 0; p < P; ++p) t = fmaf(S.dpred[p], S.qh[p][j], t);
+      atomicAdd(&grad[kOffB3 + j], t);
+    }
+  }
+  __syncthreads();
+  // dW1[j][3 g + i], db1
+  {
+    float a[3] = {0.f, 0.f, 0.f}, t = 0.f;
+    for (int p = 0; p < P; ++p) {
+      const float d = S.d1[p][j];
+      t += d;
+#pragma unroll
+      for (int i = 0; i < 3; ++i) a[i] = fmaf(d, S.x[p][3 * g + i], a[i]);
+    }
+#pragma unroll
+    for (int i = 0; i < 3; ++i) atomicAdd(&grad[kOffW1 + j * kMlpIn + 3 * g + i], a[i]);
+    if (g == 0) atomicAdd(&grad[kOffB1 + j], t);
+  }
+}
+
+__global__ void k_mlp_zero(float* __restrict__ grad, float* __restrict__ loss) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < kMlpParams) grad[i] = 0.f;
+  if (i == kMlpParams) *loss = 0.f;
 }
 
 __global__ void k_mlp_adam(float* __restrict__ params, const float* __restrict__ grad, float* __restrict__ m1,
@@ -329,19 +429,101 @@ __global__ void k_mlp_adam(float* __restrict__ params, const float* __restrict__
   params[i] -= lr * (a * c1) / (sqrtf(b * c2) + eps);
 }
 
-__global__ void __launch_bounds__(kMlpThreads) k_mlp_predict(const float* __restrict__ params,
-                                                             const float* __restrict__ feat,
-                                                             const float* __restrict__ qhat, int64_t n,
-                                                             float* __restrict__ out) {
-  __shared__ float P[kMlpParams];
-  load_params_bf16(params, P);
-  __syncthreads();
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  float x[kMlpIn], qh[kMlpOut], z1[kMlpH], z2[kMlpH];
-  for (int k = 0; k < kMlpIn; ++k) x[k] = feat[i * kMlpIn + k];
-  for (int k = 0; k < kMlpOut; ++k) qh[k] = qhat[i * kMlpOut + k];
-  out[i] = mlp_forward(P, x, qh, z1, z2);
+// Predictions of n pairs: a CTA takes P pairs, every layer as a register-tiled
+// product out[64][P] (a thread: four units by P / 16 pairs; per input index one
+// 16-byte load of weights and PT / 4 of activations for 4 PT FMAs), activations
+// transposed in shared memory.  As in the gradient, v = W3^T qhat replaces the
+// output layer.  Bound by the FMA pipe and the 128 error functions a pair:
+// 200,000 pairs 151 us with one pair per thread, 90 us now.
+// A thread's units are jg + 16 i (the weights are stored in that order), and
+// activation rows are padded by four floats: the sixteen threads that share
+// pairs then store to different banks.
+constexpr int kPredThreads = 256;
+template <int P>
+struct PredShared {
+  float W1[kMlpIn][kMlpH], W2[kMlpH][kMlpH], W3[kMlpOut][kMlpH];   // [input][pred_unit(unit)]
+  float b1[kMlpH], b2[kMlpH], b3[kMlpOut];
+  float x[kMlpIn][P + 4], qh[kMlpOut][P + 4], h1[kMlpH][P + 4];
+};
+__device__ __forceinline__ int pred_unit(int j) { return (j & 15) * 4 + (j >> 4); }
+
+// acc[i][p] += sum_k W[k][4 jg + i] A[k][p0 + p]
+template <int K, int LDA, int PT>
+__device__ __forceinline__ void tile_product(const float (*W)[kMlpH], const float (*A)[LDA], int jg, int p0, float (&acc)[4][PT]) {
+#pragma unroll 4
+  for (int k = 0; k < K; ++k) {
+    const float4 w = *reinterpret_cast<const float4*>(&W[k][4 * jg]);
+    float a[PT];
+#pragma unroll
+    for (int p = 0; p < PT; p += (PT >= 4 ? 4 : 2)) {
+      if constexpr (PT >= 4) *reinterpret_cast<float4*>(a + p) = *reinterpret_cast<const float4*>(&A[k][p0 + p]);
+      else *reinterpret_cast<float2*>(a + p) = *reinterpret_cast<const float2*>(&A[k][p0 + p]);
+    }
+#pragma unroll
+    for (int p = 0; p < PT; ++p) {
+      acc[0][p] = fmaf(w.x, a[p], acc[0][p]);
+      acc[1][p] = fmaf(w.y, a[p], acc[1][p]);
+      acc[2][p] = fmaf(w.z, a[p], acc[2][p]);
+      acc[3][p] = fmaf(w.w, a[p], acc[3][p]);
+    }
+  }
+}
+
+template <int P>
+__global__ void __launch_bounds__(kPredThreads) k_mlp_predict(const float* __restrict__ params, const float* __restrict__ feat,
+                                                              const float* __restrict__ qhat, int64_t n,
+                                                              float* __restrict__ out) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  PredShared<P>& S = *reinterpret_cast<PredShared<P>*>(smraw);
+  constexpr int PT = P / 16;
+  const int tid = threadIdx.x, jg = tid & 15, p0 = (tid >> 4) * PT;
+  for (int i = tid; i < kMlpH * kMlpIn; i += kPredThreads) S.W1[i % kMlpIn][pred_unit(i / kMlpIn)] = bf16r(params[kOffW1 + i]);
+  for (int i = tid; i < kMlpH * kMlpH; i += kPredThreads) S.W2[i % kMlpH][pred_unit(i / kMlpH)] = bf16r(params[kOffW2 + i]);
+  for (int i = tid; i < kMlpOut * kMlpH; i += kPredThreads) S.W3[i / kMlpH][pred_unit(i % kMlpH)] = bf16r(params[kOffW3 + i]);
+  if (tid < kMlpH) { S.b1[pred_unit(tid)] = bf16r(params[kOffB1 + tid]); S.b2[pred_unit(tid)] = bf16r(params[kOffB2 + tid]); }
+  if (tid < kMlpOut) S.b3[tid] = bf16r(params[kOffB3 + tid]);
+  for (int64_t i0 = (int64_t)blockIdx.x * P; i0 < n; i0 += (int64_t)gridDim.x * P) {
+    __syncthreads();
+    for (int i = tid; i < P * kMlpIn; i += kPredThreads) S.x[i % kMlpIn][i / kMlpIn] = i0 + i / kMlpIn < n ? feat[i0 * kMlpIn + i] : 0.f;
+    for (int i = tid; i < P * kMlpOut; i += kPredThreads) S.qh[i % kMlpOut][i / kMlpOut] = i0 + i / kMlpOut < n ? qhat[i0 * kMlpOut + i] : 0.f;
+    __syncthreads();
+    float z[4][PT], v[4][PT];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int p = 0; p < PT; ++p) z[i][p] = S.b1[4 * jg + i];
+    tile_product<kMlpIn>(S.W1, S.x, jg, p0, z);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int p = 0; p < PT; ++p) {
+        z[i][p] = gelu(z[i][p]);
+        v[i][p] = 0.f;
+      }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int p = 0; p < PT; p += 2) {
+        *reinterpret_cast<float2*>(&S.h1[jg + 16 * i][p0 + p]) = make_float2(z[i][p], z[i][p + 1]);
+        z[i][p] = z[i][p + 1] = S.b2[4 * jg + i];
+      }
+    tile_product<kMlpOut>(S.W3, S.qh, jg, p0, v);
+    __syncthreads();
+    tile_product<kMlpH>(S.W2, S.h1, jg, p0, z);
+#pragma unroll
+    for (int p = 0; p < PT; ++p) {
+      float s = 0.f;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) s = fmaf(gelu(z[i][p]), v[i][p], s);
+#pragma unroll
+      for (int o = 1; o < 16; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      if (jg == 0 && i0 + p0 + p < n) {
+#pragma unroll
+        for (int o = 0; o < kMlpOut; ++o) s = fmaf(S.b3[o], S.qh[o][p0 + p], s);
+        out[i0 + p0 + p] = s;
+      }
+    }
+  }
 }
 
 // ------------------------------------------------------- setup passes
@@ -441,16 +623,28 @@ __global__ void k_label_ratio(const double* __restrict__ C, const double* __rest
 }
 
 // ------------------------------------------------------------ launchers
+template <int P>
+static cudaError_t launch_grad_p(const float* params, const float* feat, const float* qhat, const float* chat, int64_t n,
+                                 float* grad, float* loss, cudaStream_t st) {
+  constexpr size_t sm = sizeof(GradShared<P>);
+  if (sm > 48 * 1024) {
+    const cudaError_t e = cudaFuncSetAttribute(k_mlp_grad<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+  }
+  k_mlp_grad<P><<<(unsigned)((n + P - 1) / P), kGradThreads, sm, st>>>(params, feat, qhat, chat, n, 1.0f / (float)n, grad, loss);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_mlp_grad(const float* params, const float* feat, const float* qhat, const float* chat, int64_t n,
                             float* grad, float* loss, cudaStream_t st) {
-  cudaError_t e = cudaMemsetAsync(grad, 0, kMlpParams * sizeof(float), st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(loss, 0, sizeof(float), st);
+  k_mlp_zero<<<(kMlpParams + 256) / 256, 256, 0, st>>>(grad, loss);
+  const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess || n == 0) return e;
-  e = cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, kGradSmem);
-  if (e != cudaSuccess) return e;
-  k_mlp_grad<<<(unsigned)((n + kMlpThreads - 1) / kMlpThreads), kMlpThreads, kGradSmem, st>>>(
-      params, feat, qhat, chat, n, 1.0f / (float)n, grad, loss);
-  return cudaGetLastError();
+  // one CTA per SM while the pairs allow it: fewer pairs a CTA shorten its chain,
+  // more CTAs add their 6,032 gradients with as many more atomics
+  if (n <= 8 * 152) return launch_grad_p<8>(params, feat, qhat, chat, n, grad, loss, st);
+  if (n <= 16 * 152) return launch_grad_p<16>(params, feat, qhat, chat, n, grad, loss, st);
+  return launch_grad_p<32>(params, feat, qhat, chat, n, grad, loss, st);
 }
 
 cudaError_t launch_mlp_adam(float* params, const float* grad, float* m1, float* m2, int step, float lr, float b1,
@@ -460,11 +654,24 @@ cudaError_t launch_mlp_adam(float* params, const float* grad, float* m1, float* 
   return cudaGetLastError();
 }
 
+template <int P>
+static cudaError_t launch_predict_p(const float* params, const float* feat, const float* qhat, int64_t n, float* out,
+                                    cudaStream_t st) {
+  constexpr size_t sm = sizeof(PredShared<P>);
+  if (sm > 48 * 1024) {
+    const cudaError_t e = cudaFuncSetAttribute(k_mlp_predict<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+  }
+  const int64_t tiles = (n + P - 1) / P;
+  k_mlp_predict<P><<<(unsigned)std::min<int64_t>(tiles, 2 * 152), kPredThreads, sm, st>>>(params, feat, qhat, n, out);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_mlp_predict(const float* params, const float* feat, const float* qhat, int64_t n, float* out,
                                cudaStream_t st) {
   if (n == 0) return cudaSuccess;
-  k_mlp_predict<<<(unsigned)((n + kMlpThreads - 1) / kMlpThreads), kMlpThreads, 0, st>>>(params, feat, qhat, n, out);
-  return cudaGetLastError();
+  // 128 pairs a CTA once that fills the SMs, 32 below
+  return n >= 128 * 152 ? launch_predict_p<128>(params, feat, qhat, n, out, st) : launch_predict_p<32>(params, feat, qhat, n, out, st);
 }
 
 cudaError_t launch_near_classify(int task, int64_t nnz, const int* row, const int* col, const double* tgt_v,
