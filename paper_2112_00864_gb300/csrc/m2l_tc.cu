@@ -581,28 +581,30 @@ __global__ void __launch_bounds__(kThreads, 1) k_m2l_tc(TcArgs args) {
   }
 }
 
-// lambda[tgt][a] = (sum over the tile's units of SH + SL) / s, in unit order
+// lambda[tgt][a] = (sum over the tile's units of SH + SL) / s, in unit order;
+// one CTA per (tile, density, a), a thread per row.  A chain of one load per
+// unit: with the a's in a loop as well it was np times as long, and the orders
+// with few tiles and many units (a tile of order 5 on the h = 1/16 cube: 57)
+// took longer here than in the MMAs: VtV's three reductions 0.73 -> 0.03 ms.
 __global__ void __launch_bounds__(kTileM) k_m2l_unit_reduce(const int4* __restrict__ splits,
                                                           const int* __restrict__ tile_tgt,
                                                           const float2* __restrict__ partial, int nslot, int npad,
-                                                          int ndp, int np, int ms,
-                                                          const double4_32a* __restrict__ box_cs,
+                                                          int ndp, int ms, const double4_32a* __restrict__ box_cs,
                                                           float* __restrict__ loc) {
   const int4 S = splits[blockIdx.x];
-  const int d = blockIdx.y, row = threadIdx.x;
+  const int d = blockIdx.y, a = blockIdx.z, row = threadIdx.x;
   const int tgt = tile_tgt[S.x * kTileM + row];
   if (tgt < 0) return;
-  const float inv_s = (float)(1.0 / box_cs[tgt].w);
-  float* out = loc + ((int64_t)tgt * ndp + d) * ms;
-  for (int a = 0; a < np; ++a) {
-    float hi = 0.f, lo = 0.f;
-    for (int u = 0; u < S.z; ++u) {
-      const float2 v = partial[(((int64_t)d * nslot + S.y + u) * npad + a) * kTileM + row];
-      two_sum(hi, lo, v.x);
-      lo += v.y;
-    }
-    out[a] = (hi + lo) * inv_s;
+  const float2* p = partial + (((int64_t)d * nslot + S.y) * npad + a) * kTileM + row;
+  float hi = 0.f, lo = 0.f;
+#pragma unroll 8
+  for (int u = 0; u < S.z; ++u) {
+    const float2 v = p[(int64_t)u * npad * kTileM];
+    two_sum(hi, lo, v.x);
+    lo += v.y;
   }
+  const float inv_s = (float)(1.0 / box_cs[tgt].w);
+  loc[((int64_t)tgt * ndp + d) * ms + a] = (hi + lo) * inv_s;
 }
 
 }  // namespace
@@ -794,8 +796,8 @@ cudaError_t launch_m2l_tc(const DevGeom& G, const DevTaskLists& L, const TcTaskS
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     if (O.nsplit_tiles > 0) {
-      k_m2l_unit_reduce<<<dim3(O.nsplit_tiles, ndp), kTileM, 0, st>>>(O.splits, L.tc_tile_tgt, partial, O.nslot,
-                                                                       a.P.npad, ndp, a.P.np, G.ms, G.box_cs, loc);
+      k_m2l_unit_reduce<<<dim3(O.nsplit_tiles, ndp, a.P.np), kTileM, 0, st>>>(O.splits, L.tc_tile_tgt, partial, O.nslot,
+                                                                               a.P.npad, ndp, G.ms, G.box_cs, loc);
       e = cudaGetLastError();
       if (e != cudaSuccess) return e;
     }
