@@ -505,10 +505,46 @@ __global__ void __launch_bounds__(kThreads, 1) k_m2l_tc(TcArgs args) {
       okw = __shfl_sync(0xffffffffu, okw, 0);
       if (!okw) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      float* lout = nullptr;
-      float2* pout = nullptr;
-      float inv_s = 0.f;
+      const uint32_t dcol = tq + (uint32_t)(db * P.dwidth);
+      // running sum SH + SL of the unit; kept short, with the output in a loop
+      // of its own: the drain and producer warps of an SM sub-partition share
+      // its instruction cache
+#pragma unroll 1
+      for (int gi = 0; gi < ngrp; ++gi) {
+        const uint32_t col = (uint32_t)(gi * 16);
+        uint32_t r0[16], r1[16], r2[16], rh[16], rl[16];
+        BCFMM_LD16(dcol + col, r0);
+        if (nreg > 1) BCFMM_LD16(dcol + (uint32_t)P.brows + col, r1);
+        if (nreg > 2) BCFMM_LD16(dcol + (uint32_t)(2 * P.brows) + col, r2);
+        BCFMM_LD16(tq + (uint32_t)P.shcol + col, rh);
+        BCFMM_LD16(tq + (uint32_t)P.slcol + col, rl);
+        tmem_wait_ld();
+        BCFMM_DEP16(r0);
+        if (nreg > 1) BCFMM_DEP16(r1);
+        if (nreg > 2) BCFMM_DEP16(r2);
+        BCFMM_DEP16(rh);
+        BCFMM_DEP16(rl);
+        float sh[16], sl[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+          // the entry's value: smaller regions first
+          float v = 0.f;
+          if (nreg > 2) v = __uint_as_float(r2[i]);
+          if (nreg > 1) v += __uint_as_float(r1[i]);
+          v += __uint_as_float(r0[i]);
+          // (a unit's first entry starts from zero; the columns held the last unit's sum)
+          sh[i] = first ? 0.f : __uint_as_float(rh[i]);
+          sl[i] = first ? 0.f : __uint_as_float(rl[i]);
+          two_sum(sh[i], sl[i], v);
+        }
+        tmem_st16(tq + (uint32_t)P.shcol + col, sh);
+        tmem_st16(tq + (uint32_t)P.slcol + col, sl);
+      }
+      asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
       if (last) {
+        float* lout = nullptr;
+        float2* pout = nullptr;
+        float inv_s = 0.f;
         const int4 U = args.units[uf & kUnitMask];
         if (U.w < 0) {
           const int tgt = args.tile_tgt[U.x * kTileM + row];
@@ -519,56 +555,27 @@ __global__ void __launch_bounds__(kThreads, 1) k_m2l_tc(TcArgs args) {
         } else {
           pout = args.partial + ((int64_t)d * args.nslot + U.w) * P.npad * kTileM + row;
         }
-      }
-      const uint32_t dcol = tq + (uint32_t)(db * P.dwidth);
-      for (int gi = 0; gi < ngrp; ++gi) {
-        const uint32_t col = (uint32_t)(gi * 16);
-        uint32_t r0[16], r1[16], r2[16], rh[16], rl[16];
-        BCFMM_LD16(dcol + col, r0);
-        if (nreg > 1) BCFMM_LD16(dcol + (uint32_t)P.brows + col, r1);
-        if (nreg > 2) BCFMM_LD16(dcol + (uint32_t)(2 * P.brows) + col, r2);
-        if (!first) {
+        __syncwarp();
+#pragma unroll 1
+        for (int gi = 0; gi < ngrp; ++gi) {
+          const uint32_t col = (uint32_t)(gi * 16);
+          uint32_t rh[16], rl[16];
           BCFMM_LD16(tq + (uint32_t)P.shcol + col, rh);
           BCFMM_LD16(tq + (uint32_t)P.slcol + col, rl);
-        }
-        tmem_wait_ld();
-        BCFMM_DEP16(r0);
-        if (nreg > 1) BCFMM_DEP16(r1);
-        if (nreg > 2) BCFMM_DEP16(r2);
-        if (!first) {
+          tmem_wait_ld();
           BCFMM_DEP16(rh);
           BCFMM_DEP16(rl);
-        }
-        float sh[16], sl[16];
+          if (lout) {
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          // the entry's value: smaller regions first
-          float v = 0.f;
-          if (nreg > 2) v = __uint_as_float(r2[i]);
-          if (nreg > 1) v += __uint_as_float(r1[i]);
-          v += __uint_as_float(r0[i]);
-          if (first) {
-            sh[i] = v;
-            sl[i] = 0.f;
-          } else {
-            sh[i] = __uint_as_float(rh[i]);
-            sl[i] = __uint_as_float(rl[i]);
-            two_sum(sh[i], sl[i], v);
+            for (int i = 0; i < 16; ++i)
+              if ((int)col + i < P.np) lout[col + i] = (__uint_as_float(rh[i]) + __uint_as_float(rl[i])) * inv_s;
+          } else if (pout) {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) pout[(int64_t)(col + i) * kTileM] = make_float2(__uint_as_float(rh[i]), __uint_as_float(rl[i]));
           }
-        }
-        if (!last) {
-          tmem_st16(tq + (uint32_t)P.shcol + col, sh);
-          tmem_st16(tq + (uint32_t)P.slcol + col, sl);
-        } else if (lout) {
-#pragma unroll
-          for (int i = 0; i < 16; ++i)
-            if ((int)col + i < P.np) lout[col + i] = (sh[i] + sl[i]) * inv_s;
-        } else if (pout) {
-#pragma unroll
-          for (int i = 0; i < 16; ++i) pout[(int64_t)(col + i) * kTileM] = make_float2(sh[i], sl[i]);
+          __syncwarp();
         }
       }
-      if (!last) asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       mbar_arrive(smem_u32(&dempty[db]));
     }
