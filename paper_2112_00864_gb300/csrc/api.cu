@@ -1529,10 +1529,6 @@ static int ensure_work(bcfmm_ctx* C, int set, int ndp) {
     if (Y.tgt) m.release(Y.tgt);
     Y.src = nullptr;
     Y.tgt = nullptr;
-    if (Y.nblk > 0) {                  // (up to four densities take the symmetric form)
-      CU(m.alloc(&Y.src, (size_t)std::min(ndp, 4) * Y.nsrc));
-      CU(m.alloc(&Y.tgt, (size_t)std::min(ndp, 4) * Y.ntgt));
-    }
   }
   if (C->tc.nsplit > 0) {
     CU(m.alloc(&w.tc_partial, std::max<size_t>((size_t)ndp * C->tc_partial_per_dens, 1)));
@@ -1543,6 +1539,22 @@ static int ensure_work(bcfmm_ctx* C, int set, int ndp) {
   if (C->ty.q > 0) {
     CU(bytes(&w.ty_momp, (size_t)C->nbox * ndp * C->ty.gpitch * es));
     CU(bytes(&w.ty_partial, std::max<size_t>((size_t)ndp * C->ty_partial_per_dens, 1) * es));
+  }
+  // the symmetric near field's slots (up to four densities) last: where the
+  // device has no room for them the directed kernel, which needs none, serves
+  for (int t = t0; t <= t1; ++t) {
+    DevSym& Y = C->task[t].sym;
+    if (Y.nblk == 0) continue;
+    cudaError_t e = m.alloc(&Y.src, (size_t)std::min(ndp, 4) * Y.nsrc);
+    if (e == cudaSuccess) e = m.alloc(&Y.tgt, (size_t)std::min(ndp, 4) * Y.ntgt);
+    if (e == cudaErrorMemoryAllocation) {
+      (void)cudaGetLastError();
+      if (Y.src) m.release(Y.src);
+      Y.src = nullptr;
+      Y.nblk = 0;
+    } else {
+      CU(e);
+    }
   }
   w.ndp = ndp;
   C->work_gen++;
