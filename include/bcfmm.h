@@ -33,8 +33,10 @@
  *  - The caller owns every pointer it passes.  The library copies the mesh
  *    at build time and never keeps a caller pointer after a call returns.
  *  - A context is bound to the CUDA device current at build time and to the
- *    stream given there; all its device work is ordered on that stream.  It
- *    is not thread-safe: one host thread at a time per context.
+ *    stream given there; all its device work is ordered on that stream: the
+ *    parts of an evaluation that run on streams of the context's own start
+ *    after the work on that stream and are joined on it before the call
+ *    returns.  It is not thread-safe: one host thread at a time per context.
  *  - Element order in inputs and outputs is the caller's.  Outputs are FP64
  *    in every precision mode.
  */
@@ -262,9 +264,12 @@ int bcfmm_eval_graph(bcfmm_ctx* ctx, int32_t task_mask, double* out_vtv, double*
  *   out_dev   FP64 device array, one value per target element; written
  *             asynchronously on the context's stream
  * The M2L keeps its partial sums (tensor cores: per work unit; Taylor
- * form: per list chunk) in a fixed static device array of 64 MiB (every GPU that loads the library holds it until
- * the process exits) instead of the context's scratch; all other buffers
- * are the context's, sized by an earlier bcfmm_set_density (required once).
+ * form: per list chunk and target) in a fixed static device array of 64 MiB
+ * (every GPU that loads the library holds it until the process exits)
+ * instead of the context's scratch; all other buffers are the context's,
+ * sized by an earlier bcfmm_set_density (required once).  Where the sums of
+ * order 8 do not fit into the array too, all of them go to the context's
+ * scratch.
  * The first call on a device looks up that array's device address (a
  * one-time set-up, per device); make that first call before any stream
  * capture.  The address is kept for the life of the process, so a device
@@ -278,8 +283,8 @@ int bcfmm_eval_graph(bcfmm_ctx* ctx, int32_t task_mask, double* out_vtv, double*
  * returned, and cleared, by the next evaluation with host output.  The
  * call records no stage timings.
  * Errors: BCFMM_ERR_ARG (null pointer, bad task, context built with
- * precision BCFMM_FP64, or a mesh whose M2L needs more scratch than the
- * array holds: the message gives both sizes), BCFMM_ERR_STATE (no earlier
+ * precision BCFMM_FP64, or a mesh whose M2L needs more scratch, order 8
+ * left out, than the array holds: the message gives both sizes), BCFMM_ERR_STATE (no earlier
  * bcfmm_set_density, or the current device is not the context's),
  * BCFMM_ERR_CUDA.
  */
@@ -374,11 +379,11 @@ void bcfmm_destroy(bcfmm_ctx* ctx);
 int bcfmm_debug_m2l_matrix(int32_t p, const double* o, double* T);
 
 /*
- * Test hook: the per-offset coefficients of the Taylor-form M2L (precision
- * BCFMM_FP32), g[gamma] = D^gamma G(o) for |gamma| <= q (same multi-index
+ * Test hook: the per-offset coefficients of the Taylor-form M2L (precisions
+ * BCFMM_FP32 and BCFMM_FP64), g[gamma] = D^gamma G(o) for |gamma| <= q (same multi-index
  * order), from which the kernel rebuilds the matrix above as
  *   T[a][b] = g[a + b] (-1)^{|b|} / (a! b!),   |a| + |b| <= q.
- * The kernel stores them in FP32.  g: host [(q+1)(q+2)(q+3)/6].
+ * The kernel stores them in the context's precision.  g: host [(q+1)(q+2)(q+3)/6].
  * Errors: BCFMM_ERR_ARG.
  */
 int bcfmm_debug_m2l_taylor_coeffs(int32_t q, const double* o, double* g);
@@ -461,11 +466,12 @@ int bcfmm_debug_near_pairs(const double* verts, int64_t nvert, const int32_t* te
  * sequence, wrong first / last flags, partial slots of cut tiles not
  * consecutive); out[9..11], per task, the faults of the Taylor-form M2L
  * schedule built for 1, 7 and 152 SMs (a list entry of a target of order
- * 1..7 missing, duplicated, invented or in a lane whose chunk is another
- * target's; a chunk not in exactly one lane; a target of another order not
- * exactly once in the generic kernel's list); out[12..14], per task, the
+ * 1..8 missing, duplicated, invented, with another offset's coefficients or
+ * in a slot that is another target's; a chunk not in exactly one slot; a
+ * target of another order not exactly once in the generic kernels' list);
+ * out[12..14], per task, the
  * faults of the packed FP32 near field's blocks built with chunks of 96
- * points and of the library's 8192 (a source point of a leaf's list in no
+ * points and of 8192 (a source point of a leaf's list in no
  * chunk or in two, a chunk over its size, the leaf's own run not whole at
  * the front of chunk 0, scratch rows not one per chunk, work increasing
  * along the block order).  out: host int64 [15].

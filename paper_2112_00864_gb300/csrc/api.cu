@@ -481,6 +481,7 @@ static int upload_task(bcfmm_ctx* C, const HostSetup& H, int t) {
       S.wb = dwb; S.wslot = dws; S.ent = den; S.tgt = dtg; S.tchunk = dtc;
       const int slot = f64 ? taylor_slot<double>(O.q) : taylor_slot<float>(O.q);
       D.tys.partial_per_dens += (size_t)O.nchunk * slot;
+      if (O.q <= kTaylorRegQ) D.tys.partial_below8 += (size_t)O.nchunk * slot;
     }
     if (!sel.empty()) {
       int* dsel;
@@ -1951,7 +1952,10 @@ extern "C" int bcfmm_eval_noalloc(bcfmm_ctx* C, int32_t task, const double* dens
   size_t cap = 0;
   CU(m2l_tc_noalloc_scratch(dev, &partial, &cap));
   // tensor cores: float2 unit sums; Taylor form: float chunk sums
-  const size_t need = tcp ? D.tcs.partial_per_dens : (D.tys.partial_per_dens + 1) / 2;
+  // (order 8 does not count: where it does not fit, the context's own buffer,
+  // sized with the others, takes all of them)
+  const size_t need = tcp ? D.tcs.partial_per_dens : (D.tys.partial_below8 + 1) / 2;
+  const bool fits = tcp || D.tys.partial_per_dens <= 2 * cap;
   if (need > cap)
     return fail(BCFMM_ERR_ARG, "eval_noalloc: the mesh needs " + std::to_string(need * sizeof(float2)) +
                                    " bytes of M2L scratch, more than the fixed " + std::to_string(cap * sizeof(float2)) +
@@ -1961,7 +1965,7 @@ extern "C" int bcfmm_eval_noalloc(bcfmm_ctx* C, int32_t task, const double* dens
   r.dens = dens_dev;
   r.ndens = r.ndp = 1;
   r.out = out_dev;
-  r.partial = partial;
+  r.partial = fits ? partial : nullptr;
   CU(run_tasks(C, &r, 1, C->st));
   C->ev_rec[task] = false;             // no stage timings recorded by this call
   return BCFMM_OK;
