@@ -64,12 +64,11 @@ def workload():
 CHOSEN = dict(p=7, q0=6, eta0=0.6, leaf_size=128, precision="fp32")
 PLAIN = dict(p=7, q0=6, eta0=0.6, leaf_size=128, precision="fp64")
 SAMPLE_TARGETS = 1024      # per task, for the accuracy gate and the CPU baseline
-# DRAM bytes (read + write) of one launch of each reported kernel on this
-# workload, from ncu --set full captures of VtV's launch under
-# "--workload kernels"; they hold for the kernels as captured and are to be
+# DRAM bytes (read + write) of the named launches on this workload, from an ncu
+# capture of VtV's launches under "--workload kernels"; they hold for the kernels as captured and are to be
 # re-taken when a kernel changes
-NCU_TRAFFIC = {"k_p2p_l2p_f32x2": (44.42e6, "ncu capture, VtV launch (16,847 chunk blocks)"),
-               "k_m2l_taylor": (61.15e6, "ncu capture, VtV's order-6 launch")}
+NCU_TRAFFIC = {"k_p2p_sym": (356342784.0, "ncu capture, VtV's two k_p2p_sym launches and k_sym_gather"),
+               "k_m2l_taylor": (11823104.0, "ncu capture, VtV's order-6 launch")}
 
 
 def dist_env():
@@ -89,8 +88,8 @@ def peaks():
 
 
 def spmv_roofline(st: dict, sums_ms: float, ndens: int, pk: dict) -> dict:
-    """Roofline of the near-correction SpMV inside the element sums
-    (k_elem_sum, VtV + VtB): algorithmic bytes 12 per near pair (int32
+    """Roofline of the near-correction SpMV with the element sums
+    (k_near_cor, VtV + VtB): algorithmic bytes 12 per near pair (int32
     column + FP64 correction) plus 8 per near pair and density (the gathered
     density), over the stage's device time, against the measured copy
     bandwidth.  The per-element sums of the point potentials ride along
@@ -98,7 +97,7 @@ def spmv_roofline(st: dict, sums_ms: float, ndens: int, pk: dict) -> dict:
     nnz = sum(int(st.get(t, {}).get("near_pairs", 0)) for t in ("vtv", "vtb"))
     byts = nnz * (12 + 8 * ndens)
     ach = byts / (sums_ms * 1e-3) / 1e9 if sums_ms > 0 else None
-    return {"kernel": "k_elem_sum", "bound": "hbm", "achieved": ach, "peak": pk["hbm_gbs"], "unit": "GB/s",
+    return {"kernel": "k_near_cor", "bound": "hbm", "achieved": ach, "peak": pk["hbm_gbs"], "unit": "GB/s",
             "frac": ach / pk["hbm_gbs"] if ach is not None else None, "traffic": None,
             "note": "near-correction SpMV: 12 B per near pair (int32 column + FP64 value) + 8 B gathered density "
                     "per pair and density, VtV + VtB, vs the measured copy bandwidth",
@@ -371,18 +370,22 @@ def run_ours(args):
         m2l_ms = sv[2]
         sm_clk = clk.get("sm_mhz") or pk.get("sm_max_mhz", 2070.0)
         pairs = st["vtv"]["p2p_pairs"] + st["vtb"]["p2p_pairs"]
-        ops_p2p = 7.0 * pairs                                        # FP32-pipe ops per pair
+        # FP32-pipe ops: VtV evaluates a pair of points once for both directions
+        # (8 ops and one rsqrt), VtB every directed pair (7 and one)
+        ops_p2p = 4.0 * st["vtv"]["p2p_pairs"] + 7.0 * st["vtb"]["p2p_pairs"]
         nsm = torch.cuda.get_device_properties(local).multi_processor_count
         fp32_peak = nsm * 128 * pk.get("sm_max_mhz", 2070.0) * 1e6  # FP32-pipe ops/s at max clock
         ffma = bcfmm.measure_ffma(local)                             # measured FMA flop/s (FMA = 2)
         m2l_pairs = st["vtv"]["m2l_pairs"]
         # box pairs of each order times 2 C(q+6, 6): one FMA per (a, b) with |a| + |b| <= q
         m2l_flop = sum(2.0 * math.comb(q + 6, 6) * n for q, n in enumerate(st["vtv"]["m2l_pairs_by_order"]))
-        roof_p2p = {"kernel": "k_p2p_l2p_f32x2", "bound": "alu", "achieved": ops_p2p / (p2p_ms * 1e-3) / 1e12,
-                    "peak": fp32_peak / 1e12, "unit": "TFLOP/s", "traffic": NCU_TRAFFIC["k_p2p_l2p_f32x2"][0],
-                    "traffic_source": NCU_TRAFFIC["k_p2p_l2p_f32x2"][1],
-                    "note": f"FP32-pipe ops (7 per pair: 3 sub, 1 mul, 2 fma, 1 fma) per s vs {nsm} SMs x 128 "
-                            "lanes x max SM clock; the rsqrt on MUFU caps it at 7/8 of this peak",
+        roof_p2p = {"kernel": "k_p2p_sym", "bound": "alu", "achieved": ops_p2p / (p2p_ms * 1e-3) / 1e12,
+                    "peak": fp32_peak / 1e12, "unit": "TFLOP/s", "traffic": NCU_TRAFFIC["k_p2p_sym"][0],
+                    "traffic_source": NCU_TRAFFIC["k_p2p_sym"][1],
+                    "note": "FP32-pipe ops over the near-field and L2P stage (VtV, symmetric: 8 per unordered pair "
+                            "of points, 3 sub, 1 mul, 4 fma; VtB: 7 per directed pair) per s vs "
+                            f"{nsm} SMs x 128 lanes x max SM clock; one rsqrt per evaluated pair on MUFU (16 a "
+                            "cycle and SM) takes as long as its 8 ops",
                     "ms_per_step": float(p2p_ms), "pairs": int(pairs),
                     "peak_ffma_measured": ffma / 2 / 1e12}
         roof_p2p["frac"] = roof_p2p["achieved"] / roof_p2p["peak"]
