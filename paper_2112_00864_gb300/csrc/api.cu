@@ -479,7 +479,7 @@ static int upload_task(bcfmm_ctx* C, const HostSetup& H, int t) {
       CU(m.upload(&dtg, O.tgt.data(), O.tgt.size(), st));
       CU(m.upload(&dtc, O.tchunk.data(), O.tchunk.size(), st));
       S.wb = dwb; S.wslot = dws; S.ent = den; S.tgt = dtg; S.tchunk = dtc;
-      const int slot = f64 ? taylor_slot<double>(O.q) : taylor_slot<float>(O.q);
+      const int slot = f64 ? taylor_partial<double>(O.q) : taylor_partial<float>(O.q);
       D.tys.partial_per_dens += (size_t)O.nchunk * slot;
       if (O.q <= kTaylorRegQ) D.tys.partial_below8 += (size_t)O.nchunk * slot;
     }

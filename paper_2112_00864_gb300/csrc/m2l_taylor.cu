@@ -101,14 +101,14 @@ struct TaylorArgs {
   int nwarp, ndp, pitch, nbox;
   const T* momp;       // [ndp][nbox][pitch]
   const T* g;          // [27 nD][taylor_row<T>(Q)]
-  T* partial;          // [nchunk][ndp][taylor_slot<T>(Q)]
+  T* partial;          // [nchunk][ndp][taylor_partial<T>(Q)]
 };
 
 // Sums of the higher orders (FP64 from 6, FP32 from 8) do not fit the
 // registers: the outputs are dealt to two to four passes (grid z), each
 // staging the rows again
 template <typename T>
-__host__ __device__ constexpr int taylor_parts(int q) { return sizeof(T) == 4 ? (q <= 7 ? 1 : 2) : (q < 6 ? 1 : q - 4); }
+__host__ __device__ constexpr int taylor_parts(int q) { return sizeof(T) == 4 ? (q <= kTaylorRegQ ? 1 : 4) : (q < 6 ? 1 : q - 4); }
 constexpr int kTaylorWarps = 4;       // warps per CTA
 constexpr int kTaylorStageRows = 22;  // 18 g rows + 4 moment rows
 template <typename T>
@@ -129,6 +129,11 @@ size_t taylor_smem(int q) {
 // tets, orders 6 and 7, 7.7 M pairs): VtV's whole M2L stage 0.86 -> 0.49 ms, the
 // order-6 launch 0.57 -> 0.33 ms; FP64, cube of 3,072 tets against the dense
 // tables, one CTA per target: 3.37 -> 0.39 ms.
+// FP32 above kTaylorRegQ: every entry's products go into a compensated sum (hi,
+// lo), as in the one-CTA-per-target kernel; 42 outputs a pass leave registers
+// for the three arrays.  With plain sums over a chunk the potentials of sources
+// far away (level-3 ball, order 8) were off by 1.85e-7 against the FP64 form,
+// 1.38e-7 with one CTA per target.
 template <typename T, int Q, int NP>
 __global__ void __launch_bounds__(kTaylorWarps * 32) k_m2l_taylor(TaylorArgs<T> A) {
   constexpr int NQ = (Q + 1) * (Q + 2) * (Q + 3) / 6;
@@ -164,9 +169,14 @@ __global__ void __launch_bounds__(kTaylorWarps * 32) k_m2l_taylor(TaylorArgs<T> 
       }
     }
   };
-  T acc[NA];
+  constexpr bool COMP = taylor_comp<T>(Q);
+  T acc[NA], lo[COMP ? NA : 1], sum[COMP ? NA : 1];
 #pragma unroll
   for (int a = 0; a < NA; ++a) acc[a] = (T)0;
+  if constexpr (COMP) {
+#pragma unroll
+    for (int a = 0; a < NA; ++a) sum[a] = lo[a] = (T)0;
+  }
   int4 cur = A.ent[wb.x], nxt = cur;
   load(cur, stage);
   cp_async_commit();
@@ -211,6 +221,13 @@ __global__ void __launch_bounds__(kTaylorWarps * 32) k_m2l_taylor(TaylorArgs<T> 
       } else {
         taylor_contract<T, Q, 3 % NP, NP>(acc, mr, gr, terms);
       }
+      if constexpr (COMP) {
+#pragma unroll
+        for (int a = 0; a < NA; ++a) {
+          two_sum(sum[a], lo[a], acc[a]);
+          acc[a] = (T)0;
+        }
+      }
     }
     __syncwarp();
     if (NS == 1 && j + 1 < wb.y) {
@@ -220,15 +237,35 @@ __global__ void __launch_bounds__(kTaylorWarps * 32) k_m2l_taylor(TaylorArgs<T> 
     cur = nxt;
     nxt = nn;
   }
+  // the four lanes of a target
+  if constexpr (COMP) {
 #pragma unroll
-  for (int a = 0; a < NA; ++a) {
-    acc[a] += __shfl_xor_sync(0xffffffffu, acc[a], 8);
-    acc[a] += __shfl_xor_sync(0xffffffffu, acc[a], 16);
+    for (int a = 0; a < NA; ++a) {
+#pragma unroll
+      for (int m = 8; m <= 16; m <<= 1) {
+        const T h = __shfl_xor_sync(0xffffffffu, sum[a], m), l = __shfl_xor_sync(0xffffffffu, lo[a], m);
+        two_sum(sum[a], lo[a], h);
+        lo[a] += l;
+      }
+    }
+  } else {
+#pragma unroll
+    for (int a = 0; a < NA; ++a) {
+      acc[a] += __shfl_xor_sync(0xffffffffu, acc[a], 8);
+      acc[a] += __shfl_xor_sync(0xffffffffu, acc[a], 16);
+    }
   }
   if (!tlive || s != 0) return;
   const int c = A.wslot[w * 8 + t];
-  T* o = A.partial + ((int64_t)c * A.ndp + d) * SLOT;
-  if constexpr (NP == 1) {
+  T* o = A.partial + ((int64_t)c * A.ndp + d) * taylor_partial<T>(Q);
+  if constexpr (COMP) {
+#pragma unroll
+    for (int a = 0; a < NA; ++a)
+      if (a * NP + (int)blockIdx.z < NQ) {
+        o[a * NP + blockIdx.z] = sum[a];
+        o[SLOT + a * NP + blockIdx.z] = lo[a];
+      }
+  } else if constexpr (NP == 1) {
 #pragma unroll
     for (int v = 0; v < SLOT / EPC; ++v) {
       T x[EPC];
@@ -244,12 +281,13 @@ __global__ void __launch_bounds__(kTaylorWarps * 32) k_m2l_taylor(TaylorArgs<T> 
 }
 
 // loc[t][d][a] = post[a] / s_t * (sum over the target's chunks, in chunk
-// order, FP32: compensated), post[a] = 1 / a!; one thread per (target, d, a)
+// order, FP32: compensated), post[a] = 1 / a!; one thread per (target, d, a).
+// slot: values of a chunk's sums; off: its lo parts' offset there (0: none)
 template <typename T>
 __global__ void __launch_bounds__(128) k_m2l_taylor_reduce(int ntgt, const int* __restrict__ tgt,
                                                           const int* __restrict__ tchunk,
-                                                          const T* __restrict__ partial, int nq, int slot, int ndp,
-                                                          int ms, const T* __restrict__ post,
+                                                          const T* __restrict__ partial, int nq, int slot, int off,
+                                                          int ndp, int ms, const T* __restrict__ post,
                                                           const double4_32a* __restrict__ box_cs,
                                                           T* __restrict__ loc) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -264,6 +302,7 @@ __global__ void __launch_bounds__(128) k_m2l_taylor_reduce(int ntgt, const int* 
     const T x = __ldg(pp + (int64_t)c * ndp * slot);
     if constexpr (sizeof(T) == 4) two_sum(hi, lo, x);
     else hi += x;
+    if (off) lo += __ldg(pp + (int64_t)c * ndp * slot + off);
   }
   loc[((int64_t)tb * ndp + d) * ms + a] = (hi + lo) * post[a] / (T)box_cs[tb].w;
 }
@@ -357,7 +396,7 @@ cudaError_t launch_order(const TaylorOrderSched& O, const TaylorTables& tab, con
   if (e != cudaSuccess) return e;
   const int64_t n = (int64_t)O.ntgt * ndp * NQ;
   k_m2l_taylor_reduce<T><<<(unsigned)((n + 127) / 128), 128, 0, st>>>(
-      O.ntgt, O.tgt, O.tchunk, partial, NQ, taylor_slot<T>(Q), ndp, G.ms,
+      O.ntgt, O.tgt, O.tchunk, partial, NQ, taylor_partial<T>(Q), taylor_comp<T>(Q) ? taylor_slot<T>(Q) : 0, ndp, G.ms,
       static_cast<const T*>(tab.fac) + tab.gpitch, G.box_cs, loc);
   return cudaGetLastError();
 }
@@ -562,7 +601,7 @@ cudaError_t launch_m2l_taylor(const DevGeom& G, const DevTaskLists& L, const Tay
       default: e = cudaErrorInvalidValue;
     }
     if (e != cudaSuccess) return e;
-    partial += (size_t)O.nchunk * ndp * taylor_slot<T>(q);
+    partial += (size_t)O.nchunk * ndp * taylor_partial<T>(q);
   }
   if (fork) {
     cudaError_t e = cudaEventRecord(side->join, side->side);

@@ -37,9 +37,9 @@ constexpr int kTaylorMaxQ = 8, kTaylorRegQ = 7;
 // consecutive rows of D's 27 (the table holds the rows of a D together).  A
 // warp walks a chunk of P's entries, lane = target slot + 8 * source slot; it
 // adds the four lanes of a target at the end and writes the sum to the
-// target's slot of that chunk.  A second kernel adds a target's slots in
-// chunk order (FP32: compensated; deterministic) and stores the local
-// expansion.
+// target's slot of that chunk (FP32 order 8: a compensated sum, hi and lo).  A
+// second kernel adds a target's slots in chunk order (FP32: compensated;
+// deterministic) and stores the local expansion.
 struct TaylorOrderSched {
   int q = 0, nwarp = 0, nchunk = 0, ntgt = 0, chunk = 0;
   int64_t pairs = 0;
@@ -93,6 +93,12 @@ template <typename T>
 __host__ __device__ constexpr int taylor_slot(int q) {
   return (int)(((q + 1) * (q + 2) * (q + 3) / 6 * sizeof(T) + 15) / 16 * 16 / sizeof(T));
 }
+// whether a chunk's sums are compensated entry by entry, (hi, lo) in its slot, and
+// the slot's elements then
+template <typename T>
+__host__ __device__ constexpr bool taylor_comp(int q) { return sizeof(T) == 4 && q > kTaylorRegQ; }
+template <typename T>
+__host__ __device__ constexpr int taylor_partial(int q) { return taylor_slot<T>(q) * (taylor_comp<T>(q) ? 2 : 1); }
 // g rows of one order for the parent offsets offs (host, FP64 -> T)
 template <typename T>
 void m2l_taylor_rows(const TaylorOffsets& offs, int q, std::vector<T>& rows);
