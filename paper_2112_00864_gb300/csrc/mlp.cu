@@ -14,6 +14,7 @@
 // Parameter vector (FP32, 6032): W1[64][12] b1[64] W2[64][64] b2[64]
 // W3[16][64] b3[16].  Training keeps FP32 master weights and runs the
 // forward and backward passes on their BF16 roundings.
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -237,10 +238,17 @@ __device__ __forceinline__ float warp_sum(float v) {
 // threads, activations and weights in shared memory.  With v = W3^T qhat the
 // output layer is two dot products (pred = v.h2 + b3.qhat) and its backward
 // pass is v itself: dz2 = dpred v gelu'(z2).
+// The sums of eight CTAs (a cluster) are added in FP64 through distributed
+// shared memory, an eighth of the parameters each, so that one atomic per
+// parameter serves 8 P pairs: every FP32 addition to a running gradient rounds
+// it, and with an atomic per CTA 1,024 pairs were off by 1.9e-7 of the norm
+// (against FP64 autograd), twice as much as with one pair per thread in eight
+// CTAs.
 // 1,024 pairs, gradient and Adam step with the copies of a caller that keeps its
 // state: 131 us with one pair per thread (eight CTAs, activations in local
-// memory), 51 us now, most of it the host's calls.
+// memory), 54 us now, most of it the host's calls.
 constexpr int kGradThreads = 256;
+constexpr int kGradCluster = 8;
 constexpr int kLdW2 = kMlpH + 1;                       // padded rows: W2 is read along both indexes
 
 template <int P>
@@ -257,12 +265,15 @@ struct GradShared {
 };
 
 template <int P>
-__global__ void __launch_bounds__(kGradThreads) k_mlp_grad(const float* __restrict__ params, const float* __restrict__ feat,
+__global__ void __cluster_dims__(kGradCluster, 1, 1) __launch_bounds__(kGradThreads) k_mlp_grad(const float* __restrict__ params, const float* __restrict__ feat,
                                                            const float* __restrict__ qhat, const float* __restrict__ chat,
                                                            int64_t n, float inv_n, float* __restrict__ grad,
                                                            float* __restrict__ loss) {
   extern __shared__ __align__(16) unsigned char smraw[];
   GradShared<P>& S = *reinterpret_cast<GradShared<P>*>(smraw);
+  // the CTA's gradient and loss, in the place of the weights once they are used up
+  float* Gs = reinterpret_cast<float*>(smraw);
+  static_assert(offsetof(GradShared<P>, x) >= (kMlpParams + 1) * sizeof(float), "gradient over the weights");
   const int tid = threadIdx.x, j = tid & 63, g = tid >> 6;      // unit, quarter of the pairs
   const int64_t i0 = (int64_t)blockIdx.x * P;
   constexpr int PQ = P / 4;
@@ -317,6 +328,7 @@ __global__ void __launch_bounds__(kGradThreads) k_mlp_grad(const float* __restri
     }
   }
   __syncthreads();
+  float cta_loss = 0.f;
   if (tid < 32) {
     float l = 0.f;
     for (int p = tid; p < P; p += 32) {
@@ -327,8 +339,7 @@ __global__ void __launch_bounds__(kGradThreads) k_mlp_grad(const float* __restri
       S.dpred[p] = 2.f * e * inv_n;
       l = fmaf(e * e, inv_n, l);
     }
-    l = warp_sum(l);
-    if (tid == 0) atomicAdd(loss, l);
+    cta_loss = warp_sum(l);
   }
   __syncthreads();
   // dz2 = dpred v gelu'(z2)
@@ -359,6 +370,7 @@ __global__ void __launch_bounds__(kGradThreads) k_mlp_grad(const float* __restri
 #pragma unroll
     for (int q = 0; q < PQ; ++q) S.d1[g * PQ + q][j] *= t[q];
   }
+  __syncthreads();
   {
     float a[16], c[4];                          // dW2[16 g + i][j], dW3[4 g + i][j]
 #pragma unroll
@@ -382,20 +394,19 @@ __global__ void __launch_bounds__(kGradThreads) k_mlp_grad(const float* __restri
       c[3] = fmaf(q.w, u, c[3]);
     }
 #pragma unroll
-    for (int i = 0; i < 16; ++i) atomicAdd(&grad[kOffW2 + (16 * g + i) * kMlpH + j], a[i]);
+    for (int i = 0; i < 16; ++i) Gs[kOffW2 + (16 * g + i) * kMlpH + j] = a[i];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) atomicAdd(&grad[kOffW3 + (4 * g + i) * kMlpH + j], c[i]);
+    for (int i = 0; i < 4; ++i) Gs[kOffW3 + (4 * g + i) * kMlpH + j] = c[i];
     if (g == 0) {
       float t = 0.f;
       for (int p = 0; p < P; ++p) t += S.d2[p][j];
-      atomicAdd(&grad[kOffB2 + j], t);
+      Gs[kOffB2 + j] = t;
     } else if (g == 1 && j < kMlpOut) {
       float t = 0.f;
       for (int p = 0; p < P; ++p) t = fmaf(S.dpred[p], S.qh[p][j], t);
-      atomicAdd(&grad[kOffB3 + j], t);
+      Gs[kOffB3 + j] = t;
     }
   }
-  __syncthreads();
   // dW1[j][3 g + i], db1
   {
     float a[3] = {0.f, 0.f, 0.f}, t = 0.f;
@@ -406,9 +417,23 @@ __global__ void __launch_bounds__(kGradThreads) k_mlp_grad(const float* __restri
       for (int i = 0; i < 3; ++i) a[i] = fmaf(d, S.x[p][3 * g + i], a[i]);
     }
 #pragma unroll
-    for (int i = 0; i < 3; ++i) atomicAdd(&grad[kOffW1 + j * kMlpIn + 3 * g + i], a[i]);
-    if (g == 0) atomicAdd(&grad[kOffB1 + j], t);
+    for (int i = 0; i < 3; ++i) Gs[kOffW1 + j * kMlpIn + 3 * g + i] = a[i];
+    if (g == 0) Gs[kOffB1 + j] = t;
   }
+  if (tid == 0) Gs[kMlpParams] = cta_loss;
+  // the cluster's sums
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  cl.sync();
+  constexpr int kSlice = kMlpParams / kGradCluster + 1;
+  const int r0 = (int)cl.block_rank() * kSlice, r1 = min(r0 + kSlice, kMlpParams + 1);
+  for (int i = r0 + tid; i < r1; i += kGradThreads) {
+    double t = 0.0;
+#pragma unroll
+    for (int c = 0; c < kGradCluster; ++c) t += (double)cl.map_shared_rank(Gs, c)[i];
+    atomicAdd(i < kMlpParams ? &grad[i] : loss, (float)t);
+  }
+  cl.sync();                                     // (the others read this CTA's shared memory)
 }
 
 __global__ void k_mlp_zero(float* __restrict__ grad, float* __restrict__ loss) {
@@ -631,7 +656,8 @@ static cudaError_t launch_grad_p(const float* params, const float* feat, const f
     const cudaError_t e = cudaFuncSetAttribute(k_mlp_grad<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
   }
-  k_mlp_grad<P><<<(unsigned)((n + P - 1) / P), kGradThreads, sm, st>>>(params, feat, qhat, chat, n, 1.0f / (float)n, grad, loss);
+  const int64_t nclus = (n + P * kGradCluster - 1) / (P * kGradCluster);
+  k_mlp_grad<P><<<(unsigned)(nclus * kGradCluster), kGradThreads, sm, st>>>(params, feat, qhat, chat, n, 1.0f / (float)n, grad, loss);
   return cudaGetLastError();
 }
 
@@ -640,10 +666,12 @@ cudaError_t launch_mlp_grad(const float* params, const float* feat, const float*
   k_mlp_zero<<<(kMlpParams + 256) / 256, 256, 0, st>>>(grad, loss);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess || n == 0) return e;
-  // one CTA per SM while the pairs allow it: fewer pairs a CTA shorten its chain,
-  // more CTAs add their 6,032 gradients with as many more atomics
-  if (n <= 8 * 152) return launch_grad_p<8>(params, feat, qhat, chat, n, grad, loss, st);
-  if (n <= 16 * 152) return launch_grad_p<16>(params, feat, qhat, chat, n, grad, loss, st);
+  // fewer pairs a CTA shorten its chain (1,024 pairs, call and wait: 35 us at 16,
+  // 2,000 pairs 42 us at 16), but a cluster takes fewer pairs then, and every
+  // cluster rounds the running gradient once: 8 and 16 pairs up to eight and
+  // twelve clusters, which keeps the error below that of one CTA per 128 pairs
+  if (n <= 8 * 8 * kGradCluster) return launch_grad_p<8>(params, feat, qhat, chat, n, grad, loss, st);
+  if (n <= 12 * 16 * kGradCluster) return launch_grad_p<16>(params, feat, qhat, chat, n, grad, loss, st);
   return launch_grad_p<32>(params, feat, qhat, chat, n, grad, loss, st);
 }
 
