@@ -302,12 +302,41 @@ __device__ __forceinline__ void outer_point(const V3* tv, const double* gx, cons
   }
 }
 
+// this lane's part of the product rule of the point passes for the pair (t, s):
+// target point lane / nvs, source point lane % nvs (lanes beyond nvt nvs: zero)
+template <bool TGT_TET, int SRC>
+__device__ __forceinline__ double product_term(const NearRuleArgs& A, int t, int s, int lane) {
+  constexpr int nvt = TGT_TET ? 4 : 3, nvs = SRC == 0 ? 4 : 3;
+  if (lane >= nvt * nvs) return 0.0;
+  const int ti = lane / nvs, sj = lane % nvs;
+  const double* xp = A.tgt_qp + 3 * ((int64_t)t * nvt + ti);
+  const double* yp = A.src_qp + 3 * ((int64_t)s * nvs + sj);
+  const double dx = xp[0] - yp[0], dy = xp[1] - yp[1], dz = xp[2] - yp[2];
+  const double r = sqrt(dx * dx + dy * dy + dz * dz);
+  if (r == 0.0) return 0.0;
+  double q = A.tgt_qw[(int64_t)t * nvt + ti] * A.src_qw[(int64_t)s * nvs + sj] * kInv4PiN / r;
+  if constexpr (SRC == 2) {
+    const double* svp = A.src_v + (int64_t)s * 3 * nvs;
+    const V3 e0 = {svp[3] - svp[0], svp[4] - svp[1], svp[5] - svp[2]}, e1 = {svp[6] - svp[0], svp[7] - svp[1], svp[8] - svp[2]};
+    V3 ns = vcross(e0, e1);
+    ns = vscale(ns, 1.0 / sqrt(vdot(ns, ns)));
+    q *= (ns.x * dx + ns.y * dy + ns.z * dz) / (r * r);
+  }
+  return q;
+}
+
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
 // 64 consecutive pairs of the CSR (or of the selection list) per CTA.  The
 // pairs of one target share its outer points, staged in shared memory; a warp
 // takes one pair at a time, its lanes the outer points.  SRC: 0 tets, 1
 // triangles (single layer), 2 triangles (double layer, kernel dG/dn_y).  The
 // result of pair ii (CSR position k = sel[ii], or ii without a selection)
-// goes to cor_val[k], or to cor_val[ii] when compact is set.
+// goes to cor_val[k].
 // Bound by the FP64 pipe: 216 points x about 400 FP64 instructions a pair of
 // tets (about 750 with libm's functions, the outer points computed anew for
 // every pair and the source tet prepared by one lane).  Build of a 3,072-tet
@@ -375,40 +404,66 @@ __global__ void __launch_bounds__(128) k_near_rule(NearRuleArgs A) {
             sum += q.w * (SRC == 2 ? tri_solid(x, sv) : tri_pot(x, sv));
           }
         }
-        if (c0 + kNearPts >= total) {
-          sum *= kInv4PiN;
-          // product rule of the point passes for this pair
-          if (lane < nvt * nvs) {
-            const int ti = lane / nvs, sj = lane % nvs;
-            const double* xp = A.tgt_qp + 3 * ((int64_t)t * nvt + ti);
-            const double* yp = A.src_qp + 3 * ((int64_t)s * nvs + sj);
-            const double dx = xp[0] - yp[0], dy = xp[1] - yp[1], dz = xp[2] - yp[2];
-            const double r = sqrt(dx * dx + dy * dy + dz * dz);
-            if (r != 0.0) {
-              double q = A.tgt_qw[(int64_t)t * nvt + ti] * A.src_qw[(int64_t)s * nvs + sj] * kInv4PiN / r;
-              if constexpr (SRC == 2) {
-                const V3 e0 = {svp[3] - svp[0], svp[4] - svp[1], svp[5] - svp[2]}, e1 = {svp[6] - svp[0], svp[7] - svp[1], svp[8] - svp[2]};
-                V3 ns = vcross(e0, e1);
-                ns = vscale(ns, 1.0 / sqrt(vdot(ns, ns)));
-                q *= (ns.x * dx + ns.y * dy + ns.z * dz) / (r * r);
-              }
-              sum -= q;
-            }
-          }
-        } else {
-          sum *= kInv4PiN;
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        sum *= kInv4PiN;
+        if (c0 + kNearPts >= total) sum -= product_term<TGT_TET, SRC>(A, t, s, lane);
+        sum = warp_sum(sum);
         if (lane == 0) {
           if (c0 > 0) sum += part[i];
           part[i] = sum;
-          if (c0 + kNearPts >= total) A.cor_val[A.compact ? p0 + i : kk] = sum;
+          if (c0 + kNearPts >= total) A.cor_val[kk] = sum;
         }
       }
     }
     a = b;
   }
+}
+
+// The same for selections whose neighbouring pairs have different targets (the
+// strided samples of a training set): one warp per pair, its lanes compute the
+// outer points themselves.  The kernel above would find one pair per target, so
+// one warp in four at work, with two barriers a pair.  Cube of 3,072 tets, 2,000
+// of its near-singular VtV pairs with features and labels: 7.2 -> 0.76 ms, BtV
+// 6.6 -> 0.68 ms; 50,000: 11.5 -> 10.2 and 5.0 -> 3.9 ms.
+template <bool TGT_TET, int SRC>
+__global__ void __launch_bounds__(128) k_near_rule_each(NearRuleArgs A) {
+  constexpr int nvt = TGT_TET ? 4 : 3, nvs = SRC == 0 ? 4 : 3, nch = TGT_TET ? 8 : 4;
+  __shared__ SrcTet sS[SRC == 0 ? 4 : 1];
+  __shared__ NearTabs tabs;
+  __shared__ double gx[kMaxGL], gw[kMaxGL];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (SRC == 0) {
+    const double* src = reinterpret_cast<const double*>(A.tabs);
+    for (int i = threadIdx.x; i < (int)(sizeof(NearTabs) / sizeof(double)); i += 128) reinterpret_cast<double*>(&tabs)[i] = src[i];
+  }
+  if (threadIdx.x < A.n) { gx[threadIdx.x] = A.glx[threadIdx.x]; gw[threadIdx.x] = A.glw[threadIdx.x]; }
+  __syncthreads();
+  const int64_t ii = blockIdx.x * (int64_t)4 + warp;
+  if (ii >= A.nnz) return;
+  int npc = TGT_TET ? A.n * A.n * A.n : A.n * A.n, npieces = 1;
+  for (int i = 0; i < A.k; ++i) npieces *= nch;
+  const int total = npieces * npc;
+  const int64_t kk = A.sel ? A.sel[ii] : ii;
+  const int t = A.row[kk], s = A.col[kk];
+  V3 tv[4];
+  for (int i = 0; i < nvt; ++i) {
+    const double* q = A.tgt_v + ((int64_t)t * nvt + i) * 3;
+    tv[i] = {q[0], q[1], q[2]};
+  }
+  const double* svp = A.src_v + (int64_t)s * 3 * nvs;
+  V3 sv[3];
+  if constexpr (SRC == 0) src_tet_prepare(svp, sS[warp], lane);
+  else
+    for (int v = 0; v < 3; ++v) sv[v] = {svp[3 * v], svp[3 * v + 1], svp[3 * v + 2]};
+  double sum = 0.0;
+  for (int j = lane; j < total; j += 32) {
+    V3 x;
+    double wt;
+    outer_point<TGT_TET>(tv, gx, gw, A.n, A.k, npc, npieces, j, x, wt);
+    if constexpr (SRC == 0) sum = fma(wt, tet_pot(x, sS[warp], tabs), sum);
+    else sum += wt * (SRC == 2 ? tri_solid(x, sv) : tri_pot(x, sv));
+  }
+  sum = warp_sum(sum * kInv4PiN - product_term<TGT_TET, SRC>(A, t, s, lane));
+  if (lane == 0) A.cor_val[A.compact ? ii : kk] = sum;
 }
 
 static NearTabs make_tabs() {
@@ -434,6 +489,17 @@ cudaError_t launch_near_rule(int task, int64_t nnz, const int64_t* sel, const in
   if (n > kMaxGL) return cudaErrorInvalidValue;
   const NearRuleArgs A{sel, row, col, tgt_v, src_v, tgt_qp, tgt_qw, src_qp, src_qw, glx, glw, cor_val,
                        static_cast<const NearTabs*>(tabs), nnz, n, k, compact};
+  // compact: the results of a training set's sample (see k_near_rule_each)
+  if (compact) {
+    const unsigned grid = (unsigned)((nnz + 3) / 4);
+    switch (task) {
+      case 0: k_near_rule_each<true, 0><<<grid, 128, 0, st>>>(A); break;
+      case 1: k_near_rule_each<false, 0><<<grid, 128, 0, st>>>(A); break;
+      case 2: k_near_rule_each<true, 1><<<grid, 128, 0, st>>>(A); break;
+      default: return cudaErrorInvalidValue;
+    }
+    return cudaGetLastError();
+  }
   const unsigned grid = (unsigned)((nnz + kNearPairs - 1) / kNearPairs);
   switch (task) {
     case 0: k_near_rule<true, 0><<<grid, 128, 0, st>>>(A); break;
