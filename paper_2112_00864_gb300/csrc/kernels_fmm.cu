@@ -879,21 +879,11 @@ __global__ void __launch_bounds__(128) k_p2p_f32x2(DevGeom G, DevTaskLists L, co
   }
 }
 
-// 1 / sqrt(x) of a normal positive double: the hardware's approximation (about
-// 20 bits) and one step of third order, y (1 + e / 2 + 3 e^2 / 8) with e = 1 -
-// x y^2, whose next term is below 2^-57: five FP64 instructions where the
-// square root and the division took some twenty.
-__device__ __forceinline__ double rsqrt_f64(double x) {
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double e = fma(-(x * y), y, 1.0);
-  return fma(e * y, fma(e, 0.375, 0.5), y);
-}
-
 // FP64 near field with L2P: a thread per target point, 128 / nt groups share the
-// sources.  FP64 instructions bound it (12 a pair, two lanes a cycle and SM).
-// 3,072-tet cube, 18.2 M pairs: 1.23 -> 0.55 ms (the target slots were padded to
-// powers of two before).
+// sources.  FP64 instructions bound it (some 14 a pair, two lanes a cycle and SM;
+// the square root and a division took some twenty).  3,072-tet cube, 18.2 M pairs:
+// 1.23 -> 0.56 ms (the target slots were padded to powers of two before); level-3
+// ball, 816 M pairs, the whole evaluation 59.1 -> 29.7 ms.
 template <int ND>
 __global__ void __launch_bounds__(128) k_p2p_l2p_f64(DevGeom G, DevTaskLists L, const double* __restrict__ W,
                                                      int64_t nsp, int64_t ntp, int ndp,
@@ -946,7 +936,7 @@ __global__ void __launch_bounds__(128) k_p2p_l2p_f64(DevGeom G, DevTaskLists L, 
           const double dx = xt - s.x, dy = yt - s.y, dz = zt - s.z;
           const double r2 = dx * dx + dy * dy + dz * dz;
           // (an integer test: a comparison would go through the FP64 pipe)
-          const double ri = (__double2hiint(r2) | __double2loint(r2)) ? rsqrt_f64(r2) : 0.0;
+          const double ri = (__double2hiint(r2) | __double2loint(r2)) ? rsqrt(r2) : 0.0;
           acc[0] += s.w * ri;
 #pragma unroll
           for (int d = 1; d < ND; ++d) acc[d] += tw[d - 1][j] * ri;
