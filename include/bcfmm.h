@@ -401,6 +401,15 @@ int bcfmm_debug_m2l_taylor_coeffs(int32_t q, const double* o, double* g);
 int bcfmm_debug_shift_matrix(int32_t kind, int32_t p, int32_t octant, double* out);
 
 /*
+ * Test hook: the near rule's own elementary functions, elementwise on the
+ * current device's default stream.  kind 0: out = a / b (normal numbers,
+ * quotient away from the ends of the range); 1: out = ln(a / b), a >= b > 0;
+ * 2: out = atan2(a, b), a > 0.  a, b, out: host [n], n in 1..2^24.
+ * Errors: BCFMM_ERR_ARG, BCFMM_ERR_CUDA.
+ */
+int bcfmm_debug_near_math(int32_t kind, int64_t n, const double* a, const double* b, double* out);
+
+/*
  * Test hook for the failure path of the bounded device waits (the paper has
  * no counterpart): enqueues on the context's stream one thread that waits,
  * through the same bounded mbarrier wait the tensor-core M2L uses, on a

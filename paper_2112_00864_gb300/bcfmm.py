@@ -26,7 +26,8 @@ EXPORTED = ["bcfmm_default_params", "bcfmm_build_bc_tree", "bcfmm_set_density", 
             "bcfmm_build_like", "bcfmm_direct_sample", "bcfmm_mlp_blob_size", "bcfmm_mlp_dataset",
             "bcfmm_mlp_grad", "bcfmm_mlp_adam", "bcfmm_mlp_predict", "bcfmm_debug_expire_wait",
             "bcfmm_debug_list_coverage", "bcfmm_debug_near_pairs", "bcfmm_debug_shift_matrix",
-            "bcfmm_debug_tree_counts", "bcfmm_debug_m2l_taylor_coeffs", "bcfmm_measure_ffma"]
+            "bcfmm_debug_tree_counts", "bcfmm_debug_m2l_taylor_coeffs", "bcfmm_measure_ffma",
+            "bcfmm_debug_near_math"]
 NEAR_MODE = {"fp64": 0, "learned": 1, "none": 2}
 TASK_BIT = {"vtv": 1, "vtb": 2, "btv": 4}
 
@@ -99,6 +100,8 @@ def load(path: str = LIB_PATH):
         L.bcfmm_mlp_predict.restype = C.c_int
         L.bcfmm_debug_expire_wait.argtypes = [p, i32]
         L.bcfmm_debug_expire_wait.restype = C.c_int
+        L.bcfmm_debug_near_math.argtypes = [i32, i64, p, p, p]
+        L.bcfmm_debug_near_math.restype = C.c_int
         L.bcfmm_debug_list_coverage.argtypes = [p, p, p, p, p, p, i32, C.POINTER(Params), p]
         L.bcfmm_debug_list_coverage.restype = C.c_int
         L.bcfmm_debug_near_pairs.argtypes = [p, i64, p, i64, p, i64, d, i32, i64, p, p, C.POINTER(C.c_int64)]
@@ -169,6 +172,17 @@ def debug_m2l_taylor_coeffs(q: int, o) -> np.ndarray:
     g = np.zeros(nterms(q))
     _check(load().bcfmm_debug_m2l_taylor_coeffs(q, o.ctypes.data, g.ctypes.data))
     return g
+
+
+def debug_near_math(kind: str, a, b) -> np.ndarray:
+    """The near rule's own functions on the GPU: "div" a / b, "log" ln(a / b) for
+    a >= b > 0, "atan" atan2(a, b) for a > 0."""
+    a, b = np.ascontiguousarray(a, np.float64), np.ascontiguousarray(b, np.float64)
+    out = np.zeros(a.shape)
+    assert a.shape == b.shape
+    _check(load().bcfmm_debug_near_math({"div": 0, "log": 1, "atan": 2}[kind], a.size, a.ctypes.data, b.ctypes.data,
+                                        out.ctypes.data))
+    return out
 
 
 def debug_shift_matrix(kind: str, p: int, octant: int) -> np.ndarray:

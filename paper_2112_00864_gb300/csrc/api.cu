@@ -2077,6 +2077,25 @@ extern "C" int bcfmm_measure_ffma(int32_t device, double* flops) {
   return BCFMM_OK;
 }
 
+extern "C" int bcfmm_debug_near_math(int32_t kind, int64_t n, const double* a, const double* b, double* out) {
+  if (kind < 0 || kind > 2 || n < 1 || n > (1 << 24) || !a || !b || !out)
+    return fail(BCFMM_ERR_ARG, "debug_near_math: kind not in 0..2, n not in 1..2^24 or null array");
+  DevAlloc m;
+  double *da = nullptr, *db = nullptr, *dout = nullptr;
+  char* dt = nullptr;
+  std::vector<char> tabs(near_rule_tabs_bytes());
+  near_rule_tabs_fill(tabs.data());
+  cudaError_t e = m.upload(&da, a, n, 0);
+  if (e == cudaSuccess) e = m.upload(&db, b, n, 0);
+  if (e == cudaSuccess) e = m.upload(&dt, tabs.data(), tabs.size(), 0);
+  if (e == cudaSuccess) e = m.alloc(&dout, n);
+  if (e == cudaSuccess) e = launch_debug_near_math(kind, n, da, db, dt, dout, 0);
+  if (e == cudaSuccess) e = cudaMemcpy(out, dout, n * sizeof(double), cudaMemcpyDeviceToHost);
+  m.free_all();
+  if (e != cudaSuccess) return fail(BCFMM_ERR_CUDA, std::string("debug_near_math: ") + cudaGetErrorString(e));
+  return BCFMM_OK;
+}
+
 extern "C" int bcfmm_debug_expire_wait(bcfmm_ctx* C, int32_t spins) {
   if (!C || spins < 1 || spins > (1 << 20)) return fail(BCFMM_ERR_ARG, "debug_expire_wait: null context or spins not in 1..2^20");
   CU(launch_debug_expire_wait(C->err, spins, C->st));

@@ -124,5 +124,8 @@ cudaError_t launch_near_rule(int task, int64_t nnz, const int64_t* sel, const in
 // tabs: device copy of the function tables (near_rule_tabs_bytes() bytes, filled on the host)
 size_t near_rule_tabs_bytes();
 void near_rule_tabs_fill(void* host);
+// the near rule's quotient (kind 0), logarithm of a ratio (1) and atan2 (2), elementwise
+cudaError_t launch_debug_near_math(int kind, int64_t n, const double* a, const double* b, const void* tabs, double* out,
+                                   cudaStream_t st);
 
 }  // namespace bcfmm

@@ -87,11 +87,17 @@ __device__ double tri_solid(V3 x, const V3* P) {
 //    are squares' differences over the same (S - l)); ln(a / b) = ln c + 2
 //    artanh((a - c b) / (a + c b)) with c the nearest of 33 table points in
 //    [1, 2] to the ratio of the mantissas, artanh by its Taylor series
-//    (|z| <= 1/127: terms to z^7, the next is below 2^-60 of z);
+//    (|z| <= 1/127: terms to z^7, the next, z^8 / 9 of z, is below 2^-59);
 //  - solid angle: tan(Omega / 2) = |h| 2A / den; atan(y / x) = atan c +
 //    atan((y - c x) / (x + c y)), c the nearest of 65 points in [0, 1],
-//    again by Taylor's series to z^7.
-// The table entries (ln c, atan c) come from the host's libm.
+//    again by Taylor's series to z^7 (|z| <= 1/127).
+// This is the table-driven scheme of P. T. P. Tang (ACM Trans. Math. Softw. 16,
+// 1990) with the functions' addition theorems in place of his products.  Errors:
+// the difference a - c b is one FMA, so z is off by at most three roundings
+// (sum, quotient, difference), and the result by at most four of 2^-52: for c = 1
+// (0) the result is the series itself, else the table's value is at least as
+// large as the series' part of it.  The table entries (ln c, atan c) come from
+// the host's libm.
 __device__ constexpr int kTetEdge[6][2] = {{0, 1}, {0, 2}, {0, 3}, {1, 2}, {1, 3}, {2, 3}};
 __device__ constexpr int kTetFace[4][3] = {{1, 2, 3}, {0, 3, 2}, {0, 1, 3}, {0, 2, 1}};
 __device__ constexpr int kFaceEdge[4][3] = {{3, 5, 4}, {2, 5, 1}, {0, 4, 2}, {1, 3, 0}};   // edge of (F[j], F[j+1])
@@ -146,8 +152,12 @@ __device__ __forceinline__ void src_tet_prepare(const double* __restrict__ v, Sr
   __syncwarp();
 }
 
-// n / d by the hardware's approximate reciprocal, one Newton step and a
-// correction of the quotient by its residual
+// n / d, both normal and the quotient far from the ends of the range: one step r <-
+// r + r (1 - d r) of Newton's iteration for 1 / d from the hardware's approximation
+// (twenty bits: e0 about 2^-19, so e0^2 = 2^-38 after it), then Markstein's
+// correction of the quotient z = n r by its residual, z + r (n - d z) (IBM J. Res.
+// Dev. 34, 1990): the residual is one FMA, so its own error is 2^-53 of 2^-38, and
+// the quotient is within one unit of 2^-52.
 __device__ __forceinline__ double div_nr(double n, double d) {
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
@@ -165,7 +175,9 @@ __device__ __forceinline__ double log_ratio(double a, double b, const NearTabs& 
   int k = (ha >> 20) - (hb >> 20);
   float rm = __fdividef(mant_f(ha), mant_f(hb));          // in (1/2, 2)
   int up = 0;
-  if (rm < 1.f) { rm *= 2.f; k -= 1; up = 1 << 20; }
+  // (k = 0: the mantissas' ratio is at least 1, whatever their leading bits give;
+  // ln 2 would cancel against the table's)
+  if (rm < 1.f && k > 0) { rm *= 2.f; k -= 1; up = 1 << 20; }
   const int i = min(kLogTab - 1, (int)fmaf(rm - 1.f, 32.f, 0.5f));
   const double2 c = T.lg[i];
   const double am = __hiloint2double(((ha & 0xfffff) | 0x3ff00000) + up, __double2loint(a));
@@ -477,6 +489,20 @@ size_t near_rule_tabs_bytes() { return sizeof(NearTabs); }
 void near_rule_tabs_fill(void* host) {
   const NearTabs T = make_tabs();
   std::memcpy(host, &T, sizeof T);
+}
+
+// out[i] = a[i] / b[i] (kind 0), ln(a / b) (1), atan2(a, b) (2) by the functions above
+__global__ void k_debug_near_math(int kind, int64_t n, const double* __restrict__ a, const double* __restrict__ b,
+                                  const NearTabs* __restrict__ tabs, double* __restrict__ out) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  out[i] = kind == 0 ? div_nr(a[i], b[i]) : kind == 1 ? log_ratio(a[i], b[i], *tabs) : atan_pos(a[i], b[i], *tabs);
+}
+cudaError_t launch_debug_near_math(int kind, int64_t n, const double* a, const double* b, const void* tabs, double* out,
+                                   cudaStream_t st) {
+  if (n == 0) return cudaSuccess;
+  k_debug_near_math<<<(unsigned)((n + 127) / 128), 128, 0, st>>>(kind, n, a, b, static_cast<const NearTabs*>(tabs), out);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_near_rule(int task, int64_t nnz, const int64_t* sel, const int* row, const int* col,
