@@ -401,6 +401,13 @@ int bcfmm_debug_m2l_taylor_coeffs(int32_t q, const double* o, double* g);
 int bcfmm_debug_shift_matrix(int32_t kind, int32_t p, int32_t octant, double* out);
 
 /*
+ * Test hook: from now on the context refuses device allocations that would
+ * bring its total (bcfmm_stats, "device_bytes") above `bytes`, as if the
+ * device had no more memory; 0: no limit.  Errors: BCFMM_ERR_ARG.
+ */
+int bcfmm_debug_memory_limit(bcfmm_ctx* ctx, int64_t bytes);
+
+/*
  * Test hook: the near rule's own elementary functions, elementwise on the
  * current device's default stream.  kind 0: out = a / b (normal numbers,
  * quotient away from the ends of the range); 1: out = ln(a / b), a >= b > 0;

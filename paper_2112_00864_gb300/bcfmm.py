@@ -27,7 +27,7 @@ EXPORTED = ["bcfmm_default_params", "bcfmm_build_bc_tree", "bcfmm_set_density", 
             "bcfmm_mlp_grad", "bcfmm_mlp_adam", "bcfmm_mlp_predict", "bcfmm_debug_expire_wait",
             "bcfmm_debug_list_coverage", "bcfmm_debug_near_pairs", "bcfmm_debug_shift_matrix",
             "bcfmm_debug_tree_counts", "bcfmm_debug_m2l_taylor_coeffs", "bcfmm_measure_ffma",
-            "bcfmm_debug_near_math"]
+            "bcfmm_debug_near_math", "bcfmm_debug_memory_limit"]
 NEAR_MODE = {"fp64": 0, "learned": 1, "none": 2}
 TASK_BIT = {"vtv": 1, "vtb": 2, "btv": 4}
 
@@ -100,6 +100,8 @@ def load(path: str = LIB_PATH):
         L.bcfmm_mlp_predict.restype = C.c_int
         L.bcfmm_debug_expire_wait.argtypes = [p, i32]
         L.bcfmm_debug_expire_wait.restype = C.c_int
+        L.bcfmm_debug_memory_limit.argtypes = [p, i64]
+        L.bcfmm_debug_memory_limit.restype = C.c_int
         L.bcfmm_debug_near_math.argtypes = [i32, i64, p, p, p]
         L.bcfmm_debug_near_math.restype = C.c_int
         L.bcfmm_debug_list_coverage.argtypes = [p, p, p, p, p, p, i32, C.POINTER(Params), p]

@@ -43,14 +43,28 @@ static int fail(int code, const std::string& msg) {
 namespace {
 
 struct DevAlloc {
-  std::vector<void*> ptrs;
+  std::vector<std::pair<void*, size_t>> ptrs;
+  size_t bytes = 0, limit = 0;         // allocated; refused above (0: no limit)
   template <typename T>
   cudaError_t alloc(T** p, size_t n) {
     *p = nullptr;
     if (n == 0) n = 1;
-    cudaError_t e = cudaMalloc((void**)p, n * sizeof(T));
-    if (e == cudaSuccess) ptrs.push_back(*p);
+    const size_t sz = n * sizeof(T);
+    if (limit > 0 && bytes + sz > limit) return cudaErrorMemoryAllocation;
+    cudaError_t e = cudaMalloc((void**)p, sz);
+    if (e == cudaSuccess) {
+      ptrs.push_back({*p, sz});
+      bytes += sz;
+    } else {
+      (void)cudaGetLastError();        // (a later launch must not report it)
+    }
     return e;
+  }
+  // bytes that an allocation can have
+  size_t room() const {
+    size_t avail = 0, total = 0;
+    if (cudaMemGetInfo(&avail, &total) != cudaSuccess) avail = 0;
+    return limit > 0 ? std::min(avail, limit > bytes ? limit - bytes : 0) : avail;
   }
   template <typename T>
   cudaError_t upload(T** p, const T* h, size_t n, cudaStream_t st) {
@@ -59,12 +73,16 @@ struct DevAlloc {
     return cudaMemcpyAsync(*p, h, n * sizeof(T), cudaMemcpyHostToDevice, st);
   }
   void release(void* p) {
-    auto it = std::find(ptrs.begin(), ptrs.end(), p);
-    if (it != ptrs.end()) { cudaFree(*it); ptrs.erase(it); }
+    auto it = std::find_if(ptrs.begin(), ptrs.end(), [p](const auto& x) { return x.first == p; });
+    if (it == ptrs.end()) return;
+    cudaFree(p);
+    bytes -= it->second;
+    ptrs.erase(it);
   }
   void free_all() {
-    for (void* p : ptrs) cudaFree(p);
+    for (const auto& x : ptrs) cudaFree(x.first);
     ptrs.clear();
+    bytes = 0;
   }
 };
 
@@ -120,13 +138,14 @@ struct bcfmm_ctx {
   double* dens[3] = {nullptr, nullptr, nullptr};
   int* err = nullptr;                  // device error word (bounded device waits)
   char* near_tabs = nullptr;           // function tables of the near rule
-  size_t tc_partial_per_dens = 0;      // largest tensor-core partial-sum need over the tasks (float2)
+  // largest tensor-core partial-sum need over the tasks of a work set (float2)
+  size_t tc_partial_per_dens[2] = {0, 0};
   // Taylor-form M2L (BCFMM_FP32 and BCFMM_FP64): offset coefficients,
-  // prescaled moments, chunk partial sums (largest need over the tasks,
-  // values per density)
+  // prescaled moments, chunk partial sums (largest need over the tasks of a
+  // work set, values per density)
   TaylorTables ty{};
   TaylorOffsets ty_offs;               // parent offsets of the tasks' schedules (build only)
-  size_t ty_partial_per_dens = 0;
+  size_t ty_partial_per_dens[2] = {0, 0};
   // work buffers, sized for the largest ndp seen: set 0 for the tasks with
   // volume sources (VtV, VtB), set 1 for those with boundary sources (BtV), so
   // that both may run at the same time.  Element type double in an FP64
@@ -140,6 +159,7 @@ struct bcfmm_ctx {
     uint8_t* tc_momb = nullptr;        // BF16 split moments of the tensor-core M2L
   } work[2];
   double* phi[3] = {nullptr, nullptr, nullptr};   // point potentials per task
+  int64_t slots_tried[2] = {0, -1};    // densities and work_gen at the last attempt to allocate VtV's slots
   double* out_dev = nullptr;           // staging of host outputs
   int out_ndp = 0;
   // streams and events of the parts of an evaluation that do not depend on
@@ -310,7 +330,7 @@ static int upload_task(bcfmm_ctx* C, const HostSetup& H, int t) {
     L.sp_grp = sg; L.grp_info = gi; L.grp_cnt = gc;
   }
   if (t == 0 && C->prm.precision != BCFMM_FP64 && p2p_sym_pays(H)) {
-    // symmetric near field (one density)
+    // symmetric near field (up to four densities)
     int nsm = 152;
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, C->device);
     HostSym Y;
@@ -447,7 +467,8 @@ static int upload_task(bcfmm_ctx* C, const HostSetup& H, int t) {
       D.tc_rows += O.rows;
       D.tc_mma_flop += 2.0 * 128 * (C->tc.nsplit == 2 ? 3 : 6) * (double)npad * npad * (double)O.nent;
     }
-    C->tc_partial_per_dens = std::max(C->tc_partial_per_dens, D.tcs.partial_per_dens);
+    size_t& need = C->tc_partial_per_dens[T.src_cls];
+    need = std::max(need, D.tcs.partial_per_dens);
   }
   // Taylor-form M2L: per order, the sibling groups' entries cut into chunks;
   // targets of orders above the kernel's range go to the wide kernel (FP32)
@@ -489,7 +510,8 @@ static int upload_task(bcfmm_ctx* C, const HostSetup& H, int t) {
       D.tys.simt_sel = dsel;
       D.tys.nsimt = (int)sel.size();
     }
-    C->ty_partial_per_dens = std::max(C->ty_partial_per_dens, D.tys.partial_per_dens);
+    size_t& need = C->ty_partial_per_dens[T.src_cls];
+    need = std::max(need, D.tys.partial_per_dens);
   }
   // near pairs + FP64 corrections computed on the device
   int64_t *cor_off;
@@ -1525,37 +1547,16 @@ static int ensure_work(bcfmm_ctx* C, int set, int ndp) {
     if (L.sp_scratch) m.release(L.sp_scratch);
     L.sp_scratch = nullptr;
     CU(m.alloc(&L.sp_scratch, (size_t)C->task[t].sp_rows * ndp * 128));
-    DevSym& Y = C->task[t].sym;
-    if (Y.src) m.release(Y.src);
-    if (Y.tgt) m.release(Y.tgt);
-    Y.src = nullptr;
-    Y.tgt = nullptr;
   }
   if (C->tc.nsplit > 0) {
-    CU(m.alloc(&w.tc_partial, std::max<size_t>((size_t)ndp * C->tc_partial_per_dens, 1)));
+    CU(m.alloc(&w.tc_partial, std::max<size_t>((size_t)ndp * C->tc_partial_per_dens[set], 1)));
     // split moments: one row per (box, density, part)
     const int kpitch = m2l_tc_kpitch(C->prm.p);
     CU(m.alloc(&w.tc_momb, (size_t)C->nbox * ndp * C->tc.nsplit * kpitch * 2));
   }
   if (C->ty.q > 0) {
     CU(bytes(&w.ty_momp, (size_t)C->nbox * ndp * C->ty.gpitch * es));
-    CU(bytes(&w.ty_partial, std::max<size_t>((size_t)ndp * C->ty_partial_per_dens, 1) * es));
-  }
-  // the symmetric near field's slots (up to four densities) last: where the
-  // device has no room for them the directed kernel, which needs none, serves
-  for (int t = t0; t <= t1; ++t) {
-    DevSym& Y = C->task[t].sym;
-    if (Y.nblk == 0) continue;
-    cudaError_t e = m.alloc(&Y.src, (size_t)std::min(ndp, 4) * Y.nsrc);
-    if (e == cudaSuccess) e = m.alloc(&Y.tgt, (size_t)std::min(ndp, 4) * Y.ntgt);
-    if (e == cudaErrorMemoryAllocation) {
-      (void)cudaGetLastError();
-      if (Y.src) m.release(Y.src);
-      Y.src = nullptr;
-      Y.nblk = 0;
-    } else {
-      CU(e);
-    }
+    CU(bytes(&w.ty_partial, std::max<size_t>((size_t)ndp * C->ty_partial_per_dens[set], 1) * es));
   }
   w.ndp = ndp;
   C->work_gen++;
@@ -1570,6 +1571,47 @@ static int ensure_out(bcfmm_ctx* C, int ndp) {
   CU(C->mem.alloc(&C->out_dev, (size_t)ndp * std::max(C->ntet, C->ntri)));
   C->out_ndp = ndp;
   return BCFMM_OK;
+}
+
+// The slots of VtV's symmetric near field, for the counts of densities that it
+// takes.  They come after every other buffer, take at most half of the memory
+// that is left, and go again when something else needs the room: without them
+// the directed kernel, which needs none, serves.
+static void release_slots(bcfmm_ctx* C) {
+  DevSym& Y = C->task[0].sym;
+  if (Y.src) C->mem.release(Y.src);
+  if (Y.tgt) C->mem.release(Y.tgt);
+  Y.src = nullptr;
+  Y.tgt = nullptr;
+  if (Y.cap > 0) C->work_gen++;
+  Y.cap = 0;
+}
+static void ensure_slots(bcfmm_ctx* C, int ndp) {
+  DevSym& Y = C->task[0].sym;
+  if (Y.nblk == 0 || ndp > kSymDens || Y.cap >= ndp || (C->slots_tried[0] == ndp && C->slots_tried[1] == C->work_gen)) return;
+  release_slots(C);
+  C->slots_tried[0] = ndp;             // (not again before other buffers change)
+  C->slots_tried[1] = C->work_gen;
+  const size_t need = (size_t)ndp * (Y.nsrc * sizeof(float) + Y.ntgt * sizeof(float2));
+  if (need > C->mem.room() / 2) return;
+  if (C->mem.alloc(&Y.src, (size_t)ndp * Y.nsrc) == cudaSuccess && C->mem.alloc(&Y.tgt, (size_t)ndp * Y.ntgt) == cudaSuccess) {
+    Y.cap = ndp;
+    C->work_gen++;
+  } else {
+    release_slots(C);
+  }
+}
+
+// A work set and the staging of host outputs (0: none), then the slots.
+static int ensure_buffers(bcfmm_ctx* C, int set, int ndp, int out_ndp) {
+  int rc = ensure_work(C, set, ndp);
+  if (rc == BCFMM_OK) rc = ensure_out(C, out_ndp);
+  if (rc == BCFMM_ERR_OOM && C->task[0].sym.cap > 0) {
+    release_slots(C);
+    rc = ensure_work(C, set, ndp);
+    if (rc == BCFMM_OK) rc = ensure_out(C, out_ndp);
+  }
+  return rc;
 }
 
 extern "C" int bcfmm_set_density(bcfmm_ctx* C, int32_t kind, const double* vals, int32_t ndens, int32_t is_device) {
@@ -1592,7 +1634,12 @@ extern "C" int bcfmm_set_density(bcfmm_ctx* C, int32_t kind, const double* vals,
   if (C->ndens[kind] < ndens) {
     if (C->dens[kind]) C->mem.release(C->dens[kind]);
     C->dens[kind] = nullptr;
-    CU(C->mem.alloc(&C->dens[kind], (size_t)16 * nel));
+    cudaError_t e = C->mem.alloc(&C->dens[kind], (size_t)16 * nel);
+    if (e == cudaErrorMemoryAllocation && C->task[0].sym.cap > 0) {
+      release_slots(C);
+      e = C->mem.alloc(&C->dens[kind], (size_t)16 * nel);
+    }
+    CU(e);
     C->work_gen++;
   }
   CU(cudaMemcpyAsync(C->dens[kind], vals, n * sizeof(double), is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
@@ -1603,10 +1650,11 @@ extern "C" int bcfmm_set_density(bcfmm_ctx* C, int32_t kind, const double* vals,
   // (the other set too, for one density: bcfmm_eval_noalloc takes any task
   // after one call of this function)
   for (int set = 0; set < 2; ++set) {
-    const int rc = ensure_work(C, set, (kind == BCFMM_VOLUME) == (set == 0) ? C->ndp[kind] : 1);
+    const int rc = ensure_buffers(C, set, (kind == BCFMM_VOLUME) == (set == 0) ? C->ndp[kind] : 1, C->ndp[kind]);
     if (rc != BCFMM_OK) return rc;
   }
-  return ensure_out(C, C->ndp[kind]);
+  ensure_slots(C, kind == BCFMM_VOLUME ? C->ndp[kind] : C->work[0].ndp);
+  return BCFMM_OK;
 }
 
 // What one task is evaluated with.
@@ -1820,7 +1868,7 @@ static int task_run(bcfmm_ctx* C, int t, TaskRun& r) {
   r.dip = t == 2 && C->ndens[BCFMM_DIPOLE] > 0 ? C->dens[BCFMM_DIPOLE] : nullptr;
   if (r.dip && C->ndens[BCFMM_DIPOLE] != r.ndens)
     return fail(BCFMM_ERR_STATE, "eval: the double-layer density's ndens differs from the boundary density's");
-  return ensure_work(C, kind, r.ndp);
+  return ensure_buffers(C, kind, r.ndp, 0);
 }
 
 // Near-field pairs from which a single task's parts run side by side: the
@@ -1836,7 +1884,7 @@ static int eval_impl(bcfmm_ctx* C, int t, double* out, int out_is_device) {
   if (!out) return fail(BCFMM_ERR_ARG, "eval: null output");
   TaskRun r;
   int rc = task_run(C, t, r);
-  if (rc == BCFMM_OK && !out_is_device) rc = ensure_out(C, r.ndp);
+  if (rc == BCFMM_OK && !out_is_device) rc = ensure_buffers(C, kind, r.ndp, r.ndp);
   if (rc != BCFMM_OK) return rc;
   cudaStream_t st = C->st;
   const bool tm = C->prm.timing && C->ev_ok;
@@ -2077,6 +2125,12 @@ extern "C" int bcfmm_measure_ffma(int32_t device, double* flops) {
   return BCFMM_OK;
 }
 
+extern "C" int bcfmm_debug_memory_limit(bcfmm_ctx* C, int64_t bytes) {
+  if (!C || bytes < 0) return fail(BCFMM_ERR_ARG, "debug_memory_limit: null context or negative limit");
+  C->mem.limit = (size_t)bytes;
+  return BCFMM_OK;
+}
+
 extern "C" int bcfmm_debug_near_math(int32_t kind, int64_t n, const double* a, const double* b, double* out) {
   if (kind < 0 || kind > 2 || n < 1 || n > (1 << 24) || !a || !b || !out)
     return fail(BCFMM_ERR_ARG, "debug_near_math: kind not in 0..2, n not in 1..2^24 or null array");
@@ -2120,6 +2174,7 @@ extern "C" int bcfmm_stats(const bcfmm_ctx* C, char* json, size_t cap) {
   kv("p", C->prm.p); kv("np", C->np); kv("eta0", C->prm.eta0); kv("n_offsets", C->ncode); kv("leaf_size", C->prm.leaf_size); kv("precision", C->prm.precision);
   kv("near_mode", C->prm.near_mode); kv("tc_unit", C->prm.tc_unit);
   kv("graph_kernels", C->graph.exec ? C->graph.nodes : 0); kv("graph_mask", C->graph.exec ? C->graph.mask : 0);
+  kv("device_bytes", (double)C->mem.bytes);
   kv("nbox", C->nbox); kv("nleaf", C->nleaf); kv("nlevels", C->nlevels);
   kv("nmesh", C->nmesh); kv("host_setup_s", C->sec_host);
   kv("setup_s", C->sec_setup); kv("tree_s", C->sec_tree); kv("lists_s", C->sec_lists);
@@ -2154,6 +2209,10 @@ extern "C" int bcfmm_stats(const bcfmm_ctx* C, char* json, size_t cap) {
     per_q += "], \"m2l_pairs_by_order\": [";
     for (int q = 0; q <= C->prm.p; ++q) per_q += std::to_string(D.m2l_pairs_q[q]) + (q < C->prm.p ? ", " : "");
     per_q += "], \"generic_m2l_targets\": " + std::to_string(C->ty.q > 0 ? D.tys.nsimt + D.tys.ord[kTaylorMaxQ].ntgt : (D.tcs.nsimt > 0 ? D.tcs.nsimt : 0));
+    if (t == 0)
+      per_q += ", \"near_sym\": {\"blocks\": " + std::to_string(D.sym.nblk) + ", \"large\": " + std::to_string(D.sym.nlarge) +
+               ", \"src_slots\": " + std::to_string(D.sym.nsrc) + ", \"tgt_slots\": " + std::to_string(D.sym.ntgt) +
+               ", \"densities\": " + std::to_string(D.sym.cap) + "}";
     per_q += ", \"p2p_sources_per_leaf\": [";
     for (int k = 0; k < 5; ++k) per_q += std::to_string(D.p2p_src_q[k]) + (k < 4 ? ", " : "]");
     snprintf(b, sizeof b,

@@ -411,7 +411,7 @@ cudaError_t launch_blocks(const DevGeom& G, const DevSym& S, int b0, int n, cons
 }
 
 cudaError_t launch_p2p_sym(const DevGeom& G, const DevSym& S, const float* W, int64_t npts, int ndp, double* phi, cudaStream_t st) {
-  if (S.nblk == 0) return cudaSuccess;
+  if (!p2p_sym_takes(S, ndp)) return cudaErrorInvalidValue;
   cudaError_t e;
   switch (ndp) {
     case 1:

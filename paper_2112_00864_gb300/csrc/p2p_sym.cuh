@@ -30,7 +30,8 @@ struct DevSym {
   const int2* base = nullptr;       // [nblk] (first src slot, first tgt slot)
   const int* self = nullptr;        // [nblk] 1: the block also holds the owner's own points
   int64_t nsrc = 0, ntgt = 0;       // slots
-  float* src = nullptr;             // [nsrc][ndp] source-side sums (sized with the work buffers)
+  int cap = 0;                      // densities that the slots hold (0: no slots)
+  float* src = nullptr;             // [nsrc][ndp] source-side sums
   float2* tgt = nullptr;            // [ntgt][ndp] owner-side sums (hi, lo)
   // gather kernel, per target leaf (most slots first)
   int nfin = 0;
@@ -56,7 +57,8 @@ int64_t p2p_sym_chunk(const HostSetup& H, int nsm);
 bool p2p_sym_pays(const HostSetup& H);
 
 // densities (padded) that the symmetric form takes; more need too many registers
-inline bool p2p_sym_takes(const DevSym& S, int ndp) { return S.nblk > 0 && ndp <= 4; }
+constexpr int kSymDens = 4;
+inline bool p2p_sym_takes(const DevSym& S, int ndp) { return ndp <= kSymDens && ndp <= S.cap; }
 // phi = near field of VtV / 4 pi (every target point; npts points per density in W and phi)
 cudaError_t launch_p2p_sym(const DevGeom& G, const DevSym& S, const float* W, int64_t npts, int ndp, double* phi, cudaStream_t st);
 
