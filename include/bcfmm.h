@@ -401,6 +401,19 @@ int bcfmm_debug_m2l_taylor_coeffs(int32_t q, const double* o, double* g);
 int bcfmm_debug_shift_matrix(int32_t kind, int32_t p, int32_t octant, double* out);
 
 /*
+ * Test hook (host only): the schedule of VtV's symmetric near field with blocks
+ * of about `chunk` sources, for the batch and parameters as in
+ * bcfmm_debug_list_coverage.  out[0]: pairs of near leaves (a leaf with itself
+ * included) not in exactly one block; out[1]: slots not written and gathered
+ * exactly once for the same point; out[2]: blocks over their size or out of
+ * order; out[3]: blocks; out[4]: 1 when a context with these parameters takes
+ * the symmetric form.  out: host int64 [5].  Errors: BCFMM_ERR_ARG, BCFMM_ERR_MESH.
+ */
+int bcfmm_debug_sym_coverage(const double* verts, const int64_t* vert_off, const int32_t* tets, const int64_t* tet_off,
+                             const int32_t* tris, const int64_t* tri_off, int32_t nmesh, const bcfmm_params* params,
+                             int64_t chunk, int64_t* out);
+
+/*
  * Test hook: from now on the context refuses device allocations that would
  * bring its total (bcfmm_stats, "device_bytes") above `bytes`, as if the
  * device had no more memory; 0: no limit.  Errors: BCFMM_ERR_ARG.

@@ -27,7 +27,7 @@ EXPORTED = ["bcfmm_default_params", "bcfmm_build_bc_tree", "bcfmm_set_density", 
             "bcfmm_mlp_grad", "bcfmm_mlp_adam", "bcfmm_mlp_predict", "bcfmm_debug_expire_wait",
             "bcfmm_debug_list_coverage", "bcfmm_debug_near_pairs", "bcfmm_debug_shift_matrix",
             "bcfmm_debug_tree_counts", "bcfmm_debug_m2l_taylor_coeffs", "bcfmm_measure_ffma",
-            "bcfmm_debug_near_math", "bcfmm_debug_memory_limit"]
+            "bcfmm_debug_near_math", "bcfmm_debug_memory_limit", "bcfmm_debug_sym_coverage"]
 NEAR_MODE = {"fp64": 0, "learned": 1, "none": 2}
 TASK_BIT = {"vtv": 1, "vtb": 2, "btv": 4}
 
@@ -100,6 +100,8 @@ def load(path: str = LIB_PATH):
         L.bcfmm_mlp_predict.restype = C.c_int
         L.bcfmm_debug_expire_wait.argtypes = [p, i32]
         L.bcfmm_debug_expire_wait.restype = C.c_int
+        L.bcfmm_debug_sym_coverage.argtypes = [p, p, p, p, p, p, i32, C.POINTER(Params), i64, p]
+        L.bcfmm_debug_sym_coverage.restype = C.c_int
         L.bcfmm_debug_memory_limit.argtypes = [p, i64]
         L.bcfmm_debug_memory_limit.restype = C.c_int
         L.bcfmm_debug_near_math.argtypes = [i32, i64, p, p, p]
@@ -444,14 +446,8 @@ def mlp_predict(params, feat, qhat, out, stream=None):
                                     _stream_handle(stream)))
 
 
-def debug_list_coverage(meshes, **kw) -> np.ndarray:
-    """Host-only check of the FMM's interaction covering for one mesh or a
-    batch: [0:3] per task the (target leaf, source point) pairs not covered
-    exactly once, [3:6] per task the interaction entries the tensor-core
-    tiles get wrong, [6:9] per task the faults of the tensor-core schedule,
-    [9:12] per task the faults of the Taylor-form M2L schedule, [12:15] per
-    task the faults of the packed near field's chunk blocks (see
-    include/bcfmm.h)."""
+def _batch_arrays(meshes):
+    """verts, vert_off, tets, tet_off, tris, tri_off of a batch, as the library takes them."""
     vo, to, ro = [0], [0], [0]
     for m in meshes:
         vo.append(vo[-1] + len(m.verts))
@@ -461,11 +457,34 @@ def debug_list_coverage(meshes, **kw) -> np.ndarray:
     tets = np.ascontiguousarray(np.concatenate([m.tets for m in meshes]), np.int32)
     tris = np.ascontiguousarray(np.concatenate([np.asarray(m.tris).reshape(-1, 3) for m in meshes]), np.int32)
     vo, to, ro = (np.asarray(x, np.int64) for x in (vo, to, ro))
+    return verts, vo, tets, to, tris, ro
+
+
+def debug_list_coverage(meshes, **kw) -> np.ndarray:
+    """Host-only check of the FMM's interaction covering for one mesh or a
+    batch: [0:3] per task the (target leaf, source point) pairs not covered
+    exactly once, [3:6] per task the interaction entries the tensor-core
+    tiles get wrong, [6:9] per task the faults of the tensor-core schedule,
+    [9:12] per task the faults of the Taylor-form M2L schedule, [12:15] per
+    task the faults of the packed near field's chunk blocks (see
+    include/bcfmm.h)."""
+    arrs = _batch_arrays(meshes)
     prm = default_params(**kw)
     out = np.zeros(15, np.int64)
-    _check(load().bcfmm_debug_list_coverage(verts.ctypes.data, vo.ctypes.data, tets.ctypes.data, to.ctypes.data,
-                                            tris.ctypes.data, ro.ctypes.data, len(meshes), C.byref(prm),
-                                            out.ctypes.data))
+    _check(load().bcfmm_debug_list_coverage(*(a.ctypes.data for a in arrs), len(meshes), C.byref(prm), out.ctypes.data))
+    return out
+
+
+def debug_sym_coverage(meshes, chunk: int, **kw) -> np.ndarray:
+    """Host-only check of the blocks of VtV's symmetric near field, of about
+    ``chunk`` sources: [0:3] faults of the leaf pairs, the slots and the
+    blocks, [3] the blocks, [4] whether a context would take this form (see
+    include/bcfmm.h)."""
+    arrs = _batch_arrays(meshes)
+    prm = default_params(**kw)
+    out = np.zeros(5, np.int64)
+    _check(load().bcfmm_debug_sym_coverage(*(a.ctypes.data for a in arrs), len(meshes), C.byref(prm), chunk,
+                                           out.ctypes.data))
     return out
 
 

@@ -1205,6 +1205,58 @@ extern "C" int bcfmm_debug_near_pairs(const double* verts, int64_t nvert, const 
   return BCFMM_OK;
 }
 
+// The tree and lists of a batch as bcfmm_build_batch builds them, for the host checks.
+static int debug_setup(const std::string& who, const double* verts, const int64_t* vert_off, const int32_t* tets,
+                       const int64_t* tet_off, const int32_t* tris, const int64_t* tri_off, int32_t nmesh,
+                       const bcfmm_params& prm, HostSetup& H) {
+  std::vector<HostSetup> parts(nmesh);
+  for (int m = 0; m < nmesh; ++m) {
+    bool me = false;
+    const int64_t nt = tet_off[m + 1] - tet_off[m], nf = tri_off[m + 1] - tri_off[m];
+    const std::string e = build_host_mesh(parts[m], verts + 3 * vert_off[m], vert_off[m + 1] - vert_off[m],
+                                          tets + 4 * tet_off[m], nt, nf > 0 ? tris + 3 * tri_off[m] : nullptr, nf,
+                                          prm, false, &me);
+    if (!e.empty()) return fail(me ? BCFMM_ERR_MESH : BCFMM_ERR_ARG, who + e);
+  }
+  if (nmesh == 1) {
+    H = std::move(parts[0]);
+    H.mesh_tet_off = {0, tet_off[1]};
+    H.mesh_tri_off = {0, tri_off[1]};
+  } else {
+    merge_setups(parts, H);
+  }
+  return BCFMM_OK;
+}
+
+// Host only: the symmetric near field's blocks (see check_p2p_sym).
+extern "C" int bcfmm_debug_sym_coverage(const double* verts, const int64_t* vert_off, const int32_t* tets,
+                                        const int64_t* tet_off, const int32_t* tris, const int64_t* tri_off,
+                                        int32_t nmesh, const bcfmm_params* prm_in, int64_t chunk, int64_t* out) {
+  if (!out || nmesh < 1 || !verts || !vert_off || !tets || !tet_off || !tri_off || chunk < 1)
+    return fail(BCFMM_ERR_ARG, "debug_sym_coverage: null argument or chunk < 1");
+  bcfmm_params prm;
+  bcfmm_default_params(&prm);
+  if (prm_in) prm = *prm_in;
+  if (prm.leaf_size < 1 || prm.leaf_size > 128 || !(prm.eta0 >= 0.3 && prm.eta0 <= 1.0))
+    return fail(BCFMM_ERR_ARG, "debug_sym_coverage: bad leaf_size or eta0");
+  try {
+    HostSetup H;
+    const int rc = debug_setup("debug_sym_coverage: ", verts, vert_off, tets, tet_off, tris, tri_off, nmesh, prm, H);
+    if (rc != BCFMM_OK) return rc;
+    HostSym S;
+    if (!build_p2p_sym(H, chunk, S)) return fail(BCFMM_ERR_ARG, "debug_sym_coverage: the slots exceed 32-bit offsets");
+    const SymFaults F = check_p2p_sym(H, chunk, S);
+    out[0] = F.pairs;
+    out[1] = F.slots;
+    out[2] = F.blocks;
+    out[3] = (int64_t)S.leaf.size();
+    out[4] = p2p_sym_pays(H);
+  } catch (const std::exception& ex) {
+    return fail(BCFMM_ERR_ARG, std::string("debug_sym_coverage: ") + ex.what());
+  }
+  return BCFMM_OK;
+}
+
 // Host only: tree and lists as bcfmm_build_batch builds them, then for
 // every task and every target leaf the source points of its mesh covered
 // by the leaf's merged near-field runs plus the interaction lists of the
@@ -1221,23 +1273,9 @@ extern "C" int bcfmm_debug_list_coverage(const double* verts, const int64_t* ver
   if (prm.leaf_size < 1 || prm.leaf_size > 128 || !(prm.eta0 >= 0.3 && prm.eta0 <= 1.0))
     return fail(BCFMM_ERR_ARG, "debug_list_coverage: bad leaf_size or eta0");
   try {
-    std::vector<HostSetup> parts(nmesh);
-    for (int m = 0; m < nmesh; ++m) {
-      bool me = false;
-      const int64_t nt = tet_off[m + 1] - tet_off[m], nf = tri_off[m + 1] - tri_off[m];
-      const std::string e = build_host_mesh(parts[m], verts + 3 * vert_off[m], vert_off[m + 1] - vert_off[m],
-                                            tets + 4 * tet_off[m], nt, nf > 0 ? tris + 3 * tri_off[m] : nullptr, nf,
-                                            prm, false, &me);
-      if (!e.empty()) return fail(me ? BCFMM_ERR_MESH : BCFMM_ERR_ARG, "debug_list_coverage: " + e);
-    }
     HostSetup H;
-    if (nmesh == 1) {
-      H = std::move(parts[0]);
-      H.mesh_tet_off = {0, tet_off[1]};
-      H.mesh_tri_off = {0, tri_off[1]};
-    } else {
-      merge_setups(parts, H);
-    }
+    const int rc = debug_setup("debug_list_coverage: ", verts, vert_off, tets, tet_off, tris, tri_off, nmesh, prm, H);
+    if (rc != BCFMM_OK) return rc;
     for (int t = 0; t < 3; ++t) {
       const HostTask& T = H.task[t];
       const int sc = T.src_cls, tc = T.tgt_cls;

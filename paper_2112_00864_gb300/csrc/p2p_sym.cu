@@ -13,6 +13,7 @@
 #include <algorithm>
 #include <climits>
 #include <cmath>
+#include <map>
 
 #include "internal.h"
 #include "p2p_sym.cuh"
@@ -551,6 +552,74 @@ bool build_p2p_sym(const HostSetup& H, int64_t chunk, HostSym& out) {
     }
   }
   return true;
+}
+
+SymFaults check_p2p_sym(const HostSetup& H, int64_t chunk, const HostSym& S) {
+  const HostTask& T = H.task[0];
+  SymFaults F;
+  auto npt = [&](int b) { return H.box[b].pt1[0] - H.box[b].pt0[0]; };
+  // near pairs of leaves as (lower box, higher box): how often they are due (1),
+  // minus how often they occur
+  std::map<std::pair<int, int>, int> due;
+  auto key = [](int a, int b) { return std::make_pair(std::min(a, b), std::max(a, b)); };
+  for (size_t i = 0; i < T.p2p_leaf.size(); ++i)
+    for (int k = T.near_off[i]; k < T.near_off[i + 1]; ++k) {
+      std::vector<int> todo(1, T.near_box[k]);     // the leaves of the near subtree
+      while (!todo.empty()) {
+        const int b = todo.back();
+        todo.pop_back();
+        const HostBox& B = H.box[b];
+        if (B.nchild == 0 && npt(b) > 0) due[key(T.p2p_leaf[i], b)] = 1;
+        for (int c = 0; c < B.nchild; ++c) todo.push_back(B.child0 + c);
+      }
+    }
+  const int nblk = (int)S.leaf.size();
+  std::vector<int> src_pt(S.nsrc, -1), tgt_pt(S.ntgt, -1);      // the point a slot was written for
+  int last = INT_MAX;
+  for (int b = 0; b < nblk; ++b) {
+    const int a = S.leaf[b], nt = npt(a);
+    if (S.self[b]) due[key(a, a)]--;
+    if ((b < S.nlarge) != (nt > 32) || nt < 1 || nt > 128 || sym_pad(nt) > last) F.blocks++;
+    last = sym_pad(nt);
+    int64_t slot = S.base[2 * b], n = 0;
+    for (int r = S.run_off[b]; r < S.run_off[b + 1]; ++r)
+      for (int q = S.runs[2 * r]; q < S.runs[2 * r + 1];) {
+        const int c = H.leaf_of[0][q];
+        if (q != H.box[c].pt0[0] || H.box[c].pt1[0] > S.runs[2 * r + 1]) { F.pairs++; break; }   // (a part of a leaf)
+        due[key(a, c)]--;
+        for (; q < H.box[c].pt1[0]; ++q, ++slot, ++n) {
+          if (slot < 0 || slot >= S.nsrc || src_pt[slot] >= 0) F.slots++;
+          else src_pt[slot] = q;
+        }
+      }
+    if (n > chunk + 128) F.blocks++;
+    for (int i = 0; i < nt; ++i) {
+      const int64_t t = (int64_t)S.base[2 * b + 1] + i;
+      if (t < 0 || t >= S.ntgt || tgt_pt[t] >= 0) F.slots++;
+      else tgt_pt[t] = H.box[a].pt0[0] + i;
+    }
+  }
+  for (const auto& d : due) F.pairs += d.second != 0;
+  // the gather: point i of a leaf takes slot f + i of every f in the leaf's lists
+  std::vector<int> leaves = S.fin_leaf, want = T.p2p_leaf;
+  std::sort(leaves.begin(), leaves.end());
+  std::sort(want.begin(), want.end());
+  if (leaves != want) F.slots++;
+  auto gather = [&](const std::vector<int>& off, const std::vector<int>& list, std::vector<int>& pt) {
+    for (size_t f = 0; f < S.fin_leaf.size(); ++f) {
+      const int lf = S.fin_leaf[f];
+      for (int e = off[f]; e < off[f + 1]; ++e)
+        for (int i = 0; i < npt(lf); ++i) {
+          const int64_t k = (int64_t)list[e] + i;
+          if (k < 0 || k >= (int64_t)pt.size() || pt[k] != H.box[lf].pt0[0] + i) F.slots++;
+          else pt[k] = -1;
+        }
+    }
+    for (int v : pt) F.slots += v >= 0;
+  };
+  gather(S.fin_src_off, S.fin_src, src_pt);
+  gather(S.fin_tgt_off, S.fin_tgt, tgt_pt);
+  return F;
 }
 
 }  // namespace bcfmm

@@ -54,6 +54,12 @@ bool build_p2p_sym(const HostSetup& H, int64_t chunk, HostSym& out);
 // sources per block: enough blocks for every SM, at most kSymChunkMax
 constexpr int64_t kSymChunkMin = 512, kSymChunkMax = 4096;
 int64_t p2p_sym_chunk(const HostSetup& H, int nsm);
+// Faults of a schedule of build_p2p_sym (host check): pairs, a pair of near leaves
+// (or of a leaf with itself) not in exactly one block; slots, a slot that is not
+// written once and gathered once, for the same point; blocks, one whose sources
+// exceed the chunk by more than a leaf, or out of the order the launches rely on.
+struct SymFaults { int64_t pairs = 0, slots = 0, blocks = 0; };
+SymFaults check_p2p_sym(const HostSetup& H, int64_t chunk, const HostSym& S);
 bool p2p_sym_pays(const HostSetup& H);
 
 // densities (padded) that the symmetric form takes; more need too many registers
