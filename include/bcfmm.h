@@ -263,28 +263,26 @@ int bcfmm_eval_graph(bcfmm_ctx* ctx, int32_t task_mask, double* out_vtv, double*
  *             read on the context's stream
  *   out_dev   FP64 device array, one value per target element; written
  *             asynchronously on the context's stream
- * The M2L keeps its partial sums (tensor cores: per work unit; Taylor
- * form: per list chunk and target) in a fixed static device array of 64 MiB
- * (every GPU that loads the library holds it until the process exits)
- * instead of the context's scratch; all other buffers are the context's,
- * sized by an earlier bcfmm_set_density (required once).  Where the sums of
- * order 8 do not fit into the array too, all of them go to the context's
- * scratch.
- * The first call on a device looks up that array's device address (a
- * one-time set-up, per device); make that first call before any stream
+ * The tensor-core M2L keeps its partial sums (per work unit) in a fixed
+ * static device array of 64 MiB (every GPU that loads the library holds it
+ * until the process exits) instead of the context's scratch; all other
+ * buffers, the Taylor form's partial sums among them, are the context's,
+ * sized by an earlier bcfmm_set_density (required once).
+ * The first tensor-core call on a device looks up that array's device address
+ * (a one-time set-up, per device); make that first call before any stream
  * capture.  The address is kept for the life of the process, so a device
  * reset (cudaDeviceReset, or a reset of the primary context) after the
- * first call on that device is not supported.  Every call on a device
- * shares the array and overwrites it completely, so nothing carries over
- * between calls, and calls that overlap on the GPU (different streams or
- * contexts on one device) race on it.
+ * first call on that device is not supported.  Every tensor-core call on a
+ * device shares the array and overwrites it completely, so nothing carries
+ * over between calls, and such calls that overlap on the GPU (different
+ * streams or contexts on one device) race on it.
  * The call does not synchronise: an expired bounded device wait of the
  * tensor-core M2L shows only in bcfmm_stats ("device_error") and is
  * returned, and cleared, by the next evaluation with host output.  The
  * call records no stage timings.
  * Errors: BCFMM_ERR_ARG (null pointer, bad task, context built with
- * precision BCFMM_FP64, or a mesh whose M2L needs more scratch, order 8
- * left out, than the array holds: the message gives both sizes), BCFMM_ERR_STATE (no earlier
+ * precision BCFMM_FP64, or a mesh whose tensor-core M2L needs more scratch
+ * than the array holds: the message gives both sizes), BCFMM_ERR_STATE (no earlier
  * bcfmm_set_density, or the current device is not the context's),
  * BCFMM_ERR_CUDA.
  */

@@ -502,7 +502,6 @@ static int upload_task(bcfmm_ctx* C, const HostSetup& H, int t) {
       S.wb = dwb; S.wslot = dws; S.ent = den; S.tgt = dtg; S.tchunk = dtc;
       const int slot = f64 ? taylor_partial<double>(O.q) : taylor_partial<float>(O.q);
       D.tys.partial_per_dens += (size_t)O.nchunk * slot;
-      if (O.q <= kTaylorRegQ) D.tys.partial_below8 += (size_t)O.nchunk * slot;
     }
     if (!sel.empty()) {
       int* dsel;
@@ -1701,7 +1700,7 @@ struct TaskRun {
   const double *dens = nullptr, *dip = nullptr;   // source density; BtV's double-layer density or null
   int ndens = 0, ndp = 0;
   double* out = nullptr;                          // device
-  void* partial = nullptr;                        // M2L partial sums in place of the work set's, or null
+  float2* partial = nullptr;                      // tensor-core partial sums in place of the work set's, or null
 };
 
 // The parts of an evaluation; T: double in an FP64 context, else float.
@@ -1741,7 +1740,7 @@ struct Parts {
     const T* mom = static_cast<T*>(w(r).mom);
     if (C->ty.q > 0) {
       cudaError_t e = launch_m2l_taylor<T>(G, L, D.tys, C->ty, r.ndp, mom, loc(r), static_cast<T*>(w(r).ty_momp),
-                                           static_cast<T*>(r.partial ? r.partial : w(r).ty_partial), st, side);
+                                           static_cast<T*>(w(r).ty_partial), st, side);
       if constexpr (f64)
         if (e == cudaSuccess && D.tys.nsimt > 0)
           e = launch_m2l_simt<double>(G, L, C->T64, r.ndp, mom, loc(r), st, D.tys.simt_sel, D.tys.nsimt);
@@ -1752,7 +1751,7 @@ struct Parts {
     } else {
       if (C->tc.nsplit == 0) return launch_m2l_simt<float>(G, L, C->T32, r.ndp, mom, loc(r), st);
       cudaError_t e = launch_m2l_tc(G, L, D.tcs, C->tc, r.ndp, mom, loc(r),
-                                    r.partial ? static_cast<float2*>(r.partial) : w(r).tc_partial, w(r).tc_momb, st);
+                                    r.partial ? r.partial : w(r).tc_partial, w(r).tc_momb, st);
       if (e == cudaSuccess && D.tcs.nsimt > 0)
         e = launch_m2l_simt<float>(G, L, C->T32, r.ndp, mom, loc(r), st, D.tcs.simt_sel, D.tcs.nsimt);
       return e;
@@ -2015,9 +2014,9 @@ extern "C" int bcfmm_eval_graph(bcfmm_ctx* C, int32_t mask, double* out_vtv, dou
 
 // One task, one density, no allocation: the tensor-core M2L writes its unit
 // partial sums into the library's fixed static device array instead of the
-// context's scratch; every other buffer was sized by an earlier
-// bcfmm_set_density.  Nothing here calls cudaMalloc, cudaFree or an
-// allocating library routine.
+// context's scratch; every other buffer, the Taylor form's chunk sums among
+// them, was sized by an earlier bcfmm_set_density.  Nothing here calls
+// cudaMalloc, cudaFree or an allocating library routine.
 extern "C" int bcfmm_eval_noalloc(bcfmm_ctx* C, int32_t task, const double* dens_dev, double* out_dev) {
   if (!C) return fail(BCFMM_ERR_ARG, "eval_noalloc: null context");
   if (task < 0 || task > 2) return fail(BCFMM_ERR_ARG, "eval_noalloc: task must be 0 (VtV), 1 (VtB) or 2 (BtV)");
@@ -2035,23 +2034,21 @@ extern "C" int bcfmm_eval_noalloc(bcfmm_ctx* C, int32_t task, const double* dens
   CU(cudaGetDevice(&dev));
   if (dev != C->device) return fail(BCFMM_ERR_STATE, "eval_noalloc: the context's device is not the current device");
   float2* partial = nullptr;
-  size_t cap = 0;
-  CU(m2l_tc_noalloc_scratch(dev, &partial, &cap));
-  // tensor cores: float2 unit sums; Taylor form: float chunk sums
-  // (order 8 does not count: where it does not fit, the context's own buffer,
-  // sized with the others, takes all of them)
-  const size_t need = tcp ? D.tcs.partial_per_dens : (D.tys.partial_below8 + 1) / 2;
-  const bool fits = tcp || D.tys.partial_per_dens <= 2 * cap;
-  if (need > cap)
-    return fail(BCFMM_ERR_ARG, "eval_noalloc: the mesh needs " + std::to_string(need * sizeof(float2)) +
-                                   " bytes of M2L scratch, more than the fixed " + std::to_string(cap * sizeof(float2)) +
-                                   " bytes (use bcfmm_eval_vtv/vtb/btv)");
+  if (tcp) {
+    size_t cap = 0;
+    CU(m2l_tc_noalloc_scratch(dev, &partial, &cap));
+    const size_t need = D.tcs.partial_per_dens;
+    if (need > cap)
+      return fail(BCFMM_ERR_ARG, "eval_noalloc: the mesh needs " + std::to_string(need * sizeof(float2)) +
+                                     " bytes of M2L scratch, more than the fixed " + std::to_string(cap * sizeof(float2)) +
+                                     " bytes (use bcfmm_eval_vtv/vtb/btv)");
+  }
   TaskRun r;
   r.t = task;
   r.dens = dens_dev;
   r.ndens = r.ndp = 1;
   r.out = out_dev;
-  r.partial = fits ? partial : nullptr;
+  r.partial = partial;
   CU(run_tasks(C, &r, 1, C->st));
   C->ev_rec[task] = false;             // no stage timings recorded by this call
   return BCFMM_OK;

@@ -58,7 +58,6 @@ struct TaylorOrderSched {
 struct TaylorTaskSched {
   TaylorOrderSched ord[kTaylorMaxQ + 1];   // index = order q (nwarp 0: none)
   size_t partial_per_dens = 0;             // values of chunk partial sums per density (all orders)
-  size_t partial_below8 = 0;               // the same without order 8
   const int* simt_sel = nullptr;           // targets (indices into the task's list) of
   int nsimt = 0;                           // higher orders: one CTA per target
 };
