@@ -648,7 +648,8 @@ __device__ __forceinline__ void p2p_pairs_x2(const float4* __restrict__ xy, cons
 // the source loop all threads reduce the group sums, one target each.
 // The weights of the densities after the first go straight to shared memory
 // (4-byte cp.async), and from four densities on the compensated sums live there
-// and are folded every other tile: the registers then hold enough targets that
+// and are folded every other tile (130 products at most; the scalar form before
+// had 256): the registers then hold enough targets that
 // the shared-memory loads of the weights do not bound the loop.
 template <int ND>
 struct P2pShape {
@@ -656,7 +657,7 @@ struct P2pShape {
   static constexpr int kTile = ND <= 4 ? 512 : 256;      // source points per tile
   static constexpr int kPairs = kTile / 2;
   static constexpr bool kSumsShared = ND >= 4;
-  static constexpr int kFold = kSumsShared ? 2 : 1;      // tiles between folds (a sum: at most 64 products)
+  static constexpr int kFold = kSumsShared ? 2 : 1;      // tiles between folds (a tile: at most 65 products a sum, 129 for ND = 2)
   static constexpr int kW2 = ND > 1 ? 2 * (ND - 1) * kPairs : 0;     // float2
   static constexpr int kRed = ND * 128 * TPT;                        // float2
   // (the sums of fewer densities are laid over the weights at the end)

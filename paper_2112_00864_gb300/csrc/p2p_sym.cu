@@ -209,7 +209,10 @@ __device__ __forceinline__ void sym_block(const DevGeom& G, const DevSym& L, con
   const int r0 = L.run_off[b], r1 = L.run_off[b + 1];
   const int2 base = L.base[b];
   float* out = L.src + (int64_t)ND * base.x;
-  int fold = 0;                                  // a lane's FP32 sum holds at most 64 products between folds
+  // a lane's FP32 sum holds at most 64 products between folds, and GS more in the
+  // first interval (the owner's own points; a fold of their own costs 3 % of the
+  // level-3 ball's step)
+  int fold = 0;
   for (int rb = r0; rb < r1; rb += kSymRuns) {
     const int nr = min(kSymRuns, r1 - rb);
     __syncthreads();
