@@ -282,11 +282,11 @@ __global__ void __launch_bounds__(kTaylorWarps * 32) k_m2l_taylor(TaylorArgs<T> 
 
 // loc[t][d][a] = post[a] / s_t * (sum over the target's chunks, in chunk
 // order, FP32: compensated), post[a] = 1 / a!; one thread per (target, d, a).
-// slot: values of a chunk's sums; off: its lo parts' offset there (0: none)
-template <typename T>
+// slot: values of a chunk's sums; OFF: its lo parts' offset there (0: none)
+template <typename T, int OFF>
 __global__ void __launch_bounds__(128) k_m2l_taylor_reduce(int ntgt, const int* __restrict__ tgt,
                                                           const int* __restrict__ tchunk,
-                                                          const T* __restrict__ partial, int nq, int slot, int off,
+                                                          const T* __restrict__ partial, int nq, int slot,
                                                           int ndp, int ms, const T* __restrict__ post,
                                                           const double4_32a* __restrict__ box_cs,
                                                           T* __restrict__ loc) {
@@ -302,7 +302,7 @@ __global__ void __launch_bounds__(128) k_m2l_taylor_reduce(int ntgt, const int* 
     const T x = __ldg(pp + (int64_t)c * ndp * slot);
     if constexpr (sizeof(T) == 4) two_sum(hi, lo, x);
     else hi += x;
-    if (off) lo += __ldg(pp + (int64_t)c * ndp * slot + off);
+    if constexpr (OFF > 0) lo += __ldg(pp + (int64_t)c * ndp * slot + OFF);
   }
   loc[((int64_t)tb * ndp + d) * ms + a] = (hi + lo) * post[a] / (T)box_cs[tb].w;
 }
@@ -395,8 +395,9 @@ cudaError_t launch_order(const TaylorOrderSched& O, const TaylorTables& tab, con
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const int64_t n = (int64_t)O.ntgt * ndp * NQ;
-  k_m2l_taylor_reduce<T><<<(unsigned)((n + 127) / 128), 128, 0, st>>>(
-      O.ntgt, O.tgt, O.tchunk, partial, NQ, taylor_partial<T>(Q), taylor_comp<T>(Q) ? taylor_slot<T>(Q) : 0, ndp, G.ms,
+  constexpr int OFF = taylor_comp<T>(Q) ? taylor_slot<T>(Q) : 0;
+  k_m2l_taylor_reduce<T, OFF><<<(unsigned)((n + 127) / 128), 128, 0, st>>>(
+      O.ntgt, O.tgt, O.tchunk, partial, NQ, taylor_partial<T>(Q), ndp, G.ms,
       static_cast<const T*>(tab.fac) + tab.gpitch, G.box_cs, loc);
   return cudaGetLastError();
 }
