@@ -266,7 +266,7 @@ static int upload_task(bcfmm_ctx* C, const HostSetup& H, int t) {
   L.src_cls = T.src_cls;
   L.tgt_cls = T.tgt_cls;
   L.n_p2p = (int)T.p2p_leaf.size();
-  int *p2p_leaf, *near_off, *near_box, *m2l_tgt, *vl_off, *vl_src, *p2m_leaf, *l2p_leaf;
+  int *p2p_leaf, *m2l_tgt, *vl_off, *vl_src, *p2m_leaf;
   uint16_t* vl_code;
   {
     // near-field blocks (one per target leaf) in descending order of work,
@@ -283,26 +283,20 @@ static int upload_task(bcfmm_ctx* C, const HostSetup& H, int t) {
       work[i] = (double)ns * (double)(B.pt1[T.tgt_cls] - B.pt0[T.tgt_cls] + 8);
     }
     std::stable_sort(ord.begin(), ord.end(), [&](int a, int b) { return work[a] > work[b]; });
-    std::vector<int> leaf(n), noff(1, 0), nbox, roff(1, 0), runs, self(n);
+    std::vector<int> leaf(n), roff(1, 0), runs;
     for (int i = 0; i < n; ++i) {
       const int o = ord[i];
       leaf[i] = T.p2p_leaf[o];
-      self[i] = T.self_len[o];
-      for (int k = T.near_off[o]; k < T.near_off[o + 1]; ++k) nbox.push_back(T.near_box[k]);
-      noff.push_back((int)nbox.size());
       for (int r = T.run_off[o]; r < T.run_off[o + 1]; ++r) { runs.push_back(T.runs[2 * r]); runs.push_back(T.runs[2 * r + 1]); }
       roff.push_back((int)runs.size() / 2);
     }
     CU(m.upload(&p2p_leaf, leaf.data(), leaf.size(), st));
-    CU(m.upload(&near_off, noff.data(), noff.size(), st));
-    CU(m.upload(&near_box, nbox.data(), nbox.size(), st));
-    L.p2p_leaf = p2p_leaf; L.near_off = near_off; L.near_box = near_box;
-    int *run_off, *self_len;
+    L.p2p_leaf = p2p_leaf;
+    int* run_off;
     int2* rd;
     CU(m.upload(&run_off, roff.data(), roff.size(), st));
-    CU(m.upload(&self_len, self.data(), self.size(), st));
     CU(m.upload(&rd, reinterpret_cast<const int2*>(runs.data()), runs.size() / 2, st));
-    L.run_off = run_off; L.runs = rd; L.self_len = self_len;
+    L.run_off = run_off; L.runs = rd;
   }
   {
     // blocks of the packed FP32 near field (long leaves cut into chunks)
@@ -366,9 +360,6 @@ static int upload_task(bcfmm_ctx* C, const HostSetup& H, int t) {
   L.n_p2m = (int)T.p2m_leaf.size();
   CU(m.upload(&p2m_leaf, T.p2m_leaf.data(), T.p2m_leaf.size(), st));
   L.p2m_leaf = p2m_leaf;
-  L.n_l2p = (int)T.l2p_leaf.size();
-  CU(m.upload(&l2p_leaf, T.l2p_leaf.data(), T.l2p_leaf.size(), st));
-  L.l2p_leaf = l2p_leaf;
   // per-level lists
   std::vector<int> flat;
   D.m2m_off.assign(1, 0);
@@ -903,7 +894,7 @@ static int build_impl(const double* verts, const int64_t* vert_off, const int32_
     const int nb = C->nbox;
     std::vector<double4_32a> cs(nb);
     std::vector<float4> bhi(nb), blo(nb);
-    std::vector<int> c0(nb), nc(nb), oc(nb), par(nb);
+    std::vector<int> c0(nb), nc(nb), oc(nb);
     std::vector<int2> rg[2] = {std::vector<int2>(nb), std::vector<int2>(nb)};
     for (int i = 0; i < nb; ++i) {
       const HostBox& B = H.box[i];
@@ -912,20 +903,20 @@ static int build_impl(const double* verts, const int64_t* vert_off, const int32_
       for (int a = 0; a < 3; ++a) { h[a] = (float)B.c[a]; l[a] = (float)(B.c[a] - (double)h[a]); }
       bhi[i] = make_float4(h[0], h[1], h[2], 0.f);
       blo[i] = make_float4(l[0], l[1], l[2], 0.f);
-      c0[i] = B.child0; nc[i] = B.nchild; oc[i] = B.octant; par[i] = B.parent;
+      c0[i] = B.child0; nc[i] = B.nchild; oc[i] = B.octant;
       for (int c = 0; c < 2; ++c) rg[c][i] = make_int2(B.pt0[c], B.pt1[c]);
     }
     const std::vector<int>& bq = box_q;
     float4 *dbh, *dbl;
-    double4_32a* dcs; int *dc0, *dnc, *doc, *dpar, *dbq; int2 *drg0, *drg1;
+    double4_32a* dcs; int *dc0, *dnc, *doc, *dbq; int2 *drg0, *drg1;
     bool ok = m.upload(&dcs, cs.data(), nb, st) == cudaSuccess && m.upload(&dc0, c0.data(), nb, st) == cudaSuccess &&
               m.upload(&dnc, nc.data(), nb, st) == cudaSuccess && m.upload(&doc, oc.data(), nb, st) == cudaSuccess &&
-              m.upload(&dpar, par.data(), nb, st) == cudaSuccess && m.upload(&drg0, rg[0].data(), nb, st) == cudaSuccess &&
+              m.upload(&drg0, rg[0].data(), nb, st) == cudaSuccess &&
               m.upload(&drg1, rg[1].data(), nb, st) == cudaSuccess && m.upload(&dbq, bq.data(), nb, st) == cudaSuccess &&
               m.upload(&dbh, bhi.data(), nb, st) == cudaSuccess && m.upload(&dbl, blo.data(), nb, st) == cudaSuccess;
     if (!ok) return cleanup(fail(BCFMM_ERR_OOM, "build: device allocation failed (boxes)"));
     G.box_hi = dbh; G.box_lo = dbl;
-    G.box_cs = dcs; G.box_child0 = dc0; G.box_nchild = dnc; G.box_octant = doc; G.box_parent = dpar;
+    G.box_cs = dcs; G.box_child0 = dc0; G.box_nchild = dnc; G.box_octant = doc;
     G.box_rng[0] = drg0; G.box_rng[1] = drg1; G.box_q = dbq;
   }
   // sorted points

@@ -48,7 +48,6 @@ struct HostTask {
   std::vector<int> p2m_leaf;                       // leaves with source points
   std::vector<std::vector<int>> m2m_parent;        // per level: non-leaf boxes with source points
   std::vector<std::vector<int>> l2l_child;         // per level: boxes (level>=3) with target points
-  std::vector<int> l2p_leaf;                       // leaves (level >= 2) with target points
   // tensor-core M2L tiles (see DevTaskLists)
   std::vector<int> tc_tile_tgt, tc_tile_off, tc_ent_code, tc_ent_src, tc_tile_q;
   // near element pairs, CSR over target elements

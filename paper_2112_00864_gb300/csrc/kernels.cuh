@@ -20,7 +20,6 @@ struct DevGeom {
   const int* box_child0;
   const int* box_nchild;
   const int* box_octant;
-  const int* box_parent;
   const int2* box_rng[2];        // point range per class
   const double4_32a* pt64[2];        // sorted points: x, y, z, quadrature weight
   const float4* pthi[2];         // float hi parts (x, y, z, weight)
@@ -33,11 +32,10 @@ struct DevGeom {
 };
 
 struct DevTaskLists {
-  int n_p2p; const int* p2p_leaf; const int* near_off; const int* near_box;
-  const int* run_off; const int2* runs; const int* self_len;   // merged source runs per target leaf
+  int n_p2p; const int* p2p_leaf;
+  const int* run_off; const int2* runs;   // merged source runs per target leaf
   int n_m2l; const int* m2l_tgt; const int* vl_off; const int* vl_src; const uint16_t* vl_code;
   int n_p2m; const int* p2m_leaf;
-  int n_l2p; const int* l2p_leaf;
   int64_t ntgt_el, nsrc_el;
   const int64_t* cor_off; const int* cor_col; const double* cor_val;
   const double* cor_val_dl;      // BtV: near-rule corrections of dG/dn_y (same CSR), or null

@@ -112,8 +112,7 @@ struct NearTabs {
 
 struct SrcTet {
   V3 v[4];
-  V3 te[6];            // unit direction of edge k (first -> second vertex)
-  double len[6];       // its length
+  double len[6];       // length of edge k
   V3 nout[4];          // outward unit normal of face f
   V3 nf[4];            // unit normal of the face's vertex order
   double nn[4];        // twice the face's area

@@ -196,13 +196,12 @@ __device__ double elem_size(const D3* v, int nv) {
 
 // ------------------------------------------------------------ network
 // forward on BF16-rounded weights held in shared memory (FP32 storage)
-__device__ float mlp_forward(const float* __restrict__ P, const float* x, const float* qhat, float* z1, float* z2) {
+__device__ float mlp_forward(const float* __restrict__ P, const float* x, const float* qhat) {
   float h1[kMlpH];
   for (int j = 0; j < kMlpH; ++j) {
     float s = P[kOffB1 + j];
 #pragma unroll
     for (int k = 0; k < kMlpIn; ++k) s = fmaf(P[kOffW1 + j * kMlpIn + k], x[k], s);
-    z1[j] = s;
     h1[j] = gelu(s);
   }
   float pred = 0.f;
@@ -210,7 +209,6 @@ __device__ float mlp_forward(const float* __restrict__ P, const float* x, const 
   for (int j = 0; j < kMlpH; ++j) {
     float s = P[kOffB2 + j];
     for (int k = 0; k < kMlpH; ++k) s = fmaf(P[kOffW2 + j * kMlpH + k], h1[k], s);
-    z2[j] = s;
     h2[j] = gelu(s);
   }
   for (int o = 0; o < kMlpOut; ++o) {
@@ -463,7 +461,7 @@ __global__ void k_mlp_adam(float* __restrict__ params, const float* __restrict__
 // A thread's units are jg + 16 i (the weights are stored in that order), and
 // activation rows are padded by four floats: the sixteen threads that share
 // pairs then store to different banks.
-constexpr int kPredThreads = 256;
+constexpr int kPredThreads = 256, kPredSms = 152;    // (the chip's SMs)
 template <int P>
 struct PredShared {
   float W1[kMlpIn][kMlpH], W2[kMlpH][kMlpH], W3[kMlpOut][kMlpH];   // [input][pred_unit(unit)]
@@ -609,10 +607,10 @@ __global__ void __launch_bounds__(kMlpThreads) k_near_mlp(int task, const int64_
   D3 tv[4], sv[4];
   load_elem(tgt_v, row[k], nvt, tv);
   load_elem(src_v, col[k], nvs, sv);
-  float x[kMlpIn], qh[kMlpOut], z1[kMlpH], z2[kMlpH];
+  float x[kMlpIn], qh[kMlpOut];
   double Q;
   pair_features(tv, nvt, elem_size(tv, nvt), sv, nvs, elem_size(sv, nvs), x, qh, &Q);
-  cor_val[k] = Q * (double)mlp_forward(P, x, qh, z1, z2);
+  cor_val[k] = Q * (double)mlp_forward(P, x, qh);
 }
 
 // Training / validation data of the pairs sel[0..n): features, qhat, Q,
@@ -691,7 +689,7 @@ static cudaError_t launch_predict_p(const float* params, const float* feat, cons
     if (e != cudaSuccess) return e;
   }
   const int64_t tiles = (n + P - 1) / P;
-  k_mlp_predict<P><<<(unsigned)std::min<int64_t>(tiles, 2 * 152), kPredThreads, sm, st>>>(params, feat, qhat, n, out);
+  k_mlp_predict<P><<<(unsigned)std::min<int64_t>(tiles, 2 * kPredSms), kPredThreads, sm, st>>>(params, feat, qhat, n, out);
   return cudaGetLastError();
 }
 
@@ -699,7 +697,7 @@ cudaError_t launch_mlp_predict(const float* params, const float* feat, const flo
                                cudaStream_t st) {
   if (n == 0) return cudaSuccess;
   // 128 pairs a CTA once that fills the SMs, 32 below
-  return n >= 128 * 152 ? launch_predict_p<128>(params, feat, qhat, n, out, st) : launch_predict_p<32>(params, feat, qhat, n, out, st);
+  return n >= 128 * kPredSms ? launch_predict_p<128>(params, feat, qhat, n, out, st) : launch_predict_p<32>(params, feat, qhat, n, out, st);
 }
 
 cudaError_t launch_near_classify(int task, int64_t nnz, const int* row, const int* col, const double* tgt_v,

@@ -323,7 +323,6 @@ void build_lists(HostSetup& H, double eta0) {
         }
         T.vl_off.push_back((int)T.vl_src.size());
         if (B.level >= 3) T.l2l_child[B.level].push_back(bi);
-        if (B.nchild == 0 && ntgt(bi) > 0) T.l2p_leaf.push_back(bi);
       }
     }
   }
@@ -688,7 +687,6 @@ void merge_setups(std::vector<HostSetup>& P, HostSetup& H) {
       for (int b : S.vl_src) T.vl_src.push_back(bm[b]);
       for (uint16_t c : S.vl_code) T.vl_code.push_back((uint16_t)cmap[m][c]);
       for (int b : S.p2m_leaf) T.p2m_leaf.push_back(bm[b]);
-      for (int b : S.l2p_leaf) T.l2p_leaf.push_back(bm[b]);
       for (size_t l = 0; l < S.m2m_parent.size(); ++l)
         for (int b : S.m2m_parent[l]) T.m2m_parent[l].push_back(bm[b]);
       for (size_t l = 0; l < S.l2l_child.size(); ++l)
