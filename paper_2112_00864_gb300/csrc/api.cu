@@ -821,7 +821,7 @@ static int build_impl(const double* verts, const int64_t* vert_off, const int32_
     // Sec. 4.3 (Eq. def:q0): q_l = q0 + L - l, L the deepest level of the
     // tree (of every mesh of a batch), capped at p
     const int L = H.nlevels - 1;
-    for (int l = 0; l < BCFMM_MAX_LEVELS; ++l) prm.p_level[l] = std::max(1, std::min(prm.p, prm.q0 + L - l));
+    for (int l = 0; l < BCFMM_MAX_LEVELS; ++l) prm.p_level[l] = std::min(prm.p, std::max(1, prm.q0 + L - l));
   }
   std::vector<int> box_q(H.box.size());
   for (size_t i = 0; i < H.box.size(); ++i) box_q[i] = level_order(prm, H.box[i].level);
@@ -1302,7 +1302,7 @@ extern "C" int bcfmm_debug_list_coverage(const double* verts, const int64_t* ver
     // tensor-core tiles: the (offset code, source box) entries of each row
     // must be exactly the row's interaction list
     if (prm.q0 > 0)
-      for (int l = 0; l < BCFMM_MAX_LEVELS; ++l) prm.p_level[l] = std::max(1, std::min(prm.p, prm.q0 + H.nlevels - 1 - l));
+      for (int l = 0; l < BCFMM_MAX_LEVELS; ++l) prm.p_level[l] = std::min(prm.p, std::max(1, prm.q0 + H.nlevels - 1 - l));
     std::vector<int> box_q(H.box.size());
     for (size_t i = 0; i < H.box.size(); ++i) box_q[i] = level_order(prm, H.box[i].level);
     const int qmax = tc_max_order(2);
