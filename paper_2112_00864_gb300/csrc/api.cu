@@ -1783,13 +1783,13 @@ struct Parts {
   }
 };
 
-// One task after the other's parts on one stream, with events between the
-// stages when ev is given.
+// One task's parts after one another on one stream, with an event between the
+// stages (bcfmm_params.timing).
 template <typename T>
 static cudaError_t run_serial(bcfmm_ctx* C, const TaskRun& r, cudaStream_t st, cudaEvent_t* ev) {
   const Parts<T> P(C);
   cudaError_t e = cudaSuccess;
-  auto mark = [&](int k) { if (ev && e == cudaSuccess) e = cudaEventRecord(ev[k], st); };
+  auto mark = [&](int k) { if (e == cudaSuccess) e = cudaEventRecord(ev[k], st); };
   auto step = [&](cudaError_t x) { if (e == cudaSuccess) e = x; };
   mark(0);
   step(P.weights(r, st));
@@ -1899,10 +1899,6 @@ static int task_run(bcfmm_ctx* C, int t, TaskRun& r) {
   return ensure_buffers(C, kind, r.ndp, 0);
 }
 
-// Near-field pairs from which a single task's parts run side by side: the
-// eight event calls cost the host about 10 us.
-constexpr int64_t kForkPairs = 100000000;
-
 static int eval_impl(bcfmm_ctx* C, int t, double* out, int out_is_device) {
   if (!C) return fail(BCFMM_ERR_ARG, "eval: null context");
   const DevTaskLists& L = C->task[t].L;
@@ -1917,9 +1913,11 @@ static int eval_impl(bcfmm_ctx* C, int t, double* out, int out_is_device) {
   cudaStream_t st = C->st;
   const bool tm = C->prm.timing && C->ev_ok;
   r.out = out_is_device ? out : C->out_dev;
-  if (!tm && C->task[t].p2p_pairs >= kForkPairs) CU(run_tasks(C, &r, 1, st));
-  else if (C->prm.precision == BCFMM_FP64) CU(run_serial<double>(C, r, st, tm ? C->ev[t] : nullptr));
-  else CU(run_serial<float>(C, r, st, tm ? C->ev[t] : nullptr));
+  // side by side unless the stages are timed: a task alone, call and wait, of 1 M
+  // near-field pairs 98 -> 89 us, 18 M 114 -> 95, 128 M 209 -> 157, 816 M 529 -> 423
+  if (!tm) CU(run_tasks(C, &r, 1, st));
+  else if (C->prm.precision == BCFMM_FP64) CU(run_serial<double>(C, r, st, C->ev[t]));
+  else CU(run_serial<float>(C, r, st, C->ev[t]));
   if (!out_is_device) {
     CU(cudaMemcpyAsync(out, C->out_dev, (size_t)r.ndens * L.ntgt_el * sizeof(double), cudaMemcpyDeviceToHost, st));
     int herr = 0;
