@@ -1621,7 +1621,8 @@ static void ensure_slots(bcfmm_ctx* C, int ndp) {
   C->slots_tried[0] = ndp;             // (not again before other buffers change)
   C->slots_tried[1] = C->work_gen;
   const size_t need = (size_t)ndp * (Y.nsrc * sizeof(float) + Y.ntgt * sizeof(float2));
-  if (need > C->mem.room() / 2) return;
+  // (asking for the free memory costs 50 us; slots of a few MB do not matter)
+  if ((need > (size_t)64 << 20 || C->mem.limit > 0) && need > C->mem.room() / 2) return;
   if (C->mem.alloc(&Y.src, (size_t)ndp * Y.nsrc) == cudaSuccess && C->mem.alloc(&Y.tgt, (size_t)ndp * Y.ntgt) == cudaSuccess) {
     Y.cap = ndp;
     C->work_gen++;
