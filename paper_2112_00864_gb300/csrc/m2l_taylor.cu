@@ -122,8 +122,8 @@ size_t taylor_smem(int q) {
 // the lanes contract one entry, the next one's 18 g rows (one contiguous
 // block) and up to four moment rows arrive by cp.async in the warp's own stage
 // (no barrier between warps).  lane = target slot + 8 * source slot.
-// Bound by the FMA pipe (57 % of its cycles at order 6, issue 68 %).  With one
-// (target, source) pair per lane and rows read by each lane from global memory
+// Bound by issue and latency at eight warps an SM (order 6: issue 68 %, FMA pipe
+// 57 % of its cycles, lanes 78 % filled).  With one (target, source) pair per lane and rows read by each lane from global memory
 // the L1 was the bound, one distinct line per cycle: 64 a pair of row pieces,
 // where an entry has 22 and fetches them coalesced.  Unit ball, level 4 (191,840
 // tets, orders 6 and 7, 7.7 M pairs): VtV's whole M2L stage 0.86 -> 0.49 ms, the
@@ -131,9 +131,10 @@ size_t taylor_smem(int q) {
 // tables, one CTA per target: 3.37 -> 0.39 ms.
 // FP32 above kTaylorRegQ: every entry's products go into a compensated sum (hi,
 // lo), as in the one-CTA-per-target kernel; 42 outputs a pass leave registers
-// for the three arrays.  With plain sums over a chunk the potentials of sources
-// far away (level-3 ball, order 8) were off by 1.85e-7 against the FP64 form,
-// 1.38e-7 with one CTA per target.
+// for the three arrays.  Potentials of sources far away (level-3 ball, order 8)
+// against the FP64 form: 1.85e-7 with plain sums over a chunk, 1.38e-7 with one CTA
+// per target, 1.20e-7 now; VtV of the level-2 ball with order 8 on every level takes
+// 239 us (200 with plain sums, 3.1 ms with one CTA per target).
 template <typename T, int Q, int NP>
 __global__ void __launch_bounds__(kTaylorWarps * 32) k_m2l_taylor(TaylorArgs<T> A) {
   constexpr int NQ = (Q + 1) * (Q + 2) * (Q + 3) / 6;
