@@ -92,7 +92,7 @@ struct NearGeom {
   double *tv = nullptr, *sv = nullptr, *tqp = nullptr, *tqw = nullptr, *sqp = nullptr, *sqw = nullptr;
   double *glx = nullptr, *glw = nullptr;
   int* row = nullptr;
-  int64_t* ns_list = nullptr;          // CSR positions of the near-singular pairs
+  int64_t* ns_list = nullptr;          // CSR positions of the near-singular pairs, ascending
 };
 
 struct TaskDev {
@@ -576,26 +576,35 @@ static int upload_task(bcfmm_ctx* C, const HostSetup& H, int t) {
     const int64_t cap = std::max<int64_t>(D.nnz, 1);
     int64_t* lists;
     unsigned long long* cnt;
-    CU(m.alloc(&lists, 4 * cap));
-    CU(m.alloc(&cnt, 4));
-    CU(cudaMemsetAsync(cnt, 0, 4 * sizeof(unsigned long long), st));
+    unsigned* singular;
+    std::vector<unsigned> bits((D.nnz + 31) / 32, 0u);
+    CU(m.alloc(&lists, 2 * cap));
+    CU(m.alloc(&cnt, 2));
+    CU(m.alloc(&singular, bits.size()));
+    CU(cudaMemsetAsync(cnt, 0, 2 * sizeof(unsigned long long), st));
     CU(cudaMemsetAsync(cor_val, 0, cap * sizeof(double), st));
     CU(launch_near_classify(t, D.nnz, cor_row, cor_col, g.tv, g.sv, C->prm.near_mode, eps, (float)C->prm.mlp_tol, lists,
-                            cnt, cap, st));
-    unsigned long long hc[4];
+                            cnt, cap, singular, st));
+    unsigned long long hc[2] = {0, 0};
+    if (!bits.empty())
+      CU(cudaMemcpyAsync(bits.data(), singular, bits.size() * sizeof(unsigned), cudaMemcpyDeviceToHost, st));
     CU(cudaMemcpyAsync(hc, cnt, sizeof hc, cudaMemcpyDeviceToHost, st));
     CU(cudaStreamSynchronize(st));
     D.n_fp64 = (int64_t)hc[0];
     D.n_learned = (int64_t)hc[1];
-    D.n_singular = (int64_t)hc[3];
+    // the near-singular pairs in CSR order (training data is drawn from them)
+    std::vector<int64_t> ns;
+    for (size_t i = 0; i < bits.size(); ++i)
+      for (unsigned b = bits[i]; b; b &= b - 1) ns.push_back((int64_t)(32 * i) + __builtin_ctz(b));
+    D.n_singular = (int64_t)ns.size();
     CU(launch_near_rule(t, D.n_fp64, lists, cor_row, cor_col, g.tv, g.sv, g.tqp, g.tqw, g.sqp, g.sqw, g.glx, g.glw,
                         C->prm.near_n, C->prm.near_k, 0, C->near_tabs, cor_val, st));
     if (learned) CU(launch_near_mlp(t, lists + cap, D.n_learned, cor_row, cor_col, g.tv, g.sv, par, cor_val, st));
-    CU(m.alloc(&g.ns_list, std::max<int64_t>(D.n_singular, 1)));
-    CU(cudaMemcpyAsync(g.ns_list, lists + 3 * cap, D.n_singular * sizeof(int64_t), cudaMemcpyDeviceToDevice, st));
+    CU(m.upload(&g.ns_list, ns.data(), ns.size(), st));
     CU(cudaStreamSynchronize(st));
     m.release(lists);
     m.release(cnt);
+    m.release(singular);
     if (eps) m.release(eps);
     if (par) m.release(par);
   }

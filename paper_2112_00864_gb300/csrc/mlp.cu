@@ -552,15 +552,16 @@ __global__ void __launch_bounds__(kPredThreads) k_mlp_predict(const float* __res
 
 // ------------------------------------------------------- setup passes
 // Classify every near pair k (CSR position): touching (gap bound <= 1e-9
-// of the radius sum) -> FP64 near rule; near-singular -> appended to the
-// near-singular list and, by mode, to the learned list (its bin's
-// calibrated error <= tol), the FP64 list (bin rejected), or nowhere
-// (mode 2: product rule only).
+// of the radius sum) -> FP64 near rule; near-singular -> its bit set in
+// `singular` (bit k % 32 of word k / 32) and, by mode, appended to the learned
+// list (its bin's calibrated error <= tol), the FP64 list (bin rejected), or
+// nowhere (mode 2: product rule only).
 __global__ void k_near_classify(int task, int64_t nnz, const int* __restrict__ row, const int* __restrict__ col,
                                 const double* __restrict__ tgt_v, const double* __restrict__ src_v, int mode,
                                 const float* __restrict__ eps_tab, float tol, int64_t* __restrict__ lists,
-                                unsigned long long* __restrict__ counts, int64_t cap) {
+                                unsigned long long* __restrict__ counts, int64_t cap, unsigned* __restrict__ singular) {
   const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const unsigned in = __ballot_sync(0xffffffffu, k < nnz);
   if (k >= nnz) return;
   const int nvt = task == 1 ? 3 : 4, nvs = task == 2 ? 3 : 4;
   D3 tv[4], sv[4];
@@ -570,11 +571,12 @@ __global__ void k_near_classify(int task, int64_t nnz, const int* __restrict__ r
   const double rs = radius(tv, nvt, ct) + radius(sv, nvs, cs);
   const double gap = sat_gap(tv, nvt, sv, nvs);
   int cls;                                   // 0 FP64 list, 1 learned list, 2 none
-  if (gap <= 1e-9 * rs) {
+  const bool touching = gap <= 1e-9 * rs;
+  const unsigned bits = __ballot_sync(in, !touching);
+  if ((threadIdx.x & 31) == 0) singular[k >> 5] = bits;
+  if (touching) {
     cls = 0;
   } else {
-    const unsigned long long s = atomicAdd(&counts[3], 1ull);
-    if ((int64_t)s < cap) lists[3 * cap + s] = k;
     if (mode == 2) {
       cls = 2;
     } else {
@@ -703,10 +705,10 @@ cudaError_t launch_mlp_predict(const float* params, const float* feat, const flo
 
 cudaError_t launch_near_classify(int task, int64_t nnz, const int* row, const int* col, const double* tgt_v,
                                  const double* src_v, int mode, const float* eps_tab, float tol, int64_t* lists,
-                                 unsigned long long* counts, int64_t cap, cudaStream_t st) {
+                                 unsigned long long* counts, int64_t cap, unsigned* singular, cudaStream_t st) {
   if (nnz == 0) return cudaSuccess;
   k_near_classify<<<(unsigned)((nnz + 127) / 128), 128, 0, st>>>(task, nnz, row, col, tgt_v, src_v, mode, eps_tab, tol,
-                                                                 lists, counts, cap);
+                                                                 lists, counts, cap, singular);
   return cudaGetLastError();
 }
 

@@ -22,10 +22,11 @@ cudaError_t launch_mlp_adam(float* params, const float* grad, float* m1, float* 
                             float b2, float eps, cudaStream_t st);
 cudaError_t launch_mlp_predict(const float* params, const float* feat, const float* qhat, int64_t n, float* out,
                                cudaStream_t st);
-// lists: [4][cap] (0 FP64 rule, 1 learned, 2 unused, 3 every near-singular pair); counts [4]
+// lists: [2][cap] (0 FP64 rule, 1 learned; in no fixed order); counts [2]; singular: a bit
+// per pair, [(nnz + 31) / 32] words
 cudaError_t launch_near_classify(int task, int64_t nnz, const int* row, const int* col, const double* tgt_v,
                                  const double* src_v, int mode, const float* eps_tab, float tol, int64_t* lists,
-                                 unsigned long long* counts, int64_t cap, cudaStream_t st);
+                                 unsigned long long* counts, int64_t cap, unsigned* singular, cudaStream_t st);
 cudaError_t launch_near_mlp(int task, const int64_t* sel, int64_t n, const int* row, const int* col,
                             const double* tgt_v, const double* src_v, const float* params, double* cor_val,
                             cudaStream_t st);
