@@ -25,7 +25,7 @@
 namespace bcfmm {
 
 constexpr double kInv4PiM = 0.079577471545947667884441881686257;
-constexpr int kMlpThreads = 128;
+constexpr int kMlpThreads = 128, kMlpSms = 152;        // (the chip's SMs)
 
 __device__ __forceinline__ float bf16r(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
 
@@ -231,23 +231,24 @@ __device__ __forceinline__ float warp_sum(float v) {
 
 // Mean loss and its gradient over n pairs (added with atomics to grad and
 // loss, which k_mlp_zero cleared).  A minibatch is small (about a thousand
-// pairs), so latency is the bound: a CTA of 256 threads takes P pairs (8, 16 or
-// 32, by the number of CTAs that n gives) and shares every layer among its
-// threads, activations and weights in shared memory.  With v = W3^T qhat the
-// output layer is two dot products (pred = v.h2 + b3.qhat) and its backward
-// pass is v itself: dz2 = dpred v gelu'(z2).
-// The sums of eight CTAs (a cluster) are added in FP64 through distributed
-// shared memory, an eighth of the parameters each, so that one atomic per
-// parameter serves 8 P pairs: every FP32 addition to a running gradient rounds
-// it, and with an atomic per CTA 1,024 pairs were off by 1.9e-7 of the norm
-// (against FP64 autograd), twice as much as with one pair per thread in eight
-// CTAs.
-// 1,024 pairs on the device: 111 us with one pair per thread (eight CTAs,
-// activations in local memory), 19.3 us with an atomic per CTA, 16.6 us now; the
+// pairs), so latency is the bound: a CTA takes P pairs and shares every layer
+// among its NT threads, activations and weights in shared memory: 8 pairs with 256
+// threads, 32 with 512, or, where they outnumber the SMs, 32 with 256.  With v =
+// W3^T qhat the output layer is two dot products (pred = v.h2 + b3.qhat) and its
+// backward pass is v itself: dz2 = dpred v gelu'(z2).
+// The sums of a cluster's CTAs are added in FP64 through distributed shared
+// memory, each CTA a share of the parameters, so that one atomic per parameter
+// serves a whole cluster: every FP32 addition to a running gradient rounds it, and
+// with an atomic per CTA 1,024 pairs were off by 1.9e-7 of the norm (against FP64
+// autograd), twice as much as with one pair per thread in eight CTAs.  Sixteen CTAs
+// of 32 pairs make two clusters of 1,024 pairs, the minibatch of a training; two
+// additions to zero give the same sum in either order, so that a training repeats
+// bit for bit.
+// On the device: 1,024 pairs 111 us with one pair per thread (eight CTAs,
+// activations in local memory), 19.3 us with an atomic per CTA, 18.2 us now; the
 // gradient and the Adam step with the copies of a caller that keeps its state: 131
-// us with one pair per thread, 54 us now, most of it the host's calls.
-constexpr int kGradThreads = 256;
-constexpr int kGradCluster = 8;
+// us with one pair per thread, 56 us now, most of it the host's calls.
+constexpr int kGradCluster = 16;                       // CTAs (opt-in; eight where the device refuses it)
 constexpr int kLdW2 = kMlpH + 1;                       // padded rows: W2 is read along both indexes
 
 template <int P>
@@ -263,8 +264,8 @@ struct GradShared {
   float part[2][P], dpred[P];
 };
 
-template <int P>
-__global__ void __cluster_dims__(kGradCluster, 1, 1) __launch_bounds__(kGradThreads) k_mlp_grad(const float* __restrict__ params, const float* __restrict__ feat,
+template <int P, int NT>
+__global__ void __launch_bounds__(NT) k_mlp_grad(const float* __restrict__ params, const float* __restrict__ feat,
                                                            const float* __restrict__ qhat, const float* __restrict__ chat,
                                                            int64_t n, float inv_n, float* __restrict__ grad,
                                                            float* __restrict__ loss) {
@@ -273,16 +274,17 @@ __global__ void __cluster_dims__(kGradCluster, 1, 1) __launch_bounds__(kGradThre
   // the CTA's gradient and loss, in the place of the weights once they are used up
   float* Gs = reinterpret_cast<float*>(smraw);
   static_assert(offsetof(GradShared<P>, x) >= (kMlpParams + 1) * sizeof(float), "gradient over the weights");
-  const int tid = threadIdx.x, j = tid & 63, g = tid >> 6;      // unit, quarter of the pairs
+  const int tid = threadIdx.x, j = tid & 63, g = tid >> 6;      // unit, group: a share of the pairs
   const int64_t i0 = (int64_t)blockIdx.x * P;
-  constexpr int PQ = P / 4;
-  for (int i = tid; i < kMlpH * kMlpIn; i += kGradThreads) S.W1[i % kMlpIn][i / kMlpIn] = bf16r(params[kOffW1 + i]);
-  for (int i = tid; i < kMlpH * kMlpH; i += kGradThreads) S.W2[i / kMlpH][i % kMlpH] = bf16r(params[kOffW2 + i]);
-  for (int i = tid; i < kMlpOut * kMlpH; i += kGradThreads) S.W3[i / kMlpH][i % kMlpH] = bf16r(params[kOffW3 + i]);
+  constexpr int NG = NT / 64, PQ = P / NG;
+  constexpr int R2 = kMlpH / NG, R3 = kMlpOut / NG;             // rows of dW2, dW3 per group
+  for (int i = tid; i < kMlpH * kMlpIn; i += NT) S.W1[i % kMlpIn][i / kMlpIn] = bf16r(params[kOffW1 + i]);
+  for (int i = tid; i < kMlpH * kMlpH; i += NT) S.W2[i / kMlpH][i % kMlpH] = bf16r(params[kOffW2 + i]);
+  for (int i = tid; i < kMlpOut * kMlpH; i += NT) S.W3[i / kMlpH][i % kMlpH] = bf16r(params[kOffW3 + i]);
   if (tid < kMlpH) { S.b1[tid] = bf16r(params[kOffB1 + tid]); S.b2[tid] = bf16r(params[kOffB2 + tid]); }
   if (tid < kMlpOut) S.b3[tid] = bf16r(params[kOffB3 + tid]);
-  for (int i = tid; i < P * kMlpIn; i += kGradThreads) S.x[i / kMlpIn][i % kMlpIn] = i0 + i / kMlpIn < n ? feat[i0 * kMlpIn + i] : 0.f;
-  for (int i = tid; i < P * kMlpOut; i += kGradThreads) S.qh[i / kMlpOut][i % kMlpOut] = i0 + i / kMlpOut < n ? qhat[i0 * kMlpOut + i] : 0.f;
+  for (int i = tid; i < P * kMlpIn; i += NT) S.x[i / kMlpIn][i % kMlpIn] = i0 + i / kMlpIn < n ? feat[i0 * kMlpIn + i] : 0.f;
+  for (int i = tid; i < P * kMlpOut; i += NT) S.qh[i / kMlpOut][i % kMlpOut] = i0 + i / kMlpOut < n ? qhat[i0 * kMlpOut + i] : 0.f;
   __syncthreads();
   // layer 1 and v
 #pragma unroll 2
@@ -371,31 +373,28 @@ __global__ void __cluster_dims__(kGradCluster, 1, 1) __launch_bounds__(kGradThre
   }
   __syncthreads();
   {
-    float a[16], c[4];                          // dW2[16 g + i][j], dW3[4 g + i][j]
+    float a[R2], c[R3];                         // dW2[R2 g + i][j], dW3[R3 g + i][j]
 #pragma unroll
-    for (int i = 0; i < 16; ++i) a[i] = 0.f;
+    for (int i = 0; i < R2; ++i) a[i] = 0.f;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) c[i] = 0.f;
+    for (int i = 0; i < R3; ++i) c[i] = 0.f;
     for (int p = 0; p < P; ++p) {
       const float h = S.h1[p][j], u = S.h2[p][j] * S.dpred[p];
 #pragma unroll
-      for (int i = 0; i < 16; i += 4) {
-        const float4 d = *reinterpret_cast<const float4*>(&S.d2[p][16 * g + i]);
+      for (int i = 0; i < R2; i += 4) {
+        const float4 d = *reinterpret_cast<const float4*>(&S.d2[p][R2 * g + i]);
         a[i] = fmaf(d.x, h, a[i]);
         a[i + 1] = fmaf(d.y, h, a[i + 1]);
         a[i + 2] = fmaf(d.z, h, a[i + 2]);
         a[i + 3] = fmaf(d.w, h, a[i + 3]);
       }
-      const float4 q = *reinterpret_cast<const float4*>(&S.qh[p][4 * g]);
-      c[0] = fmaf(q.x, u, c[0]);
-      c[1] = fmaf(q.y, u, c[1]);
-      c[2] = fmaf(q.z, u, c[2]);
-      c[3] = fmaf(q.w, u, c[3]);
+#pragma unroll
+      for (int i = 0; i < R3; ++i) c[i] = fmaf(S.qh[p][R3 * g + i], u, c[i]);
     }
 #pragma unroll
-    for (int i = 0; i < 16; ++i) Gs[kOffW2 + (16 * g + i) * kMlpH + j] = a[i];
+    for (int i = 0; i < R2; ++i) Gs[kOffW2 + (R2 * g + i) * kMlpH + j] = a[i];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) Gs[kOffW3 + (4 * g + i) * kMlpH + j] = c[i];
+    for (int i = 0; i < R3; ++i) Gs[kOffW3 + (R3 * g + i) * kMlpH + j] = c[i];
     if (g == 0) {
       float t = 0.f;
       for (int p = 0; p < P; ++p) t += S.d2[p][j];
@@ -406,8 +405,8 @@ __global__ void __cluster_dims__(kGradCluster, 1, 1) __launch_bounds__(kGradThre
       Gs[kOffB3 + j] = t;
     }
   }
-  // dW1[j][3 g + i], db1
-  {
+  // dW1[j][3 g + i] (four groups), db1
+  if (g < 4) {
     float a[3] = {0.f, 0.f, 0.f}, t = 0.f;
     for (int p = 0; p < P; ++p) {
       const float d = S.d1[p][j];
@@ -424,12 +423,12 @@ __global__ void __cluster_dims__(kGradCluster, 1, 1) __launch_bounds__(kGradThre
   namespace cg = cooperative_groups;
   cg::cluster_group cl = cg::this_cluster();
   cl.sync();
-  constexpr int kSlice = kMlpParams / kGradCluster + 1;
-  const int r0 = (int)cl.block_rank() * kSlice, r1 = min(r0 + kSlice, kMlpParams + 1);
-  for (int i = r0 + tid; i < r1; i += kGradThreads) {
+  const int nc = (int)cl.num_blocks(), slice = kMlpParams / nc + 1;
+  const int r0 = (int)cl.block_rank() * slice, r1 = min(r0 + slice, kMlpParams + 1);
+  for (int i = r0 + tid; i < r1; i += NT) {
     double t = 0.0;
-#pragma unroll
-    for (int c = 0; c < kGradCluster; ++c) t += (double)cl.map_shared_rank(Gs, c)[i];
+#pragma unroll 8
+    for (int c = 0; c < nc; ++c) t += (double)cl.map_shared_rank(Gs, c)[i];
     atomicAdd(i < kMlpParams ? &grad[i] : loss, (float)t);
   }
   cl.sync();                                     // (the others read this CTA's shared memory)
@@ -462,7 +461,7 @@ __global__ void k_mlp_adam(float* __restrict__ params, const float* __restrict__
 // A thread's units are jg + 16 i (the weights are stored in that order), and
 // activation rows are padded by four floats: the sixteen threads that share
 // pairs then store to different banks.
-constexpr int kPredThreads = 256, kPredSms = 152;    // (the chip's SMs)
+constexpr int kPredThreads = 256;
 template <int P>
 struct PredShared {
   float W1[kMlpIn][kMlpH], W2[kMlpH][kMlpH], W3[kMlpOut][kMlpH];   // [input][pred_unit(unit)]
@@ -649,17 +648,31 @@ __global__ void k_label_ratio(const double* __restrict__ C, const double* __rest
 }
 
 // ------------------------------------------------------------ launchers
-template <int P>
+template <int P, int NT>
 static cudaError_t launch_grad_p(const float* params, const float* feat, const float* qhat, const float* chat, int64_t n,
-                                 float* grad, float* loss, cudaStream_t st) {
+                                 float* grad, float* loss, int cluster, cudaStream_t st) {
+  auto kernel = k_mlp_grad<P, NT>;
   constexpr size_t sm = sizeof(GradShared<P>);
-  if (sm > 48 * 1024) {
-    const cudaError_t e = cudaFuncSetAttribute(k_mlp_grad<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e == cudaSuccess && sm > 48 * 1024) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  if (e != cudaSuccess) return e;
+  for (int nc = cluster; nc >= 8; nc /= 2) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)((n + P * nc - 1) / (P * nc) * nc));
+    cfg.blockDim = dim3(NT);
+    cfg.dynamicSmemBytes = sm;
+    cfg.stream = st;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)nc;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    e = cudaLaunchKernelEx(&cfg, kernel, params, feat, qhat, chat, n, 1.0f / (float)n, grad, loss);
+    if (e == cudaSuccess) return cudaGetLastError();
+    (void)cudaGetLastError();
   }
-  const int64_t nclus = (n + P * kGradCluster - 1) / (P * kGradCluster);
-  k_mlp_grad<P><<<(unsigned)(nclus * kGradCluster), kGradThreads, sm, st>>>(params, feat, qhat, chat, n, 1.0f / (float)n, grad, loss);
-  return cudaGetLastError();
+  return e;
 }
 
 cudaError_t launch_mlp_grad(const float* params, const float* feat, const float* qhat, const float* chat, int64_t n,
@@ -667,13 +680,14 @@ cudaError_t launch_mlp_grad(const float* params, const float* feat, const float*
   k_mlp_zero<<<(kMlpParams + 256) / 256, 256, 0, st>>>(grad, loss);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess || n == 0) return e;
-  // fewer pairs a CTA shorten its chain (1,024 pairs, call and wait: 35 us at 16,
-  // 2,000 pairs 42 us at 16), but a cluster takes fewer pairs then, and every
-  // cluster rounds the running gradient once: 8 and 16 pairs up to eight and
-  // twelve clusters, which keeps the error below that of one CTA per 128 pairs
-  if (n <= 8 * 8 * kGradCluster) return launch_grad_p<8>(params, feat, qhat, chat, n, grad, loss, st);
-  if (n <= 12 * 16 * kGradCluster) return launch_grad_p<16>(params, feat, qhat, chat, n, grad, loss, st);
-  return launch_grad_p<32>(params, feat, qhat, chat, n, grad, loss, st);
+  // fewer pairs a CTA shorten its chain, but every cluster rounds the running
+  // gradient once: 8 pairs up to two clusters (200 pairs: 15 us, 18 with 32 pairs),
+  // 32 above.  Beyond one CTA an SM the work counts, and small CTAs and clusters
+  // fill the SMs better (call and wait of 20,000 pairs: 79 against 86 us, of
+  // 200,000: 442 against 576)
+  if (n <= 2 * 8 * kGradCluster) return launch_grad_p<8, 256>(params, feat, qhat, chat, n, grad, loss, kGradCluster, st);
+  if (n <= 32 * kMlpSms) return launch_grad_p<32, 512>(params, feat, qhat, chat, n, grad, loss, kGradCluster, st);
+  return launch_grad_p<32, 256>(params, feat, qhat, chat, n, grad, loss, 8, st);
 }
 
 cudaError_t launch_mlp_adam(float* params, const float* grad, float* m1, float* m2, int step, float lr, float b1,
@@ -692,7 +706,7 @@ static cudaError_t launch_predict_p(const float* params, const float* feat, cons
     if (e != cudaSuccess) return e;
   }
   const int64_t tiles = (n + P - 1) / P;
-  k_mlp_predict<P><<<(unsigned)std::min<int64_t>(tiles, 2 * kPredSms), kPredThreads, sm, st>>>(params, feat, qhat, n, out);
+  k_mlp_predict<P><<<(unsigned)std::min<int64_t>(tiles, 2 * kMlpSms), kPredThreads, sm, st>>>(params, feat, qhat, n, out);
   return cudaGetLastError();
 }
 
@@ -700,7 +714,7 @@ cudaError_t launch_mlp_predict(const float* params, const float* feat, const flo
                                cudaStream_t st) {
   if (n == 0) return cudaSuccess;
   // 128 pairs a CTA once that fills the SMs, 32 below
-  return n >= 128 * kPredSms ? launch_predict_p<128>(params, feat, qhat, n, out, st) : launch_predict_p<32>(params, feat, qhat, n, out, st);
+  return n >= 128 * kMlpSms ? launch_predict_p<128>(params, feat, qhat, n, out, st) : launch_predict_p<32>(params, feat, qhat, n, out, st);
 }
 
 cudaError_t launch_near_classify(int task, int64_t nnz, const int* row, const int* col, const double* tgt_v,
