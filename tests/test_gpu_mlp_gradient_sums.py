@@ -13,7 +13,7 @@ def test_gradient_error(n, tol):
     """Against FP64 autograd, mean of five calls.  The rounding of the pairs' own
     values averages out (0.7e-7 of the norm at 1,024 pairs, less above, 1.5e-7 at a few hundred); what
     grows is the number of FP32 additions to a parameter's running sum, one per
-    128 to 256 pairs, each within half of 2^-24 of it: 1.8e-7 at 20,000 pairs.
+    128 to 512 pairs, each within half of 2^-24 of it: 1.8e-7 at 20,000 pairs.
     One addition per 8 to 32 pairs gives 1.7e-7 to 3.6e-7 from 1,024 pairs on."""
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
