@@ -111,8 +111,10 @@ template <typename T>
 __host__ __device__ constexpr int taylor_parts(int q) { return sizeof(T) == 4 ? (q <= kTaylorRegQ ? 1 : 4) : (q < 6 ? 1 : q - 4); }
 constexpr int kTaylorWarps = 4;       // warps per CTA
 constexpr int kTaylorStageRows = 22;  // 18 g rows + 4 moment rows
+// (one stage where two leave an SM a single CTA: FP32 order 8, every level of the
+// level-2 ball, VtV 209 us against 230)
 template <typename T>
-constexpr int taylor_stages(int q) { return sizeof(T) == 8 && q >= 7 ? 1 : 2; }
+constexpr int taylor_stages(int q) { return q >= 8 || (sizeof(T) == 8 && q >= 7) ? 1 : 2; }
 template <typename T>
 size_t taylor_smem(int q) {
   return sizeof(T) * (size_t)kTaylorWarps * taylor_stages<T>(q) * kTaylorStageRows * taylor_row<T>(q);
@@ -134,7 +136,8 @@ size_t taylor_smem(int q) {
 // for the three arrays.  Potentials of sources far away (level-3 ball, order 8)
 // against the FP64 form: 1.85e-7 with plain sums over a chunk, 1.38e-7 with one CTA
 // per target, 1.20e-7 now; VtV of the level-2 ball with order 8 on every level takes
-// 239 us (200 with plain sums, 3.1 ms with one CTA per target).
+// 209 us (194 with plain sums, 3.1 ms with one CTA per target); three, five or six
+// passes take 223, 213 and 225.
 template <typename T, int Q, int NP>
 __global__ void __launch_bounds__(kTaylorWarps * 32) k_m2l_taylor(TaylorArgs<T> A) {
   constexpr int NQ = (Q + 1) * (Q + 2) * (Q + 3) / 6;
